@@ -250,7 +250,11 @@ int lbm_set_state(lbm_t h, const void *src_host, long long t);
  * walks adapt the tile height at launch to the resident warps: fewer rows
  * (down to 2) when the grid has too few tiles to occupy them, more (up to
  * 32) when its tiles need between one and two waves; lbm_get_config reports
- * the configured 16. */
+ * the configured 16.  In the default configuration, and after lbm_tune where
+ * it measured faster, step calls on large grids (nx a multiple of 4 in FP32, of
+ * 8 in 16-bit storage) take two steps per launch, an odd last step alone;
+ * bitwise the same.  A configuration or pipeline set by the caller steps once
+ * per launch. */
 int lbm_set_config(lbm_t h, int vec, int rows, int warps);
 int lbm_get_config(lbm_t h, int *vec, int *rows, int *warps);
 

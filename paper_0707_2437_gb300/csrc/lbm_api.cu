@@ -143,7 +143,6 @@ static void drop_graphs(lbm_grid *h) {
             cudaGraphExecDestroy(h->graph[k]);
             h->graph[k] = nullptr;
         }
-    h->graph_pairs = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -282,6 +281,7 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double c2, double rho0,
     // on the legacy default stream.
     if (e == cudaSuccess) e = cudaMemsetAsync(h->scratch, 0, sizeof(double) * 16, h->stream);
     if (e == cudaSuccess) e = prepare_step(storage, h->cfg);
+    if (e == cudaSuccess) e = plan_step2(storage, 0, false, nx, ny, &h->step2);
     if (e == cudaSuccess) e = cudaMallocHost(&h->host_out, sizeof(double) * 8);
     if (e == cudaSuccess) e = cudaEventCreate(&h->ev[0]);
     if (e == cudaSuccess) e = cudaEventCreate(&h->ev[1]);
@@ -380,28 +380,42 @@ static cudaError_t launch_drive(lbm_grid *h, void *out, const uint32_t *tdev, ui
                           h->drive_period, tdev, toff, st);
 }
 
-// One step launch from buf[cur] to buf[cur ^ 1] (no bookkeeping), followed
-// by the boundary columns when the channel is driven.
-static cudaError_t launch_one(lbm_grid *h, int from) {
+// One step launch from buf[from] to buf[from ^ 1] (no bookkeeping), followed
+// by the boundary columns when the channel is driven.  The step number is
+// *tdev + toff (tdev may be NULL).
+static cudaError_t launch_one(lbm_grid *h, int from, const uint32_t *tdev, uint32_t toff,
+                              cudaStream_t st) {
     cudaError_t e =
         h->grad == LBM_GRAD_FORWARD
             ? launch_step_forward(h->cfg, h->buf[from], h->buf[from ^ 1], h->nx, h->ny, h->P,
-                                  h->coef, h->stream)
+                                  h->coef, st)
             : launch_step(h->storage, h->cfg, h->buf[from], h->buf[from ^ 1], h->nx, h->ny, h->P,
-                          h->coef, status_ptr(h), h->rounding, nullptr, (uint32_t)h->t, h->a15f,
-                          h->stream);
-    if (e == cudaSuccess && h->drive)
-        e = launch_drive(h, h->buf[from ^ 1], nullptr, (uint32_t)h->t, h->stream);
+                          h->coef, status_ptr(h), h->rounding, tdev, toff, h->a15f, st);
+    if (e == cudaSuccess && h->drive) e = launch_drive(h, h->buf[from ^ 1], tdev, toff, st);
     return e;
 }
+static cudaError_t launch_one(lbm_grid *h, int from) {
+    return launch_one(h, from, nullptr, (uint32_t)h->t, h->stream);
+}
 
-static const int kGraphPairs = 16;   // a graph holds 32 steps
+// Whether step calls take two steps per launch.
+static bool steps_in_pairs(const lbm_grid *h) {
+    return h->pairs && h->step2.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL;
+}
+
+// One launch of two steps from buf[from] to buf[from ^ 1].
+static cudaError_t launch_two(lbm_grid *h, int from, const uint32_t *tdev, uint32_t toff,
+                              cudaStream_t st) {
+    return launch_step2(h->step2, h->storage, h->buf[from], h->buf[from ^ 1], h->nx, h->ny, h->P,
+                        h->coef, h->rounding, tdev, toff, h->a15f, st);
+}
+
+static const int kGraphLaunches = 32;  // launches in a graph, an even number
 static const long long kPersistentMin = 64;  // persistent launch from this many steps
 // ... or from kPersistentMinLarge steps on grids of at least kLargeSites sites,
 // where a step is long enough that the launch's barrier costs little.
 static const long long kPersistentMinLarge = 8;
 static const long long kLargeSites = 1LL << 20;
-static const long long kGraphMin = 8; // use graphs from this many steps on
 // LBM_PERSISTENT_AUTO steps every grid with the step kernel (except slabs):
 // per step over 256- and 1024-step calls it was the faster for FP32 grids from
 // 64^2 to 8192^2 (2048^2 49.6 us against 52.2 persistent, 64^2 3.5 against
@@ -409,39 +423,29 @@ static const long long kGraphMin = 8; // use graphs from this many steps on
 // 30.8, 8192^2 372.7 against 384.8) and with a c2 field (4096^2 FP16-delta
 // 125.7 against 131.2).
 
-static int build_graphs(lbm_grid *h) {
-    drop_graphs(h);
+// The graph of kGraphLaunches step launches starting from buf[start].
+static int build_graph(lbm_grid *h, int start) {
     cudaStream_t cs;
     CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    for (int start = 0; start < 2; ++start) {
-        cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            for (int k = 0; k < 2 * kGraphPairs && e == cudaSuccess; ++k) {
-                e = h->grad == LBM_GRAD_FORWARD
-                        ? launch_step_forward(h->cfg, h->buf[(start + k) & 1],
-                                              h->buf[(start + k + 1) & 1], h->nx, h->ny, h->P,
-                                              h->coef, cs)
-                        : launch_step(h->storage, h->cfg, h->buf[(start + k) & 1],
-                                      h->buf[(start + k + 1) & 1], h->nx, h->ny, h->P, h->coef,
-                                      status_ptr(h), h->rounding, step_ptr(h), (uint32_t)k,
-                                      h->a15f, cs);
-                if (e == cudaSuccess && h->drive)
-                    e = launch_drive(h, h->buf[(start + k + 1) & 1], step_ptr(h), (uint32_t)k, cs);
-            }
-            cudaError_t e2 = cudaStreamEndCapture(cs, &g);
-            if (e == cudaSuccess) e = e2;
+    const bool two = steps_in_pairs(h);
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (int k = 0; k < kGraphLaunches && e == cudaSuccess; ++k) {
+            const int from = (start + k) & 1;
+            e = two ? launch_two(h, from, step_ptr(h), 2u * k, cs)
+                    : launch_one(h, from, step_ptr(h), (uint32_t)k, cs);
         }
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&h->graph[start], g, 0);
-        if (g) cudaGraphDestroy(g);
-        if (e != cudaSuccess) {
-            cudaStreamDestroy(cs);
-            drop_graphs(h);
-            return cuda_fail(e, "lbm_step: graph capture");
-        }
+        cudaError_t e2 = cudaStreamEndCapture(cs, &g);
+        if (e == cudaSuccess) e = e2;
     }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&h->graph[start], g, 0);
+    if (g) cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
-    h->graph_pairs = kGraphPairs;
+    if (e != cudaSuccess) {
+        h->graph[start] = nullptr;
+        return cuda_fail(e, "lbm_step: graph capture");
+    }
     return LBM_OK;
 }
 
@@ -486,25 +490,27 @@ extern "C" int lbm_step(lbm_t h, long long n) {
         }
         return lbm_batch_step(h->self_batch, n, nullptr);  // advances t and cur
     }
-    if (n >= kGraphMin) {
-        if (!h->graph_pairs) {
-            int rc = build_graphs(h);
+    const bool two = steps_in_pairs(h);
+    const long long per = (two ? 2LL : 1LL) * kGraphLaunches;
+    while (n >= per) {
+        if (!h->graph[h->cur]) {
+            int rc = build_graph(h, h->cur);
             if (rc != LBM_OK) return rc;
         }
-        long long per = 2LL * h->graph_pairs;
-        while (n >= per) {
-            if (h->rounding || h->drive)
-                CK(launch_set_u32(step_ptr(h), (uint32_t)h->t, h->stream));
-            CK(cudaGraphLaunch(h->graph[h->cur], h->stream));
-            n -= per;
-            h->t += per;  // an even number of steps leaves cur unchanged
-        }
+        if (h->rounding || h->drive)
+            CK(launch_set_u32(step_ptr(h), (uint32_t)h->t, h->stream));
+        CK(cudaGraphLaunch(h->graph[h->cur], h->stream));
+        n -= per;
+        h->t += per;  // an even number of launches leaves cur unchanged
     }
-    for (long long k = 0; k < n; ++k) {
-        cudaError_t e = launch_one(h, h->cur);
+    while (n > 0) {
+        const int took = two && n >= 2 ? 2 : 1;
+        cudaError_t e = took == 2 ? launch_two(h, h->cur, nullptr, (uint32_t)h->t, h->stream)
+                                  : launch_one(h, h->cur);
         if (e != cudaSuccess) return cuda_fail(e, "lbm_step kernel");
         h->cur ^= 1;
-        h->t += 1;
+        h->t += took;
+        n -= took;
     }
     return LBM_OK;
 }
@@ -655,6 +661,13 @@ extern "C" int lbm_set_state(lbm_t h, const void *src_host, long long t) {
 // ---------------------------------------------------------------------------
 // Tile configuration and autotuner.
 
+// A configuration of the caller's describes single-step launches; the tuner
+// turns pairs of steps back on where they are the faster.
+static void set_pairs(lbm_grid *h, bool on) {
+    if (h->pairs != on) drop_graphs(h);
+    h->pairs = on;
+}
+
 extern "C" int lbm_set_config(lbm_t h, int vec, int rows, int warps) {
     if (!h) return fail(LBM_EINVAL, "lbm_set_config: NULL handle");
     if (!valid_vec(h->storage, h->nx, vec))
@@ -674,6 +687,7 @@ extern "C" int lbm_set_config(lbm_t h, int vec, int rows, int warps) {
     h->cfg.rows = rows;
     h->cfg.warps = warps;
     h->cfg.fit_rows = false;
+    set_pairs(h, false);
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }
@@ -689,6 +703,7 @@ extern "C" int lbm_set_pipeline(lbm_t h, int stages) {
         drop_graphs(h);
     }
     h->cfg.stages = stages;
+    set_pairs(h, false);
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }
@@ -701,6 +716,7 @@ extern "C" int lbm_set_c2_field(lbm_t h, const double *c2, int on_device) {
     if (!c2) {
         if (h->a15f) cudaFree(h->a15f);
         h->a15f = nullptr;
+        CK(plan_step2(h->storage, h->rounding, false, h->nx, h->ny, &h->step2));
         return LBM_OK;
     }
     if (h->rounding) return fail(LBM_EINVAL, "lbm_set_c2_field: needs nearest rounding");
@@ -718,6 +734,7 @@ extern "C" int lbm_set_c2_field(lbm_t h, const double *c2, int on_device) {
     }
     if (h->cfg.stages >= 2) h->cfg.stages = 0;
     if (!h->a15f) CK(cudaMalloc(&h->a15f, n * sizeof(float)));
+    CK(plan_step2(h->storage, h->rounding, true, h->nx, h->ny, &h->step2));
     std::vector<double *> owned;
     double *d = nullptr;
     int rc = stage_field(h, c2, on_device, h->stream, &d, owned);
@@ -772,6 +789,7 @@ extern "C" int lbm_set_rounding(lbm_t h, int mode) {
         }
         if (h->cfg.stages >= 2) h->cfg.stages = 0;
     }
+    CK(plan_step2(h->storage, h->rounding, h->a15f != nullptr, h->nx, h->ny, &h->step2));
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }
@@ -830,9 +848,14 @@ static std::string tune_key(const lbm_grid *h) {
     return k.str();
 }
 
-// The cache file is a flat JSON object {"key": [vec, rows, warps, stages], ...}.
-static std::map<std::string, TileCfg> read_cache(const char *path) {
-    std::map<std::string, TileCfg> m;
+// The cache file is a flat JSON object {"key": [vec, rows, warps, stages, pairs],
+// ...}; files without the fifth number mean 0.
+struct Tuned {
+    TileCfg cfg;
+    int pairs = 0;  // 1: step calls run faster two steps per launch
+};
+static std::map<std::string, Tuned> read_cache(const char *path) {
+    std::map<std::string, Tuned> m;
     std::ifstream in(path);
     if (!in) return m;
     std::stringstream ss;
@@ -845,41 +868,50 @@ static std::map<std::string, TileCfg> read_cache(const char *path) {
         std::string key = s.substr(pos + 1, end - pos - 1);
         size_t lb = s.find('[', end), rb = s.find(']', end);
         if (lb == std::string::npos || rb == std::string::npos) break;
-        TileCfg c;
-        if (sscanf(s.c_str() + lb, "[%d , %d , %d , %d]", &c.vec, &c.rows, &c.warps, &c.stages) ==
-                4 ||
-            sscanf(s.c_str() + lb, "[%d,%d,%d,%d]", &c.vec, &c.rows, &c.warps, &c.stages) == 4)
-            m[key] = c;
+        Tuned t;
+        TileCfg &c = t.cfg;
+        if (sscanf(s.c_str() + lb, "[%d , %d , %d , %d , %d", &c.vec, &c.rows, &c.warps,
+                   &c.stages, &t.pairs) >= 4)
+            m[key] = t;
         pos = rb + 1;
     }
     return m;
 }
 
-static void write_cache(const char *path, const std::map<std::string, TileCfg> &m) {
+static void write_cache(const char *path, const std::map<std::string, Tuned> &m) {
     std::string tmp = std::string(path) + ".tmp";
     FILE *f = fopen(tmp.c_str(), "w");
     if (!f) return;
     fprintf(f, "{\n");
     size_t k = 0;
     for (auto &kv : m) {
-        fprintf(f, "  \"%s\": [%d, %d, %d, %d]%s\n", kv.first.c_str(), kv.second.vec,
-                kv.second.rows, kv.second.warps, kv.second.stages, (++k < m.size()) ? "," : "");
+        const TileCfg &c = kv.second.cfg;
+        fprintf(f, "  \"%s\": [%d, %d, %d, %d, %d]%s\n", kv.first.c_str(), c.vec, c.rows, c.warps,
+                c.stages, kv.second.pairs, (++k < m.size()) ? "," : "");
     }
     fprintf(f, "}\n");
     fclose(f);
     rename(tmp.c_str(), path);
 }
 
-// Times one configuration: `reps` launches from buf[cur] into the other buffer
-// (the state itself is not changed).
-static int time_cfg(lbm_grid *h, const TileCfg &c, int reps, float *ms_out) {
+// Times `reps` launches from buf[cur] into the other buffer (the state itself
+// is not changed): single steps under configuration c, or (c NULL) two steps
+// per launch.
+static int time_cfg(lbm_grid *h, const TileCfg *c, int reps, float *ms_out) {
     TileCfg saved = h->cfg;
-    h->cfg = c;
-    h->cfg.fit_rows = false;  // time the candidate's own tile height
-    cudaError_t e = prepare_step(h->storage, c);
-    if (e == cudaSuccess) e = launch_one(h, h->cur);  // warm-up
+    cudaError_t e = cudaSuccess;
+    if (c) {
+        h->cfg = *c;
+        h->cfg.fit_rows = false;  // time the candidate's own tile height
+        e = prepare_step(h->storage, *c);
+    }
+    auto launch = [&] {
+        return c ? launch_one(h, h->cur)
+                 : launch_two(h, h->cur, nullptr, (uint32_t)h->t, h->stream);
+    };
+    if (e == cudaSuccess) e = launch();  // warm-up
     if (e == cudaSuccess) e = cudaEventRecord(h->ev[0], h->stream);
-    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_one(h, h->cur);
+    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch();
     if (e == cudaSuccess) e = cudaEventRecord(h->ev[1], h->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(h->ev[1]);
     float ms = 0.f;
@@ -893,14 +925,16 @@ static int time_cfg(lbm_grid *h, const TileCfg &c, int reps, float *ms_out) {
 extern "C" int lbm_tune(lbm_t h, const char *cache_path) {
     if (!h) return fail(LBM_EINVAL, "lbm_tune: NULL handle");
     std::string key = tune_key(h);
-    std::map<std::string, TileCfg> cache;
+    std::map<std::string, Tuned> cache;
     if (cache_path) {
         cache = read_cache(cache_path);
         auto it = cache.find(key);
-        if (it != cache.end() && valid_vec(h->storage, h->nx, it->second.vec)) {
-            int rc = lbm_set_config(h, it->second.vec, it->second.rows, it->second.warps);
-            if (rc != LBM_OK) return rc;
-            return lbm_set_pipeline(h, it->second.stages);
+        if (it != cache.end() && valid_vec(h->storage, h->nx, it->second.cfg.vec)) {
+            const TileCfg &c = it->second.cfg;
+            int rc = lbm_set_config(h, c.vec, c.rows, c.warps);
+            if (rc == LBM_OK) rc = lbm_set_pipeline(h, c.stages);
+            if (rc == LBM_OK) set_pairs(h, it->second.pairs != 0);
+            return rc;
         }
     }
     CK(cudaStreamSynchronize(h->stream));
@@ -929,7 +963,7 @@ extern "C" int lbm_tune(lbm_t h, const char *cache_path) {
                     c.warps = w;
                     c.stages = nst;
                     float ms;
-                    int rc = time_cfg(h, c, reps, &ms);
+                    int rc = time_cfg(h, &c, reps, &ms);
                     if (rc != LBM_OK) return rc;
                     if (ms < best_ms) {
                         best_ms = ms;
@@ -942,8 +976,16 @@ extern "C" int lbm_tune(lbm_t h, const char *cache_path) {
     int rc = lbm_set_config(h, best.vec, best.rows, best.warps);
     if (rc == LBM_OK) rc = lbm_set_pipeline(h, best.stages);
     if (rc != LBM_OK) return rc;
+    bool pairs = false;
+    if (h->step2.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL) {
+        float ms;
+        rc = time_cfg(h, nullptr, reps, &ms);
+        if (rc != LBM_OK) return rc;
+        pairs = ms < 2 * best_ms;
+    }
+    set_pairs(h, pairs);
     if (cache_path) {
-        cache[key] = best;
+        cache[key] = Tuned{best, pairs ? 1 : 0};
         write_cache(cache_path, cache);
     }
     return LBM_OK;

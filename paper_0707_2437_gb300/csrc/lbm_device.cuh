@@ -406,11 +406,10 @@ struct SiteQ {
     float Ax, Ay;          // 3 j/tau + 3 alpha grad(rho)
 };
 
-// dr: drho at the site; dxm/dxp, dym/dyp: drho at x -/+ 1 and y -/+ 1.
+// dr: drho at the site; gx, gy: drho(x + 1) - drho(x - 1) and the same in y.
 __device__ __forceinline__ SiteQ site_quantities(float h1, float h2, float h3, float h4, float h5,
-                                                 float h6, float h7, float h8, float dr, float dxm,
-                                                 float dxp, float dym, float dyp, const Coef &c,
-                                                 float a15) {
+                                                 float h6, float h7, float h8, float dr, float gx,
+                                                 float gy, const Coef &c, float a15) {
     SiteQ q;
     float a = __fsub_rn(h5, h7);  // e_5 = (1, 1), e_7 = -e_5
     float b = __fsub_rn(h6, h8);  // e_6 = (-1, 1), e_8 = -e_6
@@ -422,8 +421,8 @@ __device__ __forceinline__ SiteQ site_quantities(float h1, float h2, float h3, f
     float ju = __fmaf_rn(q.jx, q.ux, __fmul_rn(q.jy, q.uy));
     q.wB = __fmul_rn(c.om, __fmaf_rn(-1.5f, ju, dr));
     // Central differences of Section 4: grad = (d(+1) - d(-1))/2; the 1/2 is in a15.
-    q.Ax = __fmaf_rn(c.w3, q.jx, __fmaf_rn(c.w3lo, q.jx, __fmul_rn(a15, __fsub_rn(dxp, dxm))));
-    q.Ay = __fmaf_rn(c.w3, q.jy, __fmaf_rn(c.w3lo, q.jy, __fmul_rn(a15, __fsub_rn(dyp, dym))));
+    q.Ax = __fmaf_rn(c.w3, q.jx, __fmaf_rn(c.w3lo, q.jx, __fmul_rn(a15, gx)));
+    q.Ay = __fmaf_rn(c.w3, q.jy, __fmaf_rn(c.w3lo, q.jy, __fmul_rn(a15, gy)));
     return q;
 }
 
@@ -775,10 +774,11 @@ struct Walker {
                 const float dxm = GR ? d[v] : ((v == 0) ? lft : d[v - 1]);
                 const float dxp = (v == V - 1) ? rgt : d[v + 1];
                 float *hs = h[s];
+                const float dy0 = GR ? d[v] : (swap_y ? dyp[v] : dym[v]);
+                const float dy1 = swap_y ? dym[v] : dyp[v];
                 const SiteQ q = site_quantities(hs[1], hs[2], hs[3], hs[4], hs[5], hs[6], hs[7],
-                                                hs[8], d[v], dxm, dxp,
-                                                GR ? d[v] : (swap_y ? dyp[v] : dym[v]),
-                                                swap_y ? dym[v] : dyp[v], c,
+                                                hs[8], d[v], __fsub_rn(dxp, dxm),
+                                                __fsub_rn(dy1, dy0), c,
                                                 GR ? __fmul_rn(2.f, a15v[v]) : a15v[v]);
                 float o[9];
                 o[0] = __fmaf_rn(c.om1, hs[0], q.wB);                           // rest

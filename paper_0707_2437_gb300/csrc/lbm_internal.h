@@ -73,6 +73,22 @@ Coef make_coef(double tau, double c2, double rho0);
 Err launch_step(int storage, const TileCfg &cfg, const void *fin, void *fout, int nx, int ny,
                 size_t P, const Coef &c, int *status, int rnd, const uint32_t *tdev, uint32_t toff,
                 const float *a15f, cudaStream_t st);
+// Warps of `fn` (blocks of `warps` warps, `smem` bytes of dynamic shared memory)
+// resident on the current device; 0 if the query fails.
+long long resident_warps(const void *fn, int warps, int smem);
+// Two steps per launch (lbm_step2.cu): the tiles of a grid's passes, and one
+// launch.  ok is false where the fused walk does not apply (nx not a multiple
+// of its 16-byte lanes).  Uniform alpha with either rounding, or a c2 field
+// with nearest rounding.
+struct Step2Plan {
+    bool ok = false;
+    int rows = 0, nstrips = 0;
+    long long ntiles = 0;
+};
+Err plan_step2(int storage, int rnd, bool field, int nx, int ny, Step2Plan *out);
+Err launch_step2(const Step2Plan &p, int storage, const void *fin, void *fout, int nx, int ny,
+                 size_t P, const Coef &c, int rnd, const uint32_t *tdev, uint32_t toff,
+                 const float *a15f, cudaStream_t st);
 // The forward-difference gradient (lbm_set_gradient): FP32, one site per lane.
 Err launch_step_forward(const TileCfg &cfg, const void *fin, void *fout, int nx, int ny, size_t P,
                         const Coef &c, cudaStream_t st);
@@ -117,6 +133,10 @@ struct lbm_grid {
     int device = 0;
     vss::Coef coef{};
     vss::TileCfg cfg{};
+    // Two steps per launch: the plan for the grid as configured, and whether
+    // step calls may use it (not under a tile configuration of the caller's).
+    vss::Step2Plan step2{};
+    bool pairs = true;
     int rounding = 0;             // 1: stochastic rounding of 16-bit stores
     float *a15f = nullptr;        // spatially varying alpha: 1.5 alpha per site
     int grad = 0;                 // LBM_GRAD_CENTRAL or LBM_GRAD_FORWARD
@@ -129,9 +149,8 @@ struct lbm_grid {
     double drive_amp = 0, drive_period = 0;
     double *scratch = nullptr;    // reduction partials + results
     double *host_out = nullptr;   // pinned, 8 doubles
-    // CUDA graphs of 2*graph_pairs steps starting from buffer 0 or buffer 1
+    // CUDA graphs of a fixed number of step launches starting from buffer 0 or 1
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
-    int graph_pairs = 0;
     // Long step calls run as one persistent launch through a batch holding
     // only this grid (created on first use, dropped when the tiling changes).
     int persistent = LBM_PERSISTENT_AUTO;

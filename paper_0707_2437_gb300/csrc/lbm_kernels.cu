@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "lbm_internal.h"
+#include "lbm_launch.cuh"
 
 namespace vss {
 
@@ -39,35 +40,6 @@ bool valid_vec(int storage, int nx, int vec) {
     if (vec != 1 && vec != 2 && vec != 4 && vec != 8) return false;
     if (vec == 8 && storage == ST_F32) return false;
     return nx % vec == 0;
-}
-
-// ---------------------------------------------------------------------------
-// Programmatic dependent launch.  The single-grid step kernels are launched
-// with programmatic stream serialization allowed: each block first lets the next launch on the stream
-// start (the next grid is launched once every block of this one has started
-// or exited, so its blocks only take SM slots this grid no longer needs), then
-// waits until the previous grid has completed and its memory is visible, and
-// only then touches global memory.  The next step's launch latency is thereby
-// hidden behind this step's tail.
-__device__ __forceinline__ void pdl_enter() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block,
-                              size_t smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 // ---------------------------------------------------------------------------
@@ -169,8 +141,9 @@ __global__ void __launch_bounds__(256, 2)
 }
 
 // Resident warps of a step kernel with blocks of `warps` warps on the
-// current device, found once per kernel, block size and device.
-static long long resident_warps(const void *fn, int warps) {
+// current device, found once per kernel, block size and device (a kernel is
+// always asked about with the same dynamic shared memory).
+long long resident_warps(const void *fn, int warps, int smem) {
     struct Entry {
         const void *fn;
         int warps, dev;
@@ -186,7 +159,7 @@ static long long resident_warps(const void *fn, int warps) {
             if (e.fn == fn && e.warps == warps && e.dev == dev) return e.w;
     }
     int blocks = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, 32 * warps, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, 32 * warps, smem) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return 0;
     const long long w = (long long)blocks * warps * sms;
@@ -214,7 +187,7 @@ static long long resident_warps(const void *fn, int warps) {
 // took a whole 16-row walk (31 and 25 us per launch for 512 tiles).
 static TileCfg fit_tile(const TileCfg &cfg, const void *fn, int nx, int ny) {
     if (!cfg.fit_rows) return cfg;
-    const long long wave = resident_warps(fn, cfg.warps);
+    const long long wave = resident_warps(fn, cfg.warps, 0);
     if (wave <= 0) return cfg;
     const long long nstrips = (nx + 32LL * cfg.vec - 1) / (32LL * cfg.vec);
     auto tiles = [&](int r) { return nstrips * ((ny + r - 1) / r); };

@@ -1,0 +1,40 @@
+"""Step calls that take two steps per launch (large grids) leave bit for bit
+the state of single-step calls: the fused walk repeats the single walk's
+operations in order, so nothing but equality is accepted.  The shapes put the
+strips' edges everywhere: one strip narrower than a lane pair, a last strip of
+one lane, whole strips, wrapped halo columns, short last segments of odd and
+even grids, and step counts that mix graphs, pairs and a last single step."""
+import numpy as np
+import pytest
+
+from paper_0707_2437_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+
+# (nx, ny): tiles tall enough that pairs are taken (FP32 strips of 120 columns,
+# 16-bit strips of 240).
+SHAPES = {"f32": [(4, 20011), (124, 9803), (1000, 1201), (2048, 1025)],
+          "16": [(8, 30011), (248, 15003), (1200, 2407), (2048, 3077)]}
+
+
+def _state(lbm, kind, nx, ny, calls, lens):
+    with lbm.Grid(nx, ny, 0.7, 0.2, kind.replace("-sr", "")) as g:
+        if kind.endswith("-sr"):
+            g.set_rounding("stochastic")
+        if lens:
+            g.set_c2_field(workloads.c2_lens(nx, ny, 0.2))
+        g.init(*workloads.fourier_modes(nx, ny, amp=1e-2, seed=nx + ny))
+        for n in calls:
+            g.step(n)
+        assert g.t == sum(calls)
+        return g.get_state()[0]
+
+
+@pytest.mark.parametrize("kind,lens", [("f32", False), ("f32", True), ("f16d", False),
+                                       ("bf16d", True), ("f16d-sr", False), ("bf16d-sr", False)])
+@pytest.mark.parametrize("shape", range(4))
+def test_pairs_of_steps_equal_single_steps(lbm, kind, lens, shape):
+    nx, ny = SHAPES["f32" if kind == "f32" else "16"][shape]
+    single = _state(lbm, kind, nx, ny, [1] * 77, lens)
+    pairs = _state(lbm, kind, nx, ny, [2, 71, 1, 3], lens)
+    assert np.array_equal(single, pairs)
