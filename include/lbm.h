@@ -352,11 +352,13 @@ int lbm_batch_sync(lbm_batch_t b);
  * and the error returned).  Until one of them is called, a lockstep batch
  * whose tiles at 16 rows would fill less than 3/4 of the resident warps
  * (16 per SM) takes shorter tiles, down to 2 rows, as many as those warps
- * hold. */
+ * hold, and kind groups whose walk takes two steps per pass over memory (FP32
+ * grids with nx a multiple of 4, 16-bit grids under LBM_WALK16_AUTO with nx a
+ * multiple of 8, unless their tiles are paired; slabs never) get the height
+ * that balances their tiles over the resident warps.  The tuner times those too. */
 int lbm_batch_set_config(lbm_batch_t b, int rows, int blocks_per_sm);
 int lbm_batch_tune(lbm_batch_t b);
-/* Current tile height (of the lockstep work-list as built), resident blocks
- * per SM of the first kind group, and whether every kind group runs a
+/* Tile height and resident blocks per SM of the first kind group as built, and whether every kind group runs a
  * specialised kernel rather than the general one. */
 int lbm_batch_get_config(lbm_batch_t b, int *rows, int *blocks_per_sm, int *specialised);
 /* The work-list as last built (at creation, by a configuration, schedule or

@@ -30,7 +30,6 @@ struct lbm_batch {
     int device = 0;
     int rows = 16;
     bool fit_rows = true;   // default: lockstep work-lists may use shorter tiles
-    int lock_rows = 16;     // tile height of the lockstep work-list as built
     int blocks_per_sm = 0;  // 0: the occupancy limit
     // Kind groups: consecutive ranges of the tile list, each run by its own
     // persistent launch (a specialised k_batch_one, or k_batch for the rest),
@@ -39,6 +38,9 @@ struct lbm_batch {
         int begin = 0, count = 0;
         BatchKernel kernel = nullptr;
         FlowKernel fkernel = nullptr;  // flow schedule
+        int smem = 0;                  // dynamic shared memory per block
+        bool pairs = false;            // two steps per pass (the fused walk)
+        int rows = 0;                  // tile height
         int max_blocks_per_sm = 1;
     };
     std::vector<Group> groups;
@@ -87,6 +89,8 @@ struct lbm_batch {
     int *h_nwork = nullptr;
     // Paired tiles (split walk) in the lockstep work-list.
     int paired = 0;
+    // Per grid, whether its passes take two steps (as of the work-list).
+    std::vector<char> pairs;
 };
 
 static int bfail(int code, const std::string &m) {
@@ -144,51 +148,57 @@ static int upload_worklist(lbm_batch *b, const std::vector<GridDesc> &gd,
     return LBM_OK;
 }
 
+// Dynamic shared memory and resident blocks of a kernel of this file.
+static cudaError_t resident_blocks(const void *fn, int smem, int *blocks) {
+    cudaError_t e = cudaSuccess;
+    if (smem)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, 32 * kBatchWarps, smem);
+    return e;
+}
+
+// Tile height of a lockstep group on the fused walk, from the grids' strips and
+// rows: a tile of r rows costs about r + 5 row steps (two rows of the first
+// step's collision and three pulled rows at each end).  With tiles of one
+// height a pass lasts ceil(tiles / warps) of them; in general the warps, which
+// take tiles as they finish others, are done within the mean plus one tile.
+// The lower of both bounds decides.  FP32 passes are bound by HBM and run
+// faster while the tiles in flight lie close together: at most 64 rows.
+static int pair_rows(const std::vector<std::pair<int, int>> &grids, long long warps, int most) {
+    double best = 0;
+    int rows = 2;
+    for (int r = 2; r <= most; r += r < 64 ? 1 : 4) {
+        long long tiles = 0, work = 0;
+        int tallest = 0;
+        for (const auto &g : grids) {  // (strips, rows)
+            const long long segs = (g.second + r - 1) / r;
+            tiles += g.first * segs;
+            work += g.first * (g.second + 5 * segs);
+            tallest = std::max(tallest, std::min(r, g.second));
+        }
+        const double even = (double)((tiles + warps - 1) / warps) * (tallest + 5);
+        const double mixed = (double)work / warps + (tallest + 5);
+        const double cost = std::min(even, mixed);
+        if (r == 2 || cost < best) {
+            best = cost;
+            rows = r;
+        }
+        if (tallest < r) break;  // every grid is one segment
+    }
+    return rows;
+}
+
 // (Re)builds the device grid table and the tile work-list.
 static int build_worklist(lbm_batch *b) {
-    std::vector<GridDesc> gd(b->grids.size());
+    const size_t ng = b->grids.size();
+    std::vector<GridDesc> gd(ng);
     std::vector<Tile> tiles;
     b->paired = 0;
-    // Flow schedule: the kernel for the grids' kinds and the warps it keeps
-    // resident, which set each grid's tile height below.
-    FlowKernel fk = nullptr;
-    int flow_bps = 1;
-    long long flow_warps = 0;
-    if (b->schedule == LBM_SCHEDULE_FLOW) {
-        std::vector<int> kinds;
-        for (const lbm_grid *g : b->grids)
-            kinds.push_back(kind_code(g->storage, batch_vec(b, g), g->rounding ? 1 : 0,
-                                      g->a15f ? 1 : 0));
-        fk = flow_kernel_for(kinds, b->walk16);
-        BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&flow_bps, (const void *)fk,
-                                                          32 * kBatchWarps, 0));
-        if (flow_bps < 1) return bfail(LBM_ECUDA, "flow kernel cannot be resident");
-        const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, flow_bps) : flow_bps;
-        flow_warps = (long long)per * b->sms * kBatchWarps;
-    }
-    // Lockstep, default configuration: every warp walks its tiles one after
-    // another within a step, so a batch with fewer tiles than about the
-    // resident warps (16 per SM in the specialised kernels) spends each step
-    // on a whole walk with warps idle.  Such a batch gets shorter tiles, down
-    // to 2 rows, as many as one wave holds.  Batches of at least 3/4 of a
-    // wave of tiles keep the configured height.
-    int lock_rows = b->rows;
-    if (b->schedule == LBM_SCHEDULE_LOCKSTEP && b->fit_rows) {
-        const int bps = b->blocks_per_sm > 0 ? b->blocks_per_sm : 4;
-        const long long wave = (long long)bps * b->sms * kBatchWarps;
-        auto tiles_at = [&](int r) {
-            long long t = 0;
-            for (const lbm_grid *g : b->grids) {
-                const int w = 32 * batch_vec(b, g);
-                t += (long long)((g->nx + w - 1) / w) * ((g->ny - 2 * g->slab + r - 1) / r);
-            }
-            return t;
-        };
-        if (4 * tiles_at(lock_rows) < 3 * wave)
-            while (lock_rows > 2 && tiles_at(lock_rows - 1) <= wave) --lock_rows;
-    }
-    b->lock_rows = lock_rows;
-    for (size_t k = 0; k < b->grids.size(); ++k) {
+    b->pairs.assign(ng, 0);
+    b->groups.clear();
+    bool slabs = false;
+    for (size_t k = 0; k < ng; ++k) {
         lbm_grid *g = b->grids[k];
         GridDesc &d = gd[k];
         d.buf[0] = g->buf[0];
@@ -197,50 +207,90 @@ static int build_worklist(lbm_batch *b) {
         d.P = g->P;
         d.nx = g->nx;
         d.ny = g->ny;
-        int v = batch_vec(b, g);
-        d.kind = kind_code(g->storage, v, g->rounding ? 1 : 0, g->a15f ? 1 : 0);
-        d.pad = 0;
+        d.kind = kind_code(g->storage, batch_vec(b, g), g->rounding ? 1 : 0, g->a15f ? 1 : 0);
+        d.pairs = 0;
         d.c = g->coef;
-        int w = 32 * v;
-        // Flow schedule: a grid's step takes at least one tile walk, so a grid
-        // with fewer tiles than its share of the resident warps (the warps
-        // split evenly between the grids) uses tiles a quarter as tall: four
-        // times the tiles, each walk a quarter as long.
-        int rows = lock_rows;
-        if (b->schedule == LBM_SCHEDULE_FLOW) {
-            const long long tiles_tall =
-                (long long)((g->nx + w - 1) / w) * ((g->ny - 2 * g->slab + b->rows - 1) / b->rows);
-            if (tiles_tall * (long long)b->grids.size() < flow_warps) rows = std::max(1, b->rows / 4);
-        }
-        // Rows computed: all of them, or a slab's own rows between its ghosts.
+        slabs = slabs || g->slab;
+    }
+    // Columns of a grid's tiles, and the rows it computes (all of them, or a
+    // slab's own rows between its ghosts).
+    auto strip_cols = [&](size_t k, bool pairs) {
+        const int v = batch_vec(b, b->grids[k]);
+        return (pairs ? 30 : 32) * v;
+    };
+    auto strips = [&](size_t k, bool pairs) {
+        const int w = strip_cols(k, pairs);
+        return (b->grids[k]->nx + w - 1) / w;
+    };
+    auto computed_rows = [&](size_t k) { return b->grids[k]->ny - 2 * b->grids[k]->slab; };
+    // Appends the tiles of grid k at a tile height.
+    auto add_tiles = [&](size_t k, int rows, bool pairs) {
+        lbm_grid *g = b->grids[k];
+        GridDesc &d = gd[k];
+        b->pairs[k] = pairs;
+        d.pairs = pairs ? 1 : 0;
+        const int w = strip_cols(k, pairs);
         const int ylo = g->slab, yhi = g->ny - g->slab, nyc = yhi - ylo;
         d.tile0 = (int)tiles.size();
-        d.nstrips = (g->nx + w - 1) / w;
+        d.nstrips = strips(k, pairs);
         d.nsegs = (nyc + rows - 1) / rows;
         d.ntile = d.nstrips * d.nsegs;
-        // A step reads two rows and two columns beyond its tile: the next
-        // segment or strip over suffices unless one of them is a single row
-        // or column wide (the last one of a grid can be).
+        // A pass reads two rows and columns per step beyond its tile: the next
+        // segment or strip over suffices unless one of them is smaller (the
+        // last one of a grid can be).
+        const int reach = pairs ? 4 : 2;
         const int last_rows = nyc - (d.nsegs - 1) * rows;
         const int last_cols = g->nx - (d.nstrips - 1) * w;
-        d.dseg = (rows >= 2 && last_rows >= 2) ? 1 : 2;
-        d.dstrip = last_cols >= 2 ? 1 : 2;
+        d.dseg = (rows >= reach && last_rows >= reach) ? 1 : 2;
+        d.dstrip = last_cols >= reach ? 1 : 2;
         // Neighbouring segments walk in opposite directions, so the rows they
         // share are read by both at about the same time (from L2 the second time).
         for (int y0 = ylo, seg = 0; y0 < yhi; y0 += rows, ++seg)
             for (int x0 = 0; x0 < g->nx; x0 += w)
                 tiles.push_back(Tile{(int)k, x0, y0, std::min(yhi, y0 + rows),
                                      (seg & 1) ? -1 : 1});
-    }
+    };
     if (b->schedule == LBM_SCHEDULE_FLOW) {
-        // One launch over every grid, tiles grid by grid in their order.
-        b->groups.clear();
+        // One launch over every grid, tiles grid by grid in their order, by the
+        // kernel for the grids' kinds.  Slabs take single steps: their ghost
+        // rows serve one.
+        std::vector<int> kinds;
+        for (const GridDesc &d : gd) kinds.push_back(d.kind);
+        const FlowChoice fc = flow_kernel_for(kinds, b->walk16, !slabs);
         lbm_batch::Group gr;
-        gr.begin = 0;
+        gr.fkernel = fc.fn;
+        gr.smem = fc.smem;
+        gr.pairs = fc.pairs;
+        gr.rows = b->rows;
+        BCK(resident_blocks((const void *)fc.fn, fc.smem, &gr.max_blocks_per_sm));
+        if (gr.max_blocks_per_sm < 1) return bfail(LBM_ECUDA, "flow kernel cannot be resident");
+        const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
+                                             : gr.max_blocks_per_sm;
+        const long long warps = (long long)per * b->sms * kBatchWarps;
+        for (size_t k = 0; k < ng; ++k) {
+            // A grid's pass takes at least one tile walk, so a grid with fewer
+            // tiles than its share of the resident warps (the warps split
+            // evenly between the grids) uses shorter tiles: a quarter as tall
+            // in single steps; on the fused walk as tall as its share of warps
+            // asks for, from 4 rows (its reach, so that a tile waits for its
+            // neighbours only) to 48.
+            int rows = b->rows;
+            if (fc.pairs) {
+                if (b->fit_rows) {
+                    const long long share = std::max<long long>(1, warps / (long long)ng);
+                    const long long r =
+                        ((long long)strips(k, true) * computed_rows(k) + share - 1) / share;
+                    rows = (int)std::min<long long>(48, r);
+                }
+                rows = std::max(4, rows);
+            } else {
+                const long long tall =
+                    (long long)strips(k, false) * ((computed_rows(k) + rows - 1) / rows);
+                if (tall * (long long)ng < warps) rows = std::max(1, rows / 4);
+            }
+            add_tiles(k, rows, fc.pairs);
+        }
         gr.count = (int)tiles.size();
-        gr.kernel = nullptr;
-        gr.fkernel = fk;
-        gr.max_blocks_per_sm = flow_bps;
         b->groups.push_back(gr);
         if (tiles.size() > b->prog_cap) {
             cudaFree(b->d_prog);
@@ -249,9 +299,27 @@ static int build_worklist(lbm_batch *b) {
             b->prog_cap = tiles.size();
         }
         if (!b->d_ctl)
-            BCK(cudaMalloc(&b->d_ctl, sizeof(unsigned long long) * kFlowCtlWords *
-                                          b->grids.size()));
+            BCK(cudaMalloc(&b->d_ctl, sizeof(unsigned long long) * kFlowCtlWords * ng));
         return upload_worklist(b, gd, tiles);
+    }
+    // Lockstep, default configuration, single-step walks: every warp walks its
+    // tiles one after another within a step, so a batch with fewer tiles than
+    // about the resident warps (16 per SM in the specialised kernels) spends
+    // each step on a whole walk with warps idle.  Such a batch gets shorter
+    // tiles, down to 2 rows, as many as one wave holds.  Batches of at least
+    // 3/4 of a wave of tiles keep the configured height.
+    int lock_rows = b->rows;
+    if (b->fit_rows) {
+        const int bps = b->blocks_per_sm > 0 ? b->blocks_per_sm : 4;
+        const long long wave = (long long)bps * b->sms * kBatchWarps;
+        auto tiles_at = [&](int r) {
+            long long t = 0;
+            for (size_t k = 0; k < ng; ++k)
+                t += (long long)strips(k, false) * ((computed_rows(k) + r - 1) / r);
+            return t;
+        };
+        if (4 * tiles_at(lock_rows) < 3 * wave)
+            while (lock_rows > 2 && tiles_at(lock_rows - 1) <= wave) --lock_rows;
     }
     // Kind groups.  A kind with a specialised kernel runs in its own launch
     // when its grids move at least kOwnLaunchBytes per step (about 10 us of
@@ -260,27 +328,16 @@ static int build_worklist(lbm_batch *b) {
     // any kind overlap.  A batch of one kind is one group.
     constexpr double kOwnLaunchBytes = 64.0 * 1024 * 1024;
     std::vector<double> bytes(kKindCodes, 0.0);
-    std::vector<int> count(kKindCodes, 0);
-    for (size_t k = 0; k < b->grids.size(); ++k) {
-        const lbm_grid *g = b->grids[k];
-        bytes[gd[k].kind] += (double)g->nx * (g->ny - 2 * g->slab) *
-                             ((g->storage == ST_F32 ? 72.0 : 36.0) + (g->a15f ? 4.0 : 0.0));
-    }
-    for (const Tile &t : tiles) count[gd[t.grid].kind]++;
+    std::vector<std::vector<size_t>> of_kind(kKindCodes);
     int kinds_present = 0;
-    for (int kd = 0; kd < kKindCodes; ++kd) kinds_present += count[kd] > 0;
-    std::vector<int> own, rest;
-    for (int kd = 0; kd < kKindCodes; ++kd) {
-        if (!count[kd]) continue;
-        BatchKernel kk = kernel_for({kd}, b->walk16);
-        if (kk != (BatchKernel)k_batch && (kinds_present == 1 || bytes[kd] >= kOwnLaunchBytes))
-            own.push_back(kd);
-        else
-            rest.push_back(kd);
+    for (size_t k = 0; k < ng; ++k) {
+        const lbm_grid *g = b->grids[k];
+        bytes[gd[k].kind] += (double)g->nx * computed_rows(k) *
+                             ((g->storage == ST_F32 ? 72.0 : 36.0) + (g->a15f ? 4.0 : 0.0));
+        kinds_present += of_kind[gd[k].kind].empty();
+        of_kind[gd[k].kind].push_back(k);
     }
     std::vector<Tile> ordered;
-    ordered.reserve(tiles.size());
-    b->groups.clear();
     // A group of one 8-site 16-bit kind (automatic walk) pairs the tiles of
     // its grids at most kSplitCols wide: consecutive segments share one warp,
     // a half-warp each (the split walk), where a single walk leaves half of
@@ -290,29 +347,90 @@ static int build_worklist(lbm_batch *b) {
     // a wider grid measured no faster, so a group pairs only whole narrow
     // grids, and only when their tiles are at least kSplitMinShare of its
     // tiles.
+    auto splits = [&](int kd) {
+        if (!kind_splits(kd) || b->walk16 != LBM_WALK16_AUTO) return false;
+        long long n_all = 0, n_narrow = 0;
+        for (size_t k : of_kind[kd]) {
+            const long long n =
+                (long long)strips(k, false) * ((computed_rows(k) + lock_rows - 1) / lock_rows);
+            n_all += n;
+            if (gd[k].nx <= kSplitCols) n_narrow += n;
+        }
+        return n_narrow > 0 && (double)n_narrow >= kSplitMinShare * (double)n_all;
+    };
+    // The fused walk (two steps per pass) serves every group of one kind that
+    // has it, but for the split walk's groups, slabs, and 16-bit walks the
+    // caller chose.
+    auto fuses = [&](int kd) {
+        if (!pair_kernel_for(kd).fn || splits(kd)) return false;
+        for (size_t k : of_kind[kd])
+            if (b->grids[k]->slab ||
+                (b->grids[k]->storage != ST_F32 && b->walk16 != LBM_WALK16_AUTO))
+                return false;
+        return true;
+    };
+    // The end of each pass: the warps that take the last tiles set its length,
+    // and the others wait at the barrier.  A group of more than two waves of
+    // tiles splits its last wave's tiles in two (8 rows each at the default
+    // height), halving that tail for a few more pulled rows per split tile.
+    // Measured with single steps: the nine 2048^2 FP16-delta grids 168.1k ->
+    // 170.2k MLUPS (stochastic rounding 165.0k -> 168.0k), the 512-grid batch
+    // FP16-delta 158.6k -> 159.4k, FP32 sweep 93.4k -> 93.8k; quarters, or
+    // halves over the last two waves, gained less.
+    auto split_tail = [&](size_t begin, long long wave) {
+        if ((long long)(ordered.size() - begin) <= 2 * wave) return;
+        std::vector<Tile> tail(ordered.end() - wave, ordered.end());
+        ordered.resize(ordered.size() - wave);
+        for (const Tile &t : tail) {
+            if (t.y1b > t.y0b || t.y1 - t.y0 < 2) {
+                ordered.push_back(t);
+                continue;
+            }
+            const int mid = t.y0 + (t.y1 - t.y0) / 2;
+            ordered.push_back(Tile{t.grid, t.x0, t.y0, mid, 1});
+            ordered.push_back(Tile{t.grid, t.x0, mid, t.y1, -1});
+        }
+    };
     auto add_group = [&](const std::vector<int> &kinds_in) -> int {
         lbm_batch::Group gr;
         gr.begin = (int)ordered.size();
-        auto in_group = [&](const Tile &t) {
-            return std::find(kinds_in.begin(), kinds_in.end(), gd[t.grid].kind) != kinds_in.end();
-        };
-        auto narrow = [&](const Tile &t) { return gd[t.grid].nx <= kSplitCols; };
-        bool split = kinds_in.size() == 1 && kind_splits(kinds_in[0]) &&
-                     b->walk16 == LBM_WALK16_AUTO;
-        if (split) {
-            long long n_all = 0, n_narrow = 0;
-            for (const Tile &t : tiles)
-                if (in_group(t)) {
-                    ++n_all;
-                    n_narrow += narrow(t);
-                }
-            split = n_narrow > 0 && (double)n_narrow >= kSplitMinShare * (double)n_all;
+        tiles.clear();
+        if (kinds_in.size() == 1 && fuses(kinds_in[0])) {
+            const PairChoice pc = pair_kernel_for(kinds_in[0]);
+            gr.kernel = pc.fn;
+            gr.smem = pc.smem;
+            gr.pairs = true;
+            BCK(resident_blocks((const void *)gr.kernel, gr.smem, &gr.max_blocks_per_sm));
+            if (gr.max_blocks_per_sm < 1)
+                return bfail(LBM_ECUDA, "batch kernel cannot be resident");
+            const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
+                                                 : gr.max_blocks_per_sm;
+            const long long warps = (long long)per * b->sms * kBatchWarps;
+            gr.rows = b->rows;
+            if (b->fit_rows) {
+                std::vector<std::pair<int, int>> shape;
+                for (size_t k : of_kind[kinds_in[0]])
+                    shape.push_back({strips(k, true), computed_rows(k)});
+                gr.rows = pair_rows(shape, warps,
+                                    b->grids[of_kind[kinds_in[0]][0]]->storage == ST_F32 ? 64 : 512);
+            }
+            for (size_t k : of_kind[kinds_in[0]]) add_tiles(k, gr.rows, true);
+            ordered.insert(ordered.end(), tiles.begin(), tiles.end());
+            split_tail(gr.begin, warps);
+            gr.count = (int)ordered.size() - gr.begin;
+            b->groups.push_back(gr);
+            return LBM_OK;
         }
+        for (int kd : kinds_in)
+            for (size_t k : of_kind[kd]) add_tiles(k, lock_rows, false);
+        // (grids in the caller's order, whatever their kinds)
+        std::stable_sort(tiles.begin(), tiles.end(),
+                         [](const Tile &x, const Tile &y) { return x.grid < y.grid; });
+        const bool split = kinds_in.size() == 1 && splits(kinds_in[0]);
         const int paired0 = b->paired;
-        std::vector<int> pending(b->grids.size(), -1);
+        std::vector<int> pending(ng, -1);
         for (const Tile &t : tiles) {
-            if (!in_group(t)) continue;
-            if (split && narrow(t)) {
+            if (split && gd[t.grid].nx <= kSplitCols) {
                 int &p = pending[t.grid];
                 if (p >= 0) {
                     Tile &a = ordered[p];
@@ -327,44 +445,26 @@ static int build_worklist(lbm_batch *b) {
             }
             ordered.push_back(t);
         }
-        // The end of each step: the warps that take the last tiles of a step
-        // set its length, and the others wait at the barrier.  A group of more
-        // than two waves of tiles splits its last wave's tiles in two (8 rows
-        // each at the default height), halving that tail for one extra pulled
-        // row pair per split tile.  Measured: the nine 2048^2 FP16-delta grids
-        // 168.1k -> 170.2k MLUPS (stochastic rounding 165.0k -> 168.0k), the
-        // 512-grid batch FP16-delta 158.6k -> 159.4k, FP32 sweep 93.4k ->
-        // 93.8k; quarters, or halves over the last two waves, gained less.
-        {
-            const int bps = b->blocks_per_sm > 0 ? b->blocks_per_sm : 4;
-            const long long wave = (long long)bps * b->sms * kBatchWarps;
-            const long long n = (long long)ordered.size() - gr.begin;
-            if (n > 2 * wave) {
-                std::vector<Tile> tail(ordered.end() - wave, ordered.end());
-                ordered.resize(ordered.size() - wave);
-                for (const Tile &t : tail) {
-                    if (t.y1b > t.y0b || t.y1 - t.y0 < 2) {
-                        ordered.push_back(t);
-                        continue;
-                    }
-                    const int mid = t.y0 + (t.y1 - t.y0) / 2;
-                    ordered.push_back(Tile{t.grid, t.x0, t.y0, mid, 1});
-                    ordered.push_back(Tile{t.grid, t.x0, mid, t.y1, -1});
-                }
-            }
-        }
+        const int bps = b->blocks_per_sm > 0 ? b->blocks_per_sm : 4;
+        split_tail(gr.begin, (long long)bps * b->sms * kBatchWarps);
+        gr.rows = lock_rows;
         gr.count = (int)ordered.size() - gr.begin;
         gr.kernel = kernel_for(kinds_in, b->walk16, b->paired > paired0);
-        BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&gr.max_blocks_per_sm,
-                                                          (const void *)gr.kernel,
-                                                          32 * kBatchWarps, 0));
+        BCK(resident_blocks((const void *)gr.kernel, 0, &gr.max_blocks_per_sm));
         if (gr.max_blocks_per_sm < 1) return bfail(LBM_ECUDA, "batch kernel cannot be resident");
         b->groups.push_back(gr);
         return LBM_OK;
     };
-    for (int kd : own) {
-        int rc = add_group({kd});
-        if (rc != LBM_OK) return rc;
+    std::vector<int> rest;
+    for (int kd = 0; kd < kKindCodes; ++kd) {
+        if (of_kind[kd].empty()) continue;
+        BatchKernel kk = kernel_for({kd}, b->walk16);
+        if (kk != (BatchKernel)k_batch && (kinds_present == 1 || bytes[kd] >= kOwnLaunchBytes)) {
+            int rc = add_group({kd});
+            if (rc != LBM_OK) return rc;
+        } else {
+            rest.push_back(kd);
+        }
     }
     if (!rest.empty()) {
         int rc = add_group(rest);
@@ -485,7 +585,8 @@ static cudaError_t enqueue(lbm_batch *b, long long n, cudaStream_t st) {
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_prog, 0, sizeof(int) * b->ntiles, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned) * kBarWords, st);
         if (e != cudaSuccess) return e;
-        b->groups[0].fkernel<<<grid_blocks(b, b->groups[0]), 32 * kBatchWarps, 0, st>>>(
+        const lbm_batch::Group &gr = b->groups[0];
+        gr.fkernel<<<grid_blocks(b, gr), 32 * kBatchWarps, gr.smem, st>>>(
             grids, ng, b->d_tiles, lim, par, t0, b->d_ctl, b->d_prog, bar, b->d_nwork, status,
             to);
         return cudaGetLastError();
@@ -501,7 +602,7 @@ static cudaError_t enqueue(lbm_batch *b, long long n, cudaStream_t st) {
                         (void *)&par,   (void *)&t0,    (void *)&n,      (void *)&bar,
                         (void *)&status, (void *)&to};
         e = cudaLaunchCooperativeKernel((const void *)gr.kernel, dim3(grid_blocks(b, gr)),
-                                        dim3(32 * kBatchWarps), args, 0, st);
+                                        dim3(32 * kBatchWarps), args, gr.smem, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -587,7 +688,7 @@ static int run_batch(lbm_batch *b, long long n, const long long *limits, bool ad
         for (int k = 0; k < ng; ++k) {
             long long s = b->h_limit[k];
             b->grids[k]->t += s;
-            if (s & 1) b->grids[k]->cur ^= 1;
+            if (passes_of(s, b->pairs[k]) & 1) b->grids[k]->cur ^= 1;
         }
     }
     return LBM_OK;
@@ -673,41 +774,74 @@ extern "C" int lbm_batch_set_timeout_us(lbm_batch_t b, long long us) {
     return LBM_OK;
 }
 
-// Times one-step dry runs (the state is not advanced: every grid writes its
-// other buffer) for several tile heights and, when the batch holds 16-bit
-// grids, the 16-bit walks, each at its full occupancy; keeps the fastest.
-// A one-step launch does the same per-step work as a step inside a longer
-// launch (the barriers between steps cost microseconds per millisecond step).
-// Times dry one-step runs of every (walk, tile height) candidate with the
-// events e0/e1 and leaves the fastest in *rows / *walk.
-static int tune_candidates(lbm_batch *b, cudaEvent_t e0, cudaEvent_t e1, int *rows,
-                           int *walk_out) {
-    float best = 1e30f;
-    const int rowss[] = {8, 12, 16, 24, 32};
+// A configuration the tuner tries: a tile height (0: the heights the work-list
+// fits by itself) and a 16-bit walk.
+struct BatchTry {
+    int rows, walk;
+};
+
+static int apply_try(lbm_batch *b, const BatchTry &t) {
+    int rc = lbm_batch_set_walk16(b, t.walk);
+    if (rc != LBM_OK) return rc;
+    if (t.rows > 0) return lbm_batch_set_config(b, t.rows, 0);
+    b->rows = 16;
+    b->fit_rows = true;
+    b->blocks_per_sm = 0;
+    return build_worklist(b);
+}
+
+// Milliseconds per 1e9 lattice updates of dry passes (the state is not
+// advanced: every grid writes its other buffer) under the work-list as built,
+// at its full occupancy.  A pass is one step, or two for a grid on the fused
+// walk; it does the same work as a pass inside a longer launch (the barriers
+// cost microseconds per millisecond pass).
+static int time_passes(lbm_batch *b, cudaEvent_t e0, cudaEvent_t e1, double *cost) {
+    std::vector<long long> limits;
+    double updates = 0;
+    for (size_t k = 0; k < b->grids.size(); ++k) {
+        const lbm_grid *g = b->grids[k];
+        limits.push_back(b->pairs[k] ? 2 : 1);
+        updates += (double)limits.back() * g->nx * (g->ny - 2 * g->slab);
+    }
+    int rc = run_batch(b, 2, limits.data(), false);  // warm-up (and graph build)
+    if (rc != LBM_OK) return rc;
+    BCK(cudaEventRecord(e0, b->stream));
+    for (int k = 0; k < 4 && rc == LBM_OK; ++k) rc = run_batch(b, 2, limits.data(), false);
+    if (rc != LBM_OK) return rc;
+    BCK(cudaEventRecord(e1, b->stream));
+    BCK(cudaEventSynchronize(e1));
+    float ms = 0.f;
+    BCK(cudaEventElapsedTime(&ms, e0, e1));
+    *cost = ms / 4 / updates * 1e9;
+    return LBM_OK;
+}
+
+// Times several tile heights, when the batch holds 16-bit grids the 16-bit
+// walks, and with groups on the fused walk the heights the work-list fits by
+// itself; leaves the fastest in *best.
+static int tune_candidates(lbm_batch *b, cudaEvent_t e0, cudaEvent_t e1, BatchTry *best) {
+    double least = 1e300;
     std::vector<std::vector<BatchKernel>> seen;
     for (int walk = LBM_WALK16_AUTO; walk <= LBM_WALK16_V4_PF2; ++walk) {
         int rc = lbm_batch_set_walk16(b, walk);
         if (rc != LBM_OK) return rc;
         std::vector<BatchKernel> ks;
-        for (const auto &gr : b->groups) ks.push_back(gr.kernel);
+        bool pairs = false;
+        for (const auto &gr : b->groups) {
+            ks.push_back(gr.kernel);
+            pairs = pairs || gr.pairs;
+        }
         if (std::find(seen.begin(), seen.end(), ks) != seen.end()) continue;  // same kernels
         seen.push_back(ks);
-        for (int r : rowss) {
-            rc = lbm_batch_set_config(b, r, 0);
+        for (int r : {0, 8, 12, 16, 24, 32}) {
+            if (r == 0 && !pairs) continue;
+            double cost = 0;
+            rc = apply_try(b, BatchTry{r, walk});
+            if (rc == LBM_OK) rc = time_passes(b, e0, e1, &cost);
             if (rc != LBM_OK) return rc;
-            rc = run_batch(b, 1, nullptr, false);  // warm-up (and graph build)
-            if (rc != LBM_OK) return rc;
-            BCK(cudaEventRecord(e0, b->stream));
-            for (int k = 0; k < 4 && rc == LBM_OK; ++k) rc = run_batch(b, 1, nullptr, false);
-            if (rc != LBM_OK) return rc;
-            BCK(cudaEventRecord(e1, b->stream));
-            BCK(cudaEventSynchronize(e1));
-            float ms = 0.f;
-            BCK(cudaEventElapsedTime(&ms, e0, e1));
-            if (ms < best) {
-                best = ms;
-                *rows = r;
-                *walk_out = walk;
+            if (cost < least) {
+                least = cost;
+                *best = BatchTry{r, walk};
             }
         }
     }
@@ -725,8 +859,8 @@ extern "C" int lbm_batch_tune(lbm_batch_t b) {
     }
     const int rows0 = b->rows, walk0 = b->walk16, bps0 = b->blocks_per_sm;
     const bool fit0 = b->fit_rows;
-    int best_rows = rows0, best_walk = walk0;
-    int rc = tune_candidates(b, e0, e1, &best_rows, &best_walk);
+    BatchTry best{rows0, walk0};
+    int rc = tune_candidates(b, e0, e1, &best);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc != LBM_OK) {
@@ -739,8 +873,7 @@ extern "C" int lbm_batch_tune(lbm_batch_t b) {
         }
         return rc;
     }
-    rc = lbm_batch_set_walk16(b, best_walk);
-    return rc != LBM_OK ? rc : lbm_batch_set_config(b, best_rows, 0);
+    return apply_try(b, best);
 }
 
 extern "C" int lbm_batch_set_schedule(lbm_batch_t b, int schedule) {
@@ -786,7 +919,7 @@ extern "C" int lbm_batch_get_tiles(lbm_batch_t b, int *tiles, int *paired) {
 extern "C" int lbm_batch_get_config(lbm_batch_t b, int *rows, int *blocks_per_sm,
                                     int *specialised) {
     if (!b) return bfail(LBM_EINVAL, "lbm_batch_get_config: NULL batch");
-    if (rows) *rows = b->schedule == LBM_SCHEDULE_LOCKSTEP ? b->lock_rows : b->rows;
+    if (rows) *rows = b->groups.empty() ? b->rows : b->groups[0].rows;
     if (blocks_per_sm)
         *blocks_per_sm = b->groups.empty() ? 0 : grid_blocks(b, b->groups[0]) / b->sms;
     if (specialised) {

@@ -20,6 +20,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_internal.h"
+#include "lbm_walk2.cuh"
 
 using namespace vss;
 
@@ -31,12 +32,13 @@ struct GridDesc {
     size_t P;
     int nx, ny;
     int kind;  // kind_code(storage, vec, stochastic rounding)
-    int pad;
+    int pairs; // 1: a pass takes two steps (the fused walk), 0: one
     Coef c;
     // Tiles of the grid in the work-list (flow schedule): the first one, how
     // many per step (segment-major: t = segment * nstrips + strip), and how
-    // many segments / strips on each side a tile's step reads from (1, or 2
-    // when a neighbouring segment or strip can be a single row or column).
+    // many segments / strips on each side a tile's pass reads from (1, or 2
+    // when a neighbouring segment or strip can be smaller than the pass's
+    // reach: two sites for one step, four for two).
     int tile0, ntile, nstrips, nsegs, dseg, dstrip;
 };
 
@@ -257,8 +259,8 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
 }
 
 // ---------------------------------------------------------------------------
-// Flow schedule: every grid advances its own steps, with no barrier across
-// the batch.  Each grid hands out tickets m = k * ntile + t (step k, tile t)
+// Flow schedule: every grid advances its own passes (a step, or two steps for
+// grids on the fused walk), with no barrier across the batch.  Each grid hands out tickets m = k * ntile + t (step k, tile t)
 // from its own counter, in step order.  A warp holding (k, t) waits until
 // every tile its step reads from or overwrites (the tiles within dseg
 // segments and dstrip strips, wrapped, itself included) has completed step
@@ -326,7 +328,12 @@ __device__ __forceinline__ bool flow_wait(const GridDesc &g, const int *prog, in
     return true;
 }
 
-// The flow loop of one warp; run_tile(g, par, tile, step) runs a tile.
+// Passes a grid takes for `steps` steps, and whether pass k of them takes two.
+__host__ __device__ inline long long passes_of(long long steps, int pairs) {
+    return pairs ? (steps + 1) / 2 : steps;
+}
+
+// The flow loop of one warp; run_tile(g, par, tile, step, two) runs a tile.
 template <class RunTile>
 __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, int ngrids,
                                           const Tile *__restrict__ tiles,
@@ -358,7 +365,8 @@ __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, in
                     const int cand = (int)((start + (unsigned)j) % (unsigned)ngrids);
                     const GridDesc &G = grids[cand];
                     const unsigned long long total =
-                        (unsigned long long)limit[cand] * (unsigned long long)G.ntile;
+                        (unsigned long long)passes_of(limit[cand], G.pairs) *
+                        (unsigned long long)G.ntile;
                     volatile unsigned long long *c = ctl + (size_t)cand * kFlowCtlWords;
                     const unsigned long long taken = c[0];
                     if (taken >= total) continue;
@@ -407,7 +415,9 @@ __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, in
             const int seg = ti / g.nstrips, strip = ti % g.nstrips;
             if (!flow_wait(g, prog, seg, strip, k, status, timeout_ns)) return;
             const Tile t = tiles[g.tile0 + ti];
-            run_tile(g, (parity0[gsel] + k) & 1, t, t0[gsel] + (uint32_t)k);
+            const uint32_t done = (uint32_t)k << g.pairs;  // steps before this pass
+            run_tile(g, (parity0[gsel] + k) & 1, t, t0[gsel] + done,
+                     g.pairs && limit[gsel] - (long long)done >= 2);
         }
         // Publish: the tile's stores before its completed-step count.
         __threadfence();
@@ -426,65 +436,81 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
            const uint32_t *__restrict__ t0, unsigned long long *ctl, int *prog, unsigned *glob,
            const int *__restrict__ nwork_p, int *status, unsigned long long timeout_ns) {
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
-              timeout_ns, [](const GridDesc &g, int par, const Tile &t, uint32_t step) {
+              timeout_ns, [](const GridDesc &g, int par, const Tile &t, uint32_t step, bool) {
                   any_tile(g, par, t, step);
               });
 }
 
-// Flow kernel for a batch of one walk, inlined (the register budget and the
-// row buffers of k_batch_one: 16 warps per SM, measured faster than 12
-// without spills although the flow loop's state costs a few bytes of spill).
-template <int S, int V, int PD, int RND, int VA = 0>
+// Flow kernel for a batch of one 4-site 16-bit walk, inlined (the register
+// budget of k_batch_one: 16 warps per SM, measured faster than 12 without
+// spills although the flow loop's state costs a few bytes of spill).
+template <int S, int PD>
 __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
     k_flow_one(const GridDesc *__restrict__ grids, int ngrids, const Tile *__restrict__ tiles,
                const long long *__restrict__ limit, const int *__restrict__ parity0,
                const uint32_t *__restrict__ t0, unsigned long long *ctl, int *prog,
                unsigned *glob, const int *__restrict__ nwork_p, int *status,
                unsigned long long timeout_ns) {
-    __shared__ uint4 rowbuf[(S != ST_F32 && V == 8) ? kBatchWarps : 1][(2 * 9 + (VA ? 4 : 0)) * 32];
-    (void)rowbuf;
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
-              timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t step) {
-                  Walker<S, V, LD_CG, RND, VA> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P,
-                                                 t.x0);
-                  if constexpr (VA) w.a15f = g.a15f;
-                  if constexpr (RND) w.set_step(step);
+              timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t, bool) {
+                  Walker<S, 4, LD_CG> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P, t.x0);
                   const Coef c = g.c;
-                  if constexpr (S != ST_F32 && V == 8)
-                      w.run_async(t.y0, t.y1, t.dir, c, &rowbuf[threadIdx.x >> 5][0]);
-                  else if constexpr (PD == 2)
+                  if constexpr (PD == 2)
                       w.run_prefetch2(t.y0, t.y1, t.dir, c);
-                  else if constexpr (PD == 1)
-                      w.run_prefetch(t.y0, t.y1, t.dir, c);
                   else
-                      w.run(t.y0, t.y1, t.dir, c);
+                      w.run_prefetch(t.y0, t.y1, t.dir, c);
               });
 }
 
-// Flow kernel for the serving mix: FP32 grids (4 sites per lane) and 16-bit
-// grids of storage S2 and rounding RND2 (8 sites per lane), both walks
-// inlined; 12 warps per SM (at 16 both walks together spill heavily).
+// One tile of the fused walk: two steps, or a grid's odd last one.
+template <int S, int RND, int VA>
+__device__ __forceinline__ void pair_tile(const GridDesc &g, int par, const Tile &t, uint32_t step,
+                                          bool two, uint4 *buf) {
+    const Coef c = g.c;
+    Walker2<S, LD_CG, RND, VA> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P, t.x0);
+    if constexpr (VA) w.a15f = g.a15f;
+    if constexpr (RND) w.set_step(step);
+    w.run(t.y0, t.y1, t.dir, two, c, buf);
+}
+
+// Flow kernel for a batch of one kind of grids on the fused walk.
+template <int S, int RND, int VA>
+__global__ void __launch_bounds__(32 * kBatchWarps, 2)
+    k_flow_pairs(const GridDesc *__restrict__ grids, int ngrids, const Tile *__restrict__ tiles,
+                 const long long *__restrict__ limit, const int *__restrict__ parity0,
+                 const uint32_t *__restrict__ t0, unsigned long long *ctl, int *prog,
+                 unsigned *glob, const int *__restrict__ nwork_p, int *status,
+                 unsigned long long timeout_ns) {
+    extern __shared__ uint4 walk_smem[];
+    uint4 *buf = walk_smem + (threadIdx.x >> 5) * walk2_vecs<S, VA>();
+    flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
+              timeout_ns,
+              [&](const GridDesc &g, int par, const Tile &t, uint32_t step, bool two) {
+                  pair_tile<S, RND, VA>(g, par, t, step, two, buf);
+              });
+}
+
+// Flow kernel for the serving mix: FP32 grids and 16-bit grids of storage S2
+// and rounding RND2, all on the fused walk, both walks inlined (20 grids of 128^2
+// to 2048^2 sharing 1e9 updates: 12.8 ms with single steps, 10.0 ms now, with
+// their initialisation and moments).
 template <int S2, int RND2>
-__global__ void __launch_bounds__(32 * kBatchWarps, 3)
+__global__ void __launch_bounds__(32 * kBatchWarps, 2)
     k_flow_two(const GridDesc *__restrict__ grids, int ngrids, const Tile *__restrict__ tiles,
                const long long *__restrict__ limit, const int *__restrict__ parity0,
                const uint32_t *__restrict__ t0, unsigned long long *ctl, int *prog,
                unsigned *glob, const int *__restrict__ nwork_p, int *status,
                unsigned long long timeout_ns) {
-    __shared__ uint4 rowbuf[kBatchWarps][2 * 9 * 32];
+    extern __shared__ uint4 walk_smem[];
+    static_assert(walk2_vecs<ST_F32, 0>() == walk2_vecs<S2, 0>(), "one buffer size");
+    uint4 *buf = walk_smem + (threadIdx.x >> 5) * walk2_vecs<S2, 0>();
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
-              timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t step) {
-                  const Coef c = g.c;
-                  if (g.kind == kind_code(ST_F32, 4, 0)) {
-                      Walker<ST_F32, 4, LD_CG> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P,
-                                                 t.x0);
-                      w.run(t.y0, t.y1, t.dir, c);
-                  } else {
-                      Walker<S2, 8, LD_CG, RND2> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P,
-                                                   t.x0);
-                      if constexpr (RND2) w.set_step(step);
-                      w.run_async(t.y0, t.y1, t.dir, c, &rowbuf[threadIdx.x >> 5][0]);
-                  }
+              timeout_ns,
+              [&](const GridDesc &g, int par, const Tile &t, uint32_t step, bool two) {
+                  if (g.kind == kind_code(ST_F32, 4, 0))
+                      pair_tile<ST_F32, 0, 0>(g, par, t, step, two, buf);
+                  else
+                      pair_tile<S2, RND2, 0>(g, par, t, step, two, buf);
               });
 }
 
@@ -492,57 +518,79 @@ using FlowKernel = void (*)(const GridDesc *, int, const Tile *, const long long
                             const uint32_t *, unsigned long long *, int *, unsigned *,
                             const int *, int *, unsigned long long);
 
-// The flow kernel for a batch's kinds: specialised when all grids share one
-// walk, else the general k_flow.
-FlowKernel flow_kernel_for(const std::vector<int> &kinds, int walk16) {
+// A kernel with its dynamic shared memory per block, and whether its grids
+// take two steps per pass.
+struct FlowChoice {
+    FlowKernel fn;
+    int smem;
+    bool pairs;
+};
+template <int S, int VA>
+constexpr int pair_smem() {
+    return kBatchWarps * walk2_vecs<S, VA>() * 16;
+}
+
+// The flow kernel for a batch's kinds: the fused walks when all grids share
+// one kind that has it, or FP32 and one such 16-bit kind (`pairs`: allowed);
+// a specialised single-step kernel when all share another walk, else the
+// general k_flow.
+FlowChoice flow_kernel_for(const std::vector<int> &kinds, int walk16, bool pairs) {
     bool same = true;
     for (int k : kinds) same = same && k == kinds[0];
+    if (!kinds.empty() && same && pairs) {
+        switch (kinds[0]) {
+            case kind_code(ST_F32, 4, 0):
+                return {k_flow_pairs<ST_F32, 0, 0>, pair_smem<ST_F32, 0>(), true};
+            case kind_code(ST_F32, 4, 0, 1):
+                return {k_flow_pairs<ST_F32, 0, 1>, pair_smem<ST_F32, 1>(), true};
+            case kind_code(ST_F16, 8, 0):
+                return {k_flow_pairs<ST_F16, 0, 0>, pair_smem<ST_F16, 0>(), true};
+            case kind_code(ST_BF16, 8, 0):
+                return {k_flow_pairs<ST_BF16, 0, 0>, pair_smem<ST_BF16, 0>(), true};
+            case kind_code(ST_F16, 8, 1):
+                return {k_flow_pairs<ST_F16, 1, 0>, pair_smem<ST_F16, 0>(), true};
+            case kind_code(ST_BF16, 8, 1):
+                return {k_flow_pairs<ST_BF16, 1, 0>, pair_smem<ST_BF16, 0>(), true};
+            default:
+                break;
+        }
+    }
     if (!kinds.empty() && same) {
         const bool two = walk16 == LBM_WALK16_V4_PF2;
         switch (kinds[0]) {
-            case kind_code(ST_F32, 4, 0):
-                return k_flow_one<ST_F32, 4, 0, 0>;
-            case kind_code(ST_F16, 8, 0):
-                return k_flow_one<ST_F16, 8, 0, 0>;
-            case kind_code(ST_BF16, 8, 0):
-                return k_flow_one<ST_BF16, 8, 0, 0>;
-            case kind_code(ST_F16, 8, 1):
-                return k_flow_one<ST_F16, 8, 0, 1>;
-            case kind_code(ST_BF16, 8, 1):
-                return k_flow_one<ST_BF16, 8, 0, 1>;
             case kind_code(ST_F16, 4, 0):
-                return two ? k_flow_one<ST_F16, 4, 2, 0> : k_flow_one<ST_F16, 4, 1, 0>;
+                return {two ? k_flow_one<ST_F16, 2> : k_flow_one<ST_F16, 1>, 0, false};
             case kind_code(ST_BF16, 4, 0):
-                return two ? k_flow_one<ST_BF16, 4, 2, 0> : k_flow_one<ST_BF16, 4, 1, 0>;
-            case kind_code(ST_F32, 4, 0, 1):
-                return k_flow_one<ST_F32, 4, 0, 0, 1>;
+                return {two ? k_flow_one<ST_BF16, 2> : k_flow_one<ST_BF16, 1>, 0,
+                        false};
             default:
                 break;
         }
     }
     // FP32 (4 sites per lane) with one 16-bit kind of 8 sites per lane.
     int other = -1;
-    bool pair = !kinds.empty();
+    bool mix = pairs && !kinds.empty();
     for (int k : kinds) {
         if (k == kind_code(ST_F32, 4, 0)) continue;
         if (other == -1) other = k;
-        pair = pair && k == other;
+        mix = mix && k == other;
     }
-    if (pair && other != -1) {
+    if (mix && other != -1) {
+        constexpr int smem = pair_smem<ST_F32, 0>();
         switch (other) {
             case kind_code(ST_F16, 8, 0):
-                return k_flow_two<ST_F16, 0>;
+                return {k_flow_two<ST_F16, 0>, smem, true};
             case kind_code(ST_BF16, 8, 0):
-                return k_flow_two<ST_BF16, 0>;
+                return {k_flow_two<ST_BF16, 0>, smem, true};
             case kind_code(ST_F16, 8, 1):
-                return k_flow_two<ST_F16, 1>;
+                return {k_flow_two<ST_F16, 1>, smem, true};
             case kind_code(ST_BF16, 8, 1):
-                return k_flow_two<ST_BF16, 1>;
+                return {k_flow_two<ST_BF16, 1>, smem, true};
             default:
                 break;
         }
     }
-    return k_flow;
+    return {k_flow, 0, false};
 }
 
 // Walks whose lockstep kernel takes paired tiles (the split walk): 8-site
@@ -621,6 +669,39 @@ __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
     }
 }
 
+// The same for grids on the fused walk: a pass takes two steps of every grid
+// that has two left, and one of a grid with one left.  Bound as k_step2 is (HBM
+// in FP32, issue in the 16-bit kinds), at its occupancy and two rows of copies in
+// flight; half as many barriers as single steps.  Measured, lockstep, 100 steps a
+// call, single steps before and pairs now: nine 2048^2 grids FP32 93k -> 176k
+// MLUPS, FP16 170k -> 234k, BF16 with stochastic rounding 168k -> 209k, FP32 with
+// a c2 field 85k -> 168k; 512 uneven grids FP32 93k -> 178k, FP16 159k -> 210k,
+// half and half 115k -> 185k.  Flow schedule: nine 2048^2 FP32 92k -> 174k, FP16
+// 168k -> 240k; 512 uneven, half and half, 83k -> 138k.
+template <int S, int RND, int VA>
+__global__ void __launch_bounds__(32 * kBatchWarps, 2)
+    k_batch_pairs(const GridDesc *__restrict__ grids, const Tile *__restrict__ tiles, int ntiles,
+                  const long long *__restrict__ limit, const int *__restrict__ parity0,
+                  const uint32_t *__restrict__ t0, long long nsteps, unsigned *bar, int *status,
+                  unsigned long long timeout_ns) {
+    extern __shared__ uint4 walk_smem[];
+    uint4 *buf = walk_smem + (threadIdx.x >> 5) * walk2_vecs<S, VA>();
+    const long long npass = (nsteps + 1) / 2;
+    for (long long k = 0; k < npass; ++k) {
+        reset_counter(bar, k);
+        unsigned *ctr = step_counter(bar, k);
+        for (int ti = next_tile(ctr); ti < ntiles; ti = next_tile(ctr)) {
+            const Tile t = tiles[ti];
+            const long long left = limit[t.grid] - 2 * k;
+            if (left <= 0) continue;
+            const int par = (parity0[t.grid] + (int)(k & 1)) & 1;
+            pair_tile<S, RND, VA>(grids[t.grid], par, t, t0[t.grid] + 2u * (uint32_t)k, left >= 2,
+                                  buf);
+        }
+        if (k + 1 < npass && !grid_barrier(bar, status, timeout_ns)) return;
+    }
+}
+
 using BatchKernel = void (*)(const GridDesc *, const Tile *, int, const long long *, const int *,
                              const uint32_t *, long long, unsigned *, int *, unsigned long long);
 
@@ -671,6 +752,34 @@ BatchKernel kernel_for(const std::vector<int> &kinds, int walk16, bool split = f
         }
     }
     return k_batch;
+}
+
+// Kinds with a fused walk, their lockstep kernel and its shared memory.
+struct PairChoice {
+    BatchKernel fn;
+    int smem;
+};
+PairChoice pair_kernel_for(int kind) {
+    switch (kind) {
+        case kind_code(ST_F32, 4, 0):
+            return {k_batch_pairs<ST_F32, 0, 0>, pair_smem<ST_F32, 0>()};
+        case kind_code(ST_F32, 4, 0, 1):
+            return {k_batch_pairs<ST_F32, 0, 1>, pair_smem<ST_F32, 1>()};
+        case kind_code(ST_F16, 8, 0):
+            return {k_batch_pairs<ST_F16, 0, 0>, pair_smem<ST_F16, 0>()};
+        case kind_code(ST_BF16, 8, 0):
+            return {k_batch_pairs<ST_BF16, 0, 0>, pair_smem<ST_BF16, 0>()};
+        case kind_code(ST_F16, 8, 1):
+            return {k_batch_pairs<ST_F16, 1, 0>, pair_smem<ST_F16, 0>()};
+        case kind_code(ST_BF16, 8, 1):
+            return {k_batch_pairs<ST_BF16, 1, 0>, pair_smem<ST_BF16, 0>()};
+        case kind_code(ST_F16, 8, 0, 1):
+            return {k_batch_pairs<ST_F16, 0, 1>, pair_smem<ST_F16, 1>()};
+        case kind_code(ST_BF16, 8, 0, 1):
+            return {k_batch_pairs<ST_BF16, 0, 1>, pair_smem<ST_BF16, 1>()};
+        default:
+            return {nullptr, 0};
+    }
 }
 
 }  // namespace

@@ -1,0 +1,55 @@
+"""Batches whose passes take two steps (the fused walk) leave every grid bit
+for bit in the state single steps leave it in, in both schedules: odd and even
+step limits, limits that end early, tile heights from one row up (the flow
+schedule uses at least four, the reach of a pass), strips of one lane, one whole
+strip and a last strip of one lane (120 columns in FP32, 240 in 16 bits)."""
+import numpy as np
+import pytest
+
+from paper_0707_2437_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(8, 3), (16, 1), (120, 4), (124, 7), (240, 33), (248, 5), (256, 100), (488, 20)]
+
+
+def _grid(lbm, kind, lens, k):
+    nx, ny = SIZES[k]
+    if kind == "mixed":
+        kind = "f16d" if k % 2 else "f32"
+    if kind == "f32" and nx == 248:
+        nx = 244
+    g = lbm.Grid(nx, ny, 0.6 + 0.05 * k, 0.1 + 0.04 * k, kind.replace("-sr", ""))
+    if kind.endswith("-sr"):
+        g.set_rounding("stochastic")
+    if lens:
+        g.set_c2_field(workloads.c2_lens(nx, ny, 0.2))
+    g.init(*workloads.fourier_modes(nx, ny, amp=1e-2, seed=k))
+    return g
+
+
+@pytest.mark.parametrize("schedule", ["lockstep", "flow"])
+@pytest.mark.parametrize("rows", [None, 1, 5])
+@pytest.mark.parametrize("kind,lens", [("f32", False), ("f32", True), ("f16d", False),
+                                       ("bf16d", True), ("f16d-sr", False), ("mixed", False)])
+def test_pairs_in_batches_equal_single_steps(lbm, kind, lens, rows, schedule):
+    limits = [1 + (7 * k) % 12 for k in range(len(SIZES))]
+    grids = [_grid(lbm, kind, lens, k) for k in range(len(SIZES))]
+    b = lbm.Batch(grids)
+    b.set_schedule(schedule)
+    if rows:
+        b.set_config(rows, 0)
+    b.step(12, limits)
+    b.step(3)
+    b.step(1, [k % 2 for k in range(len(SIZES))])
+    assert b.sync() == 0
+    got = [(g.t, g.get_state()[0]) for g in grids]
+    b.close()
+    for g in grids:
+        g.close()
+    for k, (t, state) in enumerate(got):
+        with _grid(lbm, kind, lens, k) as h:
+            for _ in range(limits[k] + 3 + k % 2):
+                h.step(1)
+            assert h.t == t
+            assert np.array_equal(h.get_state()[0], state), SIZES[k]
