@@ -118,14 +118,18 @@ int lbm_init(lbm_t h, const double *rho, const double *ux, const double *uy,
 
 /* Queues n >= 0 time steps of Eq. 5 (stream, moments, central grad(rho),
  * collide with force) on the handle's stream.  Calls either launch the step
- * kernel once per step with the handle's tile configuration (replayed from
- * CUDA graphs from 8 steps on), or run all n steps as one persistent launch:
- * the batched kernel (see lbm_batch_create) with this grid alone, warps
- * taking tiles dynamically, a bounded grid barrier between steps.  Which one
- * is set by lbm_set_persistent; by default (LBM_PERSISTENT_AUTO) every call
- * launches the step kernel, measured the faster for single grids of 64^2 to
- * 8192^2 in every storage.  A slab always steps persistent; a driven grid or
- * the forward-difference gradient never.  All forms give bitwise the same result.
+ * kernel once per step or pair of steps (replayed from CUDA graphs, 32 launches
+ * each), or run all n steps as one launch of one of two kinds.  Resident: the
+ * grid's tiles stay in the SMs' shared memory, one block each, and exchange
+ * their edges every few steps (bounded waits); grids of up to about 600^2
+ * sites.  Persistent: the batched kernel (see lbm_batch_create) with this grid
+ * alone, warps taking tiles dynamically, a bounded grid barrier between passes.
+ * Which one is set by lbm_set_persistent; by default (LBM_PERSISTENT_AUTO) calls
+ * of four steps or more on grids that fit run resident, all others launch the
+ * step kernel.  A slab always steps persistent; a driven grid never does, and
+ * the forward-difference gradient runs in the step kernel only.  A tile
+ * configuration or pipeline of the caller's, and a stream that is being
+ * captured, also mean the step kernel.  All forms give bitwise the same result.
  * Asynchronous: errors of the kernels surface at the next synchronising call
  * (LBM_ETIMEOUT if a bounded wait ran out). */
 int lbm_step(lbm_t h, long long n);
@@ -134,8 +138,8 @@ int lbm_step(lbm_t h, long long n);
  *   LBM_PERSISTENT_OFF   every call uses the step kernel
  *   LBM_PERSISTENT_ON    calls of 64 steps or more, or of 8 or more on grids
  *                        of at least 2^20 sites, run one persistent launch
- *   LBM_PERSISTENT_AUTO  the default: as described at lbm_step (the step
- *                        kernel, except for slabs)
+ *   LBM_PERSISTENT_AUTO  the default: as described at lbm_step (resident on
+ *                        small grids, else the step kernel, except for slabs)
  * LBM_EINVAL for other values. */
 #define LBM_PERSISTENT_OFF 0
 #define LBM_PERSISTENT_ON 1

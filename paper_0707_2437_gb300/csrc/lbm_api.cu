@@ -276,10 +276,19 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double c2, double rho0,
         if (!h->buf[0]) e = cudaMalloc(&h->buf[0], bytes);
         if (e == cudaSuccess && !h->buf[1]) e = cudaMalloc(&h->buf[1], bytes);
     }
-    if (e == cudaSuccess) e = cudaMalloc(&h->scratch, sizeof(double) * (3 * 1024 + 16));
+    if (e == cudaSuccess) e = plan_resident(nx, ny, sms > 0 ? sms : 1, &h->resident);
+    // Reduction partials and results, the status word and step counter, and
+    // the counters of a resident launch's tiles.
+    const size_t words = 3 * 1024 + 16;
+    const size_t flag_bytes =
+        sizeof(unsigned) * kResidentFlagWords * (size_t)(h->resident.tx * h->resident.ty);
+    if (e == cudaSuccess) e = cudaMalloc(&h->scratch, sizeof(double) * words + flag_bytes);
+    h->flags = reinterpret_cast<unsigned *>(h->scratch + words);
     // Stream-ordered, so that creating a grid does not wait for work running
     // on the legacy default stream.
     if (e == cudaSuccess) e = cudaMemsetAsync(h->scratch, 0, sizeof(double) * 16, h->stream);
+    if (e == cudaSuccess && flag_bytes)
+        e = cudaMemsetAsync(h->flags, 0, flag_bytes, h->stream);
     if (e == cudaSuccess) e = prepare_step(storage, h->cfg);
     if (e == cudaSuccess) e = plan_step2(storage, 0, false, nx, ny, &h->step2);
     if (e == cudaSuccess) e = cudaMallocHost(&h->host_out, sizeof(double) * 8);
@@ -403,6 +412,53 @@ static bool steps_in_pairs(const lbm_grid *h) {
     return h->pairs && h->step2.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL;
 }
 
+// Whether n steps run as one launch with the state in shared memory.  From four
+// steps on: such a launch costs about 6 us beyond its steps, a step launch 3 to 6.
+// Up to 3.6 us a step by the plan with stochastic rounding, which hashes every
+// site here but every pair of sites in the step kernel (600^2: 6.4 us against 6.3;
+// 512^2 5.0 against 6.2).  Not in a stream that is being captured: a replay would
+// repeat the exchange counters.
+static const long long kResidentMin = 4;
+static const double kResidentMostStochastic = 3.6;
+
+static bool runs_resident(const lbm_grid *h, long long n) {
+    if (!h->resident.ok || !h->pairs || h->persistent != LBM_PERSISTENT_AUTO || h->slab ||
+        h->grad != LBM_GRAD_CENTRAL || n < kResidentMin ||
+        (h->rounding && h->resident.us > kResidentMostStochastic))
+        return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess &&
+           cap == cudaStreamCaptureStatusNone;
+}
+
+static int step_resident(lbm_grid *h, long long n) {
+    ResidentArgs a{};
+    a.buf[0] = h->buf[0];
+    a.buf[1] = h->buf[1];
+    a.cur = h->cur;
+    a.nx = h->nx;
+    a.ny = h->ny;
+    a.P = h->P;
+    a.steps = n;
+    a.t0 = (uint32_t)h->t;
+    a.c = h->coef;
+    a.a15f = h->a15f;
+    a.drive = h->drive;
+    a.drive_amp = h->drive_amp;
+    a.drive_period = h->drive_period;
+    a.rho0 = h->rho0;
+    a.flags = h->flags;
+    a.epoch = h->epoch;
+    a.status = status_ptr(h);
+    cudaError_t e = launch_resident(h->resident, h->storage, h->rounding, a, h->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "lbm_step resident kernel");
+    const long long exchanges = resident_exchanges(h->resident, n);
+    h->epoch += (unsigned)exchanges;
+    if (!(exchanges & 1)) h->cur ^= 1;
+    h->t += n;
+    return LBM_OK;
+}
+
 // One launch of two steps from buf[from] to buf[from ^ 1].
 static cudaError_t launch_two(lbm_grid *h, int from, const uint32_t *tdev, uint32_t toff,
                               cudaStream_t st) {
@@ -416,8 +472,8 @@ static const long long kPersistentMin = 64;  // persistent launch from this many
 // where a step is long enough that the launch's barrier costs little.
 static const long long kPersistentMinLarge = 8;
 static const long long kLargeSites = 1LL << 20;
-// LBM_PERSISTENT_AUTO steps every grid with the step kernel (except slabs):
-// per step over 256- and 1024-step calls it was the faster for FP32 grids from
+// LBM_PERSISTENT_AUTO steps small grids resident (above) and the others with
+// the step kernel (except slabs): against the persistent launch, single steps, per step over 256- and 1024-step calls it was the faster for FP32 grids from
 // 64^2 to 8192^2 (2048^2 49.6 us against 52.2 persistent, 64^2 3.5 against
 // 6.1), for 16-bit grids with its 8-site walk (2048^2 FP16-delta 25.4 against
 // 30.8, 8192^2 372.7 against 384.8) and with a c2 field (4096^2 FP16-delta
@@ -490,6 +546,7 @@ extern "C" int lbm_step(lbm_t h, long long n) {
         }
         return lbm_batch_step(h->self_batch, n, nullptr);  // advances t and cur
     }
+    if (runs_resident(h, n)) return step_resident(h, n);
     const bool two = steps_in_pairs(h);
     const long long per = (two ? 2LL : 1LL) * kGraphLaunches;
     while (n >= per) {

@@ -89,6 +89,45 @@ Err plan_step2(int storage, int rnd, bool field, int nx, int ny, Step2Plan *out)
 Err launch_step2(const Step2Plan &p, int storage, const void *fin, void *fout, int nx, int ny,
                  size_t P, const Coef &c, int rnd, const uint32_t *tdev, uint32_t toff,
                  const float *a15f, cudaStream_t st);
+// All steps of a call in one launch with the state in shared memory
+// (lbm_resident.cu), for grids that fit.
+struct ResidentPlan {
+    bool ok = false;
+    int tx = 0, ty = 0;  // tiles in x and y, one block each
+    int T = 0;           // steps between exchanges of tile edges
+    int shape = 0;       // block shape (lbm_resident.cu)
+    int threads = 0;     // of a block
+    int lanes = 0;       // thread t has column t % lanes of band t / lanes
+    int pitch = 0;       // row pitch of a tile in shared memory
+    double us = 0;       // estimated time of a step
+};
+struct ResidentArgs {
+    void *buf[2];
+    int cur;             // buf[cur] holds the state
+    int nx, ny, tx, ty, T, lanes, pitch;
+    size_t P;
+    long long steps;
+    uint32_t t0;         // number of the first step
+    Coef c;
+    const float *a15f;
+    int drive;
+    double drive_amp, drive_period, rho0;
+    unsigned *flags;     // kResidentFlagWords words per tile
+    unsigned epoch;      // exchanges made by earlier launches on these flags
+    int *status;
+};
+constexpr int kResidentFlagWords = 32;  // a 128-byte line per tile
+// Exchanges of a launch of `steps` steps; the result is in buf[cur ^ 1] after an
+// even number of them, else in buf[cur].
+inline long long resident_exchanges(const ResidentPlan &p, long long steps) {
+    return (steps + p.T - 1) / p.T - 1;
+}
+using ResidentKernel = void (*)(ResidentArgs);
+ResidentKernel resident_kernel_f32(int rnd, bool field, int shape);
+ResidentKernel resident_kernel_f16(int rnd, bool field, int shape);
+ResidentKernel resident_kernel_bf16(int rnd, bool field, int shape);
+Err plan_resident(int nx, int ny, int sms, ResidentPlan *out);
+Err launch_resident(const ResidentPlan &p, int storage, int rnd, ResidentArgs a, cudaStream_t st);
 // The forward-difference gradient (lbm_set_gradient): FP32, one site per lane.
 Err launch_step_forward(const TileCfg &cfg, const void *fin, void *fout, int nx, int ny, size_t P,
                         const Coef &c, cudaStream_t st);
@@ -137,6 +176,10 @@ struct lbm_grid {
     // step calls may use it (not under a tile configuration of the caller's).
     vss::Step2Plan step2{};
     bool pairs = true;
+    // All steps of a call in one launch (small grids), and the exchanges made.
+    vss::ResidentPlan resident{};
+    unsigned *flags = nullptr;    // in scratch
+    unsigned epoch = 0;
     int rounding = 0;             // 1: stochastic rounding of 16-bit stores
     float *a15f = nullptr;        // spatially varying alpha: 1.5 alpha per site
     int grad = 0;                 // LBM_GRAD_CENTRAL or LBM_GRAD_FORWARD

@@ -1,0 +1,119 @@
+// Host side of the resident kernel (lbm_resident.cuh): the tiling of a grid and
+// its launch.
+#include "lbm_internal.h"
+
+namespace vss {
+
+namespace {
+
+struct Shape {
+    int threads, rows;
+};
+// Block shapes: at most `threads` threads of `rows` rows each, none of which spills
+// registers; the order is that of the kernels (resident_of).
+constexpr Shape kShapes[] = {{512, 1}, {512, 2}, {768, 2}, {768, 3}, {640, 4}, {512, 6}, {384, 10}};
+constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
+
+// Threads and row pitch of an extended tile of W columns with K rows a thread:
+// thread t has column t % Wt of band t / Wt.  K * pitch is Wt modulo 32, so the
+// 32 lanes of a warp touch 32 banks also where they span several bands; Wt is
+// W rounded up to what that needs (an idle column or three).
+inline int lanes_for(int W, int K) {
+    const int g = K & -K;  // the power of two in K
+    return (W + g - 1) / g * g;
+}
+inline int pitch_for(int W, int K) {
+    const int Wt = lanes_for(W, K);
+    int p = W;
+    while ((K * p - Wt) & 31) ++p;
+    return p;
+}
+
+bool fits(int k, int W, int H) {
+    const Shape s = kShapes[k];
+    const int Wt = lanes_for(W, s.rows);
+    return Wt <= s.threads && (s.threads / Wt) * s.rows >= H &&
+           pitch_for(W, s.rows) * H <= s.threads * s.rows;
+}
+
+// Threads of a block, in whole warps.
+int threads_for(int shape, int W, int H) {
+    const int bands = (H + kShapes[shape].rows - 1) / kShapes[shape].rows;
+    return (lanes_for(W, kShapes[shape].rows) * bands + 31) / 32 * 32;
+}
+
+int smem_of(int shape) { return 10 * kShapes[shape].threads * kShapes[shape].rows * 4; }
+
+}  // namespace
+
+// Time of a step in microseconds, fitted to measured launches (17 tilings of
+// grids from 400 x 4 to 600^2, within 20 %): two block barriers and the chain of a
+// site's arithmetic, the warps' rows, and an exchange (two passes through L2 and
+// the wait) shared by T steps.
+static double step_us(int shape, int W, int H, int hx, int hy, int T) {
+    const double warp_rows = threads_for(shape, W, H) / 32 * kShapes[shape].rows;
+    const int halo = W * H - (W - 2 * hx) * (H - 2 * hy);
+    return 0.16 + 0.018 * warp_rows + (hx || hy ? (2.4 + 0.0012 * halo) / T : 0.0);
+}
+
+// The tiling with the lowest estimate.  Grids of up to about 700^2 sites have one.
+Err plan_resident(int nx, int ny, int sms, ResidentPlan *out) {
+    *out = ResidentPlan{};
+    const long long most = 3900LL * sms;
+    if ((long long)nx * ny > most) return cudaSuccess;
+    double best = 1e30;
+    for (int tx = 1; tx <= sms && tx <= nx; ++tx)
+        for (int ty = 1; tx * ty <= sms && ty <= ny; ++ty) {
+            if ((long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty) > 3900) continue;
+            for (int T : {1, 2, 3, 4, 6, 8, 12, 16}) {
+                if (tx * ty == 1 && T > 1) break;
+                const int hx = tx > 1 ? 2 * T : 0, hy = ty > 1 ? 2 * T : 0;
+                // a tile's halo lies in its neighbours
+                if ((tx > 1 && nx / tx < hx) || (ty > 1 && ny / ty < hy)) break;
+                const int W = (nx + tx - 1) / tx + 2 * hx, H = (ny + ty - 1) / ty + 2 * hy;
+                bool any = false;
+                for (int k = 0; k < kNumShapes; ++k) {
+                    if (!fits(k, W, H)) continue;
+                    any = true;
+                    const double us = step_us(k, W, H, hx, hy, T);
+                    if (us >= best) continue;
+                    best = us;
+                    out->tx = tx;
+                    out->ty = ty;
+                    out->T = tx * ty == 1 ? 1 << 20 : T;
+                    out->shape = k;
+                    out->threads = threads_for(k, W, H);
+                    out->lanes = lanes_for(W, kShapes[k].rows);
+                    out->pitch = pitch_for(W, kShapes[k].rows);
+                    out->us = us;
+                }
+                if (!any) break;
+            }
+        }
+    out->ok = best < 1e30;
+    return cudaSuccess;
+}
+
+Err launch_resident(const ResidentPlan &p, int storage, int rnd, ResidentArgs a, cudaStream_t st) {
+    a.tx = p.tx;
+    a.ty = p.ty;
+    a.T = p.T;
+    a.lanes = p.lanes;
+    a.pitch = p.pitch;
+    const bool field = a.a15f != nullptr;
+    const ResidentKernel fn = storage == ST_F32   ? resident_kernel_f32(rnd, field, p.shape)
+                              : storage == ST_F16 ? resident_kernel_f16(rnd, field, p.shape)
+                                                  : resident_kernel_bf16(rnd, field, p.shape);
+    const int smem = smem_of(p.shape), tiles = p.tx * p.ty;
+    // (a host-side attribute of the kernel; setting it again is cheap)
+    Err e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    void *args[] = {(void *)&a};
+    if (tiles == 1)
+        return cudaLaunchKernel((const void *)fn, dim3(1), dim3(p.threads), args,
+                                (size_t)smem, st);
+    return cudaLaunchCooperativeKernel((const void *)fn, dim3(tiles),
+                                       dim3(p.threads), args, (size_t)smem, st);
+}
+
+}  // namespace vss

@@ -345,7 +345,8 @@ class Grid:
 
     def set_persistent(self, on):
         """True (long calls run one persistent launch), False (never), or
-        'auto' (the default: persistent for large 16-bit grids only)."""
+        'auto' (the default: one launch for grids that fit the SMs' shared
+        memory, the step kernel for the others)."""
         mode = 2 if on == "auto" else (1 if on else 0)
         _check(self.lib.lbm_set_persistent(self.h, mode), "lbm_set_persistent")
 
