@@ -108,22 +108,29 @@ static int *status_ptr(lbm_grid *h) { return reinterpret_cast<int *>(h->scratch 
 // Device step counter that seeds stochastic rounding inside graph replays.
 static uint32_t *step_ptr(lbm_grid *h) { return reinterpret_cast<uint32_t *>(h->scratch + 9); }
 
-// Waits for the grid's stream once and returns the status of the work on it:
-// the copies of the step kernels' status word and of the grid's own
-// persistent batch's status word to pinned host memory are queued first, so
-// one synchronisation serves the caller's results and the status.  A set
-// status word is cleared (stream-ordered) and returned as the error.
-static int sync_status(lbm_grid *h) {
-    int *hs = reinterpret_cast<int *>(h->host_out + 7);
-    CK(cudaMemcpyAsync(hs, status_ptr(h), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+// Word that the reductions count their blocks in.
+static unsigned *count_ptr(lbm_grid *h) { return reinterpret_cast<unsigned *>(h->scratch + 10); }
+// Pinned word that receives the status.
+static int *host_status_ptr(lbm_grid *h) { return reinterpret_cast<int *>(h->host_out + 7); }
+
+// Waits for the grid's stream once and returns the status of the work on it: the
+// step kernels' status word, which a kernel of the caller's has written to pinned
+// host memory (`queued`) or a copy queued here does, and the status word of the
+// grid's own persistent batch.  One synchronisation serves the caller's results
+// and the status.  A set status word is cleared (stream-ordered) and returned as
+// the error.
+static int sync_status(lbm_grid *h, bool queued = false) {
+    int *hs = host_status_ptr(h);
+    if (!queued)
+        CK(cudaMemcpyAsync(hs, status_ptr(h), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     if (h->self_batch) CK(batch_queue_status(h->self_batch, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     if (h->self_batch) {
         int rb = batch_status(h->self_batch);
         if (rb != LBM_OK) return fail(rb, "a barrier wait in the persistent step kernel ran out");
     }
-    if (*hs != 0) {
-        int st = *hs;
+    const int st = *(volatile int *)hs;
+    if (st != 0) {
         cudaMemsetAsync(status_ptr(h), 0, sizeof(int), h->stream);
         return fail(st, "a bounded wait in the step kernel ran out");
     }
@@ -600,15 +607,15 @@ extern "C" int lbm_moments(lbm_t h, double *rho, double *ux, double *uy, int on_
     size_t n = (size_t)h->nx * h->ny;
     if (on_device) {
         cudaError_t e = launch_moments(h->storage, h->buf[h->cur], h->nx, h->ny, h->P, h->rho0,
-                                       rho, ux, uy, h->stream);
+                                       rho, ux, uy, status_ptr(h), host_status_ptr(h), h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "lbm_moments kernel");
-        return sync_status(h);
+        return sync_status(h, true);
     }
     double *d = nullptr;
     CK(staging_alloc(h, &d, 3 * n * sizeof(double), h->stream));
     cudaError_t e = launch_moments(h->storage, h->buf[h->cur], h->nx, h->ny, h->P, h->rho0,
                                    rho ? d : nullptr, ux ? d + n : nullptr,
-                                   uy ? d + 2 * n : nullptr, h->stream);
+                                   uy ? d + 2 * n : nullptr, nullptr, nullptr, h->stream);
     if (e == cudaSuccess && rho)
         e = cudaMemcpyAsync(rho, d, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess && ux)
@@ -621,15 +628,17 @@ extern "C" int lbm_moments(lbm_t h, double *rho, double *ux, double *uy, int on_
     return sync_status(h);
 }
 
+static HostResults host_results(lbm_grid *h) {
+    return HostResults{h->scratch + 16, count_ptr(h), h->host_out, status_ptr(h),
+                       host_status_ptr(h)};
+}
+
 extern "C" int lbm_sums(lbm_t h, double *out3) {
     if (!h || !out3) return fail(LBM_EINVAL, "lbm_sums: NULL argument");
-    double *partials = h->scratch + 16;
-    cudaError_t e = launch_sums(h->storage, h->buf[h->cur], h->nx, h->ny, h->P, partials,
-                                h->scratch, h->stream);
+    cudaError_t e = launch_sums_host(h->storage, h->buf[h->cur], h->nx, h->ny, h->P,
+                                     host_results(h), h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "lbm_sums kernel");
-    CK(cudaMemcpyAsync(h->host_out, h->scratch, 3 * sizeof(double), cudaMemcpyDeviceToHost,
-                       h->stream));
-    int rs = sync_status(h);
+    int rs = sync_status(h, true);
     if (rs != LBM_OK) return rs;
     out3[0] = (double)h->nx * (double)h->ny * h->rho0 + h->host_out[0];
     out3[1] = h->host_out[1];
@@ -642,13 +651,10 @@ extern "C" int lbm_sums(lbm_t h, double *out3) {
 extern "C" int lbm_mode(lbm_t h, int field, int kx, int ky, double *out2) {
     if (!h || !out2 || field < 0 || field > 2)
         return fail(LBM_EINVAL, "lbm_mode: bad argument");
-    double *partials = h->scratch + 16;
     cudaError_t e = launch_mode(h->storage, h->buf[h->cur], h->nx, h->ny, h->P, h->rho0, field, kx,
-                                ky, partials, h->scratch, h->stream);
+                                ky, host_results(h), h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "lbm_mode kernel");
-    CK(cudaMemcpyAsync(h->host_out, h->scratch, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                       h->stream));
-    int rs = sync_status(h);
+    int rs = sync_status(h, true);
     if (rs != LBM_OK) return rs;
     out2[0] = h->host_out[0];
     out2[1] = h->host_out[1];

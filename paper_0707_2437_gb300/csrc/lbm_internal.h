@@ -142,8 +142,9 @@ Err launch_init(int storage, void *f, int nx, int ny, size_t P, double rho0, con
 // step just wrote; step number *tdev + toff (tdev may be NULL).
 Err launch_drive_x(int storage, void *f, int nx, int ny, size_t P, double rho0, double amp,
                    double period, const uint32_t *tdev, uint32_t toff, cudaStream_t st);
+// *status is copied to *host_status (pinned host memory; NULL: not).
 Err launch_moments(int storage, const void *f, int nx, int ny, size_t P, double rho0, double *rho,
-                   double *ux, double *uy, cudaStream_t st);
+                   double *ux, double *uy, const int *status, int *host_status, cudaStream_t st);
 // FP64 reductions: `partials` holds reduce_blocks(nx, ny) entries of the
 // output's width (at most kReduceBlocksMax); `out` (device) receives the
 // result values.
@@ -151,8 +152,20 @@ constexpr int kReduceBlocksMax = 1024;
 int reduce_blocks(int nx, int ny);
 Err launch_sums(int storage, const void *f, int nx, int ny, size_t P, double *partials,
                 double *out3, cudaStream_t st);
+// The same with the results in pinned host memory once `st` has been waited for,
+// and the status word beside them: `counter` is a word of zero, left at zero;
+// stream-ordered calls may share `partials` and it.
+struct HostResults {
+    double *partials;
+    unsigned *counter;
+    double *host_out;
+    const int *status;
+    int *host_status;
+};
+Err launch_sums_host(int storage, const void *f, int nx, int ny, size_t P, const HostResults &r,
+                     cudaStream_t st);
 Err launch_mode(int storage, const void *f, int nx, int ny, size_t P, double rho0, int field,
-                int kx, int ky, double *partials, double *out2, cudaStream_t st);
+                int kx, int ky, const HostResults &r, cudaStream_t st);
 
 bool valid_vec(int storage, int nx, int vec);
 

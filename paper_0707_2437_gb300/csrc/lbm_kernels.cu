@@ -422,16 +422,27 @@ Err launch_set_u32(uint32_t *p, uint32_t v, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// Element conversions from / to double (not on the hot path).
+// FP32 to FP64 by integer arithmetic, for kernels that keep the few FP64 lanes
+// (two per SM and clock) busy.  Normal values take it; zeros, subnormals, infinities
+// and NaNs take the conversion instruction.  Same results.
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), mag = u & 0x7fffffffu;
+    if (mag - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + 0x38000000u)),
+                                (int)(u << 29));
+    return (double)x;
+}
+
+// Element conversions from / to double.
 
 template <int S>
 __device__ __forceinline__ double ld_elem_d(const void *f, size_t idx) {
     if constexpr (S == ST_F32)
-        return (double)reinterpret_cast<const float *>(f)[idx];
+        return widen(reinterpret_cast<const float *>(f)[idx]);
     else if constexpr (S == ST_F16)
-        return (double)__half2float(reinterpret_cast<const __half *>(f)[idx]);
+        return widen(__half2float(reinterpret_cast<const __half *>(f)[idx]));
     else
-        return (double)__bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(f)[idx]);
+        return widen(__bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(f)[idx]));
 }
 
 template <int S>
@@ -444,15 +455,30 @@ __device__ __forceinline__ void st_elem_d(void *f, size_t idx, double v) {
         reinterpret_cast<__nv_bfloat16 *>(f)[idx] = __double2bfloat16(v);
 }
 
-__device__ __forceinline__ int wrapi(int a, int n) {
-    int r = a % n;
-    return r < 0 ? r + n : r;
+// Threads of the side kernels (initialisation, moments, Fourier sums): kSide a
+// block, `cols` of them side by side along a row (all of it if it is shorter), the
+// rest on the following rows, so that no thread divides by the row length.
+constexpr int kSide = 256;
+struct SideGeom {
+    int cols, par;      // columns and rows a block takes at a time
+    unsigned gx, gy;    // blocks
+};
+// gx covers every column; at most about `most` blocks, evenly loaded.
+static SideGeom side_geom(int nx, int ny, long long most, int widest = kSide) {
+    SideGeom g;
+    g.cols = nx < widest ? nx : widest;
+    g.par = kSide / g.cols;
+    const long long bx = ((long long)nx + g.cols - 1) / g.cols, by = ((long long)ny + g.par - 1) / g.par;
+    g.gx = (unsigned)bx;
+    const long long room = most / bx > 0 ? most / bx : 1;
+    const long long rounds = (by + room - 1) / room;
+    const long long gy = (by + rounds - 1) / rounds;
+    g.gy = (unsigned)(gy < 65535 ? gy : 65535);
+    return g;
 }
-
-// Weights and links in double for the FP64 side kernels.
-__device__ __forceinline__ double wd(int i) {
-    return i == 0 ? 4.0 / 9.0 : (i < 5 ? 1.0 / 9.0 : 1.0 / 36.0);
-}
+// Neighbouring indices, wrapped.
+__device__ __forceinline__ int before(int a, int n) { return a == 0 ? n - 1 : a - 1; }
+__device__ __forceinline__ int after(int a, int n) { return a + 1 == n ? 0 : a + 1; }
 
 template <int S>
 __device__ __forceinline__ float ld_elem_f(const void *f, size_t idx) {
@@ -481,22 +507,29 @@ __device__ __forceinline__ void st_elem_f(void *f, size_t idx, float v) {
 // drho = rho - rho0 is formed in FP64 (it can be far below FP32's resolution
 // of rho near 1).
 template <int S>
-__global__ void k_init(void *f, int nx, int ny, size_t P, double rho0, const double *rho,
-                       const double *ux, const double *uy) {
-    long long n = (long long)nx * ny;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-         s += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(s % nx), y = (int)(s / nx);
-        const double r = rho[s];
+__global__ void __launch_bounds__(kSide)
+    k_init(void *__restrict__ f, int nx, int ny, size_t P, double rho0, const double *__restrict__ rho,
+           const double *__restrict__ ux, const double *__restrict__ uy, int cols, int par) {
+    const int ty = threadIdx.x / cols;
+    const long long x_ = (long long)blockIdx.x * cols + threadIdx.x % cols;
+    if (ty >= par || x_ >= nx) return;
+    const int x = (int)x_, xm = before(x, nx), xp = after(x, nx);
+    // (unsigned: the last stride may pass 2^31)
+    for (unsigned y_ = blockIdx.y * par + ty; y_ < (unsigned)ny; y_ += gridDim.y * par) {
+        const int y = (int)y_;
+        const size_t r0 = (size_t)y * nx, rm = (size_t)before(y, ny) * nx,
+                     rp = (size_t)after(y, ny) * nx;
+        const double r = rho[r0 + x];
         const float dr = (float)(r - rho0);
         const float rf = (float)r;
-        const float u = (float)ux[s], v = (float)uy[s];
+        const float u = (float)ux[r0 + x], v = (float)uy[r0 + x];
         const float m15usq = -1.5f * __fmaf_rn(u, u, __fmul_rn(v, v));
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             const float eu = EXi(i) * u + EYi(i) * v;  // e components are 0 and +-1
             const float poly = __fmaf_rn(__fmul_rn(4.5f, eu), eu, __fmaf_rn(3.0f, eu, m15usq));
-            const size_t dst = (size_t)wrapi(y - EYi(i), ny) * nx + wrapi(x - EXi(i), nx);
+            const size_t dst = (EYi(i) > 0 ? rm : (EYi(i) < 0 ? rp : r0)) +
+                               (EXi(i) > 0 ? xm : (EXi(i) < 0 ? xp : x));
             st_elem_f<S>(f, (size_t)i * P + dst, __fmaf_rn(rf, poly, dr));
         }
     }
@@ -526,60 +559,69 @@ __global__ void k_drive_x(void *f, int nx, int ny, size_t P, double rho0, double
     }
 }
 
-// Moments (Section 2, Eq. 3) of the current state in FP64.
-template <int S>
-__device__ __forceinline__ void site_moments_d(const void *f, int nx, int ny, size_t P, int x,
-                                               int y, double rho0, double &dr, double &jx,
-                                               double &jy) {
-    dr = 0.0;
-    jx = 0.0;
-    jy = 0.0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        size_t src = (size_t)wrapi(y - EYi(i), ny) * nx + wrapi(x - EXi(i), nx);
-        double g = wd(i) * ld_elem_d<S>(f, (size_t)i * P + src);
-        dr += g;
-        jx += g * EXi(i);
-        jy += g * EYi(i);
-    }
-}
-
 // Moments (Section 2, Eq. 3) of every site, in FP32 arithmetic: drho = sum
 // w_i h_i and j = sum w_i h_i e_i of the pulled values, u = j / rho.  The
 // outputs are FP64 arrays with rho = rho0 + drho formed in FP64.  (The FP64
 // reductions below use FP64 per-site moments: their totals and Fourier
 // coefficients carry the accuracy of the mass checks and wave fits.)
+// rho0f: rho0 if it is an FP32 value, else 0.  Then FP32 rho = rho0 + drho needs no
+// FP64: FP64's sum is exact unless drho is below 2^-29 rho0, where both give rho0.
+// The grid's status word goes to the host with the results.
 template <int S>
-__global__ void k_moments(const void *f, int nx, int ny, size_t P, double rho0, double *rho,
-                          double *ux, double *uy) {
-    long long n = (long long)nx * ny;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-         s += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(s % nx), y = (int)(s / nx);
-        float dr = 0.f, jx = 0.f, jy = 0.f;
+__global__ void __launch_bounds__(kSide)
+    k_moments(const void *__restrict__ f, int nx, int ny, size_t P, double rho0, float rho0f,
+              double *__restrict__ rho, double *__restrict__ ux, double *__restrict__ uy, int cols,
+              int par, const int *status, int *host_status) {
+    if (host_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+        *host_status = *status;
+    const int ty = threadIdx.x / cols;
+    const long long x_ = (long long)blockIdx.x * cols + threadIdx.x % cols;
+    if (ty >= par || x_ >= nx) return;
+    const int x = (int)x_, xm = before(x, nx), xp = after(x, nx);
+    // Two rows at a time, so that eighteen loads are in flight.
+    for (unsigned y_ = blockIdx.y * par * 2 + ty; y_ < (unsigned)ny; y_ += gridDim.y * par * 2) {
+        float dr[2], jx[2], jy[2];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const size_t src = (size_t)wrapi(y - EYi(i), ny) * nx + wrapi(x - EXi(i), nx);
-            const float wi = i == 0 ? 4.0f / 9.0f : (i < 5 ? 1.0f / 9.0f : 1.0f / 36.0f);
-            const float g = __fmul_rn(wi, ld_elem_f<S>(f, (size_t)i * P + src));
-            dr = __fadd_rn(dr, g);
-            if (EXi(i)) jx = EXi(i) > 0 ? __fadd_rn(jx, g) : __fsub_rn(jx, g);
-            if (EYi(i)) jy = EYi(i) > 0 ? __fadd_rn(jy, g) : __fsub_rn(jy, g);
+        for (int u = 0; u < 2; ++u) {
+            const int y = (int)min(y_ + u * par, (unsigned)ny - 1u);
+            const size_t r0 = (size_t)y * nx, rm = (size_t)before(y, ny) * nx,
+                         rp = (size_t)after(y, ny) * nx;
+            dr[u] = jx[u] = jy[u] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const size_t src = (EYi(i) > 0 ? rm : (EYi(i) < 0 ? rp : r0)) +
+                                   (EXi(i) > 0 ? xm : (EXi(i) < 0 ? xp : x));
+                const float wi = i == 0 ? 4.0f / 9.0f : (i < 5 ? 1.0f / 9.0f : 1.0f / 36.0f);
+                const float g = __fmul_rn(wi, ld_elem_f<S>(f, (size_t)i * P + src));
+                dr[u] = __fadd_rn(dr[u], g);
+                if (EXi(i))
+                    jx[u] = EXi(i) > 0 ? __fadd_rn(jx[u], g) : __fsub_rn(jx[u], g);
+                if (EYi(i))
+                    jy[u] = EYi(i) > 0 ? __fadd_rn(jy[u], g) : __fsub_rn(jy[u], g);
+            }
         }
-        const double r = rho0 + (double)dr;
-        const float rf = (float)r;
-        if (rho) rho[s] = r;
-        if (ux) ux[s] = (double)__fdiv_rn(jx, rf);
-        if (uy) uy[s] = (double)__fdiv_rn(jy, rf);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (y_ + u * par >= (unsigned)ny) break;
+            const size_t o = (size_t)(y_ + u * par) * nx + x;
+            // (FP32's moves hide the conversions; the 16-bit kinds' do not)
+            auto wide = [](float q) { return S == ST_F32 ? (double)q : widen(q); };
+            const double r = rho0 + wide(dr[u]);
+            const float rf = rho0f != 0.f ? __fadd_rn(rho0f, dr[u]) : (float)r;
+            if (rho) rho[o] = r;
+            if (ux) ux[o] = wide(__fdiv_rn(jx[u], rf));
+            if (uy) uy[o] = wide(__fdiv_rn(jy[u], rf));
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
-// FP64 reductions in a fixed order: RB blocks of RT threads; thread k of block
-// b takes sites b*RT + k, then + RB*RT, ...; each block sums its threads in a
-// fixed tree; a second one-block kernel sums the block partials in order.
+// FP64 reductions in a fixed order: each thread sums its sites in order, each
+// block its threads in a fixed tree, and the block partials are summed in order
+// of the blocks: by the block that finishes last (counter: a word that the last
+// block leaves at zero), or by k_final.
 
-constexpr int RT = 256;
+constexpr int RT = kSide;
 constexpr int RB_MAX = kReduceBlocksMax;
 
 int reduce_blocks(int nx, int ny) {
@@ -588,22 +630,68 @@ int reduce_blocks(int nx, int ny) {
     return (int)(b < RB_MAX ? b : RB_MAX);
 }
 
+// Sum of v over the block's threads, in thread 0: a shuffle tree in each warp,
+// then the warps in order.
 template <int K>
-__device__ __forceinline__ void block_sum_store(double (&v)[K], double *out_block) {
-    __shared__ double sh[K][RT];
+__device__ __forceinline__ void block_sum(double (&v)[K]) {
+    __shared__ double sh[K][RT / 32];
 #pragma unroll
-    for (int k = 0; k < K; ++k) sh[k][threadIdx.x] = v[k];
-    __syncthreads();
-    for (int s = RT / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
+    for (int k = 0; k < K; ++k) {
 #pragma unroll
-            for (int k = 0; k < K; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + s];
-        }
-        __syncthreads();
+        for (int s = 16; s > 0; s >>= 1) v[k] += __shfl_down_sync(FULL, v[k], s);
+        if ((threadIdx.x & 31) == 0) sh[k][threadIdx.x >> 5] = v[k];
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) out_block[k] = sh[k][0];
+        for (int k = 0; k < K; ++k) {
+            v[k] = sh[k][0];
+#pragma unroll
+            for (int w = 1; w < RT / 32; ++w) v[k] += sh[k][w];
+        }
+    }
+    __syncthreads();
+}
+
+// Where a reduction's results go: device memory by k_final (counter NULL), or
+// pinned host memory by the last block, with the grid's status word.
+struct Results {
+    double *partials;
+    unsigned *counter;
+    double *host_out;
+    const int *status;
+    int *host_status;
+    double scale;
+};
+
+template <int K>
+__device__ __forceinline__ void finish_sums(double (&v)[K], const Results &r) {
+    const unsigned blocks = gridDim.x * gridDim.y;
+    const unsigned block = blockIdx.y * gridDim.x + blockIdx.x;
+    block_sum<K>(v);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) r.partials[(size_t)block * K + k] = v[k];
+    }
+    if (!r.counter) return;
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(r.counter, blocks - 1) == blocks - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = 0.0;
+    for (unsigned b = threadIdx.x; b < blocks; b += RT)
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] += __ldcg(r.partials + (size_t)b * K + k);
+    block_sum<K>(v);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) r.host_out[k] = v[k] * r.scale;
+        *r.host_status = *r.status;
     }
 }
 
@@ -617,52 +705,109 @@ __global__ void k_final(const double *partials, int nblocks, double *out) {
     }
 }
 
+// Grid totals do not depend on streaming (each plane is permuted), so the stored
+// planes are summed where they lie, each plane on its own, and weighted at the end.
 template <int S>
 __global__ void __launch_bounds__(RT)
-    k_sums(const void *f, int nx, int ny, size_t P, double *partials) {
+    k_sums(const void *__restrict__ f, int nx, int ny, size_t P, Results res) {
     long long n = (long long)nx * ny;
-    double v[3] = {0.0, 0.0, 0.0};
+    double p[9] = {};
     for (long long s = (long long)blockIdx.x * RT + threadIdx.x; s < n;
          s += (long long)gridDim.x * RT) {
-        // Grid totals do not depend on streaming (each plane is permuted), so
-        // the stored planes are summed where they lie.
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            double g = wd(i) * ld_elem_d<S>(f, (size_t)i * P + s);
-            v[0] += g;
-            v[1] += g * EXi(i);
-            v[2] += g * EYi(i);
+        for (int i = 0; i < 9; ++i) p[i] += ld_elem_d<S>(f, (size_t)i * P + s);
+    }
+    const double diag = (p[5] + p[7]) + (p[6] + p[8]), axis = (p[1] + p[3]) + (p[2] + p[4]);
+    double v[3];
+    v[0] = 4.0 / 9.0 * p[0] + 1.0 / 9.0 * axis + 1.0 / 36.0 * diag;
+    v[1] = 1.0 / 9.0 * (p[1] - p[3]) + 1.0 / 36.0 * ((p[5] - p[7]) - (p[6] - p[8]));
+    v[2] = 1.0 / 9.0 * (p[2] - p[4]) + 1.0 / 36.0 * ((p[5] - p[7]) + (p[6] - p[8]));
+    finish_sums<3>(v, res);
+}
+
+// Fourier coefficient sums of a field: sum over the sites of value * cos(phase) and
+// value * sin(phase), phase = 2 pi (kx x / nx + ky y / ny).  The phase factor is
+// the product of one of the column and one of the row: a thread sums its column's
+// values times the rows' factors (from a table a block computes for 256 rows at a
+// time; none if ky = 0) and multiplies by the column's once.  A block has 32
+// columns, so that their sines and cosines (80 FP64 instructions of 16 cycles a
+// warp) spread over the SMs.  Per site that leaves
+// the FP64 pipe (which bounds this kernel) 8 additions and products for the
+// density, scaled by 36 so that the weights are powers of two, and 1 or 2 for the
+// sum, against about 65 with sine and cosine per site and conversions: one 2048^2
+// read 910 -> 190 us.
+constexpr int kModeCols = 32;
+template <int S>
+__global__ void __launch_bounds__(RT)
+    k_mode(const void *__restrict__ f, int nx, int ny, size_t P, double rho0, int field, int kx,
+           int ky, int cols, int par, int rows_per_block, Results res) {
+    __shared__ double2 row_phase[RT], col_phase[kModeCols];
+    const int tx = threadIdx.x % cols, ty = threadIdx.x / cols;
+    const long long yb = (long long)blockIdx.y * rows_per_block;
+    const long long ye = min((long long)ny, yb + rows_per_block);
+    double v[2] = {0.0, 0.0};
+    for (long long c0 = (long long)blockIdx.x * cols; c0 < nx; c0 += (long long)gridDim.x * cols) {
+        const bool in = ty < par && c0 + tx < nx;
+        const int x = in ? (int)(c0 + tx) : 0;
+        const int xm = before(x, nx), xp = after(x, nx);
+        __syncthreads();
+        if (ty == 0 && in) {
+            // Phase reduced exactly before scaling.
+            const long long px = ((long long)kx * x) % nx;
+            double sn, cs;
+            sincospi(2.0 * ((double)px / nx), &sn, &cs);
+            col_phase[tx] = make_double2(cs, sn);
+        }
+        __syncthreads();
+        double ac = 0.0, as = 0.0;  // sum of value * row factor
+        for (long long y0 = yb; y0 < ye; y0 += RT) {
+            if (ky) {
+                __syncthreads();
+                if (y0 + threadIdx.x < ye) {
+                    const long long py = ((long long)ky * (y0 + threadIdx.x)) % ny;
+                    double sn, cs;
+                    sincospi(2.0 * ((double)py / ny), &sn, &cs);
+                    row_phase[threadIdx.x] = make_double2(cs, sn);
+                }
+                __syncthreads();
+            }
+            const int m_end = (int)min((long long)RT, ye - y0);
+            if (in)
+                for (int m = ty; m < m_end; m += par) {
+                    const int y = (int)(y0 + m);
+                    const size_t r0 = (size_t)y * nx, rm = (size_t)before(y, ny) * nx,
+                                 rp = (size_t)after(y, ny) * nx;
+                    double h[9];
+#pragma unroll
+                    for (int i = 0; i < 9; ++i)
+                        h[i] = ld_elem_d<S>(
+                            f, (size_t)i * P + (EYi(i) > 0 ? rm : (EYi(i) < 0 ? rp : r0)) +
+                                   (EXi(i) > 0 ? xm : (EXi(i) < 0 ? xp : x)));
+                    // 36 drho and 36 j (Eq. 3)
+                    const double a = h[5] - h[7], b = h[6] - h[8];
+                    double val = fma(16.0, h[0],
+                                     fma(4.0, (h[1] + h[3]) + (h[2] + h[4]),
+                                         (h[5] + h[7]) + (h[6] + h[8])));
+                    if (field) {
+                        const double j = field == 1 ? fma(4.0, h[1] - h[3], a - b)
+                                                    : fma(4.0, h[2] - h[4], a + b);
+                        val = j / fma(36.0, rho0, val);
+                    }
+                    if (ky) {
+                        ac = fma(val, row_phase[m].x, ac);
+                        as = fma(val, row_phase[m].y, as);
+                    } else {
+                        ac += val;
+                    }
+                }
+        }
+        if (in) {
+            const double2 p = col_phase[tx];
+            v[0] += ac * p.x - as * p.y;
+            v[1] += ac * p.y + as * p.x;
         }
     }
-    block_sum_store<3>(v, partials + (size_t)blockIdx.x * 3);
-}
-
-template <int S>
-__global__ void __launch_bounds__(RT)
-    k_mode(const void *f, int nx, int ny, size_t P, double rho0, int field, int kx, int ky,
-           double *partials) {
-    long long n = (long long)nx * ny;
-    double v[2] = {0.0, 0.0};
-    for (long long s = (long long)blockIdx.x * RT + threadIdx.x; s < n;
-         s += (long long)gridDim.x * RT) {
-        int x = (int)(s % nx), y = (int)(s / nx);
-        double dr, jx, jy;
-        site_moments_d<S>(f, nx, ny, P, x, y, rho0, dr, jx, jy);
-        double val = field == 0 ? dr : (field == 1 ? jx / (rho0 + dr) : jy / (rho0 + dr));
-        // Phase 2 pi (kx x / nx + ky y / ny), reduced exactly before scaling.
-        long long px = ((long long)kx * x) % nx;
-        long long py = ((long long)ky * y) % ny;
-        double ph = 2.0 * ((double)px / nx + (double)py / ny);
-        double sn, cs;
-        sincospi(ph, &sn, &cs);
-        v[0] += val * cs;
-        v[1] += val * sn;
-    }
-    block_sum_store<2>(v, partials + (size_t)blockIdx.x * 2);
-}
-
-__global__ void k_scale2(double *out, double s) {
-    if (threadIdx.x < 2) out[threadIdx.x] *= s;
+    finish_sums<2>(v, res);
 }
 
 // ---------------------------------------------------------------------------
@@ -686,16 +831,11 @@ __global__ void k_scale2(double *out, double s) {
             return cudaErrorInvalidValue;          \
     }
 
-static unsigned side_blocks(int nx, int ny) {
-    long long n = (long long)nx * ny;
-    long long b = (n + 255) / 256;
-    return (unsigned)(b < 4096 ? b : 4096);
-}
-
 Err launch_init(int storage, void *f, int nx, int ny, size_t P, double rho0, const double *rho,
                 const double *ux, const double *uy, cudaStream_t st) {
-    DISPATCH_S(storage, (k_init<S_><<<side_blocks(nx, ny), 256, 0, st>>>(f, nx, ny, P, rho0, rho,
-                                                                         ux, uy)));
+    const SideGeom g = side_geom(nx, ny, 1 << 20);  // a row a block: 4096^2 FP32 168 us of 209
+    DISPATCH_S(storage, (k_init<S_><<<dim3(g.gx, g.gy), kSide, 0, st>>>(f, nx, ny, P, rho0, rho, ux,
+                                                                        uy, g.cols, g.par)));
     return cudaGetLastError();
 }
 
@@ -709,27 +849,47 @@ Err launch_drive_x(int storage, void *f, int nx, int ny, size_t P, double rho0, 
 }
 
 Err launch_moments(int storage, const void *f, int nx, int ny, size_t P, double rho0, double *rho,
-                   double *ux, double *uy, cudaStream_t st) {
-    DISPATCH_S(storage, (k_moments<S_><<<side_blocks(nx, ny), 256, 0, st>>>(f, nx, ny, P, rho0,
-                                                                            rho, ux, uy)));
+                   double *ux, double *uy, const int *status, int *host_status, cudaStream_t st) {
+    // 4096^2: FP32 157 us (148 at the HBM peak), FP16 150; one row at a time 171, 189.
+    const SideGeom g = side_geom(nx, (ny + 1) / 2, 6144);
+    const float rho0f = (double)(float)rho0 == rho0 ? (float)rho0 : 0.f;
+    DISPATCH_S(storage, (k_moments<S_><<<dim3(g.gx, g.gy), kSide, 0, st>>>(
+                            f, nx, ny, P, rho0, rho0f, rho, ux, uy, g.cols, g.par, status,
+                            host_status)));
     return cudaGetLastError();
 }
 
 Err launch_sums(int storage, const void *f, int nx, int ny, size_t P, double *partials,
                 double *out3, cudaStream_t st) {
     int nb = reduce_blocks(nx, ny);
-    DISPATCH_S(storage, (k_sums<S_><<<nb, RT, 0, st>>>(f, nx, ny, P, partials)));
+    const Results res{partials, nullptr, nullptr, nullptr, nullptr, 1.0};
+    DISPATCH_S(storage, (k_sums<S_><<<nb, RT, 0, st>>>(f, nx, ny, P, res)));
     k_final<3><<<1, 32, 0, st>>>(partials, nb, out3);
     return cudaGetLastError();
 }
 
+Err launch_sums_host(int storage, const void *f, int nx, int ny, size_t P, const HostResults &r,
+                     cudaStream_t st) {
+    const Results res{r.partials, r.counter, r.host_out, r.status, r.host_status, 1.0};
+    DISPATCH_S(storage, (k_sums<S_><<<reduce_blocks(nx, ny), RT, 0, st>>>(f, nx, ny, P, res)));
+    return cudaGetLastError();
+}
+
 Err launch_mode(int storage, const void *f, int nx, int ny, size_t P, double rho0, int field,
-                int kx, int ky, double *partials, double *out2, cudaStream_t st) {
-    int nb = reduce_blocks(nx, ny);
-    DISPATCH_S(storage,
-               (k_mode<S_><<<nb, RT, 0, st>>>(f, nx, ny, P, rho0, field, kx, ky, partials)));
-    k_final<2><<<1, 32, 0, st>>>(partials, nb, out2);
-    k_scale2<<<1, 32, 0, st>>>(out2, 2.0 / ((double)nx * ny));
+                int kx, int ky, const HostResults &r, cudaStream_t st) {
+    // About 4 rows a thread or more; at most kReduceBlocksMax blocks.
+    SideGeom g = side_geom(nx, ny, kReduceBlocksMax, kModeCols);
+    if (g.gx > (unsigned)kReduceBlocksMax) g.gx = kReduceBlocksMax;  // (the kernel loops)
+    const long long least = 4LL * g.par;
+    long long rows = ((long long)ny + g.gy - 1) / g.gy;
+    if (rows < least) rows = least;
+    if (rows > ny) rows = ny;
+    g.gy = (unsigned)((ny + rows - 1) / rows);
+    // 2/N times the sum; the density's values come scaled by 36
+    const double scale = 2.0 / ((double)nx * ny) / (field == 0 ? 36.0 : 1.0);
+    const Results res{r.partials, r.counter, r.host_out, r.status, r.host_status, scale};
+    DISPATCH_S(storage, (k_mode<S_><<<dim3(g.gx, g.gy), kSide, 0, st>>>(
+                            f, nx, ny, P, rho0, field, kx, ky, g.cols, g.par, (int)rows, res)));
     return cudaGetLastError();
 }
 
