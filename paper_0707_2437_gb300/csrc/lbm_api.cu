@@ -283,14 +283,15 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double c2, double rho0,
         if (!h->buf[0]) e = cudaMalloc(&h->buf[0], bytes);
         if (e == cudaSuccess && !h->buf[1]) e = cudaMalloc(&h->buf[1], bytes);
     }
-    if (e == cudaSuccess) e = plan_resident(nx, ny, sms > 0 ? sms : 1, &h->resident);
     // Reduction partials and results, the status word and step counter, and
     // the counters of a resident launch's tiles.
     const size_t words = 3 * 1024 + 16;
-    const size_t flag_bytes =
-        sizeof(unsigned) * kResidentFlagWords * (size_t)(h->resident.tx * h->resident.ty);
+    h->sms = sms > 0 ? sms : 1;
+    const size_t flag_bytes = may_run_resident(nx, ny, h->sms)
+                                  ? sizeof(unsigned) * kResidentFlagWords * (size_t)h->sms
+                                  : 0;
     if (e == cudaSuccess) e = cudaMalloc(&h->scratch, sizeof(double) * words + flag_bytes);
-    h->flags = reinterpret_cast<unsigned *>(h->scratch + words);
+    if (flag_bytes) h->flags = reinterpret_cast<unsigned *>(h->scratch + words);
     // Stream-ordered, so that creating a grid does not wait for work running
     // on the legacy default stream.
     if (e == cudaSuccess) e = cudaMemsetAsync(h->scratch, 0, sizeof(double) * 16, h->stream);
@@ -428,11 +429,15 @@ static bool steps_in_pairs(const lbm_grid *h) {
 static const long long kResidentMin = 4;
 static const double kResidentMostStochastic = 3.6;
 
-static bool runs_resident(const lbm_grid *h, long long n) {
-    if (!h->resident.ok || !h->pairs || h->persistent != LBM_PERSISTENT_AUTO || h->slab ||
-        h->grad != LBM_GRAD_CENTRAL || n < kResidentMin ||
-        (h->rounding && h->resident.us > kResidentMostStochastic))
+static bool runs_resident(lbm_grid *h, long long n) {
+    if (!h->flags || !h->pairs || h->persistent != LBM_PERSISTENT_AUTO || h->slab ||
+        h->grad != LBM_GRAD_CENTRAL || n < kResidentMin)
         return false;
+    if (!h->resident_planned) {
+        if (plan_resident(h->nx, h->ny, h->sms, &h->resident) != cudaSuccess) return false;
+        h->resident_planned = true;
+    }
+    if (!h->resident.ok || (h->rounding && h->resident.us > kResidentMostStochastic)) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     return cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess &&
            cap == cudaStreamCaptureStatusNone;

@@ -126,6 +126,8 @@ using ResidentKernel = void (*)(ResidentArgs);
 ResidentKernel resident_kernel_f32(int rnd, bool field, int shape);
 ResidentKernel resident_kernel_f16(int rnd, bool field, int shape);
 ResidentKernel resident_kernel_bf16(int rnd, bool field, int shape);
+// Whether a grid is small enough to have a tiling; the tiling.
+bool may_run_resident(int nx, int ny, int sms);
 Err plan_resident(int nx, int ny, int sms, ResidentPlan *out);
 Err launch_resident(const ResidentPlan &p, int storage, int rnd, ResidentArgs a, cudaStream_t st);
 // The forward-difference gradient (lbm_set_gradient): FP32, one site per lane.
@@ -191,7 +193,9 @@ struct lbm_grid {
     bool pairs = true;
     // All steps of a call in one launch (small grids), and the exchanges made.
     vss::ResidentPlan resident{};
-    unsigned *flags = nullptr;    // in scratch
+    bool resident_planned = false;  // on the first call that may use it
+    unsigned *flags = nullptr;    // in scratch, for `sms` tiles; NULL on large grids
+    int sms = 1;
     unsigned epoch = 0;
     int rounding = 0;             // 1: stochastic rounding of 16-bit stores
     float *a15f = nullptr;        // spatially varying alpha: 1.5 alpha per site

@@ -1,5 +1,7 @@
 // Host side of the resident kernel (lbm_resident.cuh): the tiling of a grid and
 // its launch.
+#include <algorithm>
+
 #include "lbm_internal.h"
 
 namespace vss {
@@ -46,36 +48,50 @@ int smem_of(int shape) { return 10 * kShapes[shape].threads * kShapes[shape].row
 
 }  // namespace
 
-// Time of a step in microseconds, fitted to measured launches (17 tilings of
-// grids from 400 x 4 to 600^2, within 20 %): two block barriers and the chain of a
-// site's arithmetic, the warps' rows, and an exchange (two passes through L2 and
-// the wait) shared by T steps.
-static double step_us(int shape, int W, int H, int hx, int hy, int T) {
+// Time of a step in microseconds, fitted to measured launches of grids from 400 x 4
+// to 600^2: two block barriers and the chain of a site's arithmetic, the warps'
+// rows, and an exchange (two passes through L2 and the wait) shared by T steps.  An
+// exchange of tiles whose edges lie on 32-byte sectors takes a fifth less (256^2 in
+// 16 x 8 tiles 1.70 us a step, in 11 x 13 1.95; 8192 x 4 in 128 tiles 0.44, in 152
+// 0.48).
+static double exchange_us(long long halo, bool aligned) {
+    return (2.4 + 0.0012 * (double)halo) * (aligned ? 0.8 : 1.0);
+}
+static double step_us(int shape, int W, int H, int hx, int hy, int T, bool aligned) {
     const double warp_rows = threads_for(shape, W, H) / 32 * kShapes[shape].rows;
     const int halo = W * H - (W - 2 * hx) * (H - 2 * hy);
-    return 0.16 + 0.018 * warp_rows + (hx || hy ? (2.4 + 0.0012 * halo) / T : 0.0);
+    return 0.16 + 0.018 * warp_rows + (hx || hy ? exchange_us(halo, aligned) / T : 0.0);
 }
 
 // The tiling with the lowest estimate.  Grids of up to about 700^2 sites have one.
+bool may_run_resident(int nx, int ny, int sms) { return (long long)nx * ny <= 3900LL * sms; }
+
 Err plan_resident(int nx, int ny, int sms, ResidentPlan *out) {
     *out = ResidentPlan{};
-    const long long most = 3900LL * sms;
-    if ((long long)nx * ny > most) return cudaSuccess;
+    if (!may_run_resident(nx, ny, sms)) return cudaSuccess;
     double best = 1e30;
+    // (many tiles first: a good tiling early lets the bound below skip most others)
     for (int tx = 1; tx <= sms && tx <= nx; ++tx)
-        for (int ty = 1; tx * ty <= sms && ty <= ny; ++ty) {
-            if ((long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty) > 3900) continue;
+        for (int ty = std::min(sms / tx, ny); ty >= 1; --ty) {
+            if ((long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty) > 3900) break;
             for (int T : {1, 2, 3, 4, 6, 8, 12, 16}) {
                 if (tx * ty == 1 && T > 1) break;
                 const int hx = tx > 1 ? 2 * T : 0, hy = ty > 1 ? 2 * T : 0;
                 // a tile's halo lies in its neighbours
                 if ((tx > 1 && nx / tx < hx) || (ty > 1 && ny / ty < hy)) break;
                 const int W = (nx + tx - 1) / tx + 2 * hx, H = (ny + ty - 1) / ty + 2 * hy;
+                const long long sites = (long long)W * H;
+                if (sites > 3900) break;
+                const int own = (W - 2 * hx) * (H - 2 * hy);
+                const bool aligned = nx % tx == 0 && nx / tx % 8 == 0;
+                const double least = 0.16 + 0.018 * (double)sites / 32 +
+                                     (hx || hy ? exchange_us(sites - own, aligned) / T : 0.0);
+                if (least >= best) continue;  // no shape can be better
                 bool any = false;
                 for (int k = 0; k < kNumShapes; ++k) {
                     if (!fits(k, W, H)) continue;
                     any = true;
-                    const double us = step_us(k, W, H, hx, hy, T);
+                    const double us = step_us(k, W, H, hx, hy, T, aligned);
                     if (us >= best) continue;
                     best = us;
                     out->tx = tx;
