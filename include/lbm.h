@@ -118,7 +118,7 @@ int lbm_init(lbm_t h, const double *rho, const double *ux, const double *uy,
 
 /* Queues n >= 0 time steps of Eq. 5 (stream, moments, central grad(rho),
  * collide with force) on the handle's stream.  Calls either launch the step
- * kernel once per step or pair of steps (replayed from CUDA graphs, 32 launches
+ * kernel once per step, or every two or three steps (replayed from CUDA graphs, 32 launches
  * each), or run all n steps as one launch of one of two kinds.  Resident: the
  * grid's tiles stay in the SMs' shared memory, one block each, and exchange
  * their edges every few steps (bounded waits); grids of up to about 600^2
@@ -256,8 +256,7 @@ int lbm_set_state(lbm_t h, const void *src_host, long long t);
  * 32) when its tiles need between one and two waves; lbm_get_config reports
  * the configured 16.  In the default configuration, and after lbm_tune where
  * it measured faster, step calls on large grids (nx a multiple of 4 in FP32, of
- * 8 in 16-bit storage) take two steps per launch, an odd last step alone;
- * bitwise the same.  A configuration or pipeline set by the caller steps once
+ * 8 in 16-bit storage) take two or three steps per launch; bitwise the same.  A configuration or pipeline set by the caller steps once
  * per launch. */
 int lbm_set_config(lbm_t h, int vec, int rows, int warps);
 int lbm_get_config(lbm_t h, int *vec, int *rows, int *warps);
@@ -356,7 +355,7 @@ int lbm_batch_sync(lbm_batch_t b);
  * and the error returned).  Until one of them is called, a lockstep batch
  * whose tiles at 16 rows would fill less than 3/4 of the resident warps
  * (16 per SM) takes shorter tiles, down to 2 rows, as many as those warps
- * hold, and kind groups whose walk takes two steps per pass over memory (FP32
+ * hold, and kind groups whose walk takes two or three steps per pass over memory (FP32
  * grids with nx a multiple of 4, 16-bit grids under LBM_WALK16_AUTO with nx a
  * multiple of 8, unless their tiles are paired; slabs never) get the height
  * that balances their tiles over the resident warps.  The tuner times those too. */

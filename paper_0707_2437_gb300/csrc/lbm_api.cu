@@ -298,7 +298,7 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double c2, double rho0,
     if (e == cudaSuccess && flag_bytes)
         e = cudaMemsetAsync(h->flags, 0, flag_bytes, h->stream);
     if (e == cudaSuccess) e = prepare_step(storage, h->cfg);
-    if (e == cudaSuccess) e = plan_step2(storage, 0, false, nx, ny, &h->step2);
+    if (e == cudaSuccess) e = plan_fused(storage, 0, false, nx, ny, &h->fused);
     if (e == cudaSuccess) e = cudaMallocHost(&h->host_out, sizeof(double) * 8);
     if (e == cudaSuccess) e = cudaEventCreate(&h->ev[0]);
     if (e == cudaSuccess) e = cudaEventCreate(&h->ev[1]);
@@ -415,9 +415,9 @@ static cudaError_t launch_one(lbm_grid *h, int from) {
     return launch_one(h, from, nullptr, (uint32_t)h->t, h->stream);
 }
 
-// Whether step calls take two steps per launch.
-static bool steps_in_pairs(const lbm_grid *h) {
-    return h->pairs && h->step2.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL;
+// Whether step calls take several steps per launch.
+static bool steps_fused(const lbm_grid *h) {
+    return h->fuse && h->fused.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL;
 }
 
 // Whether n steps run as one launch with the state in shared memory.  From four
@@ -430,7 +430,7 @@ static const long long kResidentMin = 4;
 static const double kResidentMostStochastic = 3.6;
 
 static bool runs_resident(lbm_grid *h, long long n) {
-    if (!h->flags || !h->pairs || h->persistent != LBM_PERSISTENT_AUTO || h->slab ||
+    if (!h->flags || !h->fuse || h->persistent != LBM_PERSISTENT_AUTO || h->slab ||
         h->grad != LBM_GRAD_CENTRAL || n < kResidentMin)
         return false;
     if (!h->resident_planned) {
@@ -471,11 +471,11 @@ static int step_resident(lbm_grid *h, long long n) {
     return LBM_OK;
 }
 
-// One launch of two steps from buf[from] to buf[from ^ 1].
-static cudaError_t launch_two(lbm_grid *h, int from, const uint32_t *tdev, uint32_t toff,
-                              cudaStream_t st) {
-    return launch_step2(h->step2, h->storage, h->buf[from], h->buf[from ^ 1], h->nx, h->ny, h->P,
-                        h->coef, h->rounding, tdev, toff, h->a15f, st);
+// One launch of 1 .. h->fused.steps steps from buf[from] to buf[from ^ 1].
+static cudaError_t launch_pass(lbm_grid *h, int from, int steps, const uint32_t *tdev,
+                               uint32_t toff, cudaStream_t st) {
+    return launch_fused(h->fused, h->storage, h->buf[from], h->buf[from ^ 1], h->nx, h->ny, h->P,
+                        h->coef, steps, h->rounding, tdev, toff, h->a15f, st);
 }
 
 static const int kGraphLaunches = 32;  // launches in a graph, an even number
@@ -495,14 +495,14 @@ static const long long kLargeSites = 1LL << 20;
 static int build_graph(lbm_grid *h, int start) {
     cudaStream_t cs;
     CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    const bool two = steps_in_pairs(h);
+    const int per = steps_fused(h) ? h->fused.steps : 1;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         for (int k = 0; k < kGraphLaunches && e == cudaSuccess; ++k) {
             const int from = (start + k) & 1;
-            e = two ? launch_two(h, from, step_ptr(h), 2u * k, cs)
-                    : launch_one(h, from, step_ptr(h), (uint32_t)k, cs);
+            e = per > 1 ? launch_pass(h, from, per, step_ptr(h), (uint32_t)(per * k), cs)
+                        : launch_one(h, from, step_ptr(h), (uint32_t)k, cs);
         }
         cudaError_t e2 = cudaStreamEndCapture(cs, &g);
         if (e == cudaSuccess) e = e2;
@@ -559,8 +559,8 @@ extern "C" int lbm_step(lbm_t h, long long n) {
         return lbm_batch_step(h->self_batch, n, nullptr);  // advances t and cur
     }
     if (runs_resident(h, n)) return step_resident(h, n);
-    const bool two = steps_in_pairs(h);
-    const long long per = (two ? 2LL : 1LL) * kGraphLaunches;
+    const int each = steps_fused(h) ? h->fused.steps : 1;
+    const long long per = (long long)each * kGraphLaunches;
     while (n >= per) {
         if (!h->graph[h->cur]) {
             int rc = build_graph(h, h->cur);
@@ -573,9 +573,10 @@ extern "C" int lbm_step(lbm_t h, long long n) {
         h->t += per;  // an even number of launches leaves cur unchanged
     }
     while (n > 0) {
-        const int took = two && n >= 2 ? 2 : 1;
-        cudaError_t e = took == 2 ? launch_two(h, h->cur, nullptr, (uint32_t)h->t, h->stream)
-                                  : launch_one(h, h->cur);
+        const int took = n < each ? (int)n : each;
+        cudaError_t e = took > 1
+                            ? launch_pass(h, h->cur, took, nullptr, (uint32_t)h->t, h->stream)
+                            : launch_one(h, h->cur);
         if (e != cudaSuccess) return cuda_fail(e, "lbm_step kernel");
         h->cur ^= 1;
         h->t += took;
@@ -729,11 +730,11 @@ extern "C" int lbm_set_state(lbm_t h, const void *src_host, long long t) {
 // ---------------------------------------------------------------------------
 // Tile configuration and autotuner.
 
-// A configuration of the caller's describes single-step launches; the tuner
-// turns pairs of steps back on where they are the faster.
-static void set_pairs(lbm_grid *h, bool on) {
-    if (h->pairs != on) drop_graphs(h);
-    h->pairs = on;
+// A configuration of the caller's describes single-step launches; the tuner turns
+// passes of several steps back on where they are the faster.
+static void set_fuse(lbm_grid *h, bool on) {
+    if (h->fuse != on) drop_graphs(h);
+    h->fuse = on;
 }
 
 extern "C" int lbm_set_config(lbm_t h, int vec, int rows, int warps) {
@@ -755,7 +756,7 @@ extern "C" int lbm_set_config(lbm_t h, int vec, int rows, int warps) {
     h->cfg.rows = rows;
     h->cfg.warps = warps;
     h->cfg.fit_rows = false;
-    set_pairs(h, false);
+    set_fuse(h, false);
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }
@@ -771,7 +772,7 @@ extern "C" int lbm_set_pipeline(lbm_t h, int stages) {
         drop_graphs(h);
     }
     h->cfg.stages = stages;
-    set_pairs(h, false);
+    set_fuse(h, false);
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }
@@ -784,7 +785,7 @@ extern "C" int lbm_set_c2_field(lbm_t h, const double *c2, int on_device) {
     if (!c2) {
         if (h->a15f) cudaFree(h->a15f);
         h->a15f = nullptr;
-        CK(plan_step2(h->storage, h->rounding, false, h->nx, h->ny, &h->step2));
+        CK(plan_fused(h->storage, h->rounding, false, h->nx, h->ny, &h->fused));
         return LBM_OK;
     }
     if (h->rounding) return fail(LBM_EINVAL, "lbm_set_c2_field: needs nearest rounding");
@@ -802,7 +803,7 @@ extern "C" int lbm_set_c2_field(lbm_t h, const double *c2, int on_device) {
     }
     if (h->cfg.stages >= 2) h->cfg.stages = 0;
     if (!h->a15f) CK(cudaMalloc(&h->a15f, n * sizeof(float)));
-    CK(plan_step2(h->storage, h->rounding, true, h->nx, h->ny, &h->step2));
+    CK(plan_fused(h->storage, h->rounding, true, h->nx, h->ny, &h->fused));
     std::vector<double *> owned;
     double *d = nullptr;
     int rc = stage_field(h, c2, on_device, h->stream, &d, owned);
@@ -857,7 +858,7 @@ extern "C" int lbm_set_rounding(lbm_t h, int mode) {
         }
         if (h->cfg.stages >= 2) h->cfg.stages = 0;
     }
-    CK(plan_step2(h->storage, h->rounding, h->a15f != nullptr, h->nx, h->ny, &h->step2));
+    CK(plan_fused(h->storage, h->rounding, h->a15f != nullptr, h->nx, h->ny, &h->fused));
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }
@@ -916,11 +917,11 @@ static std::string tune_key(const lbm_grid *h) {
     return k.str();
 }
 
-// The cache file is a flat JSON object {"key": [vec, rows, warps, stages, pairs],
+// The cache file is a flat JSON object {"key": [vec, rows, warps, stages, fuse],
 // ...}; files without the fifth number mean 0.
 struct Tuned {
     TileCfg cfg;
-    int pairs = 0;  // 1: step calls run faster two steps per launch
+    int fuse = 0;  // 1: step calls run faster several steps per launch
 };
 static std::map<std::string, Tuned> read_cache(const char *path) {
     std::map<std::string, Tuned> m;
@@ -939,7 +940,7 @@ static std::map<std::string, Tuned> read_cache(const char *path) {
         Tuned t;
         TileCfg &c = t.cfg;
         if (sscanf(s.c_str() + lb, "[%d , %d , %d , %d , %d", &c.vec, &c.rows, &c.warps,
-                   &c.stages, &t.pairs) >= 4)
+                   &c.stages, &t.fuse) >= 4)
             m[key] = t;
         pos = rb + 1;
     }
@@ -955,7 +956,7 @@ static void write_cache(const char *path, const std::map<std::string, Tuned> &m)
     for (auto &kv : m) {
         const TileCfg &c = kv.second.cfg;
         fprintf(f, "  \"%s\": [%d, %d, %d, %d, %d]%s\n", kv.first.c_str(), c.vec, c.rows, c.warps,
-                c.stages, kv.second.pairs, (++k < m.size()) ? "," : "");
+                c.stages, kv.second.fuse, (++k < m.size()) ? "," : "");
     }
     fprintf(f, "}\n");
     fclose(f);
@@ -963,8 +964,8 @@ static void write_cache(const char *path, const std::map<std::string, Tuned> &m)
 }
 
 // Times `reps` launches from buf[cur] into the other buffer (the state itself
-// is not changed): single steps under configuration c, or (c NULL) two steps
-// per launch.
+// is not changed): single steps under configuration c, or (c NULL) passes of
+// several steps.
 static int time_cfg(lbm_grid *h, const TileCfg *c, int reps, float *ms_out) {
     TileCfg saved = h->cfg;
     cudaError_t e = cudaSuccess;
@@ -975,7 +976,7 @@ static int time_cfg(lbm_grid *h, const TileCfg *c, int reps, float *ms_out) {
     }
     auto launch = [&] {
         return c ? launch_one(h, h->cur)
-                 : launch_two(h, h->cur, nullptr, (uint32_t)h->t, h->stream);
+                 : launch_pass(h, h->cur, h->fused.steps, nullptr, (uint32_t)h->t, h->stream);
     };
     if (e == cudaSuccess) e = launch();  // warm-up
     if (e == cudaSuccess) e = cudaEventRecord(h->ev[0], h->stream);
@@ -1001,7 +1002,7 @@ extern "C" int lbm_tune(lbm_t h, const char *cache_path) {
             const TileCfg &c = it->second.cfg;
             int rc = lbm_set_config(h, c.vec, c.rows, c.warps);
             if (rc == LBM_OK) rc = lbm_set_pipeline(h, c.stages);
-            if (rc == LBM_OK) set_pairs(h, it->second.pairs != 0);
+            if (rc == LBM_OK) set_fuse(h, it->second.fuse != 0);
             return rc;
         }
     }
@@ -1044,16 +1045,16 @@ extern "C" int lbm_tune(lbm_t h, const char *cache_path) {
     int rc = lbm_set_config(h, best.vec, best.rows, best.warps);
     if (rc == LBM_OK) rc = lbm_set_pipeline(h, best.stages);
     if (rc != LBM_OK) return rc;
-    bool pairs = false;
-    if (h->step2.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL) {
+    bool fuse = false;
+    if (h->fused.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL) {
         float ms;
         rc = time_cfg(h, nullptr, reps, &ms);
         if (rc != LBM_OK) return rc;
-        pairs = ms < 2 * best_ms;
+        fuse = ms < h->fused.steps * best_ms;
     }
-    set_pairs(h, pairs);
+    set_fuse(h, fuse);
     if (cache_path) {
-        cache[key] = Tuned{best, pairs ? 1 : 0};
+        cache[key] = Tuned{best, fuse ? 1 : 0};
         write_cache(cache_path, cache);
     }
     return LBM_OK;

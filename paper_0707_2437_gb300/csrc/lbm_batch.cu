@@ -39,7 +39,7 @@ struct lbm_batch {
         BatchKernel kernel = nullptr;
         FlowKernel fkernel = nullptr;  // flow schedule
         int smem = 0;                  // dynamic shared memory per block
-        bool pairs = false;            // two steps per pass (the fused walk)
+        bool fused = false;            // several steps per pass (the fused walk)
         int rows = 0;                  // tile height
         int max_blocks_per_sm = 1;
     };
@@ -89,8 +89,8 @@ struct lbm_batch {
     int *h_nwork = nullptr;
     // Paired tiles (split walk) in the lockstep work-list.
     int paired = 0;
-    // Per grid, whether its passes take two steps (as of the work-list).
-    std::vector<char> pairs;
+    // Per grid, the steps of its passes (as of the work-list).
+    std::vector<int> per;
 };
 
 static int bfail(int code, const std::string &m) {
@@ -159,29 +159,29 @@ static cudaError_t resident_blocks(const void *fn, int smem, int *blocks) {
 }
 
 // Tile height of a lockstep group on the fused walk, from the grids' strips and
-// rows: a tile of r rows costs about r + 5 row steps (two rows of the first
-// step's collision and three pulled rows at each end).  With tiles of one
-// height a pass lasts ceil(tiles / warps) of them; in general the warps, which
-// take tiles as they finish others, are done within the mean plus one tile.
-// The lower of both bounds decides.  FP32 passes are bound by HBM and run
-// faster while the tiles in flight lie close together: at most 64 rows.
-static int pair_rows(const std::vector<std::pair<int, int>> &grids, long long warps, int most) {
-    double best = 0;
+// rows: a tile costs some row steps beyond its rows.  With tiles of one height a
+// pass lasts ceil(tiles / warps) of them; in general the warps, which take tiles as
+// they finish others, are done within the mean plus one tile.  The lower of both
+// bounds decides.
+// `fixed`: a height of the caller's (0: the best up to `most`).  *cost: row steps of
+// a pass.
+static int fused_rows(const std::vector<std::pair<int, int>> &grids, long long warps,
+                      int overhead, int most, int fixed, double *cost) {
     int rows = 2;
-    for (int r = 2; r <= most; r += r < 64 ? 1 : 4) {
+    for (int r = fixed ? fixed : 2; r <= (fixed ? fixed : most); r += r < 64 ? 1 : 4) {
         long long tiles = 0, work = 0;
         int tallest = 0;
         for (const auto &g : grids) {  // (strips, rows)
             const long long segs = (g.second + r - 1) / r;
             tiles += g.first * segs;
-            work += g.first * (g.second + 5 * segs);
+            work += g.first * (g.second + overhead * segs);
             tallest = std::max(tallest, std::min(r, g.second));
         }
-        const double even = (double)((tiles + warps - 1) / warps) * (tallest + 5);
-        const double mixed = (double)work / warps + (tallest + 5);
-        const double cost = std::min(even, mixed);
-        if (r == 2 || cost < best) {
-            best = cost;
+        const double even = (double)((tiles + warps - 1) / warps) * (tallest + overhead);
+        const double mixed = (double)work / warps + (tallest + overhead);
+        const double now = std::min(even, mixed);
+        if (*cost == 0 || now < *cost) {
+            *cost = now;
             rows = r;
         }
         if (tallest < r) break;  // every grid is one segment
@@ -195,7 +195,7 @@ static int build_worklist(lbm_batch *b) {
     std::vector<GridDesc> gd(ng);
     std::vector<Tile> tiles;
     b->paired = 0;
-    b->pairs.assign(ng, 0);
+    b->per.assign(ng, 1);
     b->groups.clear();
     bool slabs = false;
     for (size_t k = 0; k < ng; ++k) {
@@ -208,37 +208,33 @@ static int build_worklist(lbm_batch *b) {
         d.nx = g->nx;
         d.ny = g->ny;
         d.kind = kind_code(g->storage, batch_vec(b, g), g->rounding ? 1 : 0, g->a15f ? 1 : 0);
-        d.pairs = 0;
+        d.per = 1;
         d.c = g->coef;
         slabs = slabs || g->slab;
     }
     // Columns of a grid's tiles, and the rows it computes (all of them, or a
     // slab's own rows between its ghosts).
-    auto strip_cols = [&](size_t k, bool pairs) {
-        const int v = batch_vec(b, b->grids[k]);
-        return (pairs ? 30 : 32) * v;
-    };
-    auto strips = [&](size_t k, bool pairs) {
-        const int w = strip_cols(k, pairs);
-        return (b->grids[k]->nx + w - 1) / w;
+    auto strips = [&](size_t k, int per) {  // per: steps of a pass
+        const lbm_grid *g = b->grids[k];
+        const int w = per > 1 ? fused_cols(g->storage, per) : 32 * batch_vec(b, g);
+        return (g->nx + w - 1) / w;
     };
     auto computed_rows = [&](size_t k) { return b->grids[k]->ny - 2 * b->grids[k]->slab; };
     // Appends the tiles of grid k at a tile height.
-    auto add_tiles = [&](size_t k, int rows, bool pairs) {
+    auto add_tiles = [&](size_t k, int rows, int per) {
         lbm_grid *g = b->grids[k];
         GridDesc &d = gd[k];
-        b->pairs[k] = pairs;
-        d.pairs = pairs ? 1 : 0;
-        const int w = strip_cols(k, pairs);
+        b->per[k] = d.per = per;
+        const int w = per > 1 ? fused_cols(g->storage, per) : 32 * batch_vec(b, g);
         const int ylo = g->slab, yhi = g->ny - g->slab, nyc = yhi - ylo;
         d.tile0 = (int)tiles.size();
-        d.nstrips = strips(k, pairs);
+        d.nstrips = strips(k, per);
         d.nsegs = (nyc + rows - 1) / rows;
         d.ntile = d.nstrips * d.nsegs;
         // A pass reads two rows and columns per step beyond its tile: the next
         // segment or strip over suffices unless one of them is smaller (the
         // last one of a grid can be).
-        const int reach = pairs ? 4 : 2;
+        const int reach = 2 * d.per;
         const int last_rows = nyc - (d.nsegs - 1) * rows;
         const int last_cols = g->nx - (d.nstrips - 1) * w;
         d.dseg = (rows >= reach && last_rows >= reach) ? 1 : 2;
@@ -260,8 +256,9 @@ static int build_worklist(lbm_batch *b) {
         lbm_batch::Group gr;
         gr.fkernel = fc.fn;
         gr.smem = fc.smem;
-        gr.pairs = fc.pairs;
+        gr.fused = fc.fused;
         gr.rows = b->rows;
+        const int per_pass = fc.fused ? 2 : 1;
         BCK(resident_blocks((const void *)fc.fn, fc.smem, &gr.max_blocks_per_sm));
         if (gr.max_blocks_per_sm < 1) return bfail(LBM_ECUDA, "flow kernel cannot be resident");
         const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
@@ -272,23 +269,23 @@ static int build_worklist(lbm_batch *b) {
             // tiles than its share of the resident warps (the warps split
             // evenly between the grids) uses shorter tiles: a quarter as tall
             // in single steps; on the fused walk as tall as its share of warps
-            // asks for, from 4 rows (its reach, so that a tile waits for its
-            // neighbours only) to 48.
+            // asks for, from its reach (so that a tile waits for its neighbours
+            // only) to 48 rows.
             int rows = b->rows;
-            if (fc.pairs) {
+            if (fc.fused) {
                 if (b->fit_rows) {
                     const long long share = std::max<long long>(1, warps / (long long)ng);
                     const long long r =
-                        ((long long)strips(k, true) * computed_rows(k) + share - 1) / share;
+                        ((long long)strips(k, 2) * computed_rows(k) + share - 1) / share;
                     rows = (int)std::min<long long>(48, r);
                 }
-                rows = std::max(4, rows);
+                rows = std::max(2 * per_pass, rows);
             } else {
                 const long long tall =
-                    (long long)strips(k, false) * ((computed_rows(k) + rows - 1) / rows);
+                    (long long)strips(k, 1) * ((computed_rows(k) + rows - 1) / rows);
                 if (tall * (long long)ng < warps) rows = std::max(1, rows / 4);
             }
-            add_tiles(k, rows, fc.pairs);
+            add_tiles(k, rows, per_pass);
         }
         gr.count = (int)tiles.size();
         b->groups.push_back(gr);
@@ -315,7 +312,7 @@ static int build_worklist(lbm_batch *b) {
         auto tiles_at = [&](int r) {
             long long t = 0;
             for (size_t k = 0; k < ng; ++k)
-                t += (long long)strips(k, false) * ((computed_rows(k) + r - 1) / r);
+                t += (long long)strips(k, 1) * ((computed_rows(k) + r - 1) / r);
             return t;
         };
         if (4 * tiles_at(lock_rows) < 3 * wave)
@@ -352,17 +349,17 @@ static int build_worklist(lbm_batch *b) {
         long long n_all = 0, n_narrow = 0;
         for (size_t k : of_kind[kd]) {
             const long long n =
-                (long long)strips(k, false) * ((computed_rows(k) + lock_rows - 1) / lock_rows);
+                (long long)strips(k, 1) * ((computed_rows(k) + lock_rows - 1) / lock_rows);
             n_all += n;
             if (gd[k].nx <= kSplitCols) n_narrow += n;
         }
         return n_narrow > 0 && (double)n_narrow >= kSplitMinShare * (double)n_all;
     };
-    // The fused walk (two steps per pass) serves every group of one kind that
+    // The fused walk serves every group of one kind that
     // has it, but for the split walk's groups, slabs, and 16-bit walks the
     // caller chose.
     auto fuses = [&](int kd) {
-        if (!pair_kernel_for(kd).fn || splits(kd)) return false;
+        if (!fused_kernel_for(kd, 2).fn || splits(kd)) return false;
         for (size_t k : of_kind[kd])
             if (b->grids[k]->slab ||
                 (b->grids[k]->storage != ST_F32 && b->walk16 != LBM_WALK16_AUTO))
@@ -396,25 +393,41 @@ static int build_worklist(lbm_batch *b) {
         gr.begin = (int)ordered.size();
         tiles.clear();
         if (kinds_in.size() == 1 && fuses(kinds_in[0])) {
-            const PairChoice pc = pair_kernel_for(kinds_in[0]);
-            gr.kernel = pc.fn;
-            gr.smem = pc.smem;
-            gr.pairs = true;
-            BCK(resident_blocks((const void *)gr.kernel, gr.smem, &gr.max_blocks_per_sm));
-            if (gr.max_blocks_per_sm < 1)
-                return bfail(LBM_ECUDA, "batch kernel cannot be resident");
-            const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
-                                                 : gr.max_blocks_per_sm;
-            const long long warps = (long long)per * b->sms * kBatchWarps;
-            gr.rows = b->rows;
-            if (b->fit_rows) {
+            const std::vector<size_t> &members = of_kind[kinds_in[0]];
+            const int storage = b->grids[members[0]]->storage;
+            const bool field = b->grids[members[0]]->a15f != nullptr;
+            gr.fused = true;
+            double best = 1e300;
+            int per = 2;
+            long long warps = 1;
+            for (int steps = 2; steps <= fused_most_steps(storage, field); ++steps) {
+                const FusedChoice fc = fused_kernel_for(kinds_in[0], steps);
+                int bps = 0;
+                BCK(resident_blocks((const void *)fc.fn, fc.smem, &bps));
+                if (bps < 1) return bfail(LBM_ECUDA, "batch kernel cannot be resident");
+                const long long w =
+                    (long long)(b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, bps) : bps) *
+                    b->sms * kBatchWarps;
                 std::vector<std::pair<int, int>> shape;
-                for (size_t k : of_kind[kinds_in[0]])
-                    shape.push_back({strips(k, true), computed_rows(k)});
-                gr.rows = pair_rows(shape, warps,
-                                    b->grids[of_kind[kinds_in[0]][0]]->storage == ST_F32 ? 64 : 512);
+                for (size_t k : members) shape.push_back({strips(k, steps), computed_rows(k)});
+                double cost = 0;
+                const int rows = fused_rows(shape, w, fused_overhead(steps),
+                                            fused_most_rows(storage, steps),
+                                            b->fit_rows ? 0 : b->rows, &cost);
+                // A row step of three steps takes about 1.4 times as long as one of
+                // two here, in a launch per pass 1.22 times (nine 2048^2 grids, three
+                // steps and 296 rows 20.2 ms for 100, two and 56 rows 21.4).
+                cost /= steps == 3 ? 3 / 1.42 : 2.0;
+                if (cost >= best) continue;
+                best = cost;
+                per = steps;
+                gr.kernel = fc.fn;
+                gr.smem = fc.smem;
+                gr.max_blocks_per_sm = bps;
+                gr.rows = rows;
+                warps = w;
             }
-            for (size_t k : of_kind[kinds_in[0]]) add_tiles(k, gr.rows, true);
+            for (size_t k : members) add_tiles(k, gr.rows, per);
             ordered.insert(ordered.end(), tiles.begin(), tiles.end());
             split_tail(gr.begin, warps);
             gr.count = (int)ordered.size() - gr.begin;
@@ -422,7 +435,7 @@ static int build_worklist(lbm_batch *b) {
             return LBM_OK;
         }
         for (int kd : kinds_in)
-            for (size_t k : of_kind[kd]) add_tiles(k, lock_rows, false);
+            for (size_t k : of_kind[kd]) add_tiles(k, lock_rows, 1);
         // (grids in the caller's order, whatever their kinds)
         std::stable_sort(tiles.begin(), tiles.end(),
                          [](const Tile &x, const Tile &y) { return x.grid < y.grid; });
@@ -688,7 +701,7 @@ static int run_batch(lbm_batch *b, long long n, const long long *limits, bool ad
         for (int k = 0; k < ng; ++k) {
             long long s = b->h_limit[k];
             b->grids[k]->t += s;
-            if (passes_of(s, b->pairs[k]) & 1) b->grids[k]->cur ^= 1;
+            if (passes_of(s, b->per[k]) & 1) b->grids[k]->cur ^= 1;
         }
     }
     return LBM_OK;
@@ -792,21 +805,23 @@ static int apply_try(lbm_batch *b, const BatchTry &t) {
 
 // Milliseconds per 1e9 lattice updates of dry passes (the state is not
 // advanced: every grid writes its other buffer) under the work-list as built,
-// at its full occupancy.  A pass is one step, or two for a grid on the fused
-// walk; it does the same work as a pass inside a longer launch (the barriers
+// at its full occupancy.  A pass is one step, or several for a grid on the
+// fused walk; it does the same work as a pass inside a longer launch (the barriers
 // cost microseconds per millisecond pass).
 static int time_passes(lbm_batch *b, cudaEvent_t e0, cudaEvent_t e1, double *cost) {
     std::vector<long long> limits;
+    long long most = 1;
     double updates = 0;
     for (size_t k = 0; k < b->grids.size(); ++k) {
         const lbm_grid *g = b->grids[k];
-        limits.push_back(b->pairs[k] ? 2 : 1);
+        limits.push_back(b->per[k]);
+        most = std::max(most, limits.back());
         updates += (double)limits.back() * g->nx * (g->ny - 2 * g->slab);
     }
-    int rc = run_batch(b, 2, limits.data(), false);  // warm-up (and graph build)
+    int rc = run_batch(b, most, limits.data(), false);  // warm-up (and graph build)
     if (rc != LBM_OK) return rc;
     BCK(cudaEventRecord(e0, b->stream));
-    for (int k = 0; k < 4 && rc == LBM_OK; ++k) rc = run_batch(b, 2, limits.data(), false);
+    for (int k = 0; k < 4 && rc == LBM_OK; ++k) rc = run_batch(b, most, limits.data(), false);
     if (rc != LBM_OK) return rc;
     BCK(cudaEventRecord(e1, b->stream));
     BCK(cudaEventSynchronize(e1));
@@ -826,15 +841,15 @@ static int tune_candidates(lbm_batch *b, cudaEvent_t e0, cudaEvent_t e1, BatchTr
         int rc = lbm_batch_set_walk16(b, walk);
         if (rc != LBM_OK) return rc;
         std::vector<BatchKernel> ks;
-        bool pairs = false;
+        bool fused = false;
         for (const auto &gr : b->groups) {
             ks.push_back(gr.kernel);
-            pairs = pairs || gr.pairs;
+            fused = fused || gr.fused;
         }
         if (std::find(seen.begin(), seen.end(), ks) != seen.end()) continue;  // same kernels
         seen.push_back(ks);
         for (int r : {0, 8, 12, 16, 24, 32}) {
-            if (r == 0 && !pairs) continue;
+            if (r == 0 && !fused) continue;
             double cost = 0;
             rc = apply_try(b, BatchTry{r, walk});
             if (rc == LBM_OK) rc = time_passes(b, e0, e1, &cost);

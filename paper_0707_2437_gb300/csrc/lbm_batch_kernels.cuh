@@ -20,7 +20,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_internal.h"
-#include "lbm_walk2.cuh"
+#include "lbm_fused.cuh"
 
 using namespace vss;
 
@@ -32,13 +32,13 @@ struct GridDesc {
     size_t P;
     int nx, ny;
     int kind;  // kind_code(storage, vec, stochastic rounding)
-    int pairs; // 1: a pass takes two steps (the fused walk), 0: one
+    int per;   // steps of a pass: several on the fused walk, else 1
     Coef c;
     // Tiles of the grid in the work-list (flow schedule): the first one, how
     // many per step (segment-major: t = segment * nstrips + strip), and how
     // many segments / strips on each side a tile's pass reads from (1, or 2
     // when a neighbouring segment or strip can be smaller than the pass's
-    // reach: two sites for one step, four for two).
+    // reach: two sites a step).
     int tile0, ntile, nstrips, nsegs, dseg, dstrip;
 };
 
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
 }
 
 // ---------------------------------------------------------------------------
-// Flow schedule: every grid advances its own passes (a step, or two steps for
+// Flow schedule: every grid advances its own passes (a step, or several for
 // grids on the fused walk), with no barrier across the batch.  Each grid hands out tickets m = k * ntile + t (step k, tile t)
 // from its own counter, in step order.  A warp holding (k, t) waits until
 // every tile its step reads from or overwrites (the tiles within dseg
@@ -328,12 +328,12 @@ __device__ __forceinline__ bool flow_wait(const GridDesc &g, const int *prog, in
     return true;
 }
 
-// Passes a grid takes for `steps` steps, and whether pass k of them takes two.
-__host__ __device__ inline long long passes_of(long long steps, int pairs) {
-    return pairs ? (steps + 1) / 2 : steps;
+// Passes a grid takes for `steps` steps, `per` a pass.
+__host__ __device__ inline long long passes_of(long long steps, int per) {
+    return (steps + per - 1) / per;
 }
 
-// The flow loop of one warp; run_tile(g, par, tile, step, two) runs a tile.
+// The flow loop of one warp; run_tile(g, par, tile, step, steps) runs a tile.
 template <class RunTile>
 __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, int ngrids,
                                           const Tile *__restrict__ tiles,
@@ -365,7 +365,7 @@ __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, in
                     const int cand = (int)((start + (unsigned)j) % (unsigned)ngrids);
                     const GridDesc &G = grids[cand];
                     const unsigned long long total =
-                        (unsigned long long)passes_of(limit[cand], G.pairs) *
+                        (unsigned long long)passes_of(limit[cand], G.per) *
                         (unsigned long long)G.ntile;
                     volatile unsigned long long *c = ctl + (size_t)cand * kFlowCtlWords;
                     const unsigned long long taken = c[0];
@@ -415,9 +415,9 @@ __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, in
             const int seg = ti / g.nstrips, strip = ti % g.nstrips;
             if (!flow_wait(g, prog, seg, strip, k, status, timeout_ns)) return;
             const Tile t = tiles[g.tile0 + ti];
-            const uint32_t done = (uint32_t)k << g.pairs;  // steps before this pass
-            run_tile(g, (parity0[gsel] + k) & 1, t, t0[gsel] + done,
-                     g.pairs && limit[gsel] - (long long)done >= 2);
+            const long long done = (long long)k * g.per;  // steps before this pass
+            run_tile(g, (parity0[gsel] + k) & 1, t, t0[gsel] + (uint32_t)done,
+                     (int)min((long long)g.per, limit[gsel] - done));
         }
         // Publish: the tile's stores before its completed-step count.
         __threadfence();
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
            const uint32_t *__restrict__ t0, unsigned long long *ctl, int *prog, unsigned *glob,
            const int *__restrict__ nwork_p, int *status, unsigned long long timeout_ns) {
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
-              timeout_ns, [](const GridDesc &g, int par, const Tile &t, uint32_t step, bool) {
+              timeout_ns, [](const GridDesc &g, int par, const Tile &t, uint32_t step, int) {
                   any_tile(g, par, t, step);
               });
 }
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
                unsigned *glob, const int *__restrict__ nwork_p, int *status,
                unsigned long long timeout_ns) {
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
-              timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t, bool) {
+              timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t, int) {
                   Walker<S, 4, LD_CG> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P, t.x0);
                   const Coef c = g.c;
                   if constexpr (PD == 2)
@@ -462,31 +462,32 @@ __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
               });
 }
 
-// One tile of the fused walk: two steps, or a grid's odd last one.
-template <int S, int RND, int VA>
-__device__ __forceinline__ void pair_tile(const GridDesc &g, int par, const Tile &t, uint32_t step,
-                                          bool two, uint4 *buf) {
+// One tile of the fused walk: a pass, or what is left of a grid's steps.
+template <int S, int RND, int VA, int TS>
+__device__ __forceinline__ void fused_tile(const GridDesc &g, int par, const Tile &t, uint32_t step,
+                                           int steps, uint4 *buf) {
     const Coef c = g.c;
-    Walker2<S, LD_CG, RND, VA> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P, t.x0);
+    FusedWalk<S, LD_CG, RND, VA, TS> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P, t.x0);
     if constexpr (VA) w.a15f = g.a15f;
     if constexpr (RND) w.set_step(step);
-    w.run(t.y0, t.y1, t.dir, two, c, buf);
+    w.run(t.y0, t.y1, t.dir, steps, c, buf);
 }
 
-// Flow kernel for a batch of one kind of grids on the fused walk.
+// Flow kernel for a batch of one kind of grids on the fused walk (two steps a
+// pass: the flow schedule wants short tiles).
 template <int S, int RND, int VA>
 __global__ void __launch_bounds__(32 * kBatchWarps, 2)
-    k_flow_pairs(const GridDesc *__restrict__ grids, int ngrids, const Tile *__restrict__ tiles,
+    k_flow_fused(const GridDesc *__restrict__ grids, int ngrids, const Tile *__restrict__ tiles,
                  const long long *__restrict__ limit, const int *__restrict__ parity0,
                  const uint32_t *__restrict__ t0, unsigned long long *ctl, int *prog,
                  unsigned *glob, const int *__restrict__ nwork_p, int *status,
                  unsigned long long timeout_ns) {
     extern __shared__ uint4 walk_smem[];
-    uint4 *buf = walk_smem + (threadIdx.x >> 5) * walk2_vecs<S, VA>();
+    uint4 *buf = walk_smem + (threadIdx.x >> 5) * fused_vecs<S, VA, 2>();
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
               timeout_ns,
-              [&](const GridDesc &g, int par, const Tile &t, uint32_t step, bool two) {
-                  pair_tile<S, RND, VA>(g, par, t, step, two, buf);
+              [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int steps) {
+                  fused_tile<S, RND, VA, 2>(g, par, t, step, steps, buf);
               });
 }
 
@@ -502,15 +503,15 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 2)
                unsigned *glob, const int *__restrict__ nwork_p, int *status,
                unsigned long long timeout_ns) {
     extern __shared__ uint4 walk_smem[];
-    static_assert(walk2_vecs<ST_F32, 0>() == walk2_vecs<S2, 0>(), "one buffer size");
-    uint4 *buf = walk_smem + (threadIdx.x >> 5) * walk2_vecs<S2, 0>();
+    static_assert(fused_vecs<ST_F32, 0, 2>() == fused_vecs<S2, 0, 2>(), "one buffer size");
+    uint4 *buf = walk_smem + (threadIdx.x >> 5) * fused_vecs<S2, 0, 2>();
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
               timeout_ns,
-              [&](const GridDesc &g, int par, const Tile &t, uint32_t step, bool two) {
+              [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int steps) {
                   if (g.kind == kind_code(ST_F32, 4, 0))
-                      pair_tile<ST_F32, 0, 0>(g, par, t, step, two, buf);
+                      fused_tile<ST_F32, 0, 0, 2>(g, par, t, step, steps, buf);
                   else
-                      pair_tile<S2, RND2, 0>(g, par, t, step, two, buf);
+                      fused_tile<S2, RND2, 0, 2>(g, par, t, step, steps, buf);
               });
 }
 
@@ -518,39 +519,39 @@ using FlowKernel = void (*)(const GridDesc *, int, const Tile *, const long long
                             const uint32_t *, unsigned long long *, int *, unsigned *,
                             const int *, int *, unsigned long long);
 
-// A kernel with its dynamic shared memory per block, and whether its grids
-// take two steps per pass.
+// A kernel with its dynamic shared memory per block, and whether it is one of
+// the fused walk.
 struct FlowChoice {
     FlowKernel fn;
     int smem;
-    bool pairs;
+    bool fused;
 };
-template <int S, int VA>
-constexpr int pair_smem() {
-    return kBatchWarps * walk2_vecs<S, VA>() * 16;
+template <int S, int VA, int TS>
+constexpr int fused_smem() {
+    return kBatchWarps * fused_vecs<S, VA, TS>() * 16;
 }
 
 // The flow kernel for a batch's kinds: the fused walks when all grids share
-// one kind that has it, or FP32 and one such 16-bit kind (`pairs`: allowed);
+// one kind that has it, or FP32 and one such 16-bit kind (`fuse`: allowed);
 // a specialised single-step kernel when all share another walk, else the
 // general k_flow.
-FlowChoice flow_kernel_for(const std::vector<int> &kinds, int walk16, bool pairs) {
+FlowChoice flow_kernel_for(const std::vector<int> &kinds, int walk16, bool fuse) {
     bool same = true;
     for (int k : kinds) same = same && k == kinds[0];
-    if (!kinds.empty() && same && pairs) {
+    if (!kinds.empty() && same && fuse) {
         switch (kinds[0]) {
             case kind_code(ST_F32, 4, 0):
-                return {k_flow_pairs<ST_F32, 0, 0>, pair_smem<ST_F32, 0>(), true};
+                return {k_flow_fused<ST_F32, 0, 0>, fused_smem<ST_F32, 0, 2>(), true};
             case kind_code(ST_F32, 4, 0, 1):
-                return {k_flow_pairs<ST_F32, 0, 1>, pair_smem<ST_F32, 1>(), true};
+                return {k_flow_fused<ST_F32, 0, 1>, fused_smem<ST_F32, 1, 2>(), true};
             case kind_code(ST_F16, 8, 0):
-                return {k_flow_pairs<ST_F16, 0, 0>, pair_smem<ST_F16, 0>(), true};
+                return {k_flow_fused<ST_F16, 0, 0>, fused_smem<ST_F16, 0, 2>(), true};
             case kind_code(ST_BF16, 8, 0):
-                return {k_flow_pairs<ST_BF16, 0, 0>, pair_smem<ST_BF16, 0>(), true};
+                return {k_flow_fused<ST_BF16, 0, 0>, fused_smem<ST_BF16, 0, 2>(), true};
             case kind_code(ST_F16, 8, 1):
-                return {k_flow_pairs<ST_F16, 1, 0>, pair_smem<ST_F16, 0>(), true};
+                return {k_flow_fused<ST_F16, 1, 0>, fused_smem<ST_F16, 0, 2>(), true};
             case kind_code(ST_BF16, 8, 1):
-                return {k_flow_pairs<ST_BF16, 1, 0>, pair_smem<ST_BF16, 0>(), true};
+                return {k_flow_fused<ST_BF16, 1, 0>, fused_smem<ST_BF16, 0, 2>(), true};
             default:
                 break;
         }
@@ -569,14 +570,14 @@ FlowChoice flow_kernel_for(const std::vector<int> &kinds, int walk16, bool pairs
     }
     // FP32 (4 sites per lane) with one 16-bit kind of 8 sites per lane.
     int other = -1;
-    bool mix = pairs && !kinds.empty();
+    bool mix = fuse && !kinds.empty();
     for (int k : kinds) {
         if (k == kind_code(ST_F32, 4, 0)) continue;
         if (other == -1) other = k;
         mix = mix && k == other;
     }
     if (mix && other != -1) {
-        constexpr int smem = pair_smem<ST_F32, 0>();
+        constexpr int smem = fused_smem<ST_F32, 0, 2>();
         switch (other) {
             case kind_code(ST_F16, 8, 0):
                 return {k_flow_two<ST_F16, 0>, smem, true};
@@ -669,34 +670,34 @@ __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
     }
 }
 
-// The same for grids on the fused walk: a pass takes two steps of every grid
-// that has two left, and one of a grid with one left.  Bound as k_step2 is (HBM
-// in FP32, issue in the 16-bit kinds), at its occupancy and two rows of copies in
-// flight; half as many barriers as single steps.  Measured, lockstep, 100 steps a
-// call, single steps before and pairs now: nine 2048^2 grids FP32 93k -> 176k
-// MLUPS, FP16 170k -> 234k, BF16 with stochastic rounding 168k -> 209k, FP32 with
-// a c2 field 85k -> 168k; 512 uneven grids FP32 93k -> 178k, FP16 159k -> 210k,
-// half and half 115k -> 185k.  Flow schedule: nine 2048^2 FP32 92k -> 174k, FP16
-// 168k -> 240k; 512 uneven, half and half, 83k -> 138k.
-template <int S, int RND, int VA>
+// The same for grids on the fused walk: a pass takes several steps of every grid
+// that has them left, and the rest of a grid's steps at its end.  Bound as
+// k_step_fused is, at its occupancy and two rows of copies in flight; a half or a
+// third as many barriers as single steps.  Measured, lockstep, 100 steps a call,
+// single steps before and passes now: nine 2048^2 grids FP32 93k -> 187k MLUPS, FP16
+// 170k -> 234k, BF16 with stochastic rounding 168k -> 211k, FP32 with a c2 field 85k
+// -> 168k; 512 uneven grids FP32 93k -> 178k, FP16 159k -> 210k, half and half 115k
+// -> 185k.  Flow schedule: nine 2048^2 FP32 92k -> 174k, FP16 168k -> 238k; 512 uneven,
+// half and half, 83k -> 137k.
+template <int S, int RND, int VA, int TS>
 __global__ void __launch_bounds__(32 * kBatchWarps, 2)
-    k_batch_pairs(const GridDesc *__restrict__ grids, const Tile *__restrict__ tiles, int ntiles,
+    k_batch_fused(const GridDesc *__restrict__ grids, const Tile *__restrict__ tiles, int ntiles,
                   const long long *__restrict__ limit, const int *__restrict__ parity0,
                   const uint32_t *__restrict__ t0, long long nsteps, unsigned *bar, int *status,
                   unsigned long long timeout_ns) {
     extern __shared__ uint4 walk_smem[];
-    uint4 *buf = walk_smem + (threadIdx.x >> 5) * walk2_vecs<S, VA>();
-    const long long npass = (nsteps + 1) / 2;
+    uint4 *buf = walk_smem + (threadIdx.x >> 5) * fused_vecs<S, VA, TS>();
+    const long long npass = passes_of(nsteps, TS);
     for (long long k = 0; k < npass; ++k) {
         reset_counter(bar, k);
         unsigned *ctr = step_counter(bar, k);
         for (int ti = next_tile(ctr); ti < ntiles; ti = next_tile(ctr)) {
             const Tile t = tiles[ti];
-            const long long left = limit[t.grid] - 2 * k;
+            const long long left = limit[t.grid] - TS * k;
             if (left <= 0) continue;
             const int par = (parity0[t.grid] + (int)(k & 1)) & 1;
-            pair_tile<S, RND, VA>(grids[t.grid], par, t, t0[t.grid] + 2u * (uint32_t)k, left >= 2,
-                                  buf);
+            fused_tile<S, RND, VA, TS>(grids[t.grid], par, t, t0[t.grid] + (uint32_t)(TS * k),
+                                   (int)min((long long)TS, left), buf);
         }
         if (k + 1 < npass && !grid_barrier(bar, status, timeout_ns)) return;
     }
@@ -754,29 +755,31 @@ BatchKernel kernel_for(const std::vector<int> &kinds, int walk16, bool split = f
     return k_batch;
 }
 
-// Kinds with a fused walk, their lockstep kernel and its shared memory.
-struct PairChoice {
+// Kinds with a fused walk of `steps` steps, their lockstep kernel and its shared
+// memory.
+struct FusedChoice {
     BatchKernel fn;
     int smem;
 };
-PairChoice pair_kernel_for(int kind) {
+FusedChoice fused_kernel_for(int kind, int steps) {
     switch (kind) {
         case kind_code(ST_F32, 4, 0):
-            return {k_batch_pairs<ST_F32, 0, 0>, pair_smem<ST_F32, 0>()};
+            if (steps == 3) return {k_batch_fused<ST_F32, 0, 0, 3>, fused_smem<ST_F32, 0, 3>()};
+            return {k_batch_fused<ST_F32, 0, 0, 2>, fused_smem<ST_F32, 0, 2>()};
         case kind_code(ST_F32, 4, 0, 1):
-            return {k_batch_pairs<ST_F32, 0, 1>, pair_smem<ST_F32, 1>()};
+            return {k_batch_fused<ST_F32, 0, 1, 2>, fused_smem<ST_F32, 1, 2>()};
         case kind_code(ST_F16, 8, 0):
-            return {k_batch_pairs<ST_F16, 0, 0>, pair_smem<ST_F16, 0>()};
+            return {k_batch_fused<ST_F16, 0, 0, 2>, fused_smem<ST_F16, 0, 2>()};
         case kind_code(ST_BF16, 8, 0):
-            return {k_batch_pairs<ST_BF16, 0, 0>, pair_smem<ST_BF16, 0>()};
+            return {k_batch_fused<ST_BF16, 0, 0, 2>, fused_smem<ST_BF16, 0, 2>()};
         case kind_code(ST_F16, 8, 1):
-            return {k_batch_pairs<ST_F16, 1, 0>, pair_smem<ST_F16, 0>()};
+            return {k_batch_fused<ST_F16, 1, 0, 2>, fused_smem<ST_F16, 0, 2>()};
         case kind_code(ST_BF16, 8, 1):
-            return {k_batch_pairs<ST_BF16, 1, 0>, pair_smem<ST_BF16, 0>()};
+            return {k_batch_fused<ST_BF16, 1, 0, 2>, fused_smem<ST_BF16, 0, 2>()};
         case kind_code(ST_F16, 8, 0, 1):
-            return {k_batch_pairs<ST_F16, 0, 1>, pair_smem<ST_F16, 1>()};
+            return {k_batch_fused<ST_F16, 0, 1, 2>, fused_smem<ST_F16, 1, 2>()};
         case kind_code(ST_BF16, 8, 0, 1):
-            return {k_batch_pairs<ST_BF16, 0, 1>, pair_smem<ST_BF16, 1>()};
+            return {k_batch_fused<ST_BF16, 0, 1, 2>, fused_smem<ST_BF16, 1, 2>()};
         default:
             return {nullptr, 0};
     }

@@ -1,31 +1,30 @@
-// Two time steps per pass over memory: the fused strip walk.
+// Several time steps per pass over memory: the fused strip walk.
 //
-// A pass reads buffer A and writes the state two steps later into buffer B;
-// the state in between never leaves the SM.  One warp owns a strip of 30 V
-// columns (V = 16 bytes of elements per lane) and loads 32 V: the two outer
-// lanes hold halo columns.  A step reaches two columns (the pull, then the
-// central difference of the pulled density), two steps reach four, and V is 4
-// or 8, so the outer lanes' columns cover it and the strip needs no other halo
-// work: every shuffle stays inside the warp, and what the outer lanes compute
-// from their missing neighbours reaches no stored site.  Columns wrap lane by
-// lane, so nx must be a multiple of V.
+// A pass of T steps reads buffer A and writes the state T steps later into buffer
+// B; the states in between never leave the SM.  One warp owns a strip of columns
+// (V = 16 bytes of elements per lane) and loads halo lanes on both sides.  A step
+// reaches two columns (the pull, then the central difference of the pulled
+// density), T steps reach 2 T, which the halo lanes' columns cover (one lane a
+// side for T = 2, two for FP32's T = 3), so the strip needs no other halo work:
+// every shuffle stays inside the warp, and what the outer lanes compute from their
+// missing neighbours reaches no stored site.  Columns wrap lane by lane, so nx must
+// be a multiple of V.
 //
-// Down the rows the walk is a pipeline of two stages.  Each iteration
-//   1. takes a row of stored values, copied ahead into shared memory
-//      (cp.async), shifts it into the pulled row p and forms its drho;
-//   2. collides the row pulled before, which gives row q = p - 1 after step 1
-//      (all "-1" in walking order), rounded as a store would round it;
-//   3. assembles the pulled row s = q - 1 of step 2 from the rows q, q - 1 and
-//      q - 2 after step 1 and forms its drho;
-//   4. collides row s - 1, which gives the row after step 2, and stores it.
-// Two rows of copies are in flight.  The pulled row of step 1 waits for its
-// collision in registers, the one of step 2 and the six vectors of rows after
-// step 1 that a later row pulls wait in shared memory, at the lane that wrote
-// them.  A segment of n rows pulls n + 6 rows, collides n + 4 for step 1 and n
-// for step 2.
+// Down the rows the walk is a pipeline of T stages.  Each iteration takes a row of
+// stored values, copied ahead into shared memory (cp.async), and for each stage
+//   1. shifts it into the pulled row and forms its drho;
+//   2. collides the row the stage pulled before, which gives that row after the
+//      stage's step, rounded as a store would round it (the last stage stores it);
+//   3. assembles the next stage's pulled row, one row behind, from this row and the
+//      two before it.
+// Two rows of copies are in flight.  The first stage's pulled row waits for its
+// collision in registers; those of the later stages, and the six vectors of rows
+// between two stages that a later row pulls, wait in shared memory, at the lane
+// that wrote them.  A segment of n rows pulls n + 4 T - 2 rows; stage s = 0 .. T-1
+// collides n + 4 (T - 1 - s).
 //
-// The arithmetic is the Walker's, operation by operation, so a pass leaves
-// bit for bit the state that two single steps leave.
+// The arithmetic is the Walker's, operation by operation, so a pass leaves bit for
+// bit the state that T single steps leave.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -93,29 +92,52 @@ __device__ __forceinline__ void collide1(float (&h)[9], float dr, float gx, floa
     for (int i = 0; i < 9; ++i) h[i] = o[i];
 }
 
-template <int S>
-struct Walk2Geom {
-    static constexpr int V = (S == ST_F32) ? 4 : 8;  // sites per lane, 16 bytes
-    static constexpr int COLS = 30 * V;              // columns a strip stores
+// A walk of TS steps.  The 16-bit kinds take two steps a pass, which leaves them bound
+// by instruction issue.  FP32 takes two or three: at two it is bound by HBM and wants
+// tiles close together, at three by shared memory and issue, with more rows and
+// columns of halo, so it pays where tiles are tall (8192^2 174k against 203k MLUPS,
+// 1024^2 112k against 105k; four steps leave shared memory for six warps per SM and
+// run at 160k).  With a c2 field two: the rows of alpha values take the shared memory
+// of the third.
+template <int S, int TS>
+struct FusedGeom {
+    static constexpr int V = (S == ST_F32) ? 4 : 8;     // sites per lane, 16 bytes
+    static constexpr int HALO = (2 * TS + V - 1) / V;   // halo lanes a side
+    static constexpr int COLS = (32 - 2 * HALO) * V;    // columns a strip stores
 };
+constexpr int fused_vec(int storage) { return storage == ST_F32 ? 4 : 8; }
+constexpr int fused_cols(int storage, int steps) {
+    return storage == ST_F32 ? (steps == 3 ? FusedGeom<ST_F32, 3>::COLS : FusedGeom<ST_F32, 2>::COLS)
+                             : FusedGeom<ST_F16, 2>::COLS;
+}
+constexpr int fused_most_steps(int storage, bool field) {
+    return storage == ST_F32 && !field ? 3 : 2;
+}
+// Tallest tiles: FP32's passes of two steps are bound by HBM and run faster while the
+// tiles in flight lie close together (8192^2, 48 rows 385 us a step, 235 rows 419).
+constexpr int fused_most_rows(int storage, int steps) {
+    return storage == ST_F32 && steps == 2 ? 64 : 512;
+}
+// Row steps a tile costs beyond its rows (the pulls and collisions at its ends).
+constexpr int fused_overhead(int steps) { return 4 * steps - 3; }
 
-// Shared memory of one warp, in 16-byte vectors.
-template <int S, int VA>
-constexpr int walk2_vecs() {
-    // two landing rows, rows after step 1, the row that waits for step 2's
-    // collision; six rows of alpha values with a c2 field.
-    return 4 * 9 * 32 + (VA ? 6 * (Walk2Geom<S>::V / 4) * 32 : 0);
+// Shared memory of one warp, in 16-byte vectors: two landing rows; for each stage
+// after the first the rows held for it and the row that waits in it; with a c2
+// field the alpha values of the rows in flight.
+template <int S, int VA, int TS>
+constexpr int fused_vecs() {
+    return (2 + 2 * (TS - 1)) * 9 * 32 +
+           (VA ? (2 * TS + 2) * (FusedGeom<S, TS>::V / 4) * 32 : 0);
 }
 
-template <int S, int LD = LD_NC, int RND = 0, int VA = 0>
-struct Walker2 {
-    static constexpr int V = Walk2Geom<S>::V;
-    static constexpr int NW = Pack<S, V>::NW;
-    static constexpr int COLS = Walk2Geom<S>::COLS;
-    static_assert(NW == 4, "a lane holds one 16-byte vector per direction");
+template <int S, int LD, int RND, int VA, int TS>
+struct FusedWalk {
+    static constexpr int V = FusedGeom<S, TS>::V;
+    static constexpr int HALO = FusedGeom<S, TS>::HALO;
+    static_assert(Pack<S, V>::NW == 4, "a lane holds one 16-byte vector per direction");
     static_assert(RND == 0 || S != ST_F32, "stochastic rounding applies to 16-bit storage");
     using T = typename StoreT<S>::T;
-    uint32_t rkey1 = 0, rkey2 = 0;  // sr_step_key of the two steps
+    uint32_t rkey[TS] = {};  // sr_step_key of the steps
     const float *__restrict__ a15f = nullptr;
 
     const T *__restrict__ fin;
@@ -125,22 +147,22 @@ struct Walker2 {
     int lane, xl;
     bool act;
 
-    __device__ __forceinline__ Walker2(const void *fin_, void *fout_, int nx_, int ny_, size_t P_,
-                                       int x0)
+    __device__ __forceinline__ FusedWalk(const void *fin_, void *fout_, int nx_, int ny_, size_t P_,
+                                         int x0)
         : fin(reinterpret_cast<const T *>(fin_)),
           fout(reinterpret_cast<T *>(fout_)),
           nx(nx_),
           ny(ny_),
           P(P_) {
         lane = threadIdx.x & 31;
-        const int xu = x0 + (lane - 1) * V;  // the lane's columns, unwrapped
-        act = lane >= 1 && lane <= 30 && xu < nx;
+        const int xu = x0 + (lane - HALO) * V;  // the lane's columns, unwrapped
+        act = lane >= HALO && lane < 32 - HALO && xu < nx;
         xl = xu % nx;
         if (xl < 0) xl += nx;
     }
     __device__ __forceinline__ void set_step(uint32_t step) {
-        rkey1 = sr_step_key(step);
-        rkey2 = sr_step_key(step + 1u);
+#pragma unroll
+        for (int s = 0; s < TS; ++s) rkey[s] = sr_step_key(step + (uint32_t)s);
     }
 
     __device__ __forceinline__ static void take(uint32_t (&w)[9][4], const uint4 *s) {
@@ -280,18 +302,86 @@ struct Walker2 {
         for (int i = 0; i < 9; ++i) store_words<S, V>(dst + (size_t)i * P, w[i]);
     }
 
-    // Advances rows y0 .. y1-1 by two steps (two = false: by one), walking in
-    // direction dir.  `buf`: the warp's walk2_vecs() vectors.
-    __device__ __forceinline__ void run(int y0, int y1, int dir, bool two, const Coef &c,
+    // For stage s >= 1: the held rows, [0..2] e_y = 0 of the last row, [3..5] and
+    // [6..8] the late trio of the last two rows; the waiting row.  The alpha values.
+    __device__ __forceinline__ uint4 *held_of(uint4 *buf, int s) const {
+        return buf + (18 + 18 * (s - 1)) * 32 + lane;
+    }
+    __device__ __forceinline__ uint4 *wait_of(uint4 *buf, int s) const {
+        return buf + (27 + 18 * (s - 1)) * 32 + lane;
+    }
+    static constexpr int AV = (V / 4) * 32, AS = 2 * TS + 2;  // alpha vectors a slot, slots
+    __device__ __forceinline__ uint4 *alpha_of(uint4 *buf) const {
+        return buf + (18 + 18 * (TS - 1)) * 32 + lane;
+    }
+
+    // Iteration k of stage SG and the stages after it.  The stage pulls from iteration
+    // 4 SG on and collides from 4 SG + 2 on; u holds its waiting row.  d: drho per
+    // stage of the rows pulled two, one and zero iterations ago; row: the pulled row
+    // of the first stage, ia its alpha slot; back[s]: rows from it to stage s's.
+    template <int SG>
+    __device__ __forceinline__ void stage(int k, int dir, int steps, float sgn, const Coef &c,
+                                          int ia, uint4 *buf, uint32_t (&u)[9][4],
+                                          float (&d)[TS][3][V], int row, const int (&back)[TS]) const {
+        if (k < 4 * SG + 2) return;
+        const int as = ia - (2 * SG + 1);
+        int r = row - back[SG];
+        if (r < 0) r += ny;
+        collide(r, u, d[SG][1], d[SG][0], d[SG][2], sgn, c, rkey[SG],
+                alpha_of(buf) + (as < 0 ? as + AS : as) * AV);
+        if constexpr (SG + 1 < TS) {
+            if (SG + 1 < steps) {
+                // The row after this stage is in u.  The next stage's pulled row, one
+                // behind, takes e_y = 0 from the row before and, in walking order, one
+                // trio of an axis and two diagonals from this row and the other from
+                // two rows before.
+                uint4 *held = held_of(buf, SG + 1), *late = held + (3 + 3 * (k & 1)) * 32;
+                auto swap = [&](int i, uint4 *place) {
+                    const uint4 o = *place;
+                    *place = make_uint4(u[i][0], u[i][1], u[i][2], u[i][3]);
+                    u[i][0] = o.x;
+                    u[i][1] = o.y;
+                    u[i][2] = o.z;
+                    u[i][3] = o.w;
+                };
+                swap(0, held);
+                swap(1, held + 32);
+                swap(3, held + 64);
+                if (dir > 0) {
+                    swap(2, late);
+                    swap(5, late + 32);
+                    swap(6, late + 64);
+                } else {
+                    swap(4, late);
+                    swap(7, late + 32);
+                    swap(8, late + 64);
+                }
+                if (k >= 4 * (SG + 1)) {
+                    finish(u, d[SG + 1][2]);
+                    // This row waits; the one that waited is collided next.
+                    uint4 *wait = wait_of(buf, SG + 1);
+                    if (k >= 4 * (SG + 1) + 2) {
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) swap(i, wait + i * 32);
+                        stage<SG + 1>(k, dir, steps, sgn, c, ia, buf, u, d, row, back);
+                    } else {
+                        keep(wait, u);
+                    }
+                }
+                return;
+            }
+        }
+        store(r, u);
+    }
+
+    // Advances rows y0 .. y1-1 by `steps` (1 .. TS) steps, walking in direction
+    // dir.  `buf`: the warp's fused_vecs() vectors.
+    __device__ __forceinline__ void run(int y0, int y1, int dir, int steps, const Coef &c,
                                         uint4 *buf) const {
         uint4 *land = buf + lane;  // two slots
-        uint4 *wait2 = buf + 18 * 32 + lane;
-        uint4 *held = buf + 27 * 32 + lane;  // [0..2]: e_y = 0 of row q - 1;
-                                             // [3..5], [6..8]: the late trio of q - 1, q - 2
-        uint4 *al = buf + 36 * 32 + lane;
-        constexpr int AV = (V / 4) * 32;
+        uint4 *al = alpha_of(buf);
         const float sgn = dir > 0 ? 1.f : -1.f;
-        const int ext = two ? 3 : 1;
+        const int ext = 2 * steps - 1;
         const int K = y1 - y0 + 2 * ext;
         // The next row to copy (wrapped) and the rows before and after it.
         int q0 = (dir > 0 ? y0 - ext : y1 - 1 + ext) % ny;
@@ -309,36 +399,41 @@ struct Walker2 {
                 qm = (qm == 0) ? ny - 1 : qm - 1;
             }
         };
-        int row = q0;                // the pulled row
-        int r1 = 0, r2 = 0, r3 = 0;  // rows pulled one, two and three iterations ago
-
-        uint32_t wc[9][4] = {};  // the pulled row of step 1 that waits
-        float d2[V], d1[V], d0[V], e2[V], e1[V], e0[V];
+        int row = q0;  // the pulled row of the first stage
+        int back[TS];  // stage s collides the row pulled 2 s + 1 iterations ago
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
-            d2[v] = d1[v] = 0.f;
-            e2[v] = e1[v] = e0[v] = 0.f;
+        for (int j = 0; j < TS; ++j) {
+            back[j] = (2 * j + 1) * dir % ny;
+            if (back[j] < 0) back[j] += ny;
         }
-        int ia = 0;  // alpha slot of the pulled row, mod 6
+
+        uint32_t wc[9][4] = {};  // the first stage's waiting row
+        float d[TS][3][V];       // per stage: drho of the rows pulled two, one, zero ago
+#pragma unroll
+        for (int s = 0; s < TS; ++s)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+#pragma unroll
+                for (int v = 0; v < V; ++v) d[s][j][v] = 0.f;
+        int ia = 0;  // alpha slot of the pulled row, mod AS
         issue(qm, q0, qp, land, al);
         next();
         issue(qm, q0, qp, land + 9 * 32, al + AV);  // K >= 3
         next();
         for (int k = 0; k < K; ++k) {
-            uint32_t w[9][4];
+            uint32_t w[9][4], u[9][4];
             uint4 *slot = land + (k & 1) * 9 * 32;
             asm volatile("cp.async.wait_group 1;" ::: "memory");
             take(w, slot);
-            finish(w, d0);
+            finish(w, d[0][2]);
             // The words read from the landing row have been used (the
             // shuffles), so the next copy cannot overtake them.
             if (k + 2 < K) {
-                issue(qm, q0, qp, slot, al + (ia < 4 ? ia + 2 : ia - 4) * AV);
+                issue(qm, q0, qp, slot, al + (ia < AS - 2 ? ia + 2 : ia + 2 - AS) * AV);
                 next();
             } else {
                 asm volatile("cp.async.commit_group;" ::: "memory");  // keeps the count
             }
-            uint32_t u[9][4];
 #pragma unroll
             for (int i = 0; i < 9; ++i)
 #pragma unroll
@@ -346,66 +441,18 @@ struct Walker2 {
                     u[i][j] = wc[i][j];
                     wc[i][j] = w[i][j];
                 }
-            if (k >= 2) {
-                const uint4 *a1 = al + (ia == 0 ? 5 : ia - 1) * AV;
-                collide(r1, u, d1, d2, d0, sgn, c, rkey1, a1);
-                if (!two) {
-                    store(r1, u);
-                } else {
-                    // Row q after step 1 is in u.  The pulled row s = q - 1 of
-                    // step 2 takes e_y = 0 from row q - 1 and, in walking
-                    // order, one diagonal-and-axis trio from q and the other
-                    // from q - 2.
-                    uint4 *late = held + (3 + 3 * (k & 1)) * 32;
-                    auto swap = [&](int i, uint4 *slot) {
-                        const uint4 o = *slot;
-                        *slot = make_uint4(u[i][0], u[i][1], u[i][2], u[i][3]);
-                        u[i][0] = o.x;
-                        u[i][1] = o.y;
-                        u[i][2] = o.z;
-                        u[i][3] = o.w;
-                    };
-                    swap(0, held);
-                    swap(1, held + 32);
-                    swap(3, held + 64);
-                    if (dir > 0) {
-                        swap(2, late);
-                        swap(5, late + 32);
-                        swap(6, late + 64);
-                    } else {
-                        swap(4, late);
-                        swap(7, late + 32);
-                        swap(8, late + 64);
-                    }
-                    if (k >= 4) {
-                        finish(u, e0);
-                        if (k >= 6) {
-                            uint32_t z[9][4];
-                            take(z, wait2);
-                            keep(wait2, u);
-                            const uint4 *a2 = al + (ia >= 3 ? ia - 3 : ia + 3) * AV;
-                            collide(r3, z, e1, e2, e0, sgn, c, rkey2, a2);
-                            store(r3, z);
-                        } else {
-                            keep(wait2, u);
-                        }
-                    }
-                }
-            }
+            stage<0>(k, dir, steps, sgn, c, ia, buf, u, d, row, back);
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                d2[v] = d1[v];
-                d1[v] = d0[v];
-                e2[v] = e1[v];
-                e1[v] = e0[v];
-            }
-            r3 = r2;
-            r2 = r1;
-            r1 = row;
+            for (int s = 0; s < TS; ++s)
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    d[s][0][v] = d[s][1][v];
+                    d[s][1][v] = d[s][2][v];
+                }
             row += dir;
             if (row < 0) row += ny;
             if (row >= ny) row -= ny;
-            ia = ia == 5 ? 0 : ia + 1;
+            ia = ia == AS - 1 ? 0 : ia + 1;
         }
     }
 };

@@ -76,18 +76,19 @@ Err launch_step(int storage, const TileCfg &cfg, const void *fin, void *fout, in
 // Warps of `fn` (blocks of `warps` warps, `smem` bytes of dynamic shared memory)
 // resident on the current device; 0 if the query fails.
 long long resident_warps(const void *fn, int warps, int smem);
-// Two steps per launch (lbm_step2.cu): the tiles of a grid's passes, and one
-// launch.  ok is false where the fused walk does not apply (nx not a multiple
-// of its 16-byte lanes).  Uniform alpha with either rounding, or a c2 field
-// with nearest rounding.
-struct Step2Plan {
+// Several steps per launch (lbm_step_fused.cu): the tiles of a grid's passes, and
+// one launch of 1 .. p.steps steps.  ok is false where the fused walk does not apply
+// (nx not a multiple of its 16-byte lanes) or single steps are the faster.  Uniform
+// alpha with either rounding, or a c2 field with nearest rounding.
+struct FusedPlan {
     bool ok = false;
+    int steps = 1;  // of a pass
     int rows = 0, nstrips = 0;
     long long ntiles = 0;
 };
-Err plan_step2(int storage, int rnd, bool field, int nx, int ny, Step2Plan *out);
-Err launch_step2(const Step2Plan &p, int storage, const void *fin, void *fout, int nx, int ny,
-                 size_t P, const Coef &c, int rnd, const uint32_t *tdev, uint32_t toff,
+Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out);
+Err launch_fused(const FusedPlan &p, int storage, const void *fin, void *fout, int nx, int ny,
+                 size_t P, const Coef &c, int steps, int rnd, const uint32_t *tdev, uint32_t toff,
                  const float *a15f, cudaStream_t st);
 // All steps of a call in one launch with the state in shared memory
 // (lbm_resident.cu), for grids that fit.
@@ -187,10 +188,10 @@ struct lbm_grid {
     int device = 0;
     vss::Coef coef{};
     vss::TileCfg cfg{};
-    // Two steps per launch: the plan for the grid as configured, and whether
+    // Several steps per launch: the plan for the grid as configured, and whether
     // step calls may use it (not under a tile configuration of the caller's).
-    vss::Step2Plan step2{};
-    bool pairs = true;
+    vss::FusedPlan fused{};
+    bool fuse = true;
     // All steps of a call in one launch (small grids), and the exchanges made.
     vss::ResidentPlan resident{};
     bool resident_planned = false;  // on the first call that may use it

@@ -30,7 +30,7 @@
 #pragma once
 
 #include "lbm_internal.h"
-#include "lbm_walk2.cuh"
+#include "lbm_fused.cuh"
 
 namespace vss {
 

@@ -1,4 +1,4 @@
-"""Batches whose passes take two steps (the fused walk) leave every grid bit
+"""Batches whose passes take two or three steps (the fused walk) leave every grid bit
 for bit in the state single steps leave it in, in both schedules: odd and even
 step limits, limits that end early, tile heights from one row up (the flow
 schedule uses at least four, the reach of a pass), strips of one lane, one whole
@@ -53,3 +53,30 @@ def test_pairs_in_batches_equal_single_steps(lbm, kind, lens, rows, schedule):
                 h.step(1)
             assert h.t == t
             assert np.array_equal(h.get_state()[0], state), SIZES[k]
+
+
+def test_tall_tiles_in_a_batch_equal_single_steps(lbm):
+    """Grids tall enough for FP32's passes of three steps in lockstep (tiles over 64
+    rows on every resident warp), with limits that leave one and two steps."""
+    sizes, limits = [(8, 100003), (124, 20001)], [10, 8]
+    fields = [workloads.fourier_modes(nx, ny, amp=1e-2, seed=nx) for nx, ny in sizes]
+    grids = []
+    for (nx, ny), f in zip(sizes, fields):
+        g = lbm.Grid(nx, ny, 0.7, 0.2)
+        g.init(*f)
+        grids.append(g)
+    b = lbm.Batch(grids)
+    assert b.get_config()["rows"] > 64
+    b.step(10, limits)
+    b.step(3)
+    assert b.sync() == 0
+    got = [g.get_state()[0] for g in grids]
+    b.close()
+    for g in grids:
+        g.close()
+    for (nx, ny), f, n, state in zip(sizes, fields, limits, got):
+        with lbm.Grid(nx, ny, 0.7, 0.2) as h:
+            h.init(*f)
+            for _ in range(n + 3):
+                h.step(1)
+            assert np.array_equal(h.get_state()[0], state)

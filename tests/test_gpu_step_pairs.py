@@ -1,9 +1,10 @@
-"""Step calls that take two steps per launch (large grids) leave bit for bit
+"""Step calls that take two or three steps per launch (large grids) leave bit for bit
 the state of single-step calls: the fused walk repeats the single walk's
 operations in order, so nothing but equality is accepted.  The shapes put the
 strips' edges everywhere: one strip narrower than a lane pair, a last strip of
 one lane, whole strips, wrapped halo columns, short last segments of odd and
-even grids, and step counts that mix graphs, pairs and a last single step."""
+even grids, and step counts that mix graphs, whole and part passes and a last
+single step."""
 import numpy as np
 import pytest
 
@@ -11,8 +12,8 @@ from paper_0707_2437_gb300 import workloads
 
 pytestmark = pytest.mark.gpu
 
-# (nx, ny): tiles tall enough that pairs are taken (FP32 strips of 120 columns,
-# 16-bit strips of 240).
+# (nx, ny): tiles tall enough that passes of several steps are taken (FP32 strips of
+# 112 or 120 columns, 16-bit strips of 240).
 SHAPES = {"f32": [(4, 20011), (124, 9803), (1000, 1201), (2048, 1025)],
           "16": [(8, 30011), (248, 15003), (1200, 2407), (2048, 3077)]}
 
@@ -35,6 +36,6 @@ def _state(lbm, kind, nx, ny, calls, lens):
 @pytest.mark.parametrize("shape", range(4))
 def test_pairs_of_steps_equal_single_steps(lbm, kind, lens, shape):
     nx, ny = SHAPES["f32" if kind == "f32" else "16"][shape]
-    single = _state(lbm, kind, nx, ny, [1] * 77, lens)
-    pairs = _state(lbm, kind, nx, ny, [2, 71, 1, 3], lens)
+    single = _state(lbm, kind, nx, ny, [1] * 106, lens)
+    pairs = _state(lbm, kind, nx, ny, [2, 100, 1, 3], lens)
     assert np.array_equal(single, pairs)
