@@ -434,7 +434,11 @@ static bool runs_resident(lbm_grid *h, long long n) {
         h->grad != LBM_GRAD_CENTRAL || n < kResidentMin)
         return false;
     if (!h->resident_planned) {
-        if (plan_resident(h->nx, h->ny, h->sms, &h->resident) != cudaSuccess) return false;
+        if (plan_resident(h->nx, h->ny, h->sms, true, &h->resident) != cudaSuccess) return false;
+        if (h->resident.ok && h->resident.cluster &&
+            !cluster_fits(h->resident, h->storage, h->rounding, h->a15f != nullptr) &&
+            plan_resident(h->nx, h->ny, h->sms, false, &h->resident) != cudaSuccess)
+            return false;
         h->resident_planned = true;
     }
     if (!h->resident.ok || (h->rounding && h->resident.us > kResidentMostStochastic)) return false;

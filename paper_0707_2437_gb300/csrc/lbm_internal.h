@@ -96,6 +96,7 @@ struct ResidentPlan {
     bool ok = false;
     int tx = 0, ty = 0;  // tiles in x and y, one block each
     int T = 0;           // steps between exchanges of tile edges
+    bool cluster = false;  // the tiles are one cluster and exchange within it
     int shape = 0;       // block shape (lbm_resident.cu)
     int threads = 0;     // of a block
     int lanes = 0;       // thread t has column t % lanes of band t / lanes
@@ -106,6 +107,7 @@ struct ResidentArgs {
     void *buf[2];
     int cur;             // buf[cur] holds the state
     int nx, ny, tx, ty, T, lanes, pitch;
+    int cluster;         // the blocks are one cluster
     size_t P;
     long long steps;
     uint32_t t0;         // number of the first step
@@ -118,10 +120,10 @@ struct ResidentArgs {
     int *status;
 };
 constexpr int kResidentFlagWords = 32;  // a 128-byte line per tile
-// Exchanges of a launch of `steps` steps; the result is in buf[cur ^ 1] after an
-// even number of them, else in buf[cur].
+// Exchanges through the buffers in a launch of `steps` steps; the result is in
+// buf[cur ^ 1] after an even number of them, else in buf[cur].
 inline long long resident_exchanges(const ResidentPlan &p, long long steps) {
-    return (steps + p.T - 1) / p.T - 1;
+    return p.cluster ? 0 : (steps + p.T - 1) / p.T - 1;
 }
 using ResidentKernel = void (*)(ResidentArgs);
 ResidentKernel resident_kernel_f32(int rnd, bool field, int shape);
@@ -129,7 +131,9 @@ ResidentKernel resident_kernel_f16(int rnd, bool field, int shape);
 ResidentKernel resident_kernel_bf16(int rnd, bool field, int shape);
 // Whether a grid is small enough to have a tiling; the tiling.
 bool may_run_resident(int nx, int ny, int sms);
-Err plan_resident(int nx, int ny, int sms, ResidentPlan *out);
+Err plan_resident(int nx, int ny, int sms, bool clusters, ResidentPlan *out);
+// Whether the device can hold a plan's cluster.
+bool cluster_fits(const ResidentPlan &p, int storage, int rnd, bool field);
 Err launch_resident(const ResidentPlan &p, int storage, int rnd, ResidentArgs a, cudaStream_t st);
 // The forward-difference gradient (lbm_set_gradient): FP32, one site per lane.
 Err launch_step_forward(const TileCfg &cfg, const void *fin, void *fout, int nx, int ny, size_t P,

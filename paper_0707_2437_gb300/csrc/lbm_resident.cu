@@ -53,20 +53,25 @@ int smem_of(int shape) { return 10 * kShapes[shape].threads * kShapes[shape].row
 // rows, and an exchange (two passes through L2 and the wait) shared by T steps.  An
 // exchange of tiles whose edges lie on 32-byte sectors takes a fifth less (256^2 in
 // 16 x 8 tiles 1.70 us a step, in 11 x 13 1.95; 8192 x 4 in 128 tiles 0.44, in 152
-// 0.48).
-static double exchange_us(long long halo, bool aligned) {
+// 0.48).  Within a cluster it costs less for the few sites of a channel's tiles (400
+// x 4: 0.44 -> 0.32 us a step) and no less for tiles cut in both directions (64^2:
+// 1.06 against 1.07).
+static double exchange_us(long long halo, bool aligned, bool cluster) {
+    if (cluster) return 0.65 + 0.003 * (double)halo;
     return (2.4 + 0.0012 * (double)halo) * (aligned ? 0.8 : 1.0);
 }
-static double step_us(int shape, int W, int H, int hx, int hy, int T, bool aligned) {
+static double step_us(int shape, int W, int H, int hx, int hy, int T, bool aligned, bool cluster) {
     const double warp_rows = threads_for(shape, W, H) / 32 * kShapes[shape].rows;
     const int halo = W * H - (W - 2 * hx) * (H - 2 * hy);
-    return 0.16 + 0.018 * warp_rows + (hx || hy ? exchange_us(halo, aligned) / T : 0.0);
+    return 0.16 + 0.018 * warp_rows + (hx || hy ? exchange_us(halo, aligned, cluster) / T : 0.0);
 }
+
+constexpr int kClusterTiles = 16;  // the largest cluster (beyond the portable 8)
 
 // The tiling with the lowest estimate.  Grids of up to about 700^2 sites have one.
 bool may_run_resident(int nx, int ny, int sms) { return (long long)nx * ny <= 3900LL * sms; }
 
-Err plan_resident(int nx, int ny, int sms, ResidentPlan *out) {
+Err plan_resident(int nx, int ny, int sms, bool clusters, ResidentPlan *out) {
     *out = ResidentPlan{};
     if (!may_run_resident(nx, ny, sms)) return cudaSuccess;
     double best = 1e30;
@@ -83,20 +88,22 @@ Err plan_resident(int nx, int ny, int sms, ResidentPlan *out) {
                 const long long sites = (long long)W * H;
                 if (sites > 3900) break;
                 const int own = (W - 2 * hx) * (H - 2 * hy);
+                const bool cluster = clusters && tx * ty > 1 && tx * ty <= kClusterTiles;
                 const bool aligned = nx % tx == 0 && nx / tx % 8 == 0;
                 const double least = 0.16 + 0.018 * (double)sites / 32 +
-                                     (hx || hy ? exchange_us(sites - own, aligned) / T : 0.0);
+                                     (hx || hy ? exchange_us(sites - own, aligned, cluster) / T : 0.0);
                 if (least >= best) continue;  // no shape can be better
                 bool any = false;
                 for (int k = 0; k < kNumShapes; ++k) {
                     if (!fits(k, W, H)) continue;
                     any = true;
-                    const double us = step_us(k, W, H, hx, hy, T, aligned);
+                    const double us = step_us(k, W, H, hx, hy, T, aligned, cluster);
                     if (us >= best) continue;
                     best = us;
                     out->tx = tx;
                     out->ty = ty;
                     out->T = tx * ty == 1 ? 1 << 20 : T;
+                    out->cluster = cluster;
                     out->shape = k;
                     out->threads = threads_for(k, W, H);
                     out->lanes = lanes_for(W, kShapes[k].rows);
@@ -110,26 +117,64 @@ Err plan_resident(int nx, int ny, int sms, ResidentPlan *out) {
     return cudaSuccess;
 }
 
+static ResidentKernel kernel_for(const ResidentPlan &p, int storage, int rnd, bool field) {
+    return storage == ST_F32   ? resident_kernel_f32(rnd, field, p.shape)
+           : storage == ST_F16 ? resident_kernel_f16(rnd, field, p.shape)
+                               : resident_kernel_bf16(rnd, field, p.shape);
+}
+
+// Launch parameters of a plan (attr: room for the cluster's attribute), and the
+// attributes of its kernel, which are set again on each call at little cost.
+static Err prepare_resident(const ResidentPlan &p, ResidentKernel fn, cudaStream_t st,
+                            cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr) {
+    const int smem = smem_of(p.shape);
+    Err e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3((unsigned)(p.tx * p.ty));
+    cfg->blockDim = dim3((unsigned)p.threads);
+    cfg->dynamicSmemBytes = (size_t)smem;
+    cfg->stream = st;
+    cfg->attrs = attr;
+    if (p.cluster) {
+        e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        attr->id = cudaLaunchAttributeClusterDimension;
+        attr->val.clusterDim.x = (unsigned)(p.tx * p.ty);
+        attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+        cfg->numAttrs = 1;
+    } else if (p.tx * p.ty > 1) {
+        attr->id = cudaLaunchAttributeCooperative;
+        attr->val.cooperative = 1;
+        cfg->numAttrs = 1;
+    }
+    return e;
+}
+
+bool cluster_fits(const ResidentPlan &p, int storage, int rnd, bool field) {
+    const ResidentKernel fn = kernel_for(p, storage, rnd, field);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    int clusters = 0;
+    const bool ok = prepare_resident(p, fn, nullptr, &cfg, &attr) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, (const void *)fn, &cfg) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    return ok && clusters > 0;
+}
+
 Err launch_resident(const ResidentPlan &p, int storage, int rnd, ResidentArgs a, cudaStream_t st) {
     a.tx = p.tx;
     a.ty = p.ty;
     a.T = p.T;
     a.lanes = p.lanes;
     a.pitch = p.pitch;
-    const bool field = a.a15f != nullptr;
-    const ResidentKernel fn = storage == ST_F32   ? resident_kernel_f32(rnd, field, p.shape)
-                              : storage == ST_F16 ? resident_kernel_f16(rnd, field, p.shape)
-                                                  : resident_kernel_bf16(rnd, field, p.shape);
-    const int smem = smem_of(p.shape), tiles = p.tx * p.ty;
-    // (a host-side attribute of the kernel; setting it again is cheap)
-    Err e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    a.cluster = p.cluster ? 1 : 0;
+    const ResidentKernel fn = kernel_for(p, storage, rnd, a.a15f != nullptr);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    const Err e = prepare_resident(p, fn, st, &cfg, &attr);
     if (e != cudaSuccess) return e;
     void *args[] = {(void *)&a};
-    if (tiles == 1)
-        return cudaLaunchKernel((const void *)fn, dim3(1), dim3(p.threads), args,
-                                (size_t)smem, st);
-    return cudaLaunchCooperativeKernel((const void *)fn, dim3(tiles),
-                                       dim3(p.threads), args, (size_t)smem, st);
+    return cudaLaunchKernelExC(&cfg, (const void *)fn, args);
 }
 
 }  // namespace vss

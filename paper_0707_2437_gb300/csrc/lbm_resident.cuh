@@ -12,7 +12,8 @@
 // A thread owns K rows of one column, so the pulled values wait in registers
 // and most y neighbours are its own.
 //
-// Tiles exchange edges through the grid's own two buffers.  A tile is extended
+// Tiles exchange edges through the grid's own two buffers, or, up to 16 of them, as
+// one cluster (below).  A tile is extended
 // by a halo of 2 T columns or rows in each direction in which the grid is cut;
 // T steps use two sites of it each (the pull and the central difference), so
 // the blocks meet once in T steps: a block writes its outer ring, raises its
@@ -25,6 +26,12 @@
 // Blocks wait for one another, so launches of several tiles are cooperative (all
 // blocks resident, or none), every wait is bounded by the clock, and a wait that
 // runs out sets the handle's status word.
+//
+// Up to 16 tiles launch as one cluster instead, which the hardware schedules as a
+// whole: a block reads its halo out of its neighbours' shared memory, between two
+// cluster barriers (all tiles have done their steps; all halos have been read), of
+// which the second is waited for only before the next step writes.  That takes about
+// 0.7 us for a few dozen sites where flags and two passes through L2 take 2.2.
 //
 // The arithmetic is the Walker's, operation by operation.
 #pragma once
@@ -75,6 +82,24 @@ __device__ __forceinline__ float stored_d(double v) {
         return __bfloat162float(__double2bfloat16(v));
 }
 
+__device__ __forceinline__ void cluster_arrive() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A word of block `rank`'s shared memory, at the address `local` has here.
+__device__ __forceinline__ uint32_t peer_address(uint32_t local, int rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float peer_load(uint32_t address) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(address) : "memory");
+    return v;
+}
+
 constexpr int kDriveChunk = 128;  // boundary values computed ahead
 
 // NT threads of K rows each: up to NT * K sites of extended tile.
@@ -84,8 +109,8 @@ constexpr int kDriveChunk = 128;  // boundary values computed ahead
 // instruction issue (about 100 instructions a site, the halo's included).  The K
 // rows of a thread are independent, so they overlap; more rows than ten spill.
 // Measured per step, launches of step kernels before and resident now: 400 x 4 FP32
-// 3.5 -> 0.46 us, driven 8192 x 4 FP32 7.5 -> 0.61, 64^2 3.5 -> 1.09, 256^2 4.2 ->
-// 1.95, 509 x 381 5.4 -> 3.2, 512^2 6.6 -> 3.5; 512^2 FP16 5.6 -> 3.7, with stochastic
+// 3.5 -> 0.33 us, driven 8192 x 4 FP32 7.5 -> 0.60, 64^2 3.5 -> 1.09, 256^2 4.2 ->
+// 1.86, 509 x 381 5.4 -> 3.2, 512^2 6.6 -> 3.5; 512^2 FP16 5.6 -> 3.7, with stochastic
 // rounding 6.2 -> 5.0.
 template <int S, int RND, int VA, int NT, int K>
 __global__ void __launch_bounds__(NT, 1)
@@ -183,6 +208,45 @@ __global__ void __launch_bounds__(NT, 1)
         l = fy * Wp + fx;
         g = (size_t)cy * a.nx + cx;
     };
+    // The same site in the neighbour that owns it: its block, and the offset there.
+    const int left_w = x0 - first_of(a.nx, a.tx, wrapped(bx - 1, a.tx)) +
+                       (bx == 0 ? a.nx : 0);  // width of the tile on the left
+    const int up_h = y0 - first_of(a.ny, a.ty, wrapped(by - 1, a.ty)) + (by == 0 ? a.ny : 0);
+    auto peer_site = [&](int m, int &rank, int &l) {
+        int fx, fy;
+        halo.at(m, fx, fy);
+        int nbx = bx, nby = by, px = fx, py = fy;
+        if (fx < hx) {
+            nbx = bx == 0 ? a.tx - 1 : bx - 1;
+            px = fx + left_w;
+        } else if (fx >= W - hx) {
+            nbx = bx + 1 == a.tx ? 0 : bx + 1;
+            px = fx - (W - 2 * hx);
+        }
+        if (fy < hy) {
+            nby = by == 0 ? a.ty - 1 : by - 1;
+            py = fy + up_h;
+        } else if (fy >= H - hy) {
+            nby = by + 1 == a.ty ? 0 : by + 1;
+            py = fy - (H - 2 * hy);
+        }
+        rank = nby * a.tx + nbx;
+        l = py * Wp + px;
+    };
+    auto fetch_from_peers = [&] {
+        const uint32_t planes_at = smem_u32(F);
+        for (int m = threadIdx.x; m < halo.sites; m += blockDim.x) {
+            int rank, l, fx, fy;
+            peer_site(m, rank, l);
+            const uint32_t from = peer_address(planes_at, rank) + 4u * (uint32_t)l;
+            float v[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v[i] = peer_load(from + 4u * (uint32_t)(i * PS));
+            halo.at(m, fx, fy);
+            put_site(fy * Wp + fx, v);
+        }
+    };
+    bool peers_read = true;  // no cluster barrier is open
     auto fetch_halo = [&](const void *src) {
         for (int m = threadIdx.x; m < halo.sites; m += 2 * blockDim.x) {
             const bool two = m + (int)blockDim.x < halo.sites;
@@ -267,6 +331,10 @@ __global__ void __launch_bounds__(NT, 1)
                     for (int i = 0; i < 9; ++i) h[j][i] = stored<S>(h[j][i]);
                 }
             }
+            if (!peers_read) {  // (a cluster's first step after an exchange)
+                cluster_wait();
+                peers_read = true;
+            }
             if (edge_col) {
                 const float b = gx == 0 ? drive_h[(int)((done + s) % kDriveChunk)]
                                         : stored_d<S>(1.0 - a.rho0);
@@ -283,6 +351,15 @@ __global__ void __launch_bounds__(NT, 1)
         }
         done += steps;
         if (done >= a.steps) break;
+        if (a.cluster) {
+            cluster_arrive();
+            cluster_wait();
+            fetch_from_peers();
+            cluster_arrive();
+            peers_read = false;
+            __syncthreads();
+            continue;
+        }
         // Exchange: the outer ring of the tile's own sites out ...
         write_ring(a.buf[out]);
         ++epoch;
