@@ -264,22 +264,34 @@ static int build_worklist(lbm_batch *b) {
         const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
                                              : gr.max_blocks_per_sm;
         const long long warps = (long long)per * b->sms * kBatchWarps;
+        // A grid's pass takes at least one tile walk, so a grid with fewer tiles than
+        // its share of the resident warps (the warps split evenly between the grids)
+        // uses shorter tiles: a quarter as tall in single steps; on the fused walk as
+        // tall as seven tenths of its share of warps ask for, from its reach (so that
+        // a tile waits for its neighbours only) up to a height that depends on the
+        // whole batch: 48 rows if that still leaves two and a half tiles a warp, else
+        // 32 or 24.  Measured: 20 grids of 128^2 to 2048^2 with 1e9 updates between
+        // them 8.9, 8.7, 8.4 ms at 48, 32, 24 rows; nine 2048^2 FP32 grids 174k, 168k,
+        // 161k MLUPS; 512 uneven grids 138k, 131k, 120k.
+        auto flow_rows = [&](size_t k, int tallest) {
+            const long long share = std::max<long long>(1, 7 * warps / (10 * (long long)ng));
+            const long long r = ((long long)strips(k, 2) * computed_rows(k) + share - 1) / share;
+            return std::max(2 * per_pass, (int)std::min<long long>(tallest, r));
+        };
+        int tallest = 48;
+        if (fc.fused && b->fit_rows)
+            for (int h : {48, 32, 24}) {
+                tallest = h;
+                long long total = 0;
+                for (size_t k = 0; k < ng; ++k)
+                    total += (long long)strips(k, 2) *
+                             ((computed_rows(k) + flow_rows(k, h) - 1) / flow_rows(k, h));
+                if (2 * total >= 5 * warps) break;
+            }
         for (size_t k = 0; k < ng; ++k) {
-            // A grid's pass takes at least one tile walk, so a grid with fewer
-            // tiles than its share of the resident warps (the warps split
-            // evenly between the grids) uses shorter tiles: a quarter as tall
-            // in single steps; on the fused walk as tall as its share of warps
-            // asks for, from its reach (so that a tile waits for its neighbours
-            // only) to 48 rows.
             int rows = b->rows;
             if (fc.fused) {
-                if (b->fit_rows) {
-                    const long long share = std::max<long long>(1, warps / (long long)ng);
-                    const long long r =
-                        ((long long)strips(k, 2) * computed_rows(k) + share - 1) / share;
-                    rows = (int)std::min<long long>(48, r);
-                }
-                rows = std::max(2 * per_pass, rows);
+                rows = b->fit_rows ? flow_rows(k, tallest) : std::max(2 * per_pass, rows);
             } else {
                 const long long tall =
                     (long long)strips(k, 1) * ((computed_rows(k) + rows - 1) / rows);
