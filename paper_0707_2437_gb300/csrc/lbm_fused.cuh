@@ -97,8 +97,7 @@ __device__ __forceinline__ void collide1(float (&h)[9], float dr, float gx, floa
 // tiles close together, at three by shared memory and issue, with more rows and
 // columns of halo, so it pays where tiles are tall (8192^2 174k against 203k MLUPS,
 // 1024^2 112k against 105k; four steps leave shared memory for six warps per SM and
-// run at 160k).  With a c2 field two: the rows of alpha values take the shared memory
-// of the third.
+// run at 160k). 
 template <int S, int TS>
 struct FusedGeom {
     static constexpr int V = (S == ST_F32) ? 4 : 8;     // sites per lane, 16 bytes
@@ -110,9 +109,7 @@ constexpr int fused_cols(int storage, int steps) {
     return storage == ST_F32 ? (steps == 3 ? FusedGeom<ST_F32, 3>::COLS : FusedGeom<ST_F32, 2>::COLS)
                              : FusedGeom<ST_F16, 2>::COLS;
 }
-constexpr int fused_most_steps(int storage, bool field) {
-    return storage == ST_F32 && !field ? 3 : 2;
-}
+constexpr int fused_most_steps(int storage) { return storage == ST_F32 ? 3 : 2; }
 // Tallest tiles: FP32's passes of two steps are bound by HBM and run faster while the
 // tiles in flight lie close together (8192^2, 48 rows 385 us a step, 235 rows 419).
 constexpr int fused_most_rows(int storage, int steps) {
@@ -124,10 +121,18 @@ constexpr int fused_overhead(int steps) { return 4 * steps - 3; }
 // Shared memory of one warp, in 16-byte vectors: two landing rows; for each stage
 // after the first the rows held for it and the row that waits in it; with a c2
 // field the alpha values of the rows in flight.
+// FP32 with a c2 field takes all of it for three stages; the alpha values of the rows
+// in flight then move down five vectors of registers, one per iteration (2048^2
+// 31.2 -> 29.9 us a step against two stages, 4096^2 114.3 -> 102.4; each stage loading
+// its own row an iteration ahead took 30.4 and 104.7).
+template <int S, int TS>
+constexpr bool fused_alpha_ring() {
+    return S != ST_F32 || TS < 3;
+}
 template <int S, int VA, int TS>
 constexpr int fused_vecs() {
     return (2 + 2 * (TS - 1)) * 9 * 32 +
-           (VA ? (2 * TS + 2) * (FusedGeom<S, TS>::V / 4) * 32 : 0);
+           (VA && fused_alpha_ring<S, TS>() ? (2 * TS + 2) * (FusedGeom<S, TS>::V / 4) * 32 : 0);
 }
 
 template <int S, int LD, int RND, int VA, int TS>
@@ -137,6 +142,10 @@ struct FusedWalk {
     static_assert(Pack<S, V>::NW == 4, "a lane holds one 16-byte vector per direction");
     static_assert(RND == 0 || S != ST_F32, "stochastic rounding applies to 16-bit storage");
     using T = typename StoreT<S>::T;
+    static constexpr int AV = V / 4;      // alpha vectors of a lane's sites
+    static constexpr int AS = 2 * TS + 2;  // slots of alpha rows in shared memory
+    static constexpr int AL = 2 * TS - 1;  // rows of them kept in registers instead
+    static constexpr bool RING = VA && fused_alpha_ring<S, TS>();
     uint32_t rkey[TS] = {};  // sr_step_key of the steps
     const float *__restrict__ a15f = nullptr;
 
@@ -192,9 +201,9 @@ struct FusedWalk {
                          "l"(src)
                          : "memory");
         }
-        if constexpr (VA) {
+        if constexpr (RING) {
 #pragma unroll
-            for (int h = 0; h < V / 4; ++h)
+            for (int h = 0; h < AV; ++h)
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
                                  (uint32_t)__cvta_generic_to_shared(al + h * 32)),
                              "l"(a15f + (size_t)q0 * nx + xl + 4 * h)
@@ -238,14 +247,14 @@ struct FusedWalk {
     __device__ __forceinline__ void collide(int r, uint32_t (&w)[9][4], const float (&d)[V],
                                             const float (&before)[V], const float (&after)[V],
                                             float dir, const Coef &c, uint32_t rkey,
-                                            const uint4 *al) const {
+                                            const uint4 (&al)[AV]) const {
         const float lft = __shfl_up_sync(FULL, d[V - 1], 1);
         const float rgt = __shfl_down_sync(FULL, d[0], 1);
         float a15v[V];
         if constexpr (VA) {
 #pragma unroll
             for (int h = 0; h < V / 4; ++h) {
-                const uint4 u = al[h * 32];
+                const uint4 u = al[h];
                 a15v[4 * h + 0] = __uint_as_float(u.x);
                 a15v[4 * h + 1] = __uint_as_float(u.y);
                 a15v[4 * h + 2] = __uint_as_float(u.z);
@@ -310,7 +319,6 @@ struct FusedWalk {
     __device__ __forceinline__ uint4 *wait_of(uint4 *buf, int s) const {
         return buf + (27 + 18 * (s - 1)) * 32 + lane;
     }
-    static constexpr int AV = (V / 4) * 32, AS = 2 * TS + 2;  // alpha vectors a slot, slots
     __device__ __forceinline__ uint4 *alpha_of(uint4 *buf) const {
         return buf + (18 + 18 * (TS - 1)) * 32 + lane;
     }
@@ -322,13 +330,21 @@ struct FusedWalk {
     template <int SG>
     __device__ __forceinline__ void stage(int k, int dir, int steps, float sgn, const Coef &c,
                                           int ia, uint4 *buf, uint32_t (&u)[9][4],
-                                          float (&d)[TS][3][V], int row, const int (&back)[TS]) const {
+                                          float (&d)[TS][3][V], int row, const int (&back)[TS],
+                                          const uint4 (&alpha)[AL][AV]) const {
         if (k < 4 * SG + 2) return;
-        const int as = ia - (2 * SG + 1);
         int r = row - back[SG];
         if (r < 0) r += ny;
-        collide(r, u, d[SG][1], d[SG][0], d[SG][2], sgn, c, rkey[SG],
-                alpha_of(buf) + (as < 0 ? as + AS : as) * AV);
+        if constexpr (RING) {
+            const int as = ia - (2 * SG + 1);
+            const uint4 *from = alpha_of(buf) + (as < 0 ? as + AS : as) * AV * 32;
+            uint4 a[AV];
+#pragma unroll
+            for (int h = 0; h < AV; ++h) a[h] = from[h * 32];
+            collide(r, u, d[SG][1], d[SG][0], d[SG][2], sgn, c, rkey[SG], a);
+        } else {
+            collide(r, u, d[SG][1], d[SG][0], d[SG][2], sgn, c, rkey[SG], alpha[2 * SG]);
+        }
         if constexpr (SG + 1 < TS) {
             if (SG + 1 < steps) {
                 // The row after this stage is in u.  The next stage's pulled row, one
@@ -363,7 +379,7 @@ struct FusedWalk {
                     if (k >= 4 * (SG + 1) + 2) {
 #pragma unroll
                         for (int i = 0; i < 9; ++i) swap(i, wait + i * 32);
-                        stage<SG + 1>(k, dir, steps, sgn, c, ia, buf, u, d, row, back);
+                        stage<SG + 1>(k, dir, steps, sgn, c, ia, buf, u, d, row, back, alpha);
                     } else {
                         keep(wait, u);
                     }
@@ -416,20 +432,24 @@ struct FusedWalk {
 #pragma unroll
                 for (int v = 0; v < V; ++v) d[s][j][v] = 0.f;
         int ia = 0;  // alpha slot of the pulled row, mod AS
+        uint4 alpha[AL][AV] = {};  // of the rows pulled one iteration ago, two, ...
+        uint4 fresh = make_uint4(0, 0, 0, 0);
         issue(qm, q0, qp, land, al);
         next();
-        issue(qm, q0, qp, land + 9 * 32, al + AV);  // K >= 3
+        issue(qm, q0, qp, land + 9 * 32, al + AV * 32);  // K >= 3
         next();
         for (int k = 0; k < K; ++k) {
             uint32_t w[9][4], u[9][4];
             uint4 *slot = land + (k & 1) * 9 * 32;
+            if constexpr (VA && !RING)
+                fresh = __ldg(reinterpret_cast<const uint4 *>(a15f + (size_t)row * nx + xl));
             asm volatile("cp.async.wait_group 1;" ::: "memory");
             take(w, slot);
             finish(w, d[0][2]);
             // The words read from the landing row have been used (the
             // shuffles), so the next copy cannot overtake them.
             if (k + 2 < K) {
-                issue(qm, q0, qp, slot, al + (ia < AS - 2 ? ia + 2 : ia + 2 - AS) * AV);
+                issue(qm, q0, qp, slot, al + (ia < AS - 2 ? ia + 2 : ia + 2 - AS) * AV * 32);
                 next();
             } else {
                 asm volatile("cp.async.commit_group;" ::: "memory");  // keeps the count
@@ -441,7 +461,7 @@ struct FusedWalk {
                     u[i][j] = wc[i][j];
                     wc[i][j] = w[i][j];
                 }
-            stage<0>(k, dir, steps, sgn, c, ia, buf, u, d, row, back);
+            stage<0>(k, dir, steps, sgn, c, ia, buf, u, d, row, back, alpha);
 #pragma unroll
             for (int s = 0; s < TS; ++s)
 #pragma unroll
@@ -452,6 +472,11 @@ struct FusedWalk {
             row += dir;
             if (row < 0) row += ny;
             if (row >= ny) row -= ny;
+            if constexpr (VA && !RING) {
+#pragma unroll
+                for (int j = AL - 1; j > 0; --j) alpha[j][0] = alpha[j - 1][0];
+                alpha[0][0] = fresh;
+            }
             ia = ia == AS - 1 ? 0 : ia + 1;
         }
     }

@@ -56,8 +56,8 @@ Choice choice() {
 Choice choose(int storage, int rnd, bool field, int steps) {
     switch (storage) {
         case ST_F32:
-            return field ? choice<ST_F32, 0, 1, 2>()
-                         : (steps == 3 ? choice<ST_F32, 0, 0, 3>() : choice<ST_F32, 0, 0, 2>());
+            if (field) return steps == 3 ? choice<ST_F32, 0, 1, 3>() : choice<ST_F32, 0, 1, 2>();
+            return steps == 3 ? choice<ST_F32, 0, 0, 3>() : choice<ST_F32, 0, 0, 2>();
         case ST_F16:
             return field ? choice<ST_F16, 0, 1, 2>()
                          : (rnd ? choice<ST_F16, 1, 0, 2>() : choice<ST_F16, 0, 0, 2>());
@@ -75,7 +75,7 @@ Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out)
     *out = FusedPlan{};
     if (nx % fused_vec(storage) || (rnd && field)) return cudaSuccess;
     double best = 1e30;
-    for (int steps = 2; steps <= fused_most_steps(storage, field); ++steps) {
+    for (int steps = 2; steps <= fused_most_steps(storage); ++steps) {
         const Choice ch = choose(storage, rnd, field, steps);
         Err e = cudaFuncSetAttribute((const void *)ch.fn,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, ch.smem);
@@ -97,8 +97,12 @@ Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out)
             }
             if (r >= ny) break;
         }
-        // A row step of three steps takes about 1.22 times as long as one of two.
-        const double per_step = (double)least / (steps == 3 ? 3 / 1.22 : 2.0);
+        // A row step of three steps takes about 1.22 times as long as one of two, 1.3
+        // times with a c2 field (three steps against two: 1024^2 10.42 / 9.84 us a
+        // step, 1536^2 19.2 / 18.4, 2048^2 29.9 / 31.2, 4096^2 102.4 / 114.3, 8192^2
+        // 406 / 414).
+        const double per_step =
+            (double)least / (steps == 3 ? 3 / (field ? 1.3 : 1.22) : 2.0);
         if (per_step >= best) continue;
         best = per_step;
         out->steps = steps;

@@ -39,3 +39,11 @@ def test_pairs_of_steps_equal_single_steps(lbm, kind, lens, shape):
     single = _state(lbm, kind, nx, ny, [1] * 106, lens)
     pairs = _state(lbm, kind, nx, ny, [2, 100, 1, 3], lens)
     assert np.array_equal(single, pairs)
+
+
+@pytest.mark.parametrize("nx,ny", [(4, 50021), (1012, 4003)])
+def test_three_steps_with_a_c2_field_equal_single_steps(lbm, nx, ny):
+    """Grids tall enough for three steps a pass with alpha values in registers: one
+    lane, and nine whole strips of 112 columns and one of four."""
+    single = _state(lbm, "f32", nx, ny, [1] * 14, True)
+    assert np.array_equal(single, _state(lbm, "f32", nx, ny, [3, 8, 1, 2], True))
