@@ -165,17 +165,18 @@ static cudaError_t resident_blocks(const void *fn, int smem, int *blocks) {
 // bounds decides.
 // `fixed`: a height of the caller's (0: the best up to `most`).  *cost: row steps of
 // a pass.
-static int fused_rows(const std::vector<std::pair<int, int>> &grids, long long warps,
+static int fused_rows(const std::vector<std::pair<FusedStrips, int>> &grids, long long warps,
                       int overhead, int most, int fixed, double *cost) {
     int rows = 2;
     for (int r = fixed ? fixed : 2; r <= (fixed ? fixed : most); r += r < 64 ? 1 : 4) {
         long long tiles = 0, work = 0;
         int tallest = 0;
         for (const auto &g : grids) {  // (strips, rows)
-            const long long segs = (g.second + r - 1) / r;
-            tiles += g.first * segs;
-            work += g.first * (g.second + overhead * segs);
-            tallest = std::max(tallest, std::min(r, g.second));
+            const long long segs = (g.second + r - 1) / r, n = g.first.tiles(segs);
+            const int high = std::min(r, g.second);
+            tiles += n;
+            work += n * overhead + g.first.full * g.second + (n - g.first.full * segs) * high;
+            tallest = std::max(tallest, high);
         }
         const double even = (double)((tiles + warps - 1) / warps) * (tallest + overhead);
         const double mixed = (double)work / warps + (tallest + overhead);
@@ -245,6 +246,25 @@ static int build_worklist(lbm_batch *b) {
             for (int x0 = 0; x0 < g->nx; x0 += w)
                 tiles.push_back(Tile{(int)k, x0, y0, std::min(yhi, y0 + rows),
                                      (seg & 1) ? -1 : 1});
+    };
+    // The same for passes of `per` steps in lockstep, where a last narrow strip's
+    // segments share warps.
+    auto add_fused_tiles = [&](size_t k, int rows, int per) {
+        const lbm_grid *g = b->grids[k];
+        b->per[k] = gd[k].per = per;
+        const FusedStrips s = fused_strips(g->storage, per, g->nx);
+        const int w = fused_cols(g->storage, per), step = s.pieces ? s.pieces : 1;
+        for (int y0 = 0, seg = 0; y0 < g->ny; y0 += rows, ++seg) {
+            const int dir = (seg & 1) ? -1 : 1;
+            for (int j = 0; j < s.full; ++j)
+                tiles.push_back(Tile{(int)k, j * w, y0, std::min(g->ny, y0 + rows), dir});
+            if (!s.pieces || seg % step) continue;
+            const int y1 = (int)std::min<long long>(g->ny, y0 + (long long)step * rows);
+            Tile t{(int)k, s.full * w, y0, y1, (seg / step & 1) ? -1 : 1};
+            t.lanes = s.lanes;
+            t.rows = std::min(rows, y1 - y0);
+            tiles.push_back(t);
+        }
     };
     if (b->schedule == LBM_SCHEDULE_FLOW) {
         // One launch over every grid, tiles grid by grid in their order, by the
@@ -391,7 +411,7 @@ static int build_worklist(lbm_batch *b) {
         std::vector<Tile> tail(ordered.end() - wave, ordered.end());
         ordered.resize(ordered.size() - wave);
         for (const Tile &t : tail) {
-            if (t.y1b > t.y0b || t.y1 - t.y0 < 2) {
+            if (t.y1b > t.y0b || t.lanes || t.y1 - t.y0 < 2) {
                 ordered.push_back(t);
                 continue;
             }
@@ -421,8 +441,10 @@ static int build_worklist(lbm_batch *b) {
                 const long long w =
                     (long long)(b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, bps) : bps) *
                     b->sms * kBatchWarps;
-                std::vector<std::pair<int, int>> shape;
-                for (size_t k : members) shape.push_back({strips(k, steps), computed_rows(k)});
+                std::vector<std::pair<FusedStrips, int>> shape;
+                for (size_t k : members)
+                    shape.push_back({fused_strips(storage, steps, b->grids[k]->nx),
+                                     computed_rows(k)});
                 double cost = 0;
                 const int rows = fused_rows(shape, w, fused_overhead(steps),
                                             fused_most_rows(storage, steps),
@@ -440,7 +462,7 @@ static int build_worklist(lbm_batch *b) {
                 gr.rows = rows;
                 warps = w;
             }
-            for (size_t k : members) add_tiles(k, gr.rows, per);
+            for (size_t k : members) add_fused_tiles(k, gr.rows, per);
             ordered.insert(ordered.end(), tiles.begin(), tiles.end());
             split_tail(gr.begin, warps);
             gr.count = (int)ordered.size() - gr.begin;

@@ -50,6 +50,7 @@ struct GridDesc {
 struct __align__(16) Tile {
     int grid, x0, y0, y1, dir;
     int y0b, y1b, dirb;
+    int lanes, rows;  // fused walk: pieces of `rows` rows on `lanes` lanes each (0: one)
 };
 
 // A grid's walk in the batch kernels: storage kind, sites per lane (1, 4 or
@@ -463,14 +464,17 @@ __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
 }
 
 // One tile of the fused walk: a pass, or what is left of a grid's steps.
-template <int S, int RND, int VA, int TS>
+template <int S, int RND, int VA, int TS, bool PACK>
 __device__ __forceinline__ void fused_tile(const GridDesc &g, int par, const Tile &t, uint32_t step,
                                            int steps, uint4 *buf) {
     const Coef c = g.c;
-    FusedWalk<S, LD_CG, RND, VA, TS> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P, t.x0);
+    const bool packed = PACK && t.lanes;
+    const int rows = packed ? t.rows : t.y1 - t.y0;
+    FusedWalk<S, LD_CG, RND, VA, TS, PACK> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P, t.x0,
+                                             t.y0, t.y1, rows, packed ? t.lanes : 32);
     if constexpr (VA) w.a15f = g.a15f;
     if constexpr (RND) w.set_step(step);
-    w.run(t.y0, t.y1, t.dir, steps, c, buf);
+    w.run(rows, t.dir, steps, c, buf);
 }
 
 // Flow kernel for a batch of one kind of grids on the fused walk (two steps a
@@ -487,7 +491,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 2)
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
               timeout_ns,
               [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int steps) {
-                  fused_tile<S, RND, VA, 2>(g, par, t, step, steps, buf);
+                  fused_tile<S, RND, VA, 2, false>(g, par, t, step, steps, buf);
               });
 }
 
@@ -509,9 +513,9 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 2)
               timeout_ns,
               [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int steps) {
                   if (g.kind == kind_code(ST_F32, 4, 0))
-                      fused_tile<ST_F32, 0, 0, 2>(g, par, t, step, steps, buf);
+                      fused_tile<ST_F32, 0, 0, 2, false>(g, par, t, step, steps, buf);
                   else
-                      fused_tile<S2, RND2, 0, 2>(g, par, t, step, steps, buf);
+                      fused_tile<S2, RND2, 0, 2, false>(g, par, t, step, steps, buf);
               });
 }
 
@@ -696,8 +700,9 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 2)
             const long long left = limit[t.grid] - TS * k;
             if (left <= 0) continue;
             const int par = (parity0[t.grid] + (int)(k & 1)) & 1;
-            fused_tile<S, RND, VA, TS>(grids[t.grid], par, t, t0[t.grid] + (uint32_t)(TS * k),
-                                   (int)min((long long)TS, left), buf);
+            fused_tile<S, RND, VA, TS, fused_packs(S)>(grids[t.grid], par, t,
+                                                       t0[t.grid] + (uint32_t)(TS * k),
+                                                       (int)min((long long)TS, left), buf);
         }
         if (k + 1 < npass && !grid_barrier(bar, status, timeout_ns)) return;
     }

@@ -27,7 +27,7 @@
 // bit the state that T single steps leave.
 #pragma once
 
-#include "lbm_device.cuh"
+#include "lbm_internal.h"
 
 namespace vss {
 
@@ -115,6 +115,21 @@ constexpr int fused_most_steps(int storage) { return storage == ST_F32 ? 3 : 2; 
 constexpr int fused_most_rows(int storage, int steps) {
     return storage == ST_F32 && steps == 2 ? 64 : 512;
 }
+
+// The strips of nx columns, a multiple of fused_vec.  Packing saves walks of mostly
+// idle lanes, which pays in the 16-bit kinds, bound by issue: FP16 4096^2 76.2 -> 71.8
+// us a step, 8192^2 279 -> 272, 512 uneven FP16 grids in a batch 209k -> 229k MLUPS.
+// FP32 passes are bound by memory and gain nothing (2048^2 with three steps 26.3 /
+// 26.4 us; 512 uneven grids 178k / 174k), and as the lanes of a packed tile read and
+// write far apart it walks more slowly than the others (2048^2 with a c2 field and two
+// steps 31.2 / 39.9 us, eight pieces).
+constexpr bool fused_packs(int storage) { return storage != ST_F32; }
+inline FusedStrips fused_strips(int storage, int steps, int nx) {
+    const int vec = fused_vec(storage), use = fused_cols(storage, steps) / vec, halo = 32 - use;
+    const int n = nx / vec, rest = n % use, pieces = rest ? 32 / (rest + halo) : 0;
+    if (pieces == 1 || (rest && !fused_packs(storage))) return {n / use + 1, 0, 0};
+    return {n / use, rest + halo, pieces};
+}
 // Row steps a tile costs beyond its rows (the pulls and collisions at its ends).
 constexpr int fused_overhead(int steps) { return 4 * steps - 3; }
 
@@ -135,7 +150,9 @@ constexpr int fused_vecs() {
            (VA && fused_alpha_ring<S, TS>() ? (2 * TS + 2) * (FusedGeom<S, TS>::V / 4) * 32 : 0);
 }
 
-template <int S, int LD, int RND, int VA, int TS>
+// PACK: tiles may be packed.  Otherwise the rows are the warp's, not the lane's, which
+// saves about 1 % (nine FP32 grids of 2048^2 in the flow schedule 173.6k / 174.4k).
+template <int S, int LD, int RND, int VA, int TS, bool PACK>
 struct FusedWalk {
     static constexpr int V = FusedGeom<S, TS>::V;
     static constexpr int HALO = FusedGeom<S, TS>::HALO;
@@ -154,18 +171,23 @@ struct FusedWalk {
     int nx, ny;
     size_t P;
     int lane, xl;
-    bool act;
+    int ylo, own;  // the lane's rows: own of them from ylo (0: none)
 
+    // Columns from x0 and rows y0 .. y1-1, cut into pieces of `rows` rows (y1 - y0: one)
+    // on `lanes` lanes each (32: one).
     __device__ __forceinline__ FusedWalk(const void *fin_, void *fout_, int nx_, int ny_, size_t P_,
-                                         int x0)
+                                         int x0, int y0, int y1, int rows, int lanes)
         : fin(reinterpret_cast<const T *>(fin_)),
           fout(reinterpret_cast<T *>(fout_)),
           nx(nx_),
           ny(ny_),
           P(P_) {
         lane = threadIdx.x & 31;
-        const int xu = x0 + (lane - HALO) * V;  // the lane's columns, unwrapped
-        act = lane >= HALO && lane < 32 - HALO && xu < nx;
+        const int piece = PACK ? lane / lanes : 0, at = lane - piece * lanes;
+        const int xu = x0 + (at - HALO) * V;  // the lane's columns, unwrapped
+        ylo = y0 + piece * rows;
+        const bool act = at >= HALO && at < lanes - HALO && xu < nx && (piece + 1) * lanes <= 32;
+        own = act ? (PACK ? max(0, min(rows, y1 - ylo)) : rows) : 0;
         xl = xu % nx;
         if (xl < 0) xl += nx;
     }
@@ -305,7 +327,7 @@ struct FusedWalk {
     }
 
     __device__ __forceinline__ void store(int r, const uint32_t (&w)[9][4]) const {
-        if (!act) return;
+        if (PACK ? (unsigned)(r - ylo) >= (unsigned)own : own == 0) return;
         T *dst = fout + ((size_t)r * nx + xl);
 #pragma unroll
         for (int i = 0; i < 9; ++i) store_words<S, V>(dst + (size_t)i * P, w[i]);
@@ -390,17 +412,18 @@ struct FusedWalk {
         store(r, u);
     }
 
-    // Advances rows y0 .. y1-1 by `steps` (1 .. TS) steps, walking in direction
-    // dir.  `buf`: the warp's fused_vecs() vectors.
-    __device__ __forceinline__ void run(int y0, int y1, int dir, int steps, const Coef &c,
+    // Advances the pieces' rows (`rows` each, not above ny; walked by all pieces, stored
+    // where they are the lane's) by `steps` (1 .. TS) steps in direction dir.  `buf`:
+    // the warp's fused_vecs() vectors.
+    __device__ __forceinline__ void run(int rows, int dir, int steps, const Coef &c,
                                         uint4 *buf) const {
         uint4 *land = buf + lane;  // two slots
         uint4 *al = alpha_of(buf);
         const float sgn = dir > 0 ? 1.f : -1.f;
         const int ext = 2 * steps - 1;
-        const int K = y1 - y0 + 2 * ext;
+        const int K = rows + 2 * ext;
         // The next row to copy (wrapped) and the rows before and after it.
-        int q0 = (dir > 0 ? y0 - ext : y1 - 1 + ext) % ny;
+        int q0 = (dir > 0 ? ylo - ext : ylo + rows - 1 + ext) % ny;
         if (q0 < 0) q0 += ny;
         int qm = (q0 == 0) ? ny - 1 : q0 - 1;
         int qp = (q0 + 1 == ny) ? 0 : q0 + 1;

@@ -76,6 +76,15 @@ Err launch_step(int storage, const TileCfg &cfg, const void *fin, void *fout, in
 // Warps of `fn` (blocks of `warps` warps, `smem` bytes of dynamic shared memory)
 // resident on the current device; 0 if the query fails.
 long long resident_warps(const void *fn, int warps, int smem);
+// Strips of the fused walk: `full` ones of whole warps and, when the columns left over
+// need at most half a warp with their halo lanes, packed tiles: `pieces` segments of
+// that last strip share a warp, `lanes` lanes each, every piece on rows of its own.
+struct FusedStrips {
+    int full, lanes, pieces;  // pieces 0: none left over
+    long long tiles(long long segs) const {
+        return full * segs + (pieces ? (segs + pieces - 1) / pieces : 0);
+    }
+};
 // Several steps per launch (lbm_step_fused.cu): the tiles of a grid's passes, and
 // one launch of 1 .. p.steps steps.  ok is false where the fused walk does not apply
 // (nx not a multiple of its 16-byte lanes) or single steps are the faster.  Uniform
@@ -83,7 +92,8 @@ long long resident_warps(const void *fn, int warps, int smem);
 struct FusedPlan {
     bool ok = false;
     int steps = 1;  // of a pass
-    int rows = 0, nstrips = 0;
+    int rows = 0;
+    FusedStrips strips{};
     long long ntiles = 0;
 };
 Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out);

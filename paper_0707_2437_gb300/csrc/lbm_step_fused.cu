@@ -23,24 +23,40 @@ constexpr int kWarps = 4;  // warps per block
 template <int S, int RND, int VA, int TS>
 __global__ void __launch_bounds__(32 * kWarps, 2)
     k_step_fused(const void *__restrict__ fin, void *__restrict__ fout, int nx, int ny, size_t P,
-                 int nstrips, long long ntiles, int rows, Coef c, int steps, const uint32_t *tdev,
+                 FusedStrips strips, long long ntiles, int rows, Coef c, int steps, const uint32_t *tdev,
                  uint32_t toff, const float *__restrict__ a15f) {
     extern __shared__ uint4 walk_smem[];
     pdl_enter();
     const long long tile = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (tile >= ntiles) return;  // whole warps leave together
-    const int strip = (int)(tile % nstrips), seg = (int)(tile / nstrips);
-    const int y0 = seg * rows;
-    FusedWalk<S, LD_NC, RND, VA, TS> w(fin, fout, nx, ny, P, strip * FusedGeom<S, TS>::COLS);
+    constexpr bool PACK = fused_packs(S);
+    // Whole strips segment by segment, then the packed tiles.
+    const long long whole = (long long)strips.full * ((ny + rows - 1) / rows);
+    int seg, x0, y0, y1, lanes = 32;
+    if (!PACK || tile < whole) {
+        seg = (int)(tile / strips.full);
+        x0 = (int)(tile - (long long)seg * strips.full) * FusedGeom<S, TS>::COLS;
+        y0 = seg * rows;
+        y1 = min(ny, y0 + rows);
+    } else {
+        seg = (int)(tile - whole);
+        x0 = strips.full * FusedGeom<S, TS>::COLS;
+        y0 = seg * strips.pieces * rows;
+        y1 = min(ny, y0 + strips.pieces * rows);
+        lanes = strips.lanes;
+    }
+    const int high = min(rows, y1 - y0);
+    FusedWalk<S, LD_NC, RND, VA, TS, PACK> w(fin, fout, nx, ny, P, x0, y0, y1, high,
+                                             PACK ? lanes : 32);
     if constexpr (VA) w.a15f = a15f;
     if constexpr (RND) w.set_step((tdev ? *tdev : 0u) + toff);
     // Neighbouring segments walk in opposite directions, so the rows they
     // share are read by both at about the same time.
-    w.run(y0, min(ny, y0 + rows), (seg & 1) ? -1 : 1, steps, c,
+    w.run(high, (seg & 1) ? -1 : 1, steps, c,
           walk_smem + (threadIdx.x >> 5) * fused_vecs<S, VA, TS>());
 }
 
-using FusedKernel = void (*)(const void *, void *, int, int, size_t, int, long long, int, Coef, int,
+using FusedKernel = void (*)(const void *, void *, int, int, size_t, FusedStrips, long long, int, Coef, int,
                              const uint32_t *, uint32_t, const float *);
 
 struct Choice {
@@ -82,14 +98,14 @@ Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out)
         if (e != cudaSuccess) return e;
         const long long wave = resident_warps((const void *)ch.fn, kWarps, ch.smem);
         if (wave <= 0) return cudaErrorLaunchOutOfResources;
-        const int cols = fused_cols(storage, steps), nstrips = (nx + cols - 1) / cols;
+        const FusedStrips strips = fused_strips(storage, steps, nx);
         // Tile height: a tile costs some row steps beyond its rows, and a launch
         // lasts as many tiles as its fullest warp slot runs.
         const int most = fused_most_rows(storage, steps);
         long long least = -1;
         int rows = 2;
         for (int r = 2; r <= most; ++r) {
-            const long long tiles = (long long)nstrips * ((ny + r - 1) / r);
+            const long long tiles = strips.tiles((ny + r - 1) / r);
             const long long cost = ((tiles + wave - 1) / wave) * (r + fused_overhead(steps));
             if (least < 0 || cost < least) {
                 least = cost;
@@ -107,8 +123,8 @@ Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out)
         best = per_step;
         out->steps = steps;
         out->rows = rows;
-        out->nstrips = nstrips;
-        out->ntiles = (long long)nstrips * ((ny + rows - 1) / rows);
+        out->strips = strips;
+        out->ntiles = strips.tiles((ny + rows - 1) / rows);
     }
     // Short tiles repeat too much of the earlier steps' work, and a launch of them
     // lasts one walk of eight rows or more however small the grid: single steps are
@@ -130,7 +146,7 @@ Err launch_fused(const FusedPlan &p, int storage, const void *fin, void *fout, i
     if (!p.ok) return cudaErrorInvalidValue;
     const Choice ch = choose(storage, rnd, a15f != nullptr, p.steps);
     return launch_pdl(ch.fn, (unsigned)((p.ntiles + kWarps - 1) / kWarps), 32u * kWarps,
-                      (size_t)ch.smem, st, fin, fout, nx, ny, P, p.nstrips, p.ntiles, p.rows, c,
+                      (size_t)ch.smem, st, fin, fout, nx, ny, P, p.strips, p.ntiles, p.rows, c,
                       steps, tdev, toff, a15f);
 }
 

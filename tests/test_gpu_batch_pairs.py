@@ -58,7 +58,7 @@ def test_pairs_in_batches_equal_single_steps(lbm, kind, lens, rows, schedule):
 def test_tall_tiles_in_a_batch_equal_single_steps(lbm):
     """Grids tall enough for FP32's passes of three steps in lockstep (tiles over 64
     rows on every resident warp), with limits that leave one and two steps."""
-    sizes, limits = [(8, 100003), (124, 20001)], [10, 8]
+    sizes, limits = [(64, 100003), (124, 20001)], [10, 8]
     fields = [workloads.fourier_modes(nx, ny, amp=1e-2, seed=nx) for nx, ny in sizes]
     grids = []
     for (nx, ny), f in zip(sizes, fields):
