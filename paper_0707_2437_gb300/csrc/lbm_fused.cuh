@@ -104,6 +104,10 @@ struct FusedGeom {
     static constexpr int HALO = (2 * TS + V - 1) / V;   // halo lanes a side
     static constexpr int COLS = (32 - 2 * HALO) * V;    // columns a strip stores
 };
+// A width of a whole number of words of 4 bytes, of at least a lane's vector.
+inline bool fused_width(int storage, int nx) {
+    return storage == ST_F32 ? nx >= 4 : nx >= 8 && nx % 2 == 0;
+}
 constexpr int fused_vec(int storage) { return storage == ST_F32 ? 4 : 8; }
 constexpr int fused_cols(int storage, int steps) {
     return storage == ST_F32 ? (steps == 3 ? FusedGeom<ST_F32, 3>::COLS : FusedGeom<ST_F32, 2>::COLS)
@@ -116,7 +120,7 @@ constexpr int fused_most_rows(int storage, int steps) {
     return storage == ST_F32 && steps == 2 ? 64 : 512;
 }
 
-// The strips of nx columns, a multiple of fused_vec.  Packing saves walks of mostly
+// The strips of nx columns (a multiple of fused_vec where tiles are packed).  Packing saves walks of mostly
 // idle lanes, which pays in the 16-bit kinds, bound by issue: FP16 4096^2 76.2 -> 71.8
 // us a step, 8192^2 279 -> 272, 512 uneven FP16 grids in a batch 209k -> 229k MLUPS.
 // FP32 passes are bound by memory and gain nothing (2048^2 with three steps 26.3 /
@@ -126,8 +130,8 @@ constexpr int fused_most_rows(int storage, int steps) {
 constexpr bool fused_packs(int storage) { return storage != ST_F32; }
 inline FusedStrips fused_strips(int storage, int steps, int nx) {
     const int vec = fused_vec(storage), use = fused_cols(storage, steps) / vec, halo = 32 - use;
-    const int n = nx / vec, rest = n % use, pieces = rest ? 32 / (rest + halo) : 0;
-    if (pieces == 1 || (rest && !fused_packs(storage))) return {n / use + 1, 0, 0};
+    const int n = (nx + vec - 1) / vec, rest = n % use, pieces = rest ? 32 / (rest + halo) : 0;
+    if (pieces == 1 || (rest && (!fused_packs(storage) || nx % vec))) return {n / use + 1, 0, 0};
     return {n / use, rest + halo, pieces};
 }
 // Row steps a tile costs beyond its rows (the pulls and collisions at its ends).
@@ -144,16 +148,25 @@ template <int S, int TS>
 constexpr bool fused_alpha_ring() {
     return S != ST_F32 || TS < 3;
 }
-template <int S, int VA, int TS>
+// RAG: a staging row for the stores.
+template <int S, int VA, int TS, bool RAG = false>
 constexpr int fused_vecs() {
-    return (2 + 2 * (TS - 1)) * 9 * 32 +
+    return (2 + 2 * (TS - 1) + (RAG ? 1 : 0)) * 9 * 32 +
            (VA && fused_alpha_ring<S, TS>() ? (2 * TS + 2) * (FusedGeom<S, TS>::V / 4) * 32 : 0);
 }
 
 // PACK: tiles may be packed.  Otherwise the rows are the warp's, not the lane's, which
 // saves about 1 % (nine FP32 grids of 2048^2 in the flow schedule 173.6k / 174.4k).
-template <int S, int LD, int RND, int VA, int TS, bool PACK>
+// RAG: a width that is no multiple of the lanes' vectors.  Rows then start at any word
+// of 4 bytes, so they are copied word by word, lane after lane along the row (the
+// shared-memory image of a row is the same), and stored that way from a staging row.
+template <int S, int LD, int RND, int VA, int TS, bool PACK, bool RAG = false>
 struct FusedWalk {
+    static_assert(!RAG || (LD == LD_NC && !VA && !PACK),
+                  "4-byte copies go through L1; no alpha rows, whole strips");
+    static constexpr int WS = FusedGeom<S, TS>::V / 4;  // sites of a word
+    int col[RAG ? 4 : 1] = {};  // RAG: the column of words lane, lane + 32, ... of a row,
+    uint32_t mine = 0;          // and the ones among them that the strip stores
     static constexpr int V = FusedGeom<S, TS>::V;
     static constexpr int HALO = FusedGeom<S, TS>::HALO;
     static_assert(Pack<S, V>::NW == 4, "a lane holds one 16-byte vector per direction");
@@ -190,6 +203,16 @@ struct FusedWalk {
         own = act ? (PACK ? max(0, min(rows, y1 - ylo)) : rows) : 0;
         xl = xu % nx;
         if (xl < 0) xl += nx;
+        if constexpr (RAG) {
+            own = rows;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int w = 32 * j + lane, x = x0 + (w - 4 * HALO) * WS;
+                if (w >= 4 * HALO && w < 4 * (32 - HALO) && x < nx) mine |= 1u << j;
+                col[j] = x % nx;
+                if (col[j] < 0) col[j] += nx;
+            }
+        }
     }
     __device__ __forceinline__ void set_step(uint32_t step) {
 #pragma unroll
@@ -214,6 +237,23 @@ struct FusedWalk {
     // Copies the lane's nine vectors of pulled row q0 (and its alpha values)
     // into shared memory, as one commit group.
     __device__ __forceinline__ void issue(int qm, int q0, int qp, uint4 *land, uint4 *al) const {
+        if constexpr (RAG) {
+            __syncwarp();  // the row before has been taken by every lane
+            const uint32_t to = (uint32_t)__cvta_generic_to_shared(land - lane) + 4 * lane;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const int sr = (EYi(i) > 0) ? qm : ((EYi(i) < 0) ? qp : q0);
+                const T *src = fin + ((size_t)i * P + (size_t)sr * nx);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                                     to + 512 * i + 128 * j),
+                                 "l"(src + col[j])
+                                 : "memory");
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            return;
+        }
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             const int sr = (EYi(i) > 0) ? qm : ((EYi(i) < 0) ? qp : q0);
@@ -313,8 +353,10 @@ struct FusedWalk {
                          make_float2(a15v[v], a15v[v + 1]));
                 if constexpr (RND) {
                     // nx and v are even: the two sites are a hash pair
+                    int x = xl + v;
+                    if (RAG && x >= nx) x -= nx;
                     const uint32_t base =
-                        sr_pair_base((uint32_t)r * (uint32_t)nx + (uint32_t)(xl + v), rkey);
+                        sr_pair_base((uint32_t)r * (uint32_t)nx + (uint32_t)x, rkey);
 #pragma unroll
                     for (int i = 0; i < 9; ++i)
                         w[i][v >> 1] = sr_pack2<S>(h[i].x, h[i].y, sr_word(base, i));
@@ -326,7 +368,22 @@ struct FusedWalk {
         }
     }
 
-    __device__ __forceinline__ void store(int r, const uint32_t (&w)[9][4]) const {
+    __device__ __forceinline__ void store(int r, const uint32_t (&w)[9][4], uint4 *buf) const {
+        if constexpr (RAG) {
+            uint4 *stage = buf + (2 + 2 * (TS - 1)) * 9 * 32;
+            keep(stage + lane, w);
+            __syncwarp();
+            const uint32_t *from = reinterpret_cast<const uint32_t *>(stage) + lane;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                T *dst = fout + ((size_t)i * P + (size_t)r * nx);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (mine >> j & 1)
+                        *reinterpret_cast<uint32_t *>(dst + col[j]) = from[128 * i + 32 * j];
+            }
+            return;
+        }
         if (PACK ? (unsigned)(r - ylo) >= (unsigned)own : own == 0) return;
         T *dst = fout + ((size_t)r * nx + xl);
 #pragma unroll
@@ -409,7 +466,7 @@ struct FusedWalk {
                 return;
             }
         }
-        store(r, u);
+        store(r, u, buf);
     }
 
     // Advances the pieces' rows (`rows` each, not above ny; walked by all pieces, stored
@@ -467,6 +524,7 @@ struct FusedWalk {
             if constexpr (VA && !RING)
                 fresh = __ldg(reinterpret_cast<const uint4 *>(a15f + (size_t)row * nx + xl));
             asm volatile("cp.async.wait_group 1;" ::: "memory");
+            if constexpr (RAG) __syncwarp();  // the other lanes' copies too
             take(w, slot);
             finish(w, d[0][2]);
             // The words read from the landing row have been used (the

@@ -20,7 +20,7 @@ constexpr int kWarps = 4;  // warps per block
 // FP16 372.5 -> 274 us (245k), BF16 with stochastic rounding 371.0 -> 297; 4096^2 FP32
 // 185 -> 89.7; 2048^2 FP32 49.6 -> 26.3, FP16 25.3 -> 23.4, FP32 with a c2 field 54.0
 // -> 31.1.
-template <int S, int RND, int VA, int TS>
+template <int S, int RND, int VA, int TS, bool RAG>
 __global__ void __launch_bounds__(32 * kWarps, 2)
     k_step_fused(const void *__restrict__ fin, void *__restrict__ fout, int nx, int ny, size_t P,
                  FusedStrips strips, long long ntiles, int rows, Coef c, int steps, const uint32_t *tdev,
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2)
     pdl_enter();
     const long long tile = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (tile >= ntiles) return;  // whole warps leave together
-    constexpr bool PACK = fused_packs(S);
+    constexpr bool PACK = fused_packs(S) && !RAG;
     // Whole strips segment by segment, then the packed tiles.
     const long long whole = (long long)strips.full * ((ny + rows - 1) / rows);
     int seg, x0, y0, y1, lanes = 32;
@@ -46,27 +46,38 @@ __global__ void __launch_bounds__(32 * kWarps, 2)
         lanes = strips.lanes;
     }
     const int high = min(rows, y1 - y0);
-    FusedWalk<S, LD_NC, RND, VA, TS, PACK> w(fin, fout, nx, ny, P, x0, y0, y1, high,
-                                             PACK ? lanes : 32);
+    FusedWalk<S, LD_NC, RND, VA, TS, PACK, RAG> w(fin, fout, nx, ny, P, x0, y0, y1, high,
+                                                  PACK ? lanes : 32);
     if constexpr (VA) w.a15f = a15f;
     if constexpr (RND) w.set_step((tdev ? *tdev : 0u) + toff);
     // Neighbouring segments walk in opposite directions, so the rows they
     // share are read by both at about the same time.
     w.run(high, (seg & 1) ? -1 : 1, steps, c,
-          walk_smem + (threadIdx.x >> 5) * fused_vecs<S, VA, TS>());
+          walk_smem + (threadIdx.x >> 5) * fused_vecs<S, VA, TS, RAG>());
 }
 
-using FusedKernel = void (*)(const void *, void *, int, int, size_t, FusedStrips, long long, int, Coef, int,
-                             const uint32_t *, uint32_t, const float *);
+using FusedKernel = void (*)(const void *, void *, int, int, size_t, FusedStrips, long long, int,
+                             Coef, int, const uint32_t *, uint32_t, const float *);
 
 struct Choice {
     FusedKernel fn = nullptr;
     int smem = 0;
 };
 
-template <int S, int RND, int VA, int TS>
+template <int S, int RND, int VA, int TS, bool RAG = false>
 Choice choice() {
-    return Choice{k_step_fused<S, RND, VA, TS>, kWarps * fused_vecs<S, VA, TS>() * 16};
+    return Choice{k_step_fused<S, RND, VA, TS, RAG>, kWarps * fused_vecs<S, VA, TS, RAG>() * 16};
+}
+
+// The kernel for widths that are no multiple of the lanes' vectors (two steps).
+Choice choose_ragged(int storage, int rnd) {
+    switch (storage) {
+        case ST_F32: return choice<ST_F32, 0, 0, 2, true>();
+        case ST_F16: return rnd ? choice<ST_F16, 1, 0, 2, true>() : choice<ST_F16, 0, 0, 2, true>();
+        case ST_BF16:
+            return rnd ? choice<ST_BF16, 1, 0, 2, true>() : choice<ST_BF16, 0, 0, 2, true>();
+        default: return Choice{};
+    }
 }
 
 Choice choose(int storage, int rnd, bool field, int steps) {
@@ -89,10 +100,12 @@ Choice choose(int storage, int rnd, bool field, int steps) {
 
 Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out) {
     *out = FusedPlan{};
-    if (nx % fused_vec(storage) || (rnd && field)) return cudaSuccess;
+    const bool ragged = nx % fused_vec(storage) != 0;
+    if (!fused_width(storage, nx) || (field && (rnd || ragged))) return cudaSuccess;
     double best = 1e30;
-    for (int steps = 2; steps <= fused_most_steps(storage); ++steps) {
-        const Choice ch = choose(storage, rnd, field, steps);
+    for (int steps = 2; steps <= (ragged ? 2 : fused_most_steps(storage)); ++steps) {
+        const Choice ch = ragged ? choose_ragged(storage, rnd)
+                                 : choose(storage, rnd, field, steps);
         Err e = cudaFuncSetAttribute((const void *)ch.fn,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, ch.smem);
         if (e != cudaSuccess) return e;
@@ -126,17 +139,43 @@ Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out)
         out->strips = strips;
         out->ntiles = strips.tiles((ny + rows - 1) / rows);
     }
-    // Short tiles repeat too much of the earlier steps' work, and a launch of them
-    // lasts one walk of eight rows or more however small the grid: single steps are
-    // the faster where the tiles come out shorter than this.  Measured per step,
-    // single steps against passes (rows in brackets): FP32 768^2 7.16 / 7.15 us (5),
-    // 1024^2 10.97 / 9.41 (8), 2048^2 49.6 / 26.3 (32); with a c2 field 768^2 6.94 /
-    // 7.51, 1024^2 11.75 / 9.89; FP16 1024^2 8.85 / 10.41 (5), 1536^2 15.22 / 15.02
-    // (9), 2048^2 25.31 / 23.43 (16); with stochastic rounding, whose conversion is
-    // the slower for FP16, BF16 1536^2 16.9 / 15.9 (9), 2048^2 27.6 / 24.9 (16), FP16
-    // 2048^2 26.7 / 27.1 (16), 2048 x 4096 55.1 / 47.4 (31).
-    const int least_rows = storage == ST_F32 ? 8 : (rnd && storage == ST_F16 ? 20 : 9);
-    out->ok = out->rows >= least_rows;
+    // Passes or single steps: short tiles repeat much of the earlier steps' work, and a
+    // launch lasts one walk of some rows however small the grid.  Estimates in
+    // microseconds per step: row_us a row step of two steps in the fullest warp slot,
+    // halved; a single step takes `even` a million sites, and `idle` more for every
+    // site's worth of lanes beyond the width in its strips.  Measured per step, single
+    // steps / passes: FP32 768^2 7.16 / 7.15, 1024^2 10.97 / 9.46, 2048^2 49.6 / 26.2,
+    // 124 x 9600 11.4 / 14.8, 244 x 4800 11.1 / 11.8, 248 x 9600 27.1 / 20.4; with a
+    // c2 field 768^2 6.9 / 7.5, 1024^2 11.75 / 9.86, 16 x 100000 54.6 / 60.5; FP16
+    // 1024^2 8.85 / 10.4, 1536^2 15.2 / 15.1, 2048^2 25.3 / 23.5, 136 x 12000 20.7 /
+    // 16.0, 64 x 40000 53.8 / 17.2; with stochastic rounding, whose conversion is the
+    // slower for FP16, BF16 1536^2 16.9 / 16.2, 2048^2 27.6 / 25.3, FP16 2048^2 26.7 /
+    // 27.1, 2048 x 4096 55.1 / 47.4.  Without 16-byte lanes both move words: FP32 1022
+    // x 1024 11.2 / 12.1, 1202 x 1200 16.8 / 15.2, 242 x 4800 12.7 / 16.1, 2002 x 2004
+    // 49.5 / 36.5, 8002 x 8000 730 / 491; FP16 1302 x 1300 15.0 / 15.5, 1402 x 1400
+    // 16.3 / 15.6, 1446 x 1440 16.3 / 18.5, 2002 x 2004 35.2 / 28.2, 8002 x 8000 509 /
+    // 347; BF16 with stochastic rounding 2002 x 2004 36.7 / 30.4, FP16 37.2 / 31.7.
+    const bool wide = storage == ST_F32, slow = rnd && storage == ST_F16;
+    double row_us, even, idle;
+    int strip;  // columns of a single step's strips
+    if (ragged) {
+        row_us = wide ? 2.0 : rnd ? (slow ? 3.0 : 2.82) : 2.6;
+        even = wide ? 11.4 : rnd ? 9.0 : 8.5;
+        idle = 0;
+        strip = 32;
+    } else if (wide) {
+        row_us = 1.43;
+        even = field ? 11.2 : 9.6;
+        idle = field ? 7.0 : 4.0;
+        strip = field ? 64 : 128;
+    } else {
+        row_us = field ? 2.3 : rnd ? (slow ? 2.58 : 2.41) : 2.2;
+        even = field ? 7.0 : rnd ? (slow ? 6.4 : 7.2) : 5.8;
+        idle = 5.3;
+        strip = field ? 128 : 256;
+    }
+    const double lanes = (double)((nx + strip - 1) / strip) * strip / nx;
+    out->ok = best * row_us < 1e-6 * nx * ny * (even + idle * (lanes - 1));
     return cudaSuccess;
 }
 
@@ -144,7 +183,8 @@ Err launch_fused(const FusedPlan &p, int storage, const void *fin, void *fout, i
                  size_t P, const Coef &c, int steps, int rnd, const uint32_t *tdev, uint32_t toff,
                  const float *a15f, cudaStream_t st) {
     if (!p.ok) return cudaErrorInvalidValue;
-    const Choice ch = choose(storage, rnd, a15f != nullptr, p.steps);
+    const Choice ch = nx % fused_vec(storage) ? choose_ragged(storage, rnd)
+                                              : choose(storage, rnd, a15f != nullptr, p.steps);
     return launch_pdl(ch.fn, (unsigned)((p.ntiles + kWarps - 1) / kWarps), 32u * kWarps,
                       (size_t)ch.smem, st, fin, fout, nx, ny, P, p.strips, p.ntiles, p.rows, c,
                       steps, tdev, toff, a15f);

@@ -14,8 +14,8 @@ pytestmark = pytest.mark.gpu
 
 # (nx, ny): tiles tall enough that passes of several steps are taken (FP32 strips of
 # 112 or 120 columns, 16-bit strips of 240).
-SHAPES = {"f32": [(4, 20011), (124, 9803), (1000, 1201), (2048, 1025)],
-          "16": [(8, 30011), (248, 15003), (1200, 2407), (2048, 3077)]}
+SHAPES = {"f32": [(4, 200011), (124, 40003), (1000, 1201), (2048, 1025)],
+          "16": [(8, 30011), (248, 20003), (1200, 3607), (2048, 3077)]}
 
 
 def _state(lbm, kind, nx, ny, calls, lens):
@@ -41,9 +41,20 @@ def test_pairs_of_steps_equal_single_steps(lbm, kind, lens, shape):
     assert np.array_equal(single, pairs)
 
 
-@pytest.mark.parametrize("nx,ny", [(4, 50021), (1012, 4003)])
+@pytest.mark.parametrize("nx,ny", [(60, 50021), (1012, 4003)])
 def test_three_steps_with_a_c2_field_equal_single_steps(lbm, nx, ny):
-    """Grids tall enough for three steps a pass with alpha values in registers: one
-    lane, and nine whole strips of 112 columns and one of four."""
+    """Grids tall enough for three steps a pass with alpha values in registers: part
+    of a strip, and nine whole strips of 112 columns and one of four."""
     single = _state(lbm, "f32", nx, ny, [1] * 14, True)
     assert np.array_equal(single, _state(lbm, "f32", nx, ny, [3, 8, 1, 2], True))
+
+
+@pytest.mark.parametrize("kind,nx,ny", [
+    ("f32", 119, 12001), ("f32", 239, 9001), ("f32", 601, 4001), ("f32", 1001, 1601),
+    ("f16d", 238, 9001), ("f16d", 1202, 3001), ("bf16d", 478, 9001),
+    ("bf16d-sr", 238, 15001), ("f16d-sr", 1202, 5001)])
+def test_passes_at_widths_without_16_byte_lanes(lbm, kind, nx, ny):
+    """Rows that start at any word: strips that end inside a lane, wrapped halo columns
+    that cross the seam inside one, odd and even row alignments."""
+    single = _state(lbm, kind, nx, ny, [1] * 41, False)
+    assert np.array_equal(single, _state(lbm, kind, nx, ny, [2, 35, 1, 3], False))
