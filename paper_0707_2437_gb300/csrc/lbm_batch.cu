@@ -210,6 +210,7 @@ static int build_worklist(lbm_batch *b) {
         d.ny = g->ny;
         d.kind = kind_code(g->storage, batch_vec(b, g), g->rounding ? 1 : 0, g->a15f ? 1 : 0);
         d.per = 1;
+        d.window = 1;
         d.c = g->coef;
         slabs = slabs || g->slab;
     }
@@ -272,18 +273,23 @@ static int build_worklist(lbm_batch *b) {
         // rows serve one.
         std::vector<int> kinds;
         for (const GridDesc &d : gd) kinds.push_back(d.kind);
-        const FlowChoice fc = flow_kernel_for(kinds, b->walk16, !slabs);
+        FlowChoice fc = flow_kernel_for(kinds, b->walk16, !slabs);
         lbm_batch::Group gr;
-        gr.fkernel = fc.fn;
-        gr.smem = fc.smem;
-        gr.fused = fc.fused;
-        gr.rows = b->rows;
-        const int per_pass = fc.fused ? 2 : 1;
-        BCK(resident_blocks((const void *)fc.fn, fc.smem, &gr.max_blocks_per_sm));
-        if (gr.max_blocks_per_sm < 1) return bfail(LBM_ECUDA, "flow kernel cannot be resident");
-        const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
-                                             : gr.max_blocks_per_sm;
-        const long long warps = (long long)per * b->sms * kBatchWarps;
+        long long warps = 0;
+        auto take = [&]() -> int {
+            gr.fkernel = fc.fn;
+            gr.smem = fc.smem;
+            gr.fused = fc.fused;
+            gr.rows = b->rows;
+            BCK(resident_blocks((const void *)fc.fn, fc.smem, &gr.max_blocks_per_sm));
+            if (gr.max_blocks_per_sm < 1) return bfail(LBM_ECUDA, "flow kernel cannot be resident");
+            const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
+                                                 : gr.max_blocks_per_sm;
+            warps = (long long)per * b->sms * kBatchWarps;
+            return LBM_OK;
+        };
+        int rc = take();
+        if (rc != LBM_OK) return rc;
         // A grid's pass takes at least one tile walk, so a grid with fewer tiles than
         // its share of the resident warps (the warps split evenly between the grids)
         // uses shorter tiles: a quarter as tall in single steps; on the fused walk as
@@ -293,25 +299,89 @@ static int build_worklist(lbm_batch *b) {
         // 32 or 24.  Measured: 20 grids of 128^2 to 2048^2 with 1e9 updates between
         // them 8.9, 8.7, 8.4 ms at 48, 32, 24 rows; nine 2048^2 FP32 grids 174k, 168k,
         // 161k MLUPS; 512 uneven grids 138k, 131k, 120k.
+        int tenths = 7;  // of a grid's share of the warps
         auto flow_rows = [&](size_t k, int tallest) {
-            const long long share = std::max<long long>(1, 7 * warps / (10 * (long long)ng));
+            const long long share = std::max<long long>(1, tenths * warps / (10 * (long long)ng));
             const long long r = ((long long)strips(k, 2) * computed_rows(k) + share - 1) / share;
-            return std::max(2 * per_pass, (int)std::min<long long>(tallest, r));
+            return std::max(4, (int)std::min<long long>(tallest, r));
         };
         int tallest = 48;
-        if (fc.fused && b->fit_rows)
+        auto total = [&] {
+            long long n = 0;
+            for (size_t k = 0; k < ng; ++k) {
+                const int r = flow_rows(k, tallest);
+                n += (long long)strips(k, 2) * ((computed_rows(k) + r - 1) / r);
+            }
+            return n;
+        };
+        if (fc.fused && b->fit_rows) {
             for (int h : {48, 32, 24}) {
                 tallest = h;
-                long long total = 0;
-                for (size_t k = 0; k < ng; ++k)
-                    total += (long long)strips(k, 2) *
-                             ((computed_rows(k) + flow_rows(k, h) - 1) / flow_rows(k, h));
-                if (2 * total >= 5 * warps) break;
+                if (2 * total() >= 5 * warps) break;
             }
+            while (tenths < 10 && total() < warps) {
+                ++tenths;
+                if (total() > warps) {
+                    --tenths;
+                    break;
+                }
+            }
+        }
+        auto fused_height = [&](size_t k) {
+            return b->fit_rows ? flow_rows(k, tallest) : std::max(4, b->rows);
+        };
+        // A 16-bit batch whose strips of 240 columns are badly filled, or whose tiles
+        // come out short, is faster in single steps of 256-column strips.  Estimates of
+        // a step in microseconds, as for a single grid's passes.  Measured, single /
+        // fused, k MLUPS: FP16 64 grids of 256^2 140 / 108, nine of 512^2 147 / 113, 64
+        // of 512^2 166 / 165, 32 of 200 x 300 119 / 131, 128 of 128^2 74 / 93, nine of
+        // 2048^2 160 / 238; with stochastic rounding 64 of 256^2 109 / 93 (BF16 108 /
+        // 102), nine of 512^2 107 / 98 (BF16 106 / 111), 32 of 200 x 300 88 / 113.
+        //
+        // FP32 and 16-bit grids together take single steps where the batch is small and
+        // the fused walk's strips have a fifth more columns than those of single
+        // steps (k MLUPS, single / fused: 8 grids of 256^2 42.7 / 34.4, 16 60 / 53, four
+        // of 512^2 64 / 59, nine 71 / 90, 32 of 128^2 35.3 / 33.7, ten of 200^2 33 / 35,
+        // eight of 384^2 51 / 64).
+        const int storage = b->grids[0]->storage;
+        bool one_kind = true;
+        for (int kd : kinds) one_kind = one_kind && kd == kinds[0];
+        bool singles = false;
+        if (fc.fused && !one_kind) {
+            double sites = 0, fused = 0, single = 0;
+            for (size_t k = 0; k < ng; ++k) {
+                const lbm_grid *g = b->grids[k];
+                sites += (double)g->nx * computed_rows(k);
+                fused += (double)strips(k, 2) * fused_cols(g->storage, 2) * computed_rows(k);
+                single += 32.0 * strips(k, 1) * batch_vec(b, g) * computed_rows(k);
+            }
+            singles = sites < 1.1e6 && fused > 1.2 * single;
+        }
+        if (fc.fused && one_kind && storage != ST_F32) {
+            const bool rnd = b->grids[0]->rounding != 0;
+            double work = 0, pass = 0, sites = 0, single = rnd ? 5.0 : 4.0;
+            for (size_t k = 0; k < ng; ++k) {
+                const int r = fused_height(k), ny = computed_rows(k), nx = b->grids[k]->nx;
+                const int segs = (ny + r - 1) / r, over = fused_overhead(2);
+                work += (double)strips(k, 2) * (ny + over * segs);
+                pass = std::max(pass, (double)std::min(r, ny) + over);
+                const double lanes = 256.0 * strips(k, 1) / nx;
+                sites += (double)nx * ny;
+                single += 1e-6 * nx * ny * ((rnd ? 6.5 : 5.5) + 5.3 * (lanes - 1));
+            }
+            const double row_us = rnd ? (storage == ST_F16 ? 2.58 : 2.41) : 2.2;
+            singles = single < 0.5 * row_us * std::max(pass, work / warps) + 0.25e-6 * sites;
+        }
+        if (singles) {
+            fc = flow_kernel_for(kinds, b->walk16, false);
+            rc = take();
+            if (rc != LBM_OK) return rc;
+        }
+        const int per_pass = fc.fused ? 2 : 1;
         for (size_t k = 0; k < ng; ++k) {
             int rows = b->rows;
             if (fc.fused) {
-                rows = b->fit_rows ? flow_rows(k, tallest) : std::max(2 * per_pass, rows);
+                rows = fused_height(k);
             } else {
                 const long long tall =
                     (long long)strips(k, 1) * ((computed_rows(k) + rows - 1) / rows);
@@ -320,6 +390,7 @@ static int build_worklist(lbm_batch *b) {
             add_tiles(k, rows, per_pass);
         }
         gr.count = (int)tiles.size();
+        for (GridDesc &d : gd) d.window = gr.fused ? 1 : 2;
         b->groups.push_back(gr);
         if (tiles.size() > b->prog_cap) {
             cudaFree(b->d_prog);

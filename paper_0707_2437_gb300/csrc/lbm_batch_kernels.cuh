@@ -40,6 +40,7 @@ struct GridDesc {
     // when a neighbouring segment or strip can be smaller than the pass's
     // reach: two sites a step).
     int tile0, ntile, nstrips, nsegs, dseg, dstrip;
+    int window;  // passes that tickets may run ahead of the completed tiles
 };
 
 // A tile: one strip (x0) of one segment (rows y0 .. y1-1, walked in
@@ -260,9 +261,9 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
 }
 
 // ---------------------------------------------------------------------------
-// Flow schedule: every grid advances its own passes (a step, or several for
-// grids on the fused walk), with no barrier across the batch.  Each grid hands out tickets m = k * ntile + t (step k, tile t)
-// from its own counter, in step order.  A warp holding (k, t) waits until
+// Flow schedule: every grid advances its own passes (a step, or two on the fused
+// walk), with no barrier across the batch.  Each grid hands out tickets m = k * ntile
+// + t (pass k, tile t) from its own counter, in pass order.  A warp holding (k, t) waits until
 // every tile its step reads from or overwrites (the tiles within dseg
 // segments and dstrip strips, wrapped, itself included) has completed step
 // k - 1, runs the tile, and publishes k + 1 completed steps for it.  All
@@ -273,15 +274,16 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
 // Warps pick grids round-robin, so every grid gets about the same number of
 // tiles per unit time: small grids take many steps while large ones take
 // few, instead of every grid waiting for the whole batch at every step.  A
-// grid's tickets may run at most kFlowWindow passes ahead of its completed
+// grid's tickets may run at most `window` passes ahead of its completed
 // tiles, so that the warps a short grid's step chain would hold waiting go to
-// other grids (two passes ahead: the serving mix's launch 9.8 ms against 8.9).
+// other grids: one on the fused walk (two: the serving mix's launch 9.8 ms against
+// 8.9), two in single steps, whose tiles are more than the fused walk's (two grids of
+// 1024^2 in FP16 131k MLUPS against 124k with one).
 //
 // Control words (zeroed before each launch): per grid, tickets taken and
 // tiles completed (64-bit, each on its own 128-byte line); globally the
 // round-robin counter and the number of grids whose last ticket is taken.
 // Every wait is bounded by the same wall-clock limit as the barrier.
-constexpr int kFlowWindow = 1;
 constexpr int kFlowCtlWords = 32;  // unsigned long long words per grid: [0] taken, [16] done
 constexpr int kFlowRR = 0;         // words of `glob`
 constexpr int kFlowExh = 32;
@@ -371,7 +373,7 @@ __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, in
                     volatile unsigned long long *c = ctl + (size_t)cand * kFlowCtlWords;
                     const unsigned long long taken = c[0];
                     if (taken >= total) continue;
-                    if (taken - c[16] >= (unsigned long long)kFlowWindow * G.ntile) continue;
+                    if (taken - c[16] >= (unsigned long long)G.window * G.ntile) continue;
                     const unsigned long long mm =
                         atomicAdd(ctl + (size_t)cand * kFlowCtlWords, 1ULL);
                     if (mm >= total) continue;
@@ -442,24 +444,33 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
               });
 }
 
-// Flow kernel for a batch of one 4-site 16-bit walk, inlined (the register
-// budget of k_batch_one: 16 warps per SM, measured faster than 12 without
-// spills although the flow loop's state costs a few bytes of spill).
-template <int S, int PD>
+// Flow kernel for a batch of one single-step walk of V sites a lane, inlined
+// (the register budget of k_batch_one: 16 warps per SM, measured faster than 12
+// without spills although the flow loop's state costs a few bytes of spill).
+template <int S, int V, int PD, int RND, int VA = 0>
 __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
     k_flow_one(const GridDesc *__restrict__ grids, int ngrids, const Tile *__restrict__ tiles,
                const long long *__restrict__ limit, const int *__restrict__ parity0,
                const uint32_t *__restrict__ t0, unsigned long long *ctl, int *prog,
                unsigned *glob, const int *__restrict__ nwork_p, int *status,
                unsigned long long timeout_ns) {
+    __shared__ uint4 rowbuf[V == 8 ? kBatchWarps : 1][2 * 9 * 32];
+    (void)rowbuf;
     flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
-              timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t, int) {
-                  Walker<S, 4, LD_CG> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P, t.x0);
+              timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int) {
+                  Walker<S, V, LD_CG, RND, VA> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P,
+                                                 t.x0);
+                  if constexpr (VA) w.a15f = g.a15f;
+                  if constexpr (RND) w.set_step(step);
                   const Coef c = g.c;
-                  if constexpr (PD == 2)
+                  if constexpr (V == 8)
+                      w.run_async(t.y0, t.y1, t.dir, c, &rowbuf[threadIdx.x >> 5][0]);
+                  else if constexpr (PD == 2)
                       w.run_prefetch2(t.y0, t.y1, t.dir, c);
-                  else
+                  else if constexpr (PD == 1)
                       w.run_prefetch(t.y0, t.y1, t.dir, c);
+                  else
+                      w.run(t.y0, t.y1, t.dir, c);
               });
 }
 
@@ -519,6 +530,32 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 2)
               });
 }
 
+// The same with single steps.
+template <int S2, int RND2>
+__global__ void __launch_bounds__(32 * kBatchWarps, 3)
+    k_flow_two_single(const GridDesc *__restrict__ grids, int ngrids,
+                      const Tile *__restrict__ tiles, const long long *__restrict__ limit,
+                      const int *__restrict__ parity0, const uint32_t *__restrict__ t0,
+                      unsigned long long *ctl, int *prog, unsigned *glob,
+                      const int *__restrict__ nwork_p, int *status,
+                      unsigned long long timeout_ns) {
+    __shared__ uint4 rowbuf[kBatchWarps][2 * 9 * 32];
+    flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
+              timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int) {
+                  const Coef c = g.c;
+                  if (g.kind == kind_code(ST_F32, 4, 0)) {
+                      Walker<ST_F32, 4, LD_CG> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P,
+                                                 t.x0);
+                      w.run(t.y0, t.y1, t.dir, c);
+                  } else {
+                      Walker<S2, 8, LD_CG, RND2> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P,
+                                                   t.x0);
+                      if constexpr (RND2) w.set_step(step);
+                      w.run_async(t.y0, t.y1, t.dir, c, &rowbuf[threadIdx.x >> 5][0]);
+                  }
+              });
+}
+
 using FlowKernel = void (*)(const GridDesc *, int, const Tile *, const long long *, const int *,
                             const uint32_t *, unsigned long long *, int *, unsigned *,
                             const int *, int *, unsigned long long);
@@ -536,9 +573,9 @@ constexpr int fused_smem() {
 }
 
 // The flow kernel for a batch's kinds: the fused walks when all grids share
-// one kind that has it, or FP32 and one such 16-bit kind (`fuse`: allowed);
-// a specialised single-step kernel when all share another walk, else the
-// general k_flow.
+// one kind that has it, or FP32 and one such 16-bit kind (`fuse`: allowed), else
+// their single-step kernels; a specialised single-step kernel when all share
+// another walk, else the general k_flow.
 FlowChoice flow_kernel_for(const std::vector<int> &kinds, int walk16, bool fuse) {
     bool same = true;
     for (int k : kinds) same = same && k == kinds[0];
@@ -564,33 +601,45 @@ FlowChoice flow_kernel_for(const std::vector<int> &kinds, int walk16, bool fuse)
         const bool two = walk16 == LBM_WALK16_V4_PF2;
         switch (kinds[0]) {
             case kind_code(ST_F16, 4, 0):
-                return {two ? k_flow_one<ST_F16, 2> : k_flow_one<ST_F16, 1>, 0, false};
+                return {two ? k_flow_one<ST_F16, 4, 2, 0> : k_flow_one<ST_F16, 4, 1, 0>, 0, false};
             case kind_code(ST_BF16, 4, 0):
-                return {two ? k_flow_one<ST_BF16, 2> : k_flow_one<ST_BF16, 1>, 0,
+                return {two ? k_flow_one<ST_BF16, 4, 2, 0> : k_flow_one<ST_BF16, 4, 1, 0>, 0,
                         false};
+            case kind_code(ST_F32, 4, 0):
+                return {k_flow_one<ST_F32, 4, 0, 0>, 0, false};
+            case kind_code(ST_F32, 4, 0, 1):
+                return {k_flow_one<ST_F32, 4, 0, 0, 1>, 0, false};
+            case kind_code(ST_F16, 8, 0):
+                return {k_flow_one<ST_F16, 8, 0, 0>, 0, false};
+            case kind_code(ST_BF16, 8, 0):
+                return {k_flow_one<ST_BF16, 8, 0, 0>, 0, false};
+            case kind_code(ST_F16, 8, 1):
+                return {k_flow_one<ST_F16, 8, 0, 1>, 0, false};
+            case kind_code(ST_BF16, 8, 1):
+                return {k_flow_one<ST_BF16, 8, 0, 1>, 0, false};
             default:
                 break;
         }
     }
     // FP32 (4 sites per lane) with one 16-bit kind of 8 sites per lane.
     int other = -1;
-    bool mix = fuse && !kinds.empty();
+    bool mix = !kinds.empty();
     for (int k : kinds) {
         if (k == kind_code(ST_F32, 4, 0)) continue;
         if (other == -1) other = k;
         mix = mix && k == other;
     }
     if (mix && other != -1) {
-        constexpr int smem = fused_smem<ST_F32, 0, 2>();
+        const int smem = fuse ? fused_smem<ST_F32, 0, 2>() : 0;
         switch (other) {
             case kind_code(ST_F16, 8, 0):
-                return {k_flow_two<ST_F16, 0>, smem, true};
+                return {fuse ? k_flow_two<ST_F16, 0> : k_flow_two_single<ST_F16, 0>, smem, fuse};
             case kind_code(ST_BF16, 8, 0):
-                return {k_flow_two<ST_BF16, 0>, smem, true};
+                return {fuse ? k_flow_two<ST_BF16, 0> : k_flow_two_single<ST_BF16, 0>, smem, fuse};
             case kind_code(ST_F16, 8, 1):
-                return {k_flow_two<ST_F16, 1>, smem, true};
+                return {fuse ? k_flow_two<ST_F16, 1> : k_flow_two_single<ST_F16, 1>, smem, fuse};
             case kind_code(ST_BF16, 8, 1):
-                return {k_flow_two<ST_BF16, 1>, smem, true};
+                return {fuse ? k_flow_two<ST_BF16, 1> : k_flow_two_single<ST_BF16, 1>, smem, fuse};
             default:
                 break;
         }
