@@ -298,7 +298,9 @@ static int build_worklist(lbm_batch *b) {
         // whole batch: 48 rows if that still leaves two and a half tiles a warp, else
         // 32 or 24.  Measured: 20 grids of 128^2 to 2048^2 with 1e9 updates between
         // them 8.9, 8.7, 8.4 ms at 48, 32, 24 rows; nine 2048^2 FP32 grids 174k, 168k,
-        // 161k MLUPS; 512 uneven grids 138k, 131k, 120k.
+        // 161k MLUPS; 512 uneven grids 138k, 131k, 120k.  Where one wave holds all tiles
+        // anyway, up to the whole share: nine 512^2 FP32 grids 118k -> 134k, 32 FP16 ones
+        // of 200 x 300 109k -> 131k.
         int tenths = 7;  // of a grid's share of the warps
         auto flow_rows = [&](size_t k, int tallest) {
             const long long share = std::max<long long>(1, tenths * warps / (10 * (long long)ng));

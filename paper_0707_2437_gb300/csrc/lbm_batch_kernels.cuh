@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 2)
 
 // Flow kernel for the serving mix: FP32 grids and 16-bit grids of storage S2
 // and rounding RND2, all on the fused walk, both walks inlined (20 grids of 128^2
-// to 2048^2 sharing 1e9 updates: 12.8 ms with single steps, 10.0 ms now, with
+// to 2048^2 sharing 1e9 updates: 12.8 ms with single steps, 8.4 ms now, with
 // their initialisation and moments).
 template <int S2, int RND2>
 __global__ void __launch_bounds__(32 * kBatchWarps, 2)
@@ -728,10 +728,10 @@ __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
 // k_step_fused is, at its occupancy and two rows of copies in flight; a half or a
 // third as many barriers as single steps.  Measured, lockstep, 100 steps a call,
 // single steps before and passes now: nine 2048^2 grids FP32 93k -> 187k MLUPS, FP16
-// 170k -> 234k, BF16 with stochastic rounding 168k -> 211k, FP32 with a c2 field 85k
-// -> 168k; 512 uneven grids FP32 93k -> 178k, FP16 159k -> 210k, half and half 115k
-// -> 185k.  Flow schedule: nine 2048^2 FP32 92k -> 174k, FP16 168k -> 238k; 512 uneven,
-// half and half, 83k -> 137k.
+// 170k -> 241k, BF16 with stochastic rounding 168k -> 216k, FP32 with a c2 field 85k
+// -> 168k; 512 uneven grids FP32 93k -> 178k, FP16 159k -> 229k, half and half 115k
+// -> 191k.  Flow schedule: nine 2048^2 FP32 92k -> 174k, FP16 168k -> 237k; 512 uneven,
+// half and half, 83k -> 145k.
 template <int S, int RND, int VA, int TS>
 __global__ void __launch_bounds__(32 * kBatchWarps, 2)
     k_batch_fused(const GridDesc *__restrict__ grids, const Tile *__restrict__ tiles, int ntiles,

@@ -16,10 +16,12 @@ constexpr int kWarps = 4;  // warps per block
 // stage's waiting row in shared memory too, spent the time on shared-memory traffic
 // in FP32 (71 % of its bandwidth; 8192^2 158k against 172k MLUPS) and spilled in the
 // 16-bit kinds (214k against 245k).  Measured on one grid, per step, single steps
-// before and passes now: 8192^2 FP32 705.7 -> 353 us (190k MLUPS; 24 B an update),
-// FP16 372.5 -> 274 us (245k), BF16 with stochastic rounding 371.0 -> 297; 4096^2 FP32
-// 185 -> 89.7; 2048^2 FP32 49.6 -> 26.3, FP16 25.3 -> 23.4, FP32 with a c2 field 54.0
-// -> 31.1.
+// before and passes now: 8192^2 FP32 705.7 -> 354 us (190k MLUPS; 24 B an update),
+// FP16 372.5 -> 271 us (248k), BF16 with stochastic rounding 371.0 -> 295; 4096^2 FP32
+// 185 -> 89.8, FP16 107 -> 71.7; 2048^2 FP32 49.6 -> 26.3, FP16 25.3 -> 23.5, FP32 with
+// a c2 field 54.0 -> 29.8.  RAG (rows copied and stored word by word, coalesced, which
+// adds a staging row and some 100 of 1200 instructions a row step): 2002 x 2004 FP32
+// 49.5 -> 36.5, FP16 35.2 -> 28.2.
 template <int S, int RND, int VA, int TS, bool RAG>
 __global__ void __launch_bounds__(32 * kWarps, 2)
     k_step_fused(const void *__restrict__ fin, void *__restrict__ fout, int nx, int ny, size_t P,

@@ -80,3 +80,34 @@ def test_tall_tiles_in_a_batch_equal_single_steps(lbm):
             for _ in range(n + 3):
                 h.step(1)
             assert np.array_equal(h.get_state()[0], state)
+
+
+@pytest.mark.parametrize("kind", ["f16d", "bf16d", "f16d-sr", "bf16d-sr", "mixed"])
+@pytest.mark.parametrize("nx,ny", [(256, 40), (264, 33)])
+def test_small_flow_batches_equal_solo_grids(lbm, kind, nx, ny):
+    """Few grids whose strips of 240 columns are badly filled (one column beyond a strip
+    of single steps too): the flow schedule steps them one step at a time."""
+    def make(k):
+        st = ("f32" if k % 2 else "f16d") if kind == "mixed" else kind
+        g = lbm.Grid(nx, ny, 0.6 + 0.1 * k, 0.2, st.replace("-sr", ""))
+        if st.endswith("-sr"):
+            g.set_rounding("stochastic")
+        g.init(*workloads.fourier_modes(nx, ny, amp=1e-2, seed=k))
+        return g
+
+    limits = [5, 12, 9]
+    grids = [make(k) for k in range(3)]
+    b = lbm.Batch(grids)
+    b.set_schedule("flow")
+    b.step(12, limits)
+    b.step(3)
+    assert b.sync() == 0
+    got = [g.get_state()[0] for g in grids]
+    b.close()
+    for g in grids:
+        g.close()
+    for k, state in enumerate(got):
+        with make(k) as h:
+            for _ in range(limits[k] + 3):
+                h.step(1)
+            assert np.array_equal(h.get_state()[0], state)
