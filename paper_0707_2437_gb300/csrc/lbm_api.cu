@@ -34,6 +34,7 @@ static int fail(int code, const std::string &msg) {
 
 static int cuda_fail(cudaError_t e, const char *where) {
     g_last_error = std::string(where) + ": " + cudaGetErrorString(e);
+    cudaGetLastError();  // reported here: a later launch does not meet it again
     return e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
 }
 

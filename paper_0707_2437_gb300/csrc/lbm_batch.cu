@@ -91,6 +91,9 @@ struct lbm_batch {
     int paired = 0;
     // Per grid, the steps of its passes (as of the work-list).
     std::vector<int> per;
+    // The work-list on the device is the one of the settings above.  A build that fails
+    // leaves none, and the next step call builds again before it launches anything.
+    bool built = false;
 };
 
 static int bfail(int code, const std::string &m) {
@@ -100,6 +103,7 @@ static int bfail(int code, const std::string &m) {
 
 static int bcuda(cudaError_t e, const char *where) {
     set_error(std::string(where) + ": " + cudaGetErrorString(e));
+    cudaGetLastError();  // reported here: a later launch does not meet it again
     return e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
 }
 
@@ -144,7 +148,7 @@ static int upload_worklist(lbm_batch *b, const std::vector<GridDesc> &gd,
         b->built_a15f.push_back(g->a15f);
         b->built_rounding.push_back(g->rounding);
     }
-    drop_graph(b);
+    b->built = true;
     return LBM_OK;
 }
 
@@ -192,6 +196,8 @@ static int fused_rows(const std::vector<std::pair<FusedStrips, int>> &grids, lon
 
 // (Re)builds the device grid table and the tile work-list.
 static int build_worklist(lbm_batch *b) {
+    b->built = false;
+    drop_graph(b);  // (it launches on the old list)
     const size_t ng = b->grids.size();
     std::vector<GridDesc> gd(ng);
     std::vector<Tile> tiles;
@@ -397,6 +403,7 @@ static int build_worklist(lbm_batch *b) {
         if (tiles.size() > b->prog_cap) {
             cudaFree(b->d_prog);
             b->d_prog = nullptr;
+            b->prog_cap = 0;
             BCK(cudaMalloc(&b->d_prog, sizeof(int) * tiles.size()));
             b->prog_cap = tiles.size();
         }
@@ -820,7 +827,7 @@ extern "C" int lbm_batch_step(lbm_batch_t b, long long n, const long long *limit
     if (b->schedule == LBM_SCHEDULE_FLOW && n > 0x7fffffffLL)
         return bfail(LBM_EINVAL, "lbm_batch_step: flow schedule takes at most 2^31 - 1 steps a call");
     if (n == 0) return LBM_OK;
-    bool stale = false;
+    bool stale = !b->built;
     for (size_t k = 0; k < b->grids.size(); ++k) {
         const lbm_grid *g = b->grids[k];
         if (g->drive) return bfail(LBM_EINVAL, "lbm_batch_step: a grid has a drive");
@@ -829,7 +836,8 @@ extern "C" int lbm_batch_step(lbm_batch_t b, long long n, const long long *limit
         stale = stale || g->a15f != b->built_a15f[k] || g->rounding != b->built_rounding[k];
     }
     if (stale) {
-        // A grid's c2 field or rounding changed since the work-list was built.
+        // A grid's c2 field or rounding changed since the work-list was built, or its
+        // last build failed.
         BCK(cudaStreamSynchronize(b->stream));
         int rc = build_worklist(b);
         if (rc != LBM_OK) return rc;
@@ -858,7 +866,7 @@ extern "C" int lbm_batch_set_config(lbm_batch_t b, int rows, int blocks_per_sm) 
         return bfail(LBM_EINVAL, "lbm_batch_set_config: bad argument");
     BCK(cudaStreamSynchronize(b->stream));
     b->blocks_per_sm = blocks_per_sm;
-    if (rows != b->rows || b->fit_rows) {
+    if (rows != b->rows || b->fit_rows || !b->built) {
         b->rows = rows;
         b->fit_rows = false;
         return build_worklist(b);
@@ -871,7 +879,7 @@ extern "C" int lbm_batch_set_walk16(lbm_batch_t b, int walk) {
     if (!b || walk < LBM_WALK16_AUTO || walk > LBM_WALK16_V4_PF2)
         return bfail(LBM_EINVAL, "lbm_batch_set_walk16: unknown walk");
     BCK(cudaStreamSynchronize(b->stream));
-    if (walk == b->walk16) return LBM_OK;
+    if (walk == b->walk16 && b->built) return LBM_OK;
     b->walk16 = walk;
     return build_worklist(b);
 }
@@ -1003,7 +1011,7 @@ extern "C" int lbm_batch_set_schedule(lbm_batch_t b, int schedule) {
     if (!b || schedule < LBM_SCHEDULE_LOCKSTEP || schedule > LBM_SCHEDULE_FLOW)
         return bfail(LBM_EINVAL, "lbm_batch_set_schedule: unknown schedule");
     BCK(cudaStreamSynchronize(b->stream));
-    if (schedule == b->schedule) return LBM_OK;
+    if (schedule == b->schedule && b->built) return LBM_OK;
     b->schedule = schedule;
     return build_worklist(b);
 }
