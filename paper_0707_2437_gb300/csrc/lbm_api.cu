@@ -435,6 +435,7 @@ static bool runs_resident(lbm_grid *h, long long n) {
         h->grad != LBM_GRAD_CENTRAL || n < kResidentMin)
         return false;
     if (!h->resident_planned) {
+        h->resident_refused = false;
         if (plan_resident(h->nx, h->ny, h->sms, true, &h->resident) != cudaSuccess) return false;
         if (h->resident.ok && h->resident.cluster &&
             !cluster_fits(h->resident, h->storage, h->rounding, h->a15f != nullptr) &&
@@ -442,13 +443,17 @@ static bool runs_resident(lbm_grid *h, long long n) {
             return false;
         h->resident_planned = true;
     }
-    if (!h->resident.ok || (h->rounding && h->resident.us > kResidentMostStochastic)) return false;
+    if (!h->resident.ok || h->resident_refused || (h->rounding && h->resident.us > kResidentMostStochastic)) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     return cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess &&
            cap == cudaStreamCaptureStatusNone;
 }
 
-static int step_resident(lbm_grid *h, long long n) {
+// False if the launch is refused, with nothing queued: a group of blocks that wait for
+// one another has to fit the SMs that the stream may use, which can be fewer than the
+// device's (a green context's stream, an MPS client).  The step kernels run there, so
+// they take this call and the following ones, until the plan is made again.
+static bool step_resident(lbm_grid *h, long long n) {
     ResidentArgs a{};
     a.buf[0] = h->buf[0];
     a.buf[1] = h->buf[1];
@@ -467,13 +472,16 @@ static int step_resident(lbm_grid *h, long long n) {
     a.flags = h->flags;
     a.epoch = h->epoch;
     a.status = status_ptr(h);
-    cudaError_t e = launch_resident(h->resident, h->storage, h->rounding, a, h->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "lbm_step resident kernel");
+    if (launch_resident(h->resident, h->storage, h->rounding, a, h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        h->resident_refused = true;
+        return false;
+    }
     const long long exchanges = resident_exchanges(h->resident, n);
     h->epoch += (unsigned)exchanges;
     if (!(exchanges & 1)) h->cur ^= 1;
     h->t += n;
-    return LBM_OK;
+    return true;
 }
 
 // One launch of 1 .. h->fused.steps steps from buf[from] to buf[from ^ 1].
@@ -563,7 +571,7 @@ extern "C" int lbm_step(lbm_t h, long long n) {
         }
         return lbm_batch_step(h->self_batch, n, nullptr);  // advances t and cur
     }
-    if (runs_resident(h, n)) return step_resident(h, n);
+    if (runs_resident(h, n) && step_resident(h, n)) return LBM_OK;
     const int each = steps_fused(h) ? h->fused.steps : 1;
     const long long per = (long long)each * kGraphLaunches;
     while (n >= per) {
@@ -694,6 +702,7 @@ extern "C" int lbm_set_stream(lbm_t h, void *cuda_stream) {
     cudaEventDestroy(ev);  // released once recorded work completes
     if (e != cudaSuccess) return cuda_fail(e, "lbm_set_stream");
     h->stream = s;
+    h->resident_planned = false;
     return LBM_OK;
 }
 
@@ -787,6 +796,7 @@ extern "C" int lbm_set_c2_field(lbm_t h, const double *c2, int on_device) {
     CK(cudaStreamSynchronize(h->stream));
     drop_graphs(h);
     drop_self_batch(h);
+    h->resident_planned = false;  // (the field and the rounding choose the kernel)
     if (!c2) {
         if (h->a15f) cudaFree(h->a15f);
         h->a15f = nullptr;
@@ -853,6 +863,7 @@ extern "C" int lbm_set_rounding(lbm_t h, int mode) {
     drop_graphs(h);
     drop_self_batch(h);
     h->rounding = mode;
+    h->resident_planned = false;
     if (mode == LBM_ROUND_STOCHASTIC) {
         // Stochastic rounding runs on the register walks with vec <= 4 and on
         // the shared-memory row walk at vec 8 with 4 warps per block; other

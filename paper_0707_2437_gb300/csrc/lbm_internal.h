@@ -209,6 +209,7 @@ struct lbm_grid {
     // All steps of a call in one launch (small grids), and the exchanges made.
     vss::ResidentPlan resident{};
     bool resident_planned = false;  // on the first call that may use it
+    bool resident_refused = false;  // such a launch was refused on this stream
     unsigned *flags = nullptr;    // in scratch, for `sms` tiles; NULL on large grids
     int sms = 1;
     unsigned epoch = 0;

@@ -79,3 +79,24 @@ def test_failed_work_list_is_built_again_by_the_next_step(fake_lib, change):
             assert g.t == 7
             assert np.array_equal(g.get_state()[0], alone(nx, ny, 7, st))
     """)
+
+
+@pytest.mark.parametrize("nx,ny,tiles", [(400, 4, "one cluster"), (256, 256, "all SMs")])
+def test_refused_resident_launch_steps_by_the_step_kernel(fake_lib, nx, ny, tiles):
+    """A stream that owns too few SMs for a grid's tiles still steps it: the call whose
+    launch is refused, the next one, and one after the grid has moved to a stream that
+    takes such launches."""
+    _run(fake_lib, f"""
+        g = grid({nx}, {ny})
+        g.step(10)
+        group.value = 1
+        g.step(11)
+        g.step(12)
+        g.sync()
+        assert g.t == 33
+        assert np.array_equal(g.get_state()[0], alone({nx}, {ny}, 33)), "{tiles}"
+        group.value = 0
+        g.set_stream(lbm.new_stream())
+        g.step(13)
+        assert np.array_equal(g.get_state()[0], alone({nx}, {ny}, 46))
+    """)
