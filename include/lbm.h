@@ -134,6 +134,18 @@ int lbm_init(lbm_t h, const double *rho, const double *ux, const double *uy,
  * (LBM_ETIMEOUT if a bounded wait ran out). */
 int lbm_step(lbm_t h, long long n);
 
+/* How a call lbm_step(h, n) would run as the handle stands (n >= 1):
+ *   *form   LBM_FORM_LAUNCHES    launches of the step kernel
+ *           LBM_FORM_RESIDENT    one launch, tiles in shared memory
+ *           LBM_FORM_PERSISTENT  one launch of the batch kernel
+ *   *steps  time steps of a launch: 1, 2 or 3 with LBM_FORM_LAUNCHES (the last launch
+ *           of a call can take fewer), else n, at most 2^31 - 1
+ * Either pointer may be NULL.  Queues nothing. */
+#define LBM_FORM_LAUNCHES 0
+#define LBM_FORM_RESIDENT 1
+#define LBM_FORM_PERSISTENT 2
+int lbm_get_step_form(lbm_t h, long long n, int *form, int *steps);
+
 /* Persistent mode of lbm_step:
  *   LBM_PERSISTENT_OFF   every call uses the step kernel
  *   LBM_PERSISTENT_ON    calls of 64 steps or more, or of 8 or more on grids

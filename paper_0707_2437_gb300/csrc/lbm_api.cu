@@ -530,6 +530,27 @@ static int build_graph(lbm_grid *h, int start) {
     return LBM_OK;
 }
 
+// The form of a step call of n >= 1 steps.
+static int form_of(lbm_grid *h, long long n) {
+    if (h->timing) return LBM_FORM_LAUNCHES;
+    if (h->slab) return LBM_FORM_PERSISTENT;
+    const long long sites = (long long)h->nx * h->ny;
+    if (h->persistent == LBM_PERSISTENT_ON && !h->drive && h->grad == LBM_GRAD_CENTRAL &&
+        (n >= kPersistentMin || (sites >= kLargeSites && n >= kPersistentMinLarge)))
+        return LBM_FORM_PERSISTENT;
+    return runs_resident(h, n) ? LBM_FORM_RESIDENT : LBM_FORM_LAUNCHES;
+}
+
+extern "C" int lbm_get_step_form(lbm_t h, long long n, int *form, int *steps) {
+    if (!h || n < 1) return fail(LBM_EINVAL, "lbm_get_step_form: bad handle or n < 1");
+    const int f = form_of(h, n);
+    const long long each = h->timing || !steps_fused(h) ? 1 : h->fused.steps;
+    if (form) *form = f;
+    if (steps)
+        *steps = (int)std::min(f == LBM_FORM_LAUNCHES ? std::min(n, each) : n, 0x7fffffffLL);
+    return LBM_OK;
+}
+
 extern "C" int lbm_step(lbm_t h, long long n) {
     if (!h || n < 0) return fail(LBM_EINVAL, "lbm_step: bad handle or n < 0");
     if (n == 0) return LBM_OK;
@@ -555,11 +576,8 @@ extern "C" int lbm_step(lbm_t h, long long n) {
     if (h->slab && n != 1)
         return fail(LBM_EINVAL, "lbm_step: a slab takes one step at a time (its ghost rows "
                                 "are refreshed between steps)");
-    const long long sites = (long long)h->nx * h->ny;
-    bool persistent = false;
-    if (h->persistent == LBM_PERSISTENT_ON)
-        persistent = n >= kPersistentMin || (sites >= kLargeSites && n >= kPersistentMinLarge);
-    if (h->slab || (persistent && !h->drive && h->grad == LBM_GRAD_CENTRAL)) {
+    const int form = form_of(h, n);
+    if (form == LBM_FORM_PERSISTENT) {
         // Slabs always step here: the batch's tile list covers only their
         // own rows.
         // One persistent launch of all n steps (dynamic tile scheduling,
@@ -571,7 +589,7 @@ extern "C" int lbm_step(lbm_t h, long long n) {
         }
         return lbm_batch_step(h->self_batch, n, nullptr);  // advances t and cur
     }
-    if (runs_resident(h, n) && step_resident(h, n)) return LBM_OK;
+    if (form == LBM_FORM_RESIDENT && step_resident(h, n)) return LBM_OK;
     const int each = steps_fused(h) ? h->fused.steps : 1;
     const long long per = (long long)each * kGraphLaunches;
     while (n >= per) {

@@ -75,6 +75,7 @@ def load() -> ctypes.CDLL:
             "lbm_get_pipeline": ([vp, ctypes.POINTER(i), ctypes.POINTER(i)], i),
             "lbm_set_timing": ([vp, i], i),
             "lbm_set_persistent": ([vp, i], i),
+            "lbm_get_step_form": ([vp, ll, ctypes.POINTER(i), ctypes.POINTER(i)], i),
             "lbm_kernel_ms": ([vp, dp, ctypes.POINTER(ll)], i),
             "lbm_batch_create": ([ctypes.POINTER(vp), i, ctypes.POINTER(vp)], i),
             "lbm_batch_destroy": ([vp], i),
@@ -349,6 +350,14 @@ class Grid:
         memory, the step kernel for the others)."""
         mode = 2 if on == "auto" else (1 if on else 0)
         _check(self.lib.lbm_set_persistent(self.h, mode), "lbm_set_persistent")
+
+    def step_form(self, n: int):
+        """How step(n) would run as the grid stands: ('launches', steps a launch),
+        ('resident', n) or ('persistent', n)."""
+        form, steps = ctypes.c_int(), ctypes.c_int()
+        _check(self.lib.lbm_get_step_form(self.h, int(n), ctypes.byref(form),
+                                          ctypes.byref(steps)), "lbm_get_step_form")
+        return ["launches", "resident", "persistent"][form.value], steps.value
 
     def set_timing(self, on: bool):
         _check(self.lib.lbm_set_timing(self.h, 1 if on else 0), "lbm_set_timing")
