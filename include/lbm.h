@@ -319,9 +319,13 @@ int lbm_set_gradient(lbm_t h, int mode);
 int lbm_get_gradient(lbm_t h, int *mode);
 
 /* Autotuner: times the valid tile configurations on this grid (without
- * changing its state) and keeps the fastest.  If cache_path is not NULL the
- * choice is read from / stored in that JSON file, keyed by device, storage
- * and grid size.  Waits for the stream. */
+ * changing its state) and keeps the fastest, and then the other forms of step
+ * calls that the grid can take (passes of several steps, a resident call of 256
+ * steps), each kept where it is faster than single steps.  A form that the grid
+ * cannot take now stays as it is by default.  If cache_path is not NULL the
+ * choice is read from / stored in that JSON file, keyed by device, storage, grid
+ * size and options (rounding, c2 field, drive, gradient, slab); forms that the
+ * entry says nothing of are timed and added to it.  Waits for the stream. */
 int lbm_tune(lbm_t h, const char *cache_path);
 
 /* Mean device time in milliseconds of the step kernel over the last

@@ -431,7 +431,7 @@ static const long long kResidentMin = 4;
 static const double kResidentMostStochastic = 3.6;
 
 static bool runs_resident(lbm_grid *h, long long n) {
-    if (!h->flags || !h->fuse || h->persistent != LBM_PERSISTENT_AUTO || h->slab ||
+    if (!h->flags || !h->reside || h->persistent != LBM_PERSISTENT_AUTO || h->slab ||
         h->grad != LBM_GRAD_CENTRAL || n < kResidentMin)
         return false;
     if (!h->resident_planned) {
@@ -449,14 +449,13 @@ static bool runs_resident(lbm_grid *h, long long n) {
            cap == cudaStreamCaptureStatusNone;
 }
 
-// False if the launch is refused, with nothing queued: a group of blocks that wait for
-// one another has to fit the SMs that the stream may use, which can be fewer than the
-// device's (a green context's stream, an MPS client).  The step kernels run there, so
-// they take this call and the following ones, until the plan is made again.
-static bool step_resident(lbm_grid *h, long long n) {
+// Launches n steps resident from `state`, a buffer of the grid's, with buf[cur ^ 1].  The
+// plan's exchanges go through both, and the result is in the second after an even number
+// of them.
+static cudaError_t launch_resident_steps(lbm_grid *h, void *state, long long n) {
     ResidentArgs a{};
-    a.buf[0] = h->buf[0];
-    a.buf[1] = h->buf[1];
+    a.buf[h->cur] = state;
+    a.buf[h->cur ^ 1] = h->buf[h->cur ^ 1];
     a.cur = h->cur;
     a.nx = h->nx;
     a.ny = h->ny;
@@ -472,14 +471,22 @@ static bool step_resident(lbm_grid *h, long long n) {
     a.flags = h->flags;
     a.epoch = h->epoch;
     a.status = status_ptr(h);
-    if (launch_resident(h->resident, h->storage, h->rounding, a, h->stream) != cudaSuccess) {
+    const cudaError_t e = launch_resident(h->resident, h->storage, h->rounding, a, h->stream);
+    if (e == cudaSuccess) h->epoch += (unsigned)resident_exchanges(h->resident, n);
+    return e;
+}
+
+// False if the launch is refused, with nothing queued: a group of blocks that wait for
+// one another has to fit the SMs that the stream may use, which can be fewer than the
+// device's (a green context's stream, an MPS client).  The step kernels run there, so
+// they take this call and the following ones, until the plan is made again.
+static bool step_resident(lbm_grid *h, long long n) {
+    if (launch_resident_steps(h, h->buf[h->cur], n) != cudaSuccess) {
         cudaGetLastError();
         h->resident_refused = true;
         return false;
     }
-    const long long exchanges = resident_exchanges(h->resident, n);
-    h->epoch += (unsigned)exchanges;
-    if (!(exchanges & 1)) h->cur ^= 1;
+    if (!(resident_exchanges(h->resident, n) & 1)) h->cur ^= 1;
     h->t += n;
     return true;
 }
@@ -762,11 +769,13 @@ extern "C" int lbm_set_state(lbm_t h, const void *src_host, long long t) {
 // ---------------------------------------------------------------------------
 // Tile configuration and autotuner.
 
-// A configuration of the caller's describes single-step launches; the tuner turns
-// passes of several steps back on where they are the faster.
-static void set_fuse(lbm_grid *h, bool on) {
-    if (h->fuse != on) drop_graphs(h);
-    h->fuse = on;
+// The forms that step calls may take beside single-step launches.  A configuration of
+// the caller's describes those alone; the tuner lets the other forms back in where they
+// are the faster.
+static void allow_forms(lbm_grid *h, bool passes, bool resident) {
+    if (h->fuse != passes) drop_graphs(h);
+    h->fuse = passes;
+    h->reside = resident;
 }
 
 extern "C" int lbm_set_config(lbm_t h, int vec, int rows, int warps) {
@@ -788,7 +797,7 @@ extern "C" int lbm_set_config(lbm_t h, int vec, int rows, int warps) {
     h->cfg.rows = rows;
     h->cfg.warps = warps;
     h->cfg.fit_rows = false;
-    set_fuse(h, false);
+    allow_forms(h, false, false);
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }
@@ -804,7 +813,7 @@ extern "C" int lbm_set_pipeline(lbm_t h, int stages) {
         drop_graphs(h);
     }
     h->cfg.stages = stages;
-    set_fuse(h, false);
+    allow_forms(h, false, false);
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }
@@ -942,20 +951,28 @@ extern "C" int lbm_get_config(lbm_t h, int *vec, int *rows, int *warps) {
     return LBM_OK;
 }
 
+// A grid's options choose its kernels and forms, so each set of them is tuned by itself.
 static std::string tune_key(const lbm_grid *h) {
     cudaDeviceProp p;
     std::string dev = "dev";
     if (cudaGetDeviceProperties(&p, h->device) == cudaSuccess) dev = p.name;
     std::ostringstream k;
     k << dev << "|s" << h->storage << "|" << h->nx << "x" << h->ny;
+    if (h->rounding) k << "|sr";
+    if (h->a15f) k << "|c2";
+    if (h->drive) k << "|drive";
+    if (h->grad == LBM_GRAD_FORWARD) k << "|forward";
+    if (h->slab) k << "|slab";
     return k.str();
 }
 
-// The cache file is a flat JSON object {"key": [vec, rows, warps, stages, fuse],
-// ...}; files without the fifth number mean 0.
+// The cache file is a flat JSON object {"key": [vec, rows, warps, stages, passes,
+// resident], ...}.  The last two: whether that form of step calls was faster (1) or
+// slower (0) than single steps, -1 if it was not timed.  Entries with fewer numbers are
+// older and say nothing of the forms.
 struct Tuned {
     TileCfg cfg;
-    int fuse = 0;  // 1: step calls run faster several steps per launch
+    int passes = -1, resident = -1;
 };
 static std::map<std::string, Tuned> read_cache(const char *path) {
     std::map<std::string, Tuned> m;
@@ -973,9 +990,10 @@ static std::map<std::string, Tuned> read_cache(const char *path) {
         if (lb == std::string::npos || rb == std::string::npos) break;
         Tuned t;
         TileCfg &c = t.cfg;
-        if (sscanf(s.c_str() + lb, "[%d , %d , %d , %d , %d", &c.vec, &c.rows, &c.warps,
-                   &c.stages, &t.fuse) >= 4)
-            m[key] = t;
+        const int got = sscanf(s.c_str() + lb, "[%d , %d , %d , %d , %d , %d", &c.vec, &c.rows,
+                               &c.warps, &c.stages, &t.passes, &t.resident);
+        if (got < 6) t.passes = t.resident = -1;
+        if (got >= 4) m[key] = t;
         pos = rb + 1;
     }
     return m;
@@ -989,8 +1007,9 @@ static void write_cache(const char *path, const std::map<std::string, Tuned> &m)
     size_t k = 0;
     for (auto &kv : m) {
         const TileCfg &c = kv.second.cfg;
-        fprintf(f, "  \"%s\": [%d, %d, %d, %d, %d]%s\n", kv.first.c_str(), c.vec, c.rows, c.warps,
-                c.stages, kv.second.fuse, (++k < m.size()) ? "," : "");
+        fprintf(f, "  \"%s\": [%d, %d, %d, %d, %d, %d]%s\n", kv.first.c_str(), c.vec, c.rows,
+                c.warps, c.stages, kv.second.passes, kv.second.resident,
+                (++k < m.size()) ? "," : "");
     }
     fprintf(f, "}\n");
     fclose(f);
@@ -1025,9 +1044,77 @@ static int time_cfg(lbm_grid *h, const TileCfg *c, int reps, float *ms_out) {
     return LBM_OK;
 }
 
+static const long long kTuneSteps = 256;  // of a resident launch timed by the tuner
+
+// Times a resident call, in milliseconds per step, on a copy of the state: its exchanges
+// write to the buffer it starts from.  *ms_out is left alone where the copy or the launch
+// does not fit.
+static int time_resident(lbm_grid *h, int reps, float *ms_out) {
+    void *copy = nullptr;
+    if (cudaMalloc(&copy, state_bytes(h)) != cudaSuccess) {
+        cudaGetLastError();
+        return LBM_OK;
+    }
+    float total = 0.f;
+    bool refused = false;
+    cudaError_t e = cudaSuccess;
+    for (int r = 0; r <= reps && e == cudaSuccess; ++r) {  // (the first: warm-up)
+        float ms = 0.f;
+        e = cudaMemcpyAsync(copy, h->buf[h->cur], state_bytes(h), cudaMemcpyDeviceToDevice,
+                            h->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev[0], h->stream);
+        if (e == cudaSuccess && launch_resident_steps(h, copy, kTuneSteps) != cudaSuccess) {
+            cudaGetLastError();
+            refused = true;
+            break;
+        }
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev[1], h->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(h->ev[1]);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, h->ev[0], h->ev[1]);
+        if (r) total += ms;
+    }
+    cudaStreamSynchronize(h->stream);
+    cudaFree(copy);
+    if (e != cudaSuccess) return cuda_fail(e, "lbm_tune");
+    if (!refused) *ms_out = total / reps / kTuneSteps;
+    return LBM_OK;
+}
+
+// Times the forms of t that have not been and that the grid can take, against single
+// steps under t.cfg; `ms`: the time of one, or negative if not known.  *timed: whether
+// there were any.
+static int tune_forms(lbm_grid *h, int reps, float ms, Tuned *t, bool *timed) {
+    allow_forms(h, true, true);
+    const bool passes = t->passes < 0 && steps_fused(h);
+    const bool resident = t->resident < 0 && runs_resident(h, kTuneSteps);
+    *timed = passes || resident;
+    if (*timed && ms < 0) {
+        const int rc = time_cfg(h, &t->cfg, reps, &ms);
+        if (rc != LBM_OK) return rc;
+    }
+    if (passes) {
+        float each = 0.f;
+        const int rc = time_cfg(h, nullptr, reps, &each);
+        if (rc != LBM_OK) return rc;
+        each /= (float)h->fused.steps;
+        t->passes = each < ms;
+        ms = std::min(ms, each);
+    }
+    if (resident) {
+        float each = -1.f;
+        const int rc = time_resident(h, 3, &each);
+        if (rc != LBM_OK) return rc;
+        if (each >= 0) t->resident = each < ms;
+    }
+    allow_forms(h, t->passes != 0, t->resident != 0);
+    return LBM_OK;
+}
+
 extern "C" int lbm_tune(lbm_t h, const char *cache_path) {
     if (!h) return fail(LBM_EINVAL, "lbm_tune: NULL handle");
     std::string key = tune_key(h);
+    long long sites = (long long)h->nx * h->ny;
+    int reps = (int)std::max<long long>(3, std::min<long long>(50, 200000000LL / (sites + 1)));
     std::map<std::string, Tuned> cache;
     if (cache_path) {
         cache = read_cache(cache_path);
@@ -1036,13 +1123,13 @@ extern "C" int lbm_tune(lbm_t h, const char *cache_path) {
             const TileCfg &c = it->second.cfg;
             int rc = lbm_set_config(h, c.vec, c.rows, c.warps);
             if (rc == LBM_OK) rc = lbm_set_pipeline(h, c.stages);
-            if (rc == LBM_OK) set_fuse(h, it->second.fuse != 0);
+            bool timed = false;
+            if (rc == LBM_OK) rc = tune_forms(h, reps, -1.f, &it->second, &timed);
+            if (rc == LBM_OK && timed) write_cache(cache_path, cache);
             return rc;
         }
     }
     CK(cudaStreamSynchronize(h->stream));
-    long long sites = (long long)h->nx * h->ny;
-    int reps = (int)std::max<long long>(3, std::min<long long>(50, 200000000LL / (sites + 1)));
     TileCfg best = h->cfg;
     float best_ms = 1e30f;
     const int vecs[] = {1, 2, 4, 8};
@@ -1079,16 +1166,13 @@ extern "C" int lbm_tune(lbm_t h, const char *cache_path) {
     int rc = lbm_set_config(h, best.vec, best.rows, best.warps);
     if (rc == LBM_OK) rc = lbm_set_pipeline(h, best.stages);
     if (rc != LBM_OK) return rc;
-    bool fuse = false;
-    if (h->fused.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL) {
-        float ms;
-        rc = time_cfg(h, nullptr, reps, &ms);
-        if (rc != LBM_OK) return rc;
-        fuse = ms < h->fused.steps * best_ms;
-    }
-    set_fuse(h, fuse);
+    Tuned t;
+    t.cfg = best;
+    bool timed = false;
+    rc = tune_forms(h, reps, best_ms, &t, &timed);
+    if (rc != LBM_OK) return rc;
     if (cache_path) {
-        cache[key] = Tuned{best, fuse ? 1 : 0};
+        cache[key] = t;
         write_cache(cache_path, cache);
     }
     return LBM_OK;

@@ -203,11 +203,13 @@ struct lbm_grid {
     vss::Coef coef{};
     vss::TileCfg cfg{};
     // Several steps per launch: the plan for the grid as configured, and whether
-    // step calls may use it (not under a tile configuration of the caller's).
+    // step calls may use it (not under a tile configuration of the caller's, nor
+    // where the tuner measured single steps the faster).
     vss::FusedPlan fused{};
     bool fuse = true;
-    // All steps of a call in one launch (small grids), and the exchanges made.
+    // All steps of a call in one launch (small grids), the same, and the exchanges made.
     vss::ResidentPlan resident{};
+    bool reside = true;
     bool resident_planned = false;  // on the first call that may use it
     bool resident_refused = false;  // such a launch was refused on this stream
     unsigned *flags = nullptr;    // in scratch, for `sms` tiles; NULL on large grids
