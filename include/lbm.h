@@ -121,12 +121,15 @@ int lbm_init(lbm_t h, const double *rho, const double *ux, const double *uy,
  * kernel once per step, or every two or three steps (replayed from CUDA graphs, 32 launches
  * each), or run all n steps as one launch of one of two kinds.  Resident: the
  * grid's tiles stay in the SMs' shared memory, one block each, and exchange
- * their edges every few steps (bounded waits); grids of up to about 600^2
+ * their edges every few steps (bounded waits); grids of up to about 660^2
  * sites.  Persistent: the batched kernel (see lbm_batch_create) with this grid
  * alone, warps taking tiles dynamically, a bounded grid barrier between passes.
  * Which one is set by lbm_set_persistent; by default (LBM_PERSISTENT_AUTO) calls
- * of four steps or more on grids that fit run resident, all others launch the
- * step kernel.  A slab always steps persistent; a driven grid never does, and
+ * of four steps or more on grids that fit run resident where that is estimated to
+ * be the faster, all others launch the step kernel.  A resident launch of a grid
+ * of 128^2 or more has nearly all SMs to itself, while step launches of small
+ * grids on several streams overlap: the estimate counts the streams that small
+ * grids of the process are on.  A slab always steps persistent; a driven grid never does, and
  * the forward-difference gradient runs in the step kernel only.  A tile
  * configuration or pipeline of the caller's, and a stream that is being
  * captured, also mean the step kernel.  All forms give bitwise the same result.

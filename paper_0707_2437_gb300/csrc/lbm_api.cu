@@ -9,6 +9,7 @@
 #include <fstream>
 #include <map>
 #include <mutex>
+#include <new>
 #include <sstream>
 #include <string>
 #include <vector>
@@ -191,6 +192,42 @@ static cudaError_t copy_stream(int device, cudaStream_t *out) {
     return cudaSuccess;
 }
 
+// Small grids (those that may run resident) per device and stream: as many streams as
+// hold some may step them at the same time.
+static std::mutex g_small_mu;
+static std::map<std::pair<int, cudaStream_t>, int> g_small;
+
+static std::pair<int, cudaStream_t> small_key(const lbm_grid *h) {
+    return {h->device, h->stream == cudaStreamLegacy ? nullptr : h->stream};
+}
+static void uncount_small(lbm_grid *h) {
+    if (!h->counted) return;
+    std::lock_guard<std::mutex> lk(g_small_mu);
+    auto it = g_small.find(small_key(h));
+    if (it != g_small.end() && --it->second == 0) g_small.erase(it);
+    h->counted = false;
+}
+// (Not counted if the host is out of memory.)
+static void count_small(lbm_grid *h) {
+    if (!h->flags || h->counted) return;
+    std::lock_guard<std::mutex> lk(g_small_mu);
+    try {
+        ++g_small[small_key(h)];
+        h->counted = true;
+    } catch (const std::bad_alloc &) {
+    }
+}
+static int small_streams(int device) {
+    std::lock_guard<std::mutex> lk(g_small_mu);
+    int n = 0;
+    for (const auto &kv : g_small) n += kv.first.first == device;
+    return n;
+}
+void never_resident(lbm_grid *h) {
+    uncount_small(h);
+    h->flags = nullptr;
+}
+
 static cudaError_t staging_alloc(lbm_grid *h, double **p, size_t bytes, cudaStream_t st) {
     cudaMemPool_t pool = nullptr;
     {
@@ -310,6 +347,7 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double c2, double rho0,
         cudaGetLastError();
         return rc;
     }
+    count_small(h);
     *out = h;
     return c2 > 1.2656 ? LBM_WUNSTABLE : LBM_OK;
 }
@@ -321,6 +359,7 @@ extern "C" int lbm_create(int nx, int ny, double tau, double c2, int storage, vo
 
 extern "C" int lbm_destroy(lbm_t h) {
     if (!h) return LBM_OK;
+    uncount_small(h);
     if (h->stream || h->buf[0]) cudaStreamSynchronize(h->stream);
     drop_self_batch(h);
     drop_graphs(h);
@@ -421,14 +460,11 @@ static bool steps_fused(const lbm_grid *h) {
     return h->fuse && h->fused.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL;
 }
 
-// Whether n steps run as one launch with the state in shared memory.  From four
-// steps on: such a launch costs about 6 us beyond its steps, a step launch 3 to 6.
-// Up to 3.6 us a step by the plan with stochastic rounding, which hashes every
-// site here but every pair of sites in the step kernel (600^2: 6.4 us against 6.3;
-// 512^2 5.0 against 6.2).  Not in a stream that is being captured: a replay would
+// Whether n steps run as one launch with the state in shared memory: from four steps on
+// (such a launch costs 3 to 10 us beyond its steps, a step launch 3 to 6), where that is
+// the faster (resident_pays).  Not in a stream that is being captured: a replay would
 // repeat the exchange counters.
 static const long long kResidentMin = 4;
-static const double kResidentMostStochastic = 3.6;
 
 static bool runs_resident(lbm_grid *h, long long n) {
     if (!h->flags || !h->reside || h->persistent != LBM_PERSISTENT_AUTO || h->slab ||
@@ -443,7 +479,10 @@ static bool runs_resident(lbm_grid *h, long long n) {
             return false;
         h->resident_planned = true;
     }
-    if (!h->resident.ok || h->resident_refused || (h->rounding && h->resident.us > kResidentMostStochastic)) return false;
+    if (!h->resident.ok || h->resident_refused ||
+        !resident_pays(h->resident, h->storage, h->rounding, h->a15f != nullptr, h->drive,
+                       (long long)h->nx * h->ny, h->sms, small_streams(h->device), n))
+        return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     return cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess &&
            cap == cudaStreamCaptureStatusNone;
@@ -726,7 +765,9 @@ extern "C" int lbm_set_stream(lbm_t h, void *cuda_stream) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev, 0);
     cudaEventDestroy(ev);  // released once recorded work completes
     if (e != cudaSuccess) return cuda_fail(e, "lbm_set_stream");
+    uncount_small(h);
     h->stream = s;
+    count_small(h);
     h->resident_planned = false;
     return LBM_OK;
 }

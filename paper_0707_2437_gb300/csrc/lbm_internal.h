@@ -142,6 +142,10 @@ ResidentKernel resident_kernel_bf16(int rnd, bool field, int shape);
 // Whether a grid is small enough to have a tiling; the tiling.
 bool may_run_resident(int nx, int ny, int sms);
 Err plan_resident(int nx, int ny, int sms, bool clusters, ResidentPlan *out);
+// Whether a call of n >= 4 steps is faster resident than by the step kernel, with small
+// grids on `streams` streams of the device.
+bool resident_pays(const ResidentPlan &p, int storage, int rnd, bool field, bool drive,
+                   long long sites, int sms, int streams, long long n);
 // Whether the device can hold a plan's cluster.
 bool cluster_fits(const ResidentPlan &p, int storage, int rnd, bool field);
 Err launch_resident(const ResidentPlan &p, int storage, int rnd, ResidentArgs a, cudaStream_t st);
@@ -213,6 +217,7 @@ struct lbm_grid {
     bool resident_planned = false;  // on the first call that may use it
     bool resident_refused = false;  // such a launch was refused on this stream
     unsigned *flags = nullptr;    // in scratch, for `sms` tiles; NULL on large grids
+    bool counted = false;         // among the small grids of its stream
     int sms = 1;
     unsigned epoch = 0;
     int rounding = 0;             // 1: stochastic rounding of 16-bit stores
@@ -240,6 +245,9 @@ struct lbm_grid {
     cudaEvent_t ev[2] = {nullptr, nullptr};
     cudaEvent_t staged = nullptr;  // lbm_init: host fields copied
 };
+
+// Takes a grid that will never run resident out of the count of small grids.
+void never_resident(lbm_grid *h);
 
 // Status word of a batch's kernels: batch_queue_status queues its copy to
 // pinned host memory on `st`; once `st` has been synchronised, batch_status

@@ -68,7 +68,7 @@ static double step_us(int shape, int W, int H, int hx, int hy, int T, bool align
 
 constexpr int kClusterTiles = 16;  // the largest cluster (beyond the portable 8)
 
-// The tiling with the lowest estimate.  Grids of up to about 700^2 sites have one.
+// The tiling with the lowest estimate.  Grids of up to about 660^2 sites have one.
 bool may_run_resident(int nx, int ny, int sms) { return (long long)nx * ny <= 3900LL * sms; }
 
 Err plan_resident(int nx, int ny, int sms, bool clusters, ResidentPlan *out) {
@@ -115,6 +115,51 @@ Err plan_resident(int nx, int ny, int sms, bool clusters, ResidentPlan *out) {
         }
     out->ok = best < 1e30;
     return cudaSuccess;
+}
+
+// Where a resident call pays.  A call of n steps costs about n r + L, r the step time of
+// its kind and L the launch, the first load and the last store; the step kernel n t, or
+// more in short calls, whose launches are not replayed.  Fitted to 600 pairs of
+// measurements (100 sizes from 16^2 to 661^2 and from 4 to 16384 wide, calls of 4 to 512
+// steps, each kind): the choice is the slower by more than 3 % for one in 200 of them.  The
+// step kernel's time scatters by a fifth with where a grid's buffers lie in L2 (FP16 400 x
+// 400 4.1 us, 400 x 408 5.1).  Step kernel / resident, us a step, calls of 4 and of 512
+// steps: FP32 512^2 7.0 / 6.2 and 6.6 / 3.7, 640^2 7.3 / 8.2 and 6.8 / 6.0; FP32 with a c2
+// field 512^2 5.2 / 6.7 and 4.8 / 4.4, 640^2 6.2 / 8.9 and 5.8 / 6.7; FP16 400^2 4.4 /
+// 4.7 and 4.1 / 2.9, 640^2 6.2 / 8.7 and 5.9 / 6.2; FP16 with stochastic rounding, which
+// hashes every site here but every pair of sites there, 400^2 4.4 / 6.0 and 4.4 / 4.0.
+//
+// `streams`: streams with small grids in use.  Their step kernels overlap, and so do
+// resident calls as long as their tiles find SMs of their own, which is two grids of 64^2,
+// eleven of 400 x 4, and none of 128^2 and more.  Measured, us per step and grid, step
+// kernel / resident: FP32 64^2 on 4 streams 0.97 / 0.56, on 8 0.54 / 0.56; 128^2 on 2
+// 1.93 / 1.17, on 8 0.64 / 1.17; 256^2 on 2 2.9 / 1.8, on 4 1.5 / 1.8, on 16 0.72 / 1.84;
+// 512^2 on 2 3.6 / 3.7, on 4 2.3 / 3.7; FP16 512^2 on 4 1.9 / 4.0.
+bool resident_pays(const ResidentPlan &p, int storage, int rnd, bool field, bool drive,
+                   long long sites, int sms, int streams, long long n) {
+    struct Kind {
+        double t, per_site, most;           // of the step kernel
+        double per_row, per_band, exchange; // beyond the plan's estimate
+    };
+    constexpr Kind kF32{2.6, 13e-6, 7.0, 0, 0.064, 0.9}, kF32Field{3.2, 7e-6, 5.8, 0, 0.11, 1.2};
+    constexpr Kind k16{3.0, 10e-6, 6.0, 0, 0.088, 1.0}, k16Field{2.8, 15e-6, 6.0, 0, 0.135, 1.45};
+    constexpr Kind kHash{3.6, 9e-6, 6.4, 0.0096, 0.145, 1.55};
+    const bool wide = storage == ST_F32;
+    const Kind k = wide ? (field ? kF32Field : kF32) : rnd ? kHash : field ? k16Field : k16;
+    const int tiles = p.tx * p.ty;
+    const double warp_rows = p.threads / 32 * kShapes[p.shape].rows;
+    double t = std::min(k.t + k.per_site * (double)sites, k.most);
+    if (drive) t += 2.5;  // the boundary kernel of every step
+    double r = p.us - 0.24 + k.per_row * warp_rows + k.per_band * kShapes[p.shape].rows +
+               (tiles > 1 ? k.exchange / p.T : 0.0);
+    double fixed = 1.5 + 0.055 * warp_rows;
+    if (streams > 1) {
+        t = std::max({1.1 * t / streams, 0.45, (wide ? 8.5e-6 : 7e-6) * (double)sites});
+        const int together = std::min(streams, std::max(1, sms / tiles));
+        r /= together;
+        fixed /= together;
+    }
+    return (double)n * (t - r) >= fixed;
 }
 
 static ResidentKernel kernel_for(const ResidentPlan &p, int storage, int rnd, bool field) {

@@ -35,6 +35,7 @@ extern "C" int lbm_slab_create(int nx, int ny_local, double tau, double c2, int 
     int rc = lbm_create(nx, ny_local + 2 * kGhost, tau, c2, storage, cuda_stream, &h);
     if (rc < 0) return rc;
     h->slab = kGhost;
+    never_resident(h);
     *out = h;
     return rc;
 }

@@ -99,6 +99,53 @@ def test_sizes_of_the_resident_tests_run_resident(lbm, nx, ny, kind, option):
         assert g.step_form(150)[0] == "launches"
 
 
+@pytest.mark.parametrize("kind,option,nx,ny,n,resident", [
+    ("f32", "", 64, 64, 4, True), ("f32", "", 509, 381, 4, True), ("f32", "", 640, 640, 4, False),
+    ("f32", "", 640, 640, 64, True), ("f32", "field", 512, 512, 4, False),
+    ("f32", "field", 512, 512, 64, True), ("f32", "field", 640, 640, 512, False),
+    ("f16d", "", 256, 256, 4, True), ("f16d", "", 512, 512, 4, False),
+    ("f16d", "", 512, 512, 16, True), ("bf16d", "", 640, 640, 512, False),
+    ("f16d", "drive", 640, 640, 64, True), ("bf16d", "field", 600, 600, 6, False),
+    ("f16d-sr", "", 256, 256, 8, True), ("f16d-sr", "", 512, 512, 4, False),
+    ("bf16d-sr", "", 600, 600, 512, False)])
+def test_resident_where_it_is_the_faster(lbm, kind, option, nx, ny, n, resident):
+    """Both sides of the line, at sizes where the two forms differ by a tenth or more."""
+    with _grid(lbm, nx, ny, kind, option) as g:
+        assert (g.step_form(n)[0] == "resident") == resident
+
+
+def test_small_grids_on_several_streams(lbm):
+    """Grids of 256^2 take turns on the SMs when they run resident: on eight streams
+    their step launches overlap instead.  Grids of one tile have an SM each, and a large
+    grid's stream does not count."""
+    streams = [lbm.new_stream() for _ in range(8)]
+    big = lbm.Grid(2048, 2048, 0.8, 0.2, stream=lbm.new_stream())
+    grids = [lbm.Grid(256, 256, 0.8, 0.2, stream=s) for s in streams]
+    tiny = lbm.Grid(16, 16, 0.8, 0.2, stream=streams[0])
+    fields = workloads.fourier_modes(256, 256, amp=1e-2, seed=1)
+    for g in grids:
+        g.init(*fields)
+        assert g.step_form(100)[0] == "launches"
+        g.step(100)
+    assert tiny.step_form(100)[0] == "resident"
+    for g in grids[1:4]:
+        g.close()
+    for g in grids[4:]:
+        g.set_stream(streams[0])
+    rest = [grids[0]] + grids[4:]
+    for g in rest:
+        assert g.step_form(100)[0] == "resident"
+        g.step(20)
+    states = [g.get_state()[0] for g in rest]
+    for g in rest + [tiny, big]:
+        g.close()
+    with lbm.Grid(256, 256, 0.8, 0.2) as h:
+        h.set_persistent(False)
+        h.init(*fields)
+        h.step(120)
+        assert all(np.array_equal(h.get_state()[0], s) for s in states)
+
+
 def test_forms_under_settings(lbm):
     with lbm.Grid(256, 256, 0.8, 0.2) as g:
         g.set_persistent(True)
