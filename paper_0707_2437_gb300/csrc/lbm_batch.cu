@@ -365,9 +365,10 @@ static int build_worklist(lbm_batch *b) {
             }
             singles = sites < 1.1e6 && fused > 1.2 * single;
         }
-        if (fc.fused && one_kind && storage != ST_F32) {
-            const bool rnd = b->grids[0]->rounding != 0;
+        if (fc.fused && one_kind) {
+            const bool rnd = b->grids[0]->rounding != 0, field = b->grids[0]->a15f != nullptr;
             double work = 0, pass = 0, sites = 0, single = rnd ? 5.0 : 4.0;
+            double strip_sites = 0, extra = 0;
             for (size_t k = 0; k < ng; ++k) {
                 const int r = fused_height(k), ny = computed_rows(k), nx = b->grids[k]->nx;
                 const int segs = (ny + r - 1) / r, over = fused_overhead(2);
@@ -376,9 +377,23 @@ static int build_worklist(lbm_batch *b) {
                 const double lanes = 256.0 * strips(k, 1) / nx;
                 sites += (double)nx * ny;
                 single += 1e-6 * nx * ny * ((rnd ? 6.5 : 5.5) + 5.3 * (lanes - 1));
+                strip_sites += 128.0 * strips(k, 1) * ny;
+                extra += (double)(strips(k, 2) - strips(k, 1)) * ny;
             }
-            const double row_us = rnd ? (storage == ST_F16 ? 2.58 : 2.41) : 2.2;
-            singles = single < 0.5 * row_us * std::max(pass, work / warps) + 0.25e-6 * sites;
+            const double passes = std::max(pass, work / warps);
+            if (storage != ST_F32) {
+                const double row_us = rnd ? (storage == ST_F16 ? 2.58 : 2.41) : 2.2;
+                singles = single < 0.5 * row_us * passes + 0.25e-6 * sites;
+            } else if (extra > 0) {
+                // FP32: strips of 120 columns where single steps have fewer of 128, which
+                // shows while the tiles are one wave (single / fused, us a step: 64 grids
+                // of 124 x 128 13.3 / 15.5, 128 of 124 x 64 13.9 / 16.1, 32 of 128 x 256
+                // 12.5 / 13.3, 16 of 128 x 512 12.6 / 13.0, nine of 128 x 4096 61 / 48, 64
+                // of 248 x 128 28 / 20; with a c2 field 64 of 124 x 128 14.8 / 16.3).
+                singles = std::max((field ? 9.9 : 8.5) + 4.3e-6 * strip_sites + 0.008 * ng,
+                                   (field ? 14.2e-6 : 12.9e-6) * strip_sites) <
+                          (field ? 0.73 : 0.715) * passes + 0.25e-6 * sites + 0.006 * ng;
+            }
         }
         if (singles) {
             fc = flow_kernel_for(kinds, b->walk16, false);
@@ -504,14 +519,14 @@ static int build_worklist(lbm_batch *b) {
         lbm_batch::Group gr;
         gr.begin = (int)ordered.size();
         tiles.clear();
-        if (kinds_in.size() == 1 && fuses(kinds_in[0])) {
+        bool fused = kinds_in.size() == 1 && fuses(kinds_in[0]);
+        int per = 2;
+        long long warps = 1;
+        if (fused) {
             const std::vector<size_t> &members = of_kind[kinds_in[0]];
             const int storage = b->grids[members[0]]->storage;
             const bool field = b->grids[members[0]]->a15f != nullptr;
-            gr.fused = true;
             double best = 1e300;
-            int per = 2;
-            long long warps = 1;
             // (with a c2 field three steps gain nothing here: 22.5 ms against 22.4)
             for (int steps = 2; steps <= (field ? 2 : fused_most_steps(storage)); ++steps) {
                 const FusedChoice fc = fused_kernel_for(kinds_in[0], steps);
@@ -542,13 +557,34 @@ static int build_worklist(lbm_batch *b) {
                 gr.rows = rows;
                 warps = w;
             }
-            for (size_t k : members) add_fused_tiles(k, gr.rows, per);
+            // FP32 strips are 120 columns here and 128 in single steps, so widths of 121 to
+            // 128 (or 241 to 256, less so) have one more; a batch of less than a wave of
+            // tiles then is the faster in single steps.  Estimates of a step as above.
+            // Single / fused, us a step: 64 grids of 124 x 128 14.6 / 15.8, 128 of 124 x 64
+            // 14.6 / 16.5, 256 of 124 x 32 14.6 / 16.5, 16 of 124 x 512 14.6 / 15.2, 64 of
+            // 124 x 256 27.1 / 26.1, 64 of 116 x 128 14.6 / 10.0, 64 of 248 x 128 27 / 20;
+            // with a c2 field 128 of 124 x 64 16.3 / 16.7.
+            if (storage == ST_F32 && b->fit_rows && lock_rows < b->rows) {
+                double strip_sites = 0, extra = 0;
+                for (size_t k : members) {
+                    strip_sites += 128.0 * strips(k, 1) * computed_rows(k);
+                    extra += (double)(strips(k, 2) - strips(k, 1)) * computed_rows(k);
+                }
+                const double single = std::max((field ? 7.3 : 6.5) + (field ? 2.2 : 2.05) * lock_rows,
+                                               13.3e-6 * strip_sites);
+                if (extra > 0 && single < (field ? 1.46 : 1.43) * best + 1.5) fused = false;
+            }
+        }
+        if (fused) {
+            gr.fused = true;
+            for (size_t k : of_kind[kinds_in[0]]) add_fused_tiles(k, gr.rows, per);
             ordered.insert(ordered.end(), tiles.begin(), tiles.end());
             split_tail(gr.begin, warps);
             gr.count = (int)ordered.size() - gr.begin;
             b->groups.push_back(gr);
             return LBM_OK;
         }
+        gr.smem = 0;
         for (int kd : kinds_in)
             for (size_t k : of_kind[kd]) add_tiles(k, lock_rows, 1);
         // (grids in the caller's order, whatever their kinds)
