@@ -215,8 +215,7 @@ static int build_worklist(lbm_batch *b) {
         d.nx = g->nx;
         d.ny = g->ny;
         d.kind = kind_code(g->storage, batch_vec(b, g), g->rounding ? 1 : 0, g->a15f ? 1 : 0);
-        d.per = 1;
-        d.window = 1;
+        d.pad = 0;
         d.c = g->coef;
         slabs = slabs || g->slab;
     }
@@ -232,7 +231,7 @@ static int build_worklist(lbm_batch *b) {
     auto add_tiles = [&](size_t k, int rows, int per) {
         lbm_grid *g = b->grids[k];
         GridDesc &d = gd[k];
-        b->per[k] = d.per = per;
+        b->per[k] = per;
         const int w = per > 1 ? fused_cols(g->storage, per) : 32 * batch_vec(b, g);
         const int ylo = g->slab, yhi = g->ny - g->slab, nyc = yhi - ylo;
         d.tile0 = (int)tiles.size();
@@ -242,7 +241,7 @@ static int build_worklist(lbm_batch *b) {
         // A pass reads two rows and columns per step beyond its tile: the next
         // segment or strip over suffices unless one of them is smaller (the
         // last one of a grid can be).
-        const int reach = 2 * d.per;
+        const int reach = 2 * per;
         const int last_rows = nyc - (d.nsegs - 1) * rows;
         const int last_cols = g->nx - (d.nstrips - 1) * w;
         d.dseg = (rows >= reach && last_rows >= reach) ? 1 : 2;
@@ -258,7 +257,7 @@ static int build_worklist(lbm_batch *b) {
     // segments share warps.
     auto add_fused_tiles = [&](size_t k, int rows, int per) {
         const lbm_grid *g = b->grids[k];
-        b->per[k] = gd[k].per = per;
+        b->per[k] = per;
         const FusedStrips s = fused_strips(g->storage, per, g->nx);
         const int w = fused_cols(g->storage, per), step = s.pieces ? s.pieces : 1;
         for (int y0 = 0, seg = 0; y0 < g->ny; y0 += rows, ++seg) {
@@ -413,7 +412,6 @@ static int build_worklist(lbm_batch *b) {
             add_tiles(k, rows, per_pass);
         }
         gr.count = (int)tiles.size();
-        for (GridDesc &d : gd) d.window = gr.fused ? 1 : 2;
         b->groups.push_back(gr);
         if (tiles.size() > b->prog_cap) {
             cudaFree(b->d_prog);

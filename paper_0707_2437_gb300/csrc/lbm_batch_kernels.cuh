@@ -32,7 +32,7 @@ struct GridDesc {
     size_t P;
     int nx, ny;
     int kind;  // kind_code(storage, vec, stochastic rounding)
-    int per;   // steps of a pass: several on the fused walk, else 1
+    int pad;
     Coef c;
     // Tiles of the grid in the work-list (flow schedule): the first one, how
     // many per step (segment-major: t = segment * nstrips + strip), and how
@@ -40,19 +40,27 @@ struct GridDesc {
     // when a neighbouring segment or strip can be smaller than the pass's
     // reach: two sites a step).
     int tile0, ntile, nstrips, nsegs, dseg, dstrip;
-    int window;  // passes that tickets may run ahead of the completed tiles
 };
 
 // A tile: one strip (x0) of one segment (rows y0 .. y1-1, walked in
 // direction dir) of a grid.  A paired tile (y1b > y0b; lockstep kernels of
 // 8-site 16-bit walks only) adds a second segment, rows y0b .. y1b-1 in
 // direction dirb, of a grid at most 16*8 columns wide: the two halves of the
-// warp walk one segment each (the split walk).
+// warp walk one segment each (the split walk).  A packed tile (lockstep kernels of the
+// fused walk only) has pieces of `rows` rows on `lanes` lanes each; lanes 0: one piece.
 struct __align__(16) Tile {
     int grid, x0, y0, y1, dir;
-    int y0b, y1b, dirb;
-    int lanes, rows;  // fused walk: pieces of `rows` rows on `lanes` lanes each (0: one)
+    union {
+        int y0b;
+        int lanes;
+    };
+    union {
+        int y1b;
+        int rows;
+    };
+    int dirb;
 };
+static_assert(sizeof(Tile) == 32, "a sector");
 
 // A grid's walk in the batch kernels: storage kind, sites per lane (1, 4 or
 // 8), stochastic rounding, and a per-site c2 field.
@@ -274,7 +282,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
 // Warps pick grids round-robin, so every grid gets about the same number of
 // tiles per unit time: small grids take many steps while large ones take
 // few, instead of every grid waiting for the whole batch at every step.  A
-// grid's tickets may run at most `window` passes ahead of its completed
+// grid's tickets may run at most a window of passes ahead of its completed
 // tiles, so that the warps a short grid's step chain would hold waiting go to
 // other grids: one on the fused walk (two: the serving mix's launch 9.8 ms against
 // 8.9), two in single steps, whose tiles are more than the fused walk's (two grids of
@@ -336,8 +344,10 @@ __host__ __device__ inline long long passes_of(long long steps, int per) {
     return (steps + per - 1) / per;
 }
 
-// The flow loop of one warp; run_tile(g, par, tile, step, steps) runs a tile.
-template <class RunTile>
+// The flow loop of one warp, PER steps a pass; run_tile(g, par, tile, step, steps) runs a
+// tile.  (As run-time values of the grid, the steps of a pass and the window made the
+// single-step kernels 2 to 7 % slower: FP16 64 grids of 256 x 128 16.3 / 16.6 us a step.)
+template <int PER, class RunTile>
 __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, int ngrids,
                                           const Tile *__restrict__ tiles,
                                           const long long *__restrict__ limit,
@@ -346,6 +356,7 @@ __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, in
                                           unsigned long long *ctl, int *prog, unsigned *glob,
                                           const int *__restrict__ nwork_p, int *status,
                                           unsigned long long timeout_ns, RunTile run_tile) {
+    constexpr int kWindow = PER > 1 ? 1 : 2;  // passes that tickets may run ahead
     const int lane = threadIdx.x & 31;
     // The warp's ticket and idle timer live in shared memory while a tile
     // runs, leaving the walk the registers it has in the lockstep kernels.
@@ -368,12 +379,12 @@ __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, in
                     const int cand = (int)((start + (unsigned)j) % (unsigned)ngrids);
                     const GridDesc &G = grids[cand];
                     const unsigned long long total =
-                        (unsigned long long)passes_of(limit[cand], G.per) *
+                        (unsigned long long)passes_of(limit[cand], PER) *
                         (unsigned long long)G.ntile;
                     volatile unsigned long long *c = ctl + (size_t)cand * kFlowCtlWords;
                     const unsigned long long taken = c[0];
                     if (taken >= total) continue;
-                    if (taken - c[16] >= (unsigned long long)G.window * G.ntile) continue;
+                    if (taken - c[16] >= (unsigned long long)kWindow * G.ntile) continue;
                     const unsigned long long mm =
                         atomicAdd(ctl + (size_t)cand * kFlowCtlWords, 1ULL);
                     if (mm >= total) continue;
@@ -418,9 +429,9 @@ __device__ __forceinline__ void flow_loop(const GridDesc *__restrict__ grids, in
             const int seg = ti / g.nstrips, strip = ti % g.nstrips;
             if (!flow_wait(g, prog, seg, strip, k, status, timeout_ns)) return;
             const Tile t = tiles[g.tile0 + ti];
-            const long long done = (long long)k * g.per;  // steps before this pass
+            const long long done = (long long)k * PER;  // steps before this pass
             run_tile(g, (parity0[gsel] + k) & 1, t, t0[gsel] + (uint32_t)done,
-                     (int)min((long long)g.per, limit[gsel] - done));
+                     PER > 1 ? (int)min((long long)PER, limit[gsel] - done) : 1);
         }
         // Publish: the tile's stores before its completed-step count.
         __threadfence();
@@ -438,7 +449,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
            const long long *__restrict__ limit, const int *__restrict__ parity0,
            const uint32_t *__restrict__ t0, unsigned long long *ctl, int *prog, unsigned *glob,
            const int *__restrict__ nwork_p, int *status, unsigned long long timeout_ns) {
-    flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
+    flow_loop<1>(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
               timeout_ns, [](const GridDesc &g, int par, const Tile &t, uint32_t step, int) {
                   any_tile(g, par, t, step);
               });
@@ -456,7 +467,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
                unsigned long long timeout_ns) {
     __shared__ uint4 rowbuf[V == 8 ? kBatchWarps : 1][2 * 9 * 32];
     (void)rowbuf;
-    flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
+    flow_loop<1>(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
               timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int) {
                   Walker<S, V, LD_CG, RND, VA> w(g.buf[par], g.buf[par ^ 1], g.nx, g.ny, g.P,
                                                  t.x0);
@@ -499,7 +510,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 2)
                  unsigned long long timeout_ns) {
     extern __shared__ uint4 walk_smem[];
     uint4 *buf = walk_smem + (threadIdx.x >> 5) * fused_vecs<S, VA, 2>();
-    flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
+    flow_loop<2>(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
               timeout_ns,
               [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int steps) {
                   fused_tile<S, RND, VA, 2, false>(g, par, t, step, steps, buf);
@@ -520,7 +531,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 2)
     extern __shared__ uint4 walk_smem[];
     static_assert(fused_vecs<ST_F32, 0, 2>() == fused_vecs<S2, 0, 2>(), "one buffer size");
     uint4 *buf = walk_smem + (threadIdx.x >> 5) * fused_vecs<S2, 0, 2>();
-    flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
+    flow_loop<2>(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
               timeout_ns,
               [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int steps) {
                   if (g.kind == kind_code(ST_F32, 4, 0))
@@ -540,7 +551,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 3)
                       const int *__restrict__ nwork_p, int *status,
                       unsigned long long timeout_ns) {
     __shared__ uint4 rowbuf[kBatchWarps][2 * 9 * 32];
-    flow_loop(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
+    flow_loop<1>(grids, ngrids, tiles, limit, parity0, t0, ctl, prog, glob, nwork_p, status,
               timeout_ns, [&](const GridDesc &g, int par, const Tile &t, uint32_t step, int) {
                   const Coef c = g.c;
                   if (g.kind == kind_code(ST_F32, 4, 0)) {
