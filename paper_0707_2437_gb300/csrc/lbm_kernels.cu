@@ -619,7 +619,8 @@ __global__ void __launch_bounds__(kSide)
 // FP64 reductions in a fixed order: each thread sums its sites in order, each
 // block its threads in a fixed tree, and the block partials are summed in order
 // of the blocks: by the block that finishes last (counter: a word that the last
-// block leaves at zero), or by k_final.
+// block leaves at zero), or by k_final, in the same order, so that lbm_sums and
+// lbm_sums_noalloc agree bit for bit.
 
 constexpr int RT = kSide;
 constexpr int RB_MAX = kReduceBlocksMax;
@@ -664,6 +665,18 @@ struct Results {
     double scale;
 };
 
+// Sum of the block partials over one block's threads, in thread 0.
+template <int K>
+__device__ __forceinline__ void sum_partials(double (&v)[K], const double *partials,
+                                             unsigned blocks) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = 0.0;
+    for (unsigned b = threadIdx.x; b < blocks; b += RT)
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] += __ldcg(partials + (size_t)b * K + k);
+    block_sum<K>(v);
+}
+
 template <int K>
 __device__ __forceinline__ void finish_sums(double (&v)[K], const Results &r) {
     const unsigned blocks = gridDim.x * gridDim.y;
@@ -682,12 +695,7 @@ __device__ __forceinline__ void finish_sums(double (&v)[K], const Results &r) {
     }
     __syncthreads();
     if (!last) return;
-#pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = 0.0;
-    for (unsigned b = threadIdx.x; b < blocks; b += RT)
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] += __ldcg(r.partials + (size_t)b * K + k);
-    block_sum<K>(v);
+    sum_partials<K>(v, r.partials, blocks);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < K; ++k) r.host_out[k] = v[k] * r.scale;
@@ -696,12 +704,13 @@ __device__ __forceinline__ void finish_sums(double (&v)[K], const Results &r) {
 }
 
 template <int K>
-__global__ void k_final(const double *partials, int nblocks, double *out) {
-    // One block: thread k sums partial k of every block in block order.
-    if (threadIdx.x < K) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * K + threadIdx.x];
-        out[threadIdx.x] = s;
+__global__ void __launch_bounds__(RT)
+    k_final(const double *__restrict__ partials, int nblocks, double *__restrict__ out) {
+    double v[K];
+    sum_partials<K>(v, partials, (unsigned)nblocks);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) out[k] = v[k];
     }
 }
 
@@ -864,7 +873,7 @@ Err launch_sums(int storage, const void *f, int nx, int ny, size_t P, double *pa
     int nb = reduce_blocks(nx, ny);
     const Results res{partials, nullptr, nullptr, nullptr, nullptr, 1.0};
     DISPATCH_S(storage, (k_sums<S_><<<nb, RT, 0, st>>>(f, nx, ny, P, res)));
-    k_final<3><<<1, 32, 0, st>>>(partials, nb, out3);
+    k_final<3><<<1, RT, 0, st>>>(partials, nb, out3);
     return cudaGetLastError();
 }
 
