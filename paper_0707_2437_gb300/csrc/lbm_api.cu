@@ -321,22 +321,23 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double c2, double rho0,
         if (!h->buf[0]) e = cudaMalloc(&h->buf[0], bytes);
         if (e == cudaSuccess && !h->buf[1]) e = cudaMalloc(&h->buf[1], bytes);
     }
-    // Reduction partials and results, the status word and step counter, and
-    // the counters of a resident launch's tiles.
-    const size_t words = 3 * 1024 + 16;
+    // The status word, the step counter and the reductions' block count; the counters of
+    // a resident launch's tiles; reduction partials.
     h->sms = sms > 0 ? sms : 1;
     const size_t flag_bytes = may_run_resident(nx, ny, h->sms)
                                   ? sizeof(unsigned) * kResidentFlagWords * (size_t)h->sms
                                   : 0;
-    if (e == cudaSuccess) e = cudaMalloc(&h->scratch, sizeof(double) * words + flag_bytes);
-    if (flag_bytes) h->flags = reinterpret_cast<unsigned *>(h->scratch + words);
-    // Stream-ordered, so that creating a grid does not wait for work running
-    // on the legacy default stream.
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->scratch, 0, sizeof(double) * 16, h->stream);
-    if (e == cudaSuccess && flag_bytes)
-        e = cudaMemsetAsync(h->flags, 0, flag_bytes, h->stream);
+    const size_t zeroed = sizeof(double) * 16 + flag_bytes;
+    if (e == cudaSuccess)
+        e = cudaMalloc(&h->scratch, zeroed + sizeof(double) * 3 * kReduceBlocksMax);
+    if (e == cudaSuccess) {
+        if (flag_bytes) h->flags = reinterpret_cast<unsigned *>(h->scratch + 16);
+        h->partials = h->scratch + zeroed / sizeof(double);
+        // Stream-ordered, so that creating a grid does not wait for work running
+        // on the legacy default stream.
+        e = cudaMemsetAsync(h->scratch, 0, zeroed, h->stream);
+    }
     if (e == cudaSuccess) e = prepare_step(storage, h->cfg);
-    if (e == cudaSuccess) e = plan_fused(storage, 0, false, nx, ny, &h->fused);
     if (e == cudaSuccess) e = cudaMallocHost(&h->host_out, sizeof(double) * 8);
     if (e == cudaSuccess) e = cudaEventCreate(&h->ev[0]);
     if (e == cudaSuccess) e = cudaEventCreate(&h->ev[1]);
@@ -455,9 +456,20 @@ static cudaError_t launch_one(lbm_grid *h, int from) {
     return launch_one(h, from, nullptr, (uint32_t)h->t, h->stream);
 }
 
-// Whether step calls take several steps per launch.
-static bool steps_fused(const lbm_grid *h) {
-    return h->fuse && h->fused.ok && !h->drive && !h->slab && h->grad == LBM_GRAD_CENTRAL;
+// Whether step calls take several steps per launch.  The plan is made on the first call
+// that asks and again after a change of the rounding or the field (a grid that steps
+// resident or in a batch needs none); without one, single steps.
+static bool steps_fused(lbm_grid *h) {
+    if (!h->fuse || h->drive || h->slab || h->grad != LBM_GRAD_CENTRAL) return false;
+    if (!h->fused_planned) {
+        if (plan_fused(h->storage, h->rounding, h->a15f != nullptr, h->nx, h->ny, &h->fused) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            h->fused = FusedPlan{};
+        }
+        h->fused_planned = true;
+    }
+    return h->fused.ok;
 }
 
 // Whether n steps run as one launch with the state in shared memory: from four steps on
@@ -712,7 +724,7 @@ extern "C" int lbm_moments(lbm_t h, double *rho, double *ux, double *uy, int on_
 }
 
 static HostResults host_results(lbm_grid *h) {
-    return HostResults{h->scratch + 16, count_ptr(h), h->host_out, status_ptr(h),
+    return HostResults{h->partials, count_ptr(h), h->host_out, status_ptr(h),
                        host_status_ptr(h)};
 }
 
@@ -864,11 +876,10 @@ extern "C" int lbm_set_c2_field(lbm_t h, const double *c2, int on_device) {
     CK(cudaStreamSynchronize(h->stream));
     drop_graphs(h);
     drop_self_batch(h);
-    h->resident_planned = false;  // (the field and the rounding choose the kernel)
+    h->resident_planned = h->fused_planned = false;  // (the field and the rounding choose the kernels)
     if (!c2) {
         if (h->a15f) cudaFree(h->a15f);
         h->a15f = nullptr;
-        CK(plan_fused(h->storage, h->rounding, false, h->nx, h->ny, &h->fused));
         return LBM_OK;
     }
     if (h->rounding) return fail(LBM_EINVAL, "lbm_set_c2_field: needs nearest rounding");
@@ -886,7 +897,6 @@ extern "C" int lbm_set_c2_field(lbm_t h, const double *c2, int on_device) {
     }
     if (h->cfg.stages >= 2) h->cfg.stages = 0;
     if (!h->a15f) CK(cudaMalloc(&h->a15f, n * sizeof(float)));
-    CK(plan_fused(h->storage, h->rounding, true, h->nx, h->ny, &h->fused));
     std::vector<double *> owned;
     double *d = nullptr;
     int rc = stage_field(h, c2, on_device, h->stream, &d, owned);
@@ -931,7 +941,7 @@ extern "C" int lbm_set_rounding(lbm_t h, int mode) {
     drop_graphs(h);
     drop_self_batch(h);
     h->rounding = mode;
-    h->resident_planned = false;
+    h->resident_planned = h->fused_planned = false;
     if (mode == LBM_ROUND_STOCHASTIC) {
         // Stochastic rounding runs on the register walks with vec <= 4 and on
         // the shared-memory row walk at vec 8 with 4 warps per block; other
@@ -942,7 +952,6 @@ extern "C" int lbm_set_rounding(lbm_t h, int mode) {
         }
         if (h->cfg.stages >= 2) h->cfg.stages = 0;
     }
-    CK(plan_fused(h->storage, h->rounding, h->a15f != nullptr, h->nx, h->ny, &h->fused));
     CK(prepare_step(h->storage, h->cfg));
     return LBM_OK;
 }

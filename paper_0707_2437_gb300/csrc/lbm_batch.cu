@@ -152,14 +152,13 @@ static int upload_worklist(lbm_batch *b, const std::vector<GridDesc> &gd,
     return LBM_OK;
 }
 
-// Dynamic shared memory and resident blocks of a kernel of this file.
-static cudaError_t resident_blocks(const void *fn, int smem, int *blocks) {
-    cudaError_t e = cudaSuccess;
-    if (smem)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, 32 * kBatchWarps, smem);
-    return e;
+// Resident blocks per SM of a kernel of this file, at least one.
+static int resident_blocks(const lbm_batch *b, const void *fn, int smem, int *blocks) {
+    *blocks = (int)(resident_warps(fn, kBatchWarps, smem) / kBatchWarps / b->sms);
+    if (*blocks >= 1) return LBM_OK;
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? bcuda(e, "occupancy of a batch kernel")
+                            : bfail(LBM_ECUDA, "batch kernel cannot be resident");
 }
 
 // Tile height of a lockstep group on the fused walk, from the grids' strips and
@@ -286,8 +285,8 @@ static int build_worklist(lbm_batch *b) {
             gr.smem = fc.smem;
             gr.fused = fc.fused;
             gr.rows = b->rows;
-            BCK(resident_blocks((const void *)fc.fn, fc.smem, &gr.max_blocks_per_sm));
-            if (gr.max_blocks_per_sm < 1) return bfail(LBM_ECUDA, "flow kernel cannot be resident");
+            int rc = resident_blocks(b, (const void *)fc.fn, fc.smem, &gr.max_blocks_per_sm);
+            if (rc != LBM_OK) return rc;
             const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
                                                  : gr.max_blocks_per_sm;
             warps = (long long)per * b->sms * kBatchWarps;
@@ -529,8 +528,8 @@ static int build_worklist(lbm_batch *b) {
             for (int steps = 2; steps <= (field ? 2 : fused_most_steps(storage)); ++steps) {
                 const FusedChoice fc = fused_kernel_for(kinds_in[0], steps);
                 int bps = 0;
-                BCK(resident_blocks((const void *)fc.fn, fc.smem, &bps));
-                if (bps < 1) return bfail(LBM_ECUDA, "batch kernel cannot be resident");
+                int rc = resident_blocks(b, (const void *)fc.fn, fc.smem, &bps);
+                if (rc != LBM_OK) return rc;
                 const long long w =
                     (long long)(b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, bps) : bps) *
                     b->sms * kBatchWarps;
@@ -612,8 +611,8 @@ static int build_worklist(lbm_batch *b) {
         gr.rows = lock_rows;
         gr.count = (int)ordered.size() - gr.begin;
         gr.kernel = kernel_for(kinds_in, b->walk16, b->paired > paired0);
-        BCK(resident_blocks((const void *)gr.kernel, 0, &gr.max_blocks_per_sm));
-        if (gr.max_blocks_per_sm < 1) return bfail(LBM_ECUDA, "batch kernel cannot be resident");
+        int rc = resident_blocks(b, (const void *)gr.kernel, 0, &gr.max_blocks_per_sm);
+        if (rc != LBM_OK) return rc;
         b->groups.push_back(gr);
         return LBM_OK;
     };

@@ -73,8 +73,8 @@ Coef make_coef(double tau, double c2, double rho0);
 Err launch_step(int storage, const TileCfg &cfg, const void *fin, void *fout, int nx, int ny,
                 size_t P, const Coef &c, int *status, int rnd, const uint32_t *tdev, uint32_t toff,
                 const float *a15f, cudaStream_t st);
-// Warps of `fn` (blocks of `warps` warps, `smem` bytes of dynamic shared memory)
-// resident on the current device; 0 if the query fails.
+// Warps of `fn` (blocks of `warps` warps, `smem` bytes of dynamic shared memory, which
+// it is allowed from then on) resident on the current device; 0 if the query fails.
 long long resident_warps(const void *fn, int warps, int smem);
 // Strips of the fused walk: `full` ones of whole warps and, when the columns left over
 // need at most half a warp with their halo lanes, packed tiles: `pieces` segments of
@@ -210,6 +210,7 @@ struct lbm_grid {
     // step calls may use it (not under a tile configuration of the caller's, nor
     // where the tuner measured single steps the faster).
     vss::FusedPlan fused{};
+    bool fused_planned = false;   // on the first call that may use it
     bool fuse = true;
     // All steps of a call in one launch (small grids), the same, and the exchanges made.
     vss::ResidentPlan resident{};
@@ -230,7 +231,8 @@ struct lbm_grid {
     // Driven channel in x (lbm_set_drive): boundary columns after every step.
     bool drive = false;
     double drive_amp = 0, drive_period = 0;
-    double *scratch = nullptr;    // reduction partials + results
+    double *scratch = nullptr;    // status and counters, flags, reduction partials
+    double *partials = nullptr;   // in scratch
     double *host_out = nullptr;   // pinned, 8 doubles
     // CUDA graphs of a fixed number of step launches starting from buffer 0 or 1
     cudaGraphExec_t graph[2] = {nullptr, nullptr};

@@ -140,9 +140,10 @@ __global__ void __launch_bounds__(256, 2)
     w.run(y0, y1, (seg & 1) ? -1 : 1, c, status);
 }
 
-// Resident warps of a step kernel with blocks of `warps` warps on the
+// Resident warps of a step or batch kernel with blocks of `warps` warps on the
 // current device, found once per kernel, block size and device (a kernel is
-// always asked about with the same dynamic shared memory).
+// always asked about with the same dynamic shared memory), when the kernel is
+// also allowed that shared memory.
 long long resident_warps(const void *fn, int warps, int smem) {
     struct Entry {
         const void *fn;
@@ -159,6 +160,9 @@ long long resident_warps(const void *fn, int warps, int smem) {
             if (e.fn == fn && e.warps == warps && e.dev == dev) return e.w;
     }
     int blocks = 0, sms = 0;
+    if (smem && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+                    cudaSuccess)
+        return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, 32 * warps, smem) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return 0;

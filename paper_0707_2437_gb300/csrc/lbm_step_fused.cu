@@ -108,9 +108,6 @@ Err plan_fused(int storage, int rnd, bool field, int nx, int ny, FusedPlan *out)
     for (int steps = 2; steps <= (ragged ? 2 : fused_most_steps(storage)); ++steps) {
         const Choice ch = ragged ? choose_ragged(storage, rnd)
                                  : choose(storage, rnd, field, steps);
-        Err e = cudaFuncSetAttribute((const void *)ch.fn,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, ch.smem);
-        if (e != cudaSuccess) return e;
         const long long wave = resident_warps((const void *)ch.fn, kWarps, ch.smem);
         if (wave <= 0) return cudaErrorLaunchOutOfResources;
         const FusedStrips strips = fused_strips(storage, steps, nx);

@@ -159,3 +159,33 @@ def test_forms_under_settings(lbm):
         assert g.step_form(64) == ("launches", 1)
     with lbm.Slab(256, 64, 0.8, 0.2) as s:
         assert s.step_form(1) == ("persistent", 1)
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 64), (2048, 1025)])
+def test_first_step_call_under_capture(lbm, nx, ny):
+    """Plans are made by the first call that needs them, which may be one into a stream
+    that is being captured: launches of the step kernel, single or passes, that a replay
+    repeats."""
+    import torch
+    fields = workloads.fourier_modes(nx, ny, amp=1e-2, seed=nx)
+    stream = torch.cuda.Stream()
+    with lbm.Grid(nx, ny, 0.7, 0.2, stream=stream) as warm:  # (kernels are loaded)
+        warm.init(*fields)
+        warm.step(1)
+        warm.step(7)
+        warm.sync()
+    with lbm.Grid(nx, ny, 0.7, 0.2, stream=stream) as g:
+        g.init(*fields)
+        g.sync()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            assert g.step_form(7)[0] == "launches"
+            g.step(7)
+        with torch.cuda.stream(stream):
+            graph.replay()
+        state = g.get_state()[0]
+        g.set_persistent(False)
+        g.init(*fields)
+        for _ in range(7):
+            g.step(1)
+        assert np.array_equal(g.get_state()[0], state)
