@@ -137,6 +137,12 @@ int lbm_init(lbm_t h, const double *rho, const double *ux, const double *uy,
  * (LBM_ETIMEOUT if a bounded wait ran out). */
 int lbm_step(lbm_t h, long long n);
 
+/* Limit of a wait inside a resident launch, in microseconds (default 1e6; 0: a wait
+ * runs out at its first look, for tests of what follows).  Launches of a single tile or
+ * of one cluster have no such waits.  A launch in which a wait runs out ends early, the next synchronising call on the handle
+ * returns LBM_ETIMEOUT, and the state is undefined until lbm_init or lbm_set_state. */
+int lbm_set_timeout_us(lbm_t h, long long us);
+
 /* How a call lbm_step(h, n) would run as the handle stands (n >= 1):
  *   *form   LBM_FORM_LAUNCHES    launches of the step kernel
  *           LBM_FORM_RESIDENT    one launch, tiles in shared memory

@@ -521,6 +521,8 @@ static cudaError_t launch_resident_steps(lbm_grid *h, void *state, long long n) 
     a.rho0 = h->rho0;
     a.flags = h->flags;
     a.epoch = h->epoch;
+    a.wait_ns = h->wait_ns;
+    a.wait_polls = h->wait_ns < 1000000 ? 0u : 255u;
     a.status = status_ptr(h);
     const cudaError_t e = launch_resident(h->resident, h->storage, h->rounding, a, h->stream);
     if (e == cudaSuccess) h->epoch += (unsigned)resident_exchanges(h->resident, n);
@@ -681,6 +683,12 @@ extern "C" int lbm_set_persistent(lbm_t h, int on) {
     CK(cudaStreamSynchronize(h->stream));
     h->persistent = on;
     if (on == LBM_PERSISTENT_OFF) drop_self_batch(h);
+    return LBM_OK;
+}
+
+extern "C" int lbm_set_timeout_us(lbm_t h, long long us) {
+    if (!h || us < 0) return fail(LBM_EINVAL, "lbm_set_timeout_us: bad argument");
+    h->wait_ns = (unsigned long long)us * 1000ULL;
     return LBM_OK;
 }
 

@@ -127,6 +127,8 @@ struct ResidentArgs {
     double drive_amp, drive_period, rho0;
     unsigned *flags;     // kResidentFlagWords words per tile
     unsigned epoch;      // exchanges made by earlier launches on these flags
+    unsigned wait_polls; // the clock is read when these bits of the poll count are set
+    unsigned long long wait_ns;  // limit of a wait
     int *status;
 };
 constexpr int kResidentFlagWords = 32;  // a 128-byte line per tile
@@ -221,6 +223,7 @@ struct lbm_grid {
     bool counted = false;         // among the small grids of its stream
     int sms = 1;
     unsigned epoch = 0;
+    unsigned long long wait_ns = 1000000000ULL;  // limit of a resident launch's waits
     int rounding = 0;             // 1: stochastic rounding of 16-bit stores
     float *a15f = nullptr;        // spatially varying alpha: 1.5 alpha per site
     int grad = 0;                 // LBM_GRAD_CENTRAL or LBM_GRAD_FORWARD

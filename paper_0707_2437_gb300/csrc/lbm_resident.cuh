@@ -24,8 +24,11 @@
 // tile wraps on itself.
 //
 // Blocks wait for one another, so launches of several tiles are cooperative (all
-// blocks resident, or none), every wait is bounded by the clock, and a wait that
-// runs out sets the handle's status word.
+// blocks resident, or none), every wait is bounded by the clock (lbm_set_timeout_us,
+// read every 256 polls, or at every one under a limit of less than a millisecond), and
+// a wait that runs out sets the handle's status word, at which the others give up too.
+// Cluster barriers have no limit: the hardware starts a cluster whole, and every block
+// reaches every one of them.
 //
 // Up to 16 tiles launch as one cluster instead, which the hardware schedules as a
 // whole: a block reads its halo out of its neighbours' shared memory, between two
@@ -42,8 +45,6 @@
 namespace vss {
 
 namespace {
-
-constexpr unsigned long long kWaitNs = 1000000000ULL;  // 1 s per wait
 
 __device__ __forceinline__ int first_of(int n, int parts, int i) {
     return (int)((long long)n * i / parts);
@@ -384,10 +385,10 @@ __global__ void __launch_bounds__(NT, 1)
                                  : "l"(flag)
                                  : "memory");
                     if ((int)(v - epoch) >= 0) break;
-                    if ((it & 255u) == 255u) {
+                    if ((it & a.wait_polls) == a.wait_polls) {
                         const unsigned long long now = globaltimer_ns();
                         if (began == 0) began = now;
-                        if (now - began > kWaitNs || *(volatile int *)a.status != 0) {
+                        if (now - began >= a.wait_ns || *(volatile int *)a.status != 0) {
                             atomicCAS(a.status, 0, STATUS_TIMEOUT);
                             ok = false;
                             break;

@@ -75,6 +75,7 @@ def load() -> ctypes.CDLL:
             "lbm_get_pipeline": ([vp, ctypes.POINTER(i), ctypes.POINTER(i)], i),
             "lbm_set_timing": ([vp, i], i),
             "lbm_set_persistent": ([vp, i], i),
+            "lbm_set_timeout_us": ([vp, ll], i),
             "lbm_get_step_form": ([vp, ll, ctypes.POINTER(i), ctypes.POINTER(i)], i),
             "lbm_kernel_ms": ([vp, dp, ctypes.POINTER(ll)], i),
             "lbm_batch_create": ([ctypes.POINTER(vp), i, ctypes.POINTER(vp)], i),
@@ -350,6 +351,10 @@ class Grid:
         memory, the step kernel for the others)."""
         mode = 2 if on == "auto" else (1 if on else 0)
         _check(self.lib.lbm_set_persistent(self.h, mode), "lbm_set_persistent")
+
+    def set_timeout_us(self, us: int):
+        """Limit of a wait inside a resident launch, in microseconds."""
+        _check(self.lib.lbm_set_timeout_us(self.h, int(us)), "lbm_set_timeout_us")
 
     def step_form(self, n: int):
         """How step(n) would run as the grid stands: ('launches', steps a launch),
