@@ -195,7 +195,7 @@ def serve_comparison(args, stream=None):
             trace07, realtime=True).summary()
     # The same two traces with the flow schedule (each grid advances on its
     # own; launches share a budget of lattice updates by size^0.5), and with
-    # the server's default: flow while at most 24 grids are resident,
+    # the server's default: flow while few grids are resident,
     # lockstep above.
     for sched in ("flow", "auto"):
         if sched not in args.serve_schedules.split(","):

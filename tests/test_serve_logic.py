@@ -293,3 +293,16 @@ def test_flow_shares_weighted_by_size(monkeypatch):
         if w == 0.5:
             assert by_size[0][1] >= by_size[-1][1]
             assert by_size[0][0] * by_size[0][1] <= by_size[-1][0] * by_size[-1][1] * 1.01 + by_size[-1][0]
+
+
+def test_default_schedule_is_lockstep_beyond_two_grids(monkeypatch):
+    """The default keeps lockstep's throughput and p99: flow only while one or two
+    grids are resident."""
+    dev = _FakeDevice(total=1 << 40)
+    monkeypatch.setattr(serve, "lbm", _fake_lbm(dev))
+    reqs = _requests(n=16)
+    stats = serve.Server(reserve_bytes=0).run(reqs, realtime=False)
+    assert len(stats.results) == len(reqs)
+    assert {(sch, len(calls) > 2) for sch, calls in dev.steps} <= {("lockstep", True),
+                                                                   ("flow", False)}
+    assert ("lockstep", True) in {(sch, len(calls) > 2) for sch, calls in dev.steps}
