@@ -386,9 +386,15 @@ int lbm_batch_sync(lbm_batch_t b);
  * that balances their tiles over the resident warps.  The tuner times those too. */
 int lbm_batch_set_config(lbm_batch_t b, int rows, int blocks_per_sm);
 int lbm_batch_tune(lbm_batch_t b);
-/* Tile height and resident blocks per SM of the first kind group as built, and whether every kind group runs a
- * specialised kernel rather than the general one. */
+/* Tile height of the first kind group as built (in the flow schedule, where grids have
+ * heights of their own, that of the first grid), resident blocks per SM of the first kind
+ * group, and whether every kind group runs a specialised kernel rather than the general
+ * one. */
 int lbm_batch_get_config(lbm_batch_t b, int *rows, int *blocks_per_sm, int *specialised);
+/* Time steps of a pass over memory (1, 2 or 3) of member `grid`, 0 to n-1 in the order of
+ * lbm_batch_create, in the work-list as last built; the last pass of a call can take
+ * fewer. */
+int lbm_batch_get_pass(lbm_batch_t b, int grid, int *steps);
 /* The work-list as last built (at creation, by a configuration, schedule or
  * walk change, or by a step call that found a grid's field or rounding
  * changed): *tiles = warp walks per time step, *paired = how many of them

@@ -284,7 +284,6 @@ static int build_worklist(lbm_batch *b) {
             gr.fkernel = fc.fn;
             gr.smem = fc.smem;
             gr.fused = fc.fused;
-            gr.rows = b->rows;
             int rc = resident_blocks(b, (const void *)fc.fn, fc.smem, &gr.max_blocks_per_sm);
             if (rc != LBM_OK) return rc;
             const int per = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, gr.max_blocks_per_sm)
@@ -409,6 +408,7 @@ static int build_worklist(lbm_batch *b) {
                 if (tall * (long long)ng < warps) rows = std::max(1, rows / 4);
             }
             add_tiles(k, rows, per_pass);
+            if (k == 0) gr.rows = rows;
         }
         gr.count = (int)tiles.size();
         b->groups.push_back(gr);
@@ -1077,6 +1077,13 @@ extern "C" int lbm_batch_get_tiles(lbm_batch_t b, int *tiles, int *paired) {
     if (!b) return bfail(LBM_EINVAL, "lbm_batch_get_tiles: NULL batch");
     if (tiles) *tiles = b->ntiles;
     if (paired) *paired = b->paired;
+    return LBM_OK;
+}
+
+extern "C" int lbm_batch_get_pass(lbm_batch_t b, int grid, int *steps) {
+    if (!b || !steps || grid < 0 || grid >= (int)b->grids.size())
+        return bfail(LBM_EINVAL, "lbm_batch_get_pass: bad argument");
+    *steps = b->per[grid];
     return LBM_OK;
 }
 

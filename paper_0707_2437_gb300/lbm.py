@@ -89,6 +89,7 @@ def load() -> ctypes.CDLL:
             "lbm_batch_get_groups": ([vp, ctypes.POINTER(i)], i),
             "lbm_batch_get_config": ([vp, ctypes.POINTER(i), ctypes.POINTER(i),
                                       ctypes.POINTER(i)], i),
+            "lbm_batch_get_pass": ([vp, i, ctypes.POINTER(i)], i),
             "lbm_batch_get_tiles": ([vp, ctypes.POINTER(i), ctypes.POINTER(i)], i),
             "lbm_set_gradient": ([vp, i], i),
             "lbm_get_gradient": ([vp, ctypes.POINTER(i)], i),
@@ -474,6 +475,12 @@ class Batch:
         return {"rows": r.value, "blocks_per_sm": b.value, "specialised": bool(sp.value),
                 "walk16": WALK16_NAMES[wk.value], "groups": ng.value, "tiles": nt.value,
                 "paired_tiles": npair.value}
+
+    def steps_per_pass(self, grid: int = 0) -> int:
+        """Time steps of a pass over memory of grid number `grid`: 1, 2 or 3."""
+        n = ctypes.c_int()
+        _check(self.lib.lbm_batch_get_pass(self.b, grid, ctypes.byref(n)), "lbm_batch_get_pass")
+        return n.value
 
     def set_walk16(self, walk: str):
         """Walk of the batch's 16-bit grids: 'auto' (the default, 'v8'), 'v8'
