@@ -39,13 +39,17 @@ ONE_STEP_NOTE = ("achieved and frac count the bytes of one step per pass over me
 METRIC = "MLUPS (million lattice updates per second), D2Q9 variable-speed-of-sound step"
 WORKLOAD = "2048x2048 periodic D2Q9, 9 runs c2=0.05..0.45, tau~U[0.55,1.5], acoustic+shear wave"
 PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "batch_sweep2048_traffic.json")
-KERNEL_SOURCES = [os.path.join(ROOT, "paper_0707_2437_gb300", "csrc", f)
+CSRC = os.path.join(ROOT, "paper_0707_2437_gb300", "csrc")
+KERNEL_SOURCES = [os.path.join(CSRC, f)
                   for f in ("lbm_device.cuh", "lbm_kernels.cu", "lbm_batch_kernels.cuh")]
+# The walk that the batch kernels include, and the code that chooses their tiles and the
+# steps of their passes.
+WALK_SOURCES = [os.path.join(CSRC, f) for f in ("lbm_fused.cuh", "lbm_batch.cu")]
 
 
 def kernel_source_hash() -> str:
     h = hashlib.sha256()
-    for p in KERNEL_SOURCES:
+    for p in KERNEL_SOURCES + WALK_SOURCES:
         h.update(open(p, "rb").read())
     return h.hexdigest()[:16]
 
@@ -427,8 +431,10 @@ def run_native(args):
     alg_bytes = per_step_bytes * (spl if batch is not None else 1)
     peak, peak_kind = measured_peak()
     # The recorded traffic is that of the nine-grid sweep on the batch path.
-    traffic = (recorded_traffic(storage, args.rounding, spl)
-               if batch is not None and args.workload == "sweep2048" and len(runs) == 9
+    default_batch = (batch is not None and args.schedule == "lockstep" and not args.walk16
+                     and not args.batch_rows and not args.tune)
+    traffic = (recorded_traffic(storage, args.rounding, spl, batch.steps_per_pass())
+               if default_batch and args.workload == "sweep2048" and len(runs) == 9
                and not args.c2_field else None)
 
     # The same batch with one step per launch, for the launch overhead, and
@@ -637,7 +643,8 @@ def run_native(args):
                      "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)"
                      if peak_kind == "measured" else "fallback 6.8 TB/s",
                      "note": ONE_STEP_NOTE if batch is not None and spl > 1 else None,
-                     "kernel": (f"k_batch_fused (persistent, 9 grids, {spl} steps per launch)"
+                     "kernel": (f"{batch_kernel(batch, args.schedule)}, persistent, {len(runs)} "
+                                f"grid(s), {spl} steps per launch"
                                 if batch is not None
                                 else f"k_step_tma<{storage},stages={stages}>"
                                 if pipelined and stages >= 2
@@ -689,19 +696,30 @@ def run_native(args):
         print(json.dumps(line), flush=True)
 
 
-def recorded_traffic(storage: str, rounding: str, spl: int):
-    """DRAM bytes of one launch of `spl` steps of the nine-grid sweep on the
-    batch path, from the ncu record under profiles/, or None when the record
-    does not cover these kernel sources, this storage or this rounding."""
+def recorded_traffic(storage: str, rounding: str, spl: int, per: int):
+    """DRAM bytes of one launch of `spl` steps, `per` of them a pass, of the nine-grid
+    sweep on the batch path in its default configuration, from the ncu record under
+    profiles/, or None when the record does not cover these sources, this storage, this
+    rounding or passes of this length."""
     if not os.path.exists(PROFILE_TRAFFIC) or rounding != "nearest":
         return None
-    tj = json.load(open(PROFILE_TRAFFIC))
-    entry = tj.get("storage", {}).get(storage)
-    if entry and tj.get("source_hash") == kernel_source_hash() and tj.get("path") == "batch":
-        # Captured on one-step launches of the same kernel; a launch of `spl`
-        # steps makes the same accesses `spl` times.
-        return entry["dram_bytes_per_step"] * spl
-    return None
+    passes = json.load(open(PROFILE_TRAFFIC)).get("passes", {})
+    entry = passes.get("storage", {}).get(storage)
+    if not entry or passes.get("source_hash") != kernel_source_hash() \
+            or entry["steps_per_pass"] != per:
+        return None
+    # Captured on launches of one pass; a launch makes the same accesses in each of its
+    # passes, the last of which can take fewer steps.
+    return entry["dram_bytes_per_pass"] * -(-spl // per)
+
+
+def batch_kernel(batch, schedule: str) -> str:
+    """Name of the kernel that the grids of a batch of one kind run."""
+    kind = "k_flow" if schedule == "flow" else "k_batch"
+    if not batch.get_config()["specialised"]:
+        return kind
+    per = batch.steps_per_pass()
+    return f"{kind}_fused ({per} steps a pass)" if per > 1 else f"{kind}_one"
 
 
 def sweep_leg(args, storage: str, stream, single_mlups):
@@ -735,6 +753,7 @@ def sweep_leg(args, storage: str, stream, single_mlups):
         status = b.sync()
         launch = b.get_launch()
         bcfg = b.get_config()
+        per, kernel = b.steps_per_pass(), batch_kernel(b, "lockstep")
         b.close()
         for g in grids:
             g.close()
@@ -750,9 +769,9 @@ def sweep_leg(args, storage: str, stream, single_mlups):
             "ratio_over_single_grid_kernel": mlups / single_mlups if single_mlups else None,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
-                         "traffic": recorded_traffic(storage, "nearest", spl),
+                         "traffic": recorded_traffic(storage, "nearest", spl, per),
                          "bytes_per_update": BYTES_PER_LU[storage], "note": ONE_STEP_NOTE,
-                         "kernel": f"k_batch_fused<{storage}>",
+                         "kernel": f"{kernel}, {storage}",
                          "algorithmic_bytes_per_launch": per_launch,
                          "mean_launch_ms": statistics.mean(ms)},
             "batch_config": bcfg, "batch_launch": launch, "batch_status": status}
@@ -864,7 +883,9 @@ def run_batch_workload(args):
                    "path": "one lbm_batch_step call of all steps: one persistent cooperative "
                            "launch per kind group"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": None, "kernel": "k_batch_one / k_batch",
+                     "frac": achieved / peak, "traffic": None,
+                     "kernel": ("k_flow_two / k_flow_fused / k_flow_one" if args.schedule == "flow"
+                                else "k_batch_fused / k_batch_one / k_batch"),
                      "algorithmic_bytes_per_step": r["alg_bytes_per_step"]},
         "gpu_launches": r["batch_config"]["groups"], "clocks": clk, "batch_status": r["status"],
     }
