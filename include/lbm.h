@@ -393,11 +393,12 @@ int lbm_batch_tune(lbm_batch_t b);
 int lbm_batch_get_config(lbm_batch_t b, int *rows, int *blocks_per_sm, int *specialised);
 /* Time steps of a pass over memory (1, 2 or 3) of member `grid`, 0 to n-1 in the order of
  * lbm_batch_create, in the work-list as last built; the last pass of a call can take
- * fewer. */
+ * fewer, and calls of one step run single-step walks (of a list that the first such call
+ * makes, waiting for the batch's stream). */
 int lbm_batch_get_pass(lbm_batch_t b, int grid, int *steps);
 /* The work-list as last built (at creation, by a configuration, schedule or
  * walk change, or by a step call that found a grid's field or rounding
- * changed): *tiles = warp walks per time step, *paired = how many of them
+ * changed): *tiles = warp walks per pass, *paired = how many of them
  * walk two segments of a narrow grid, a half-warp each (lockstep kind groups
  * of one 8-site 16-bit kind under LBM_WALK16_AUTO pair the tiles of grids at
  * most 128 columns wide when those are at least a fifth of the group's tiles;

@@ -22,10 +22,6 @@
 
 struct lbm_batch {
     std::vector<lbm_grid *> grids;
-    // Per grid, the c2 field pointer and rounding mode the work-list was built
-    // for (a change rebuilds it at the next step call).
-    std::vector<const float *> built_a15f;
-    std::vector<int> built_rounding;
     cudaStream_t stream = nullptr;
     int device = 0;
     int rows = 16;
@@ -43,14 +39,33 @@ struct lbm_batch {
         int rows = 0;                  // tile height
         int max_blocks_per_sm = 1;
     };
-    std::vector<Group> groups;
+    // A work-list: the grids' records and tiles on the device, the groups that run them.
+    struct List {
+        std::vector<Group> groups;
+        GridDesc *d_grids = nullptr;
+        Tile *d_tiles = nullptr;
+        int ntiles = 0;
+        int paired = 0;        // tiles with two segments (split walk)
+        std::vector<int> per;  // per grid, the steps of its passes
+        // graph cache (one step count)
+        cudaGraphExec_t graph = nullptr;
+        long long graph_n = -1;
+        // The list on the device is the one of the batch's settings.  A build that fails
+        // leaves none, and the next step call builds again before it launches anything;
+        // so does one that finds another c2 field or rounding than the list was built for.
+        bool built = false;
+        std::vector<const float *> built_a15f;
+        std::vector<int> built_rounding;
+    };
+    // The list of step calls, and one of single-step walks for calls of one step where
+    // the first takes several a pass, made by the first such call: a pass cut to one step
+    // reads the halo of several and walks narrower strips (one step of nine 2048^2 grids
+    // FP32 545 us in such a pass, 417 in single steps; FP16 291 / 236).
+    List list[2];
     int walk16 = LBM_WALK16_AUTO;  // walk of 16-bit grids (lbm_batch_set_walk16)
     int sms = 1;
     unsigned long long timeout_ns = 1000000000ULL;
     // device
-    GridDesc *d_grids = nullptr;
-    Tile *d_tiles = nullptr;
-    int ntiles = 0;
     long long *d_limit = nullptr;
     int *d_parity = nullptr;
     uint32_t *d_t0 = nullptr;
@@ -67,9 +82,6 @@ struct lbm_batch {
     std::vector<cudaStream_t> xs;
     std::vector<cudaEvent_t> xev;
     cudaEvent_t done = nullptr;
-    // graph cache (one step count)
-    cudaGraphExec_t graph = nullptr;
-    long long graph_n = -1;
     // Launch mode (lbm_batch_set_launch): LBM_LAUNCH_AUTO tries a graph and
     // falls back to direct launches if capture fails, LBM_LAUNCH_GRAPH
     // requires the graph, LBM_LAUNCH_DIRECT never captures.  `capture_failed`
@@ -87,13 +99,6 @@ struct lbm_batch {
     size_t prog_cap = 0;
     int *d_nwork = nullptr;
     int *h_nwork = nullptr;
-    // Paired tiles (split walk) in the lockstep work-list.
-    int paired = 0;
-    // Per grid, the steps of its passes (as of the work-list).
-    std::vector<int> per;
-    // The work-list on the device is the one of the settings above.  A build that fails
-    // leaves none, and the next step call builds again before it launches anything.
-    bool built = false;
 };
 
 static int bfail(int code, const std::string &m) {
@@ -113,10 +118,13 @@ static int bcuda(cudaError_t e, const char *where) {
         if (e_ != cudaSuccess) return bcuda(e_, #call);     \
     } while (0)
 
-static void drop_graph(lbm_batch *b) {
-    if (b->graph) cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-    b->graph_n = -1;
+static void drop_graph(lbm_batch::List &w) {
+    if (w.graph) cudaGraphExecDestroy(w.graph);
+    w.graph = nullptr;
+    w.graph_n = -1;
+}
+static void drop_graphs(lbm_batch *b) {
+    for (lbm_batch::List &w : b->list) drop_graph(w);
 }
 
 // Sites per lane of a grid's walk.  FP32: 4 (128-bit loads) when nx is a
@@ -133,22 +141,23 @@ static int batch_vec(const lbm_batch *b, const lbm_grid *g) {
 }
 
 // Copies the grid table and the tile list to the device.
-static int upload_worklist(lbm_batch *b, const std::vector<GridDesc> &gd,
+static int upload_worklist(lbm_batch *b, lbm_batch::List &w, const std::vector<GridDesc> &gd,
                            const std::vector<Tile> &ordered) {
-    if (b->d_tiles) cudaFree(b->d_tiles);
-    b->d_tiles = nullptr;
-    BCK(cudaMalloc(&b->d_tiles, sizeof(Tile) * std::max<size_t>(1, ordered.size())));
-    BCK(cudaMemcpy(b->d_grids, gd.data(), sizeof(GridDesc) * gd.size(), cudaMemcpyHostToDevice));
-    BCK(cudaMemcpy(b->d_tiles, ordered.data(), sizeof(Tile) * ordered.size(),
+    if (w.d_tiles) cudaFree(w.d_tiles);
+    w.d_tiles = nullptr;
+    BCK(cudaMalloc(&w.d_tiles, sizeof(Tile) * std::max<size_t>(1, ordered.size())));
+    if (!w.d_grids) BCK(cudaMalloc(&w.d_grids, sizeof(GridDesc) * gd.size()));
+    BCK(cudaMemcpy(w.d_grids, gd.data(), sizeof(GridDesc) * gd.size(), cudaMemcpyHostToDevice));
+    BCK(cudaMemcpy(w.d_tiles, ordered.data(), sizeof(Tile) * ordered.size(),
                    cudaMemcpyHostToDevice));
-    b->ntiles = (int)ordered.size();
-    b->built_a15f.clear();
-    b->built_rounding.clear();
+    w.ntiles = (int)ordered.size();
+    w.built_a15f.clear();
+    w.built_rounding.clear();
     for (const lbm_grid *g : b->grids) {
-        b->built_a15f.push_back(g->a15f);
-        b->built_rounding.push_back(g->rounding);
+        w.built_a15f.push_back(g->a15f);
+        w.built_rounding.push_back(g->rounding);
     }
-    b->built = true;
+    w.built = true;
     return LBM_OK;
 }
 
@@ -193,16 +202,16 @@ static int fused_rows(const std::vector<std::pair<FusedStrips, int>> &grids, lon
     return rows;
 }
 
-// (Re)builds the device grid table and the tile work-list.
-static int build_worklist(lbm_batch *b) {
-    b->built = false;
-    drop_graph(b);  // (it launches on the old list)
+// (Re)builds a work-list; singles_only: of single-step walks.
+static int build_list(lbm_batch *b, lbm_batch::List &w, bool singles_only) {
+    w.built = false;
+    drop_graph(w);  // (it launches on the old list)
     const size_t ng = b->grids.size();
     std::vector<GridDesc> gd(ng);
     std::vector<Tile> tiles;
-    b->paired = 0;
-    b->per.assign(ng, 1);
-    b->groups.clear();
+    w.paired = 0;
+    w.per.assign(ng, 1);
+    w.groups.clear();
     bool slabs = false;
     for (size_t k = 0; k < ng; ++k) {
         lbm_grid *g = b->grids[k];
@@ -230,7 +239,7 @@ static int build_worklist(lbm_batch *b) {
     auto add_tiles = [&](size_t k, int rows, int per) {
         lbm_grid *g = b->grids[k];
         GridDesc &d = gd[k];
-        b->per[k] = per;
+        w.per[k] = per;
         const int w = per > 1 ? fused_cols(g->storage, per) : 32 * batch_vec(b, g);
         const int ylo = g->slab, yhi = g->ny - g->slab, nyc = yhi - ylo;
         d.tile0 = (int)tiles.size();
@@ -256,7 +265,7 @@ static int build_worklist(lbm_batch *b) {
     // segments share warps.
     auto add_fused_tiles = [&](size_t k, int rows, int per) {
         const lbm_grid *g = b->grids[k];
-        b->per[k] = per;
+        w.per[k] = per;
         const FusedStrips s = fused_strips(g->storage, per, g->nx);
         const int w = fused_cols(g->storage, per), step = s.pieces ? s.pieces : 1;
         for (int y0 = 0, seg = 0; y0 < g->ny; y0 += rows, ++seg) {
@@ -277,7 +286,7 @@ static int build_worklist(lbm_batch *b) {
         // rows serve one.
         std::vector<int> kinds;
         for (const GridDesc &d : gd) kinds.push_back(d.kind);
-        FlowChoice fc = flow_kernel_for(kinds, b->walk16, !slabs);
+        FlowChoice fc = flow_kernel_for(kinds, b->walk16, !slabs && !singles_only);
         lbm_batch::Group gr;
         long long warps = 0;
         auto take = [&]() -> int {
@@ -411,17 +420,18 @@ static int build_worklist(lbm_batch *b) {
             if (k == 0) gr.rows = rows;
         }
         gr.count = (int)tiles.size();
-        b->groups.push_back(gr);
+        w.groups.push_back(gr);
         if (tiles.size() > b->prog_cap) {
+            int *prog = nullptr;
+            BCK(cudaMalloc(&prog, sizeof(int) * tiles.size()));
             cudaFree(b->d_prog);
-            b->d_prog = nullptr;
-            b->prog_cap = 0;
-            BCK(cudaMalloc(&b->d_prog, sizeof(int) * tiles.size()));
+            b->d_prog = prog;
             b->prog_cap = tiles.size();
+            drop_graphs(b);  // (both lists' launches use it)
         }
         if (!b->d_ctl)
             BCK(cudaMalloc(&b->d_ctl, sizeof(unsigned long long) * kFlowCtlWords * ng));
-        return upload_worklist(b, gd, tiles);
+        return upload_worklist(b, w, gd, tiles);
     }
     // Lockstep, default configuration, single-step walks: every warp walks its
     // tiles one after another within a step, so a batch with fewer tiles than
@@ -483,7 +493,7 @@ static int build_worklist(lbm_batch *b) {
     // has it, but for the split walk's groups, slabs, and 16-bit walks the
     // caller chose.
     auto fuses = [&](int kd) {
-        if (!fused_kernel_for(kd, 2).fn || splits(kd)) return false;
+        if (singles_only || !fused_kernel_for(kd, 2).fn || splits(kd)) return false;
         for (size_t k : of_kind[kd])
             if (b->grids[k]->slab ||
                 (b->grids[k]->storage != ST_F32 && b->walk16 != LBM_WALK16_AUTO))
@@ -578,7 +588,7 @@ static int build_worklist(lbm_batch *b) {
             ordered.insert(ordered.end(), tiles.begin(), tiles.end());
             split_tail(gr.begin, warps);
             gr.count = (int)ordered.size() - gr.begin;
-            b->groups.push_back(gr);
+            w.groups.push_back(gr);
             return LBM_OK;
         }
         gr.smem = 0;
@@ -588,7 +598,7 @@ static int build_worklist(lbm_batch *b) {
         std::stable_sort(tiles.begin(), tiles.end(),
                          [](const Tile &x, const Tile &y) { return x.grid < y.grid; });
         const bool split = kinds_in.size() == 1 && splits(kinds_in[0]);
-        const int paired0 = b->paired;
+        const int paired0 = w.paired;
         std::vector<int> pending(ng, -1);
         for (const Tile &t : tiles) {
             if (split && gd[t.grid].nx <= kSplitCols) {
@@ -599,7 +609,7 @@ static int build_worklist(lbm_batch *b) {
                     a.y1b = t.y1;
                     a.dirb = t.dir;
                     p = -1;
-                    ++b->paired;
+                    ++w.paired;
                     continue;
                 }
                 p = (int)ordered.size();
@@ -610,10 +620,10 @@ static int build_worklist(lbm_batch *b) {
         split_tail(gr.begin, (long long)bps * b->sms * kBatchWarps);
         gr.rows = lock_rows;
         gr.count = (int)ordered.size() - gr.begin;
-        gr.kernel = kernel_for(kinds_in, b->walk16, b->paired > paired0);
+        gr.kernel = kernel_for(kinds_in, b->walk16, w.paired > paired0);
         int rc = resident_blocks(b, (const void *)gr.kernel, 0, &gr.max_blocks_per_sm);
         if (rc != LBM_OK) return rc;
-        b->groups.push_back(gr);
+        w.groups.push_back(gr);
         return LBM_OK;
     };
     std::vector<int> rest;
@@ -631,15 +641,24 @@ static int build_worklist(lbm_batch *b) {
         int rc = add_group(rest);
         if (rc != LBM_OK) return rc;
     }
-    return upload_worklist(b, gd, ordered);
+    return upload_worklist(b, w, gd, ordered);
+}
+
+// (Re)builds the batch's work-list after a change of its settings; the list for calls of
+// one step follows when one needs it.
+static int build_worklist(lbm_batch *b) {
+    b->list[1].built = false;
+    return build_list(b, b->list[0], false);
 }
 
 extern "C" int lbm_batch_destroy(lbm_batch_t b) {
     if (!b) return LBM_OK;
-    if (b->stream || b->d_grids) cudaStreamSynchronize(b->stream);
-    drop_graph(b);
-    cudaFree(b->d_grids);
-    cudaFree(b->d_tiles);
+    if (b->stream || b->d_limit) cudaStreamSynchronize(b->stream);
+    drop_graphs(b);
+    for (lbm_batch::List &w : b->list) {
+        cudaFree(w.d_grids);
+        cudaFree(w.d_tiles);
+    }
     cudaFree(b->d_limit);
     cudaFree(b->d_parity);
     cudaFree(b->d_t0);
@@ -684,7 +703,6 @@ extern "C" int lbm_batch_create(const lbm_t *grids, int n, lbm_batch_t *out) {
     // One attribute (a full cudaGetDeviceProperties is slow, and servers
     // re-create batches often).
     cudaError_t e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_grids, sizeof(GridDesc) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_limit, sizeof(long long) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_parity, sizeof(int) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_t0, sizeof(uint32_t) * n);
@@ -720,7 +738,7 @@ static int grid_blocks(const lbm_batch *b, const lbm_batch::Group &g) {
 }
 
 // Queues: copy per-call arrays, reset barrier and status, cooperative launch.
-static cudaError_t enqueue(lbm_batch *b, long long n, cudaStream_t st) {
+static cudaError_t enqueue(lbm_batch *b, lbm_batch::List &w, long long n, cudaStream_t st) {
     int ng = (int)b->grids.size();
     cudaError_t e = cudaMemcpyAsync(b->d_limit, b->h_limit, sizeof(long long) * ng,
                                     cudaMemcpyHostToDevice, st);
@@ -731,7 +749,7 @@ static cudaError_t enqueue(lbm_batch *b, long long n, cudaStream_t st) {
         e = cudaMemcpyAsync(b->d_t0, b->h_t0, sizeof(uint32_t) * ng, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_status, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    const GridDesc *grids = b->d_grids;
+    const GridDesc *grids = w.d_grids;
     const long long *lim = b->d_limit;
     const int *par = b->d_parity;
     const uint32_t *t0 = b->d_t0;
@@ -743,21 +761,21 @@ static cudaError_t enqueue(lbm_batch *b, long long n, cudaStream_t st) {
         if (e == cudaSuccess)
             e = cudaMemsetAsync(b->d_ctl, 0,
                                 sizeof(unsigned long long) * kFlowCtlWords * ng, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(b->d_prog, 0, sizeof(int) * b->ntiles, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(b->d_prog, 0, sizeof(int) * w.ntiles, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned) * kBarWords, st);
         if (e != cudaSuccess) return e;
-        const lbm_batch::Group &gr = b->groups[0];
+        const lbm_batch::Group &gr = w.groups[0];
         gr.fkernel<<<grid_blocks(b, gr), 32 * kBatchWarps, gr.smem, st>>>(
-            grids, ng, b->d_tiles, lim, par, t0, b->d_ctl, b->d_prog, bar, b->d_nwork, status,
+            grids, ng, w.d_tiles, lim, par, t0, b->d_ctl, b->d_prog, bar, b->d_nwork, status,
             to);
         return cudaGetLastError();
     }
     // The groups hold disjoint grids: each launch advances its grids by all n
     // steps.  Barrier words and tile counters start at zero for every launch.
-    for (const lbm_batch::Group &gr : b->groups) {
+    for (const lbm_batch::Group &gr : w.groups) {
         e = cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned) * kBarWords, st);
         if (e != cudaSuccess) return e;
-        const Tile *tiles = b->d_tiles + gr.begin;
+        const Tile *tiles = w.d_tiles + gr.begin;
         int ntiles = gr.count;
         void *args[] = {(void *)&grids, (void *)&tiles, (void *)&ntiles, (void *)&lim,
                         (void *)&par,   (void *)&t0,    (void *)&n,      (void *)&bar,
@@ -769,7 +787,8 @@ static cudaError_t enqueue(lbm_batch *b, long long n, cudaStream_t st) {
     return cudaSuccess;
 }
 
-static int run_batch(lbm_batch *b, long long n, const long long *limits, bool advance) {
+static int run_batch(lbm_batch *b, lbm_batch::List &w, long long n, const long long *limits,
+                     bool advance) {
     int ng = (int)b->grids.size();
     // The previous call's copies must have read the pinned arrays first.
     BCK(cudaEventSynchronize(b->copied));
@@ -805,37 +824,37 @@ static int run_batch(lbm_batch *b, long long n, const long long *limits, bool ad
                             (b->launch_mode == LBM_LAUNCH_AUTO && !b->capture_failed);
     bool graphed = false;
     if (want_graph) {
-        if (b->graph_n != n) {
-            drop_graph(b);
+        if (w.graph_n != n) {
+            drop_graph(w);
             cudaStream_t cs;
             BCK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
             cudaGraph_t g = nullptr;
             e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
-                cudaError_t e1 = enqueue(b, n, cs);
+                cudaError_t e1 = enqueue(b, w, n, cs);
                 cudaError_t e2 = cudaStreamEndCapture(cs, &g);
                 e = e1 != cudaSuccess ? e1 : e2;
             }
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
+            if (e == cudaSuccess) e = cudaGraphInstantiate(&w.graph, g, 0);
             if (g) cudaGraphDestroy(g);
             cudaStreamDestroy(cs);
             if (e != cudaSuccess) {
                 cudaGetLastError();
-                drop_graph(b);
+                drop_graph(w);
                 if (b->launch_mode == LBM_LAUNCH_GRAPH)
                     return bcuda(e, "lbm_batch_step: capturing the persistent launch in a CUDA graph");
                 // AUTO: recorded (lbm_batch_get_launch) and never retried.
                 b->capture_failed = true;
             } else {
-                b->graph_n = n;
+                w.graph_n = n;
             }
         }
-        if (b->graph) {
-            e = cudaGraphLaunch(b->graph, b->stream);
+        if (w.graph) {
+            e = cudaGraphLaunch(w.graph, b->stream);
             graphed = true;
         }
     }
-    if (!graphed) e = enqueue(b, n, b->stream);
+    if (!graphed) e = enqueue(b, w, n, b->stream);
     if (e != cudaSuccess) return bcuda(e, "lbm_batch_step launch");
     b->last_launch = graphed ? LBM_LAUNCH_GRAPH : LBM_LAUNCH_DIRECT;
     BCK(cudaEventRecord(b->copied, b->stream));
@@ -849,10 +868,22 @@ static int run_batch(lbm_batch *b, long long n, const long long *limits, bool ad
         for (int k = 0; k < ng; ++k) {
             long long s = b->h_limit[k];
             b->grids[k]->t += s;
-            if (passes_of(s, b->per[k]) & 1) b->grids[k]->cur ^= 1;
+            if (passes_of(s, w.per[k]) & 1) b->grids[k]->cur ^= 1;
         }
     }
     return LBM_OK;
+}
+
+// Builds a list that is not the one of the batch's settings and grids.
+static int ready(lbm_batch *b, lbm_batch::List &w, bool singles_only) {
+    bool stale = !w.built;
+    for (size_t k = 0; k < b->grids.size() && !stale; ++k) {
+        const lbm_grid *g = b->grids[k];
+        stale = g->a15f != w.built_a15f[k] || g->rounding != w.built_rounding[k];
+    }
+    if (!stale) return LBM_OK;
+    BCK(cudaStreamSynchronize(b->stream));
+    return build_list(b, w, singles_only);
 }
 
 extern "C" int lbm_batch_step(lbm_batch_t b, long long n, const long long *limits) {
@@ -860,22 +891,17 @@ extern "C" int lbm_batch_step(lbm_batch_t b, long long n, const long long *limit
     if (b->schedule == LBM_SCHEDULE_FLOW && n > 0x7fffffffLL)
         return bfail(LBM_EINVAL, "lbm_batch_step: flow schedule takes at most 2^31 - 1 steps a call");
     if (n == 0) return LBM_OK;
-    bool stale = !b->built;
-    for (size_t k = 0; k < b->grids.size(); ++k) {
-        const lbm_grid *g = b->grids[k];
+    for (const lbm_grid *g : b->grids) {
         if (g->drive) return bfail(LBM_EINVAL, "lbm_batch_step: a grid has a drive");
         if (g->grad != LBM_GRAD_CENTRAL)
             return bfail(LBM_EINVAL, "lbm_batch_step: a grid uses the forward difference");
-        stale = stale || g->a15f != b->built_a15f[k] || g->rounding != b->built_rounding[k];
     }
-    if (stale) {
-        // A grid's c2 field or rounding changed since the work-list was built, or its
-        // last build failed.
-        BCK(cudaStreamSynchronize(b->stream));
-        int rc = build_worklist(b);
-        if (rc != LBM_OK) return rc;
-    }
-    return run_batch(b, n, limits, true);
+    int rc = ready(b, b->list[0], false);
+    if (rc != LBM_OK) return rc;
+    const std::vector<int> &per = b->list[0].per;
+    const bool single = n == 1 && *std::max_element(per.begin(), per.end()) > 1;
+    if (single && (rc = ready(b, b->list[1], true)) != LBM_OK) return rc;
+    return run_batch(b, b->list[single ? 1 : 0], n, limits, true);
 }
 
 cudaError_t batch_queue_status(lbm_batch *b, cudaStream_t st) {
@@ -899,12 +925,12 @@ extern "C" int lbm_batch_set_config(lbm_batch_t b, int rows, int blocks_per_sm) 
         return bfail(LBM_EINVAL, "lbm_batch_set_config: bad argument");
     BCK(cudaStreamSynchronize(b->stream));
     b->blocks_per_sm = blocks_per_sm;
-    if (rows != b->rows || b->fit_rows || !b->built) {
+    if (rows != b->rows || b->fit_rows || !b->list[0].built) {
         b->rows = rows;
         b->fit_rows = false;
         return build_worklist(b);
     }
-    drop_graph(b);
+    drop_graphs(b);
     return LBM_OK;
 }
 
@@ -912,7 +938,7 @@ extern "C" int lbm_batch_set_walk16(lbm_batch_t b, int walk) {
     if (!b || walk < LBM_WALK16_AUTO || walk > LBM_WALK16_V4_PF2)
         return bfail(LBM_EINVAL, "lbm_batch_set_walk16: unknown walk");
     BCK(cudaStreamSynchronize(b->stream));
-    if (walk == b->walk16 && b->built) return LBM_OK;
+    if (walk == b->walk16 && b->list[0].built) return LBM_OK;
     b->walk16 = walk;
     return build_worklist(b);
 }
@@ -925,14 +951,14 @@ extern "C" int lbm_batch_get_walk16(lbm_batch_t b, int *walk) {
 
 extern "C" int lbm_batch_get_groups(lbm_batch_t b, int *groups) {
     if (!b || !groups) return bfail(LBM_EINVAL, "lbm_batch_get_groups: bad argument");
-    *groups = (int)b->groups.size();
+    *groups = (int)b->list[0].groups.size();
     return LBM_OK;
 }
 
 extern "C" int lbm_batch_set_timeout_us(lbm_batch_t b, long long us) {
     if (!b || us < 1) return bfail(LBM_EINVAL, "lbm_batch_set_timeout_us: bad argument");
     b->timeout_ns = (unsigned long long)us * 1000ULL;
-    drop_graph(b);
+    drop_graphs(b);
     return LBM_OK;
 }
 
@@ -963,14 +989,14 @@ static int time_passes(lbm_batch *b, cudaEvent_t e0, cudaEvent_t e1, double *cos
     double updates = 0;
     for (size_t k = 0; k < b->grids.size(); ++k) {
         const lbm_grid *g = b->grids[k];
-        limits.push_back(b->per[k]);
+        limits.push_back(b->list[0].per[k]);
         most = std::max(most, limits.back());
         updates += (double)limits.back() * g->nx * (g->ny - 2 * g->slab);
     }
-    int rc = run_batch(b, most, limits.data(), false);  // warm-up (and graph build)
+    int rc = run_batch(b, b->list[0], most, limits.data(), false);  // warm-up (and graph build)
     if (rc != LBM_OK) return rc;
     BCK(cudaEventRecord(e0, b->stream));
-    for (int k = 0; k < 4 && rc == LBM_OK; ++k) rc = run_batch(b, most, limits.data(), false);
+    for (int k = 0; k < 4 && rc == LBM_OK; ++k) rc = run_batch(b, b->list[0], most, limits.data(), false);
     if (rc != LBM_OK) return rc;
     BCK(cudaEventRecord(e1, b->stream));
     BCK(cudaEventSynchronize(e1));
@@ -991,7 +1017,7 @@ static int tune_candidates(lbm_batch *b, cudaEvent_t e0, cudaEvent_t e1, BatchTr
         if (rc != LBM_OK) return rc;
         std::vector<BatchKernel> ks;
         bool fused = false;
-        for (const auto &gr : b->groups) {
+        for (const auto &gr : b->list[0].groups) {
             ks.push_back(gr.kernel);
             fused = fused || gr.fused;
         }
@@ -1044,7 +1070,7 @@ extern "C" int lbm_batch_set_schedule(lbm_batch_t b, int schedule) {
     if (!b || schedule < LBM_SCHEDULE_LOCKSTEP || schedule > LBM_SCHEDULE_FLOW)
         return bfail(LBM_EINVAL, "lbm_batch_set_schedule: unknown schedule");
     BCK(cudaStreamSynchronize(b->stream));
-    if (schedule == b->schedule && b->built) return LBM_OK;
+    if (schedule == b->schedule && b->list[0].built) return LBM_OK;
     b->schedule = schedule;
     return build_worklist(b);
 }
@@ -1061,7 +1087,7 @@ extern "C" int lbm_batch_set_launch(lbm_batch_t b, int mode) {
     BCK(cudaStreamSynchronize(b->stream));
     b->launch_mode = mode;
     b->capture_failed = false;
-    drop_graph(b);
+    drop_graphs(b);
     return LBM_OK;
 }
 
@@ -1075,27 +1101,27 @@ extern "C" int lbm_batch_get_launch(lbm_batch_t b, int *mode, int *last, int *ca
 
 extern "C" int lbm_batch_get_tiles(lbm_batch_t b, int *tiles, int *paired) {
     if (!b) return bfail(LBM_EINVAL, "lbm_batch_get_tiles: NULL batch");
-    if (tiles) *tiles = b->ntiles;
-    if (paired) *paired = b->paired;
+    if (tiles) *tiles = b->list[0].ntiles;
+    if (paired) *paired = b->list[0].paired;
     return LBM_OK;
 }
 
 extern "C" int lbm_batch_get_pass(lbm_batch_t b, int grid, int *steps) {
     if (!b || !steps || grid < 0 || grid >= (int)b->grids.size())
         return bfail(LBM_EINVAL, "lbm_batch_get_pass: bad argument");
-    *steps = b->per[grid];
+    *steps = b->list[0].per[grid];
     return LBM_OK;
 }
 
 extern "C" int lbm_batch_get_config(lbm_batch_t b, int *rows, int *blocks_per_sm,
                                     int *specialised) {
     if (!b) return bfail(LBM_EINVAL, "lbm_batch_get_config: NULL batch");
-    if (rows) *rows = b->groups.empty() ? b->rows : b->groups[0].rows;
+    if (rows) *rows = b->list[0].groups.empty() ? b->rows : b->list[0].groups[0].rows;
     if (blocks_per_sm)
-        *blocks_per_sm = b->groups.empty() ? 0 : grid_blocks(b, b->groups[0]) / b->sms;
+        *blocks_per_sm = b->list[0].groups.empty() ? 0 : grid_blocks(b, b->list[0].groups[0]) / b->sms;
     if (specialised) {
         *specialised = 1;
-        for (const auto &gr : b->groups)
+        for (const auto &gr : b->list[0].groups)
             if (gr.kernel == (BatchKernel)k_batch || gr.fkernel == (FlowKernel)k_flow)
                 *specialised = 0;
     }

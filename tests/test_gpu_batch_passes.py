@@ -109,6 +109,38 @@ def test_mixed_passes_in_flow_equal_single_steps(lbm, kind):
              range(len(sizes)))
 
 
+@pytest.mark.parametrize("schedule", ["lockstep", "flow"])
+@pytest.mark.parametrize("kind", ["f32", "f16d", "bf16d-sr", "mixed"])
+def test_calls_of_one_step_between_others(lbm, schedule, kind):
+    """Calls of one step run on a list of single-step walks: mixed with longer calls, and
+    with a grid's rounding or field changed in between (both lists are built again)."""
+    sizes = [(120, 64), (240, 300), (240, 96), (480, 200)]
+    make = _maker(lbm, sizes, ["f32", "f16d"] if kind == "mixed" else [kind])
+    grids = [make(k) for k in range(len(sizes))]
+    b = lbm.Batch(grids)
+    b.set_schedule(schedule)
+    b.step(5)
+    for n in (1, 1, 4, 1):
+        b.step(n)
+    lens = workloads.c2_lens(*sizes[0], 0.2)
+    if not kind.endswith("-sr"):
+        grids[0].set_c2_field(lens)
+    b.step(1)
+    b.step(3, [1, 0, 3, 2])
+    b.step(1, [0, 1, 1, 0])
+    assert b.sync() == 0
+    got = [(g.t, g.get_state()[0]) for g in grids]
+    _close(b, grids)
+    for k, (t, state) in enumerate(got):
+        assert t == 13 + [1, 1, 4, 2][k]
+        with make(k) as h:
+            for n in range(t):
+                if n == 12 and k == 0 and not kind.endswith("-sr"):
+                    h.set_c2_field(lens)
+                h.step(1)
+            assert np.array_equal(h.get_state()[0], state), sizes[k]
+
+
 def test_tall_batch_takes_three_steps(lbm):
     """The grids of the test of tall tiles in a batch."""
     grids = [lbm.Grid(nx, ny, 0.7, 0.2) for nx, ny in [(64, 100003), (124, 20001)]]

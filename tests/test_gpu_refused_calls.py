@@ -81,6 +81,36 @@ def test_failed_work_list_is_built_again_by_the_next_step(fake_lib, change):
     """)
 
 
+@pytest.mark.parametrize("schedule", ["lockstep", "flow"])
+def test_failed_list_for_calls_of_one_step(fake_lib, schedule):
+    """Calls of one step have a list of their own, made by the first of them; where it
+    cannot be allocated that call fails, and others run."""
+    _run(fake_lib, f"""
+        sizes = [(120, 40), (116, 33), (240, 64)]
+        grids = [grid(*s) for s in sizes]
+        b = lbm.Batch(grids)
+        b.set_schedule("{schedule}")
+        assert b.steps_per_pass() == 2
+        b.step(4)
+        malloc.value = 1
+        try:
+            b.step(1)
+        except lbm.LbmError as e:
+            assert e.status == lbm.LBM_ENOMEM, e
+        else:
+            raise AssertionError("no error")
+        b.step(4)
+        malloc.value = 0
+        b.step(1)
+        b.step(4)
+        b.step(1)
+        assert b.sync() == 0
+        for g, s in zip(grids, sizes):
+            assert g.t == 14
+            assert np.array_equal(g.get_state()[0], alone(*s, 14))
+    """)
+
+
 @pytest.mark.parametrize("nx,ny,tiles", [(400, 4, "one cluster"), (256, 256, "all SMs")])
 def test_refused_resident_launch_steps_by_the_step_kernel(fake_lib, nx, ny, tiles):
     """A stream that owns too few SMs for a grid's tiles still steps it: the call whose
