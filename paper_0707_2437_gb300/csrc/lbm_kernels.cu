@@ -742,19 +742,21 @@ __global__ void __launch_bounds__(RT)
 // value * sin(phase), phase = 2 pi (kx x / nx + ky y / ny).  The phase factor is
 // the product of one of the column and one of the row: a thread sums its column's
 // values times the rows' factors (from a table a block computes for 256 rows at a
-// time; none if ky = 0) and multiplies by the column's once.  A block has 32
-// columns, so that their sines and cosines (80 FP64 instructions of 16 cycles a
-// warp) spread over the SMs.  Per site that leaves
+// time, once if it has no more; none if ky = 0) and multiplies by the column's once.
+// A block has 32 columns, so that their sines and cosines (80 FP64 instructions of 16
+// cycles a warp) spread over the SMs; more where a grid of a few rows has more columns
+// than that for every block.  Per site that leaves
 // the FP64 pipe (which bounds this kernel) 8 additions and products for the
 // density, scaled by 36 so that the weights are powers of two, and 1 or 2 for the
 // sum, against about 65 with sine and cosine per site and conversions: one 2048^2
 // read 910 -> 190 us.
 constexpr int kModeCols = 32;
+constexpr int kModeRows = 64;  // rows a block takes at least, so that theirs spread too
 template <int S>
 __global__ void __launch_bounds__(RT)
     k_mode(const void *__restrict__ f, int nx, int ny, size_t P, double rho0, int field, int kx,
            int ky, int cols, int par, int rows_per_block, Results res) {
-    __shared__ double2 row_phase[RT], col_phase[kModeCols];
+    __shared__ double2 row_phase[RT], col_phase[RT];
     const int tx = threadIdx.x % cols, ty = threadIdx.x / cols;
     const long long yb = (long long)blockIdx.y * rows_per_block;
     const long long ye = min((long long)ny, yb + rows_per_block);
@@ -771,16 +773,20 @@ __global__ void __launch_bounds__(RT)
             sincospi(2.0 * ((double)px / nx), &sn, &cs);
             col_phase[tx] = make_double2(cs, sn);
         }
-        __syncthreads();
+        // The rows' factors from the last threads down: other warps than the columns',
+        // at the same time.
+        const bool table = ky && (ye - yb > RT || c0 < cols * (long long)gridDim.x);
+        if (!table) __syncthreads();
         double ac = 0.0, as = 0.0;  // sum of value * row factor
         for (long long y0 = yb; y0 < ye; y0 += RT) {
-            if (ky) {
-                __syncthreads();
-                if (y0 + threadIdx.x < ye) {
-                    const long long py = ((long long)ky * (y0 + threadIdx.x)) % ny;
+            if (table) {
+                if (y0 > yb) __syncthreads();
+                const int m = RT - 1 - (int)threadIdx.x;
+                if (y0 + m < ye) {
+                    const long long py = ((long long)ky * (y0 + m)) % ny;
                     double sn, cs;
                     sincospi(2.0 * ((double)py / ny), &sn, &cs);
-                    row_phase[threadIdx.x] = make_double2(cs, sn);
+                    row_phase[m] = make_double2(cs, sn);
                 }
                 __syncthreads();
             }
@@ -890,10 +896,12 @@ Err launch_sums_host(int storage, const void *f, int nx, int ny, size_t P, const
 
 Err launch_mode(int storage, const void *f, int nx, int ny, size_t P, double rho0, int field,
                 int kx, int ky, const HostResults &r, cudaStream_t st) {
-    // About 4 rows a thread or more; at most kReduceBlocksMax blocks.
-    SideGeom g = side_geom(nx, ny, kReduceBlocksMax, kModeCols);
+    // At most kReduceBlocksMax blocks.
+    int widest = kModeCols;
+    while (2LL * widest * ny <= kSide && nx > (long long)widest * kReduceBlocksMax) widest *= 2;
+    SideGeom g = side_geom(nx, ny, kReduceBlocksMax, widest);
     if (g.gx > (unsigned)kReduceBlocksMax) g.gx = kReduceBlocksMax;  // (the kernel loops)
-    const long long least = 4LL * g.par;
+    const long long least = 4 * g.par < kModeRows ? 4 * g.par : kModeRows;
     long long rows = ((long long)ny + g.gy - 1) / g.gy;
     if (rows < least) rows = least;
     if (rows > ny) rows = ny;
