@@ -50,17 +50,9 @@ struct GridDesc {
 // fused walk only) has pieces of `rows` rows on `lanes` lanes each; lanes 0: one piece.
 struct __align__(16) Tile {
     int grid, x0, y0, y1, dir;
-    union {
-        int y0b;
-        int lanes;
-    };
-    union {
-        int y1b;
-        int rows;
-    };
-    int dirb;
+    int y0b, y1b, dirb;
+    int lanes, rows;
 };
-static_assert(sizeof(Tile) == 32, "a sector");
 
 // A grid's walk in the batch kernels: storage kind, sites per lane (1, 4 or
 // 8), stochastic rounding, and a per-site c2 field.
