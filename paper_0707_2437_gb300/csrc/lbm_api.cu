@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <fstream>
 #include <map>
 #include <mutex>
@@ -193,9 +194,12 @@ static cudaError_t copy_stream(int device, cudaStream_t *out) {
 }
 
 // Small grids (those that may run resident) per device and stream: as many streams as
-// hold some may step them at the same time.
+// hold some may step them at the same time.  The number of streams is kept beside the
+// table, for step calls to read.
+static constexpr int kDevices = 64;
 static std::mutex g_small_mu;
 static std::map<std::pair<int, cudaStream_t>, int> g_small;
+static std::atomic<int> g_small_streams[kDevices];
 
 static std::pair<int, cudaStream_t> small_key(const lbm_grid *h) {
     return {h->device, h->stream == cudaStreamLegacy ? nullptr : h->stream};
@@ -204,24 +208,24 @@ static void uncount_small(lbm_grid *h) {
     if (!h->counted) return;
     std::lock_guard<std::mutex> lk(g_small_mu);
     auto it = g_small.find(small_key(h));
-    if (it != g_small.end() && --it->second == 0) g_small.erase(it);
+    if (it != g_small.end() && --it->second == 0) {
+        g_small.erase(it);
+        --g_small_streams[h->device];
+    }
     h->counted = false;
 }
-// (Not counted if the host is out of memory.)
+// (Not counted if the host is out of memory, or on a 65th device.)
 static void count_small(lbm_grid *h) {
-    if (!h->flags || h->counted) return;
+    if (!h->flags || h->counted || h->device >= kDevices) return;
     std::lock_guard<std::mutex> lk(g_small_mu);
     try {
-        ++g_small[small_key(h)];
+        if (g_small[small_key(h)]++ == 0) ++g_small_streams[h->device];
         h->counted = true;
     } catch (const std::bad_alloc &) {
     }
 }
 static int small_streams(int device) {
-    std::lock_guard<std::mutex> lk(g_small_mu);
-    int n = 0;
-    for (const auto &kv : g_small) n += kv.first.first == device;
-    return n;
+    return device < kDevices ? g_small_streams[device].load(std::memory_order_relaxed) : 1;
 }
 void never_resident(lbm_grid *h) {
     uncount_small(h);
