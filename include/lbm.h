@@ -118,8 +118,8 @@ int lbm_init(lbm_t h, const double *rho, const double *ux, const double *uy,
 
 /* Queues n >= 0 time steps of Eq. 5 (stream, moments, central grad(rho),
  * collide with force) on the handle's stream.  Calls either launch the step
- * kernel once per step, or every two or three steps (replayed from CUDA graphs, 32 launches
- * each), or run all n steps as one launch of one of two kinds.  Resident: the
+ * kernel once per step, or every two or three steps (replayed from CUDA graphs,
+ * 32 launches each), or run all n steps as one launch of one of two kinds.  Resident: the
  * grid's tiles stay in the SMs' shared memory, one block each, and exchange
  * their edges every few steps (bounded waits); grids of up to about 660^2
  * sites.  Persistent: the batched kernel (see lbm_batch_create) with this grid
@@ -203,9 +203,9 @@ int lbm_mode(lbm_t h, int field, int kx, int ky, double *out2);
  *   on         1 to drive, 0 to return to a fully periodic grid
  *   amplitude  |amplitude| < 1 (the paper's runs are small-amplitude)
  *   period     steps per cycle, finite and > 0 (500 in the paper)
- * Needs nx >= 4.  Each step then runs one extra small kernel (27 ny
- * stores), and long step calls use CUDA graphs instead of the persistent
- * launch.  A driven grid cannot join a batch: lbm_batch_create and
+ * Needs nx >= 4.  A resident call sets the columns within its steps.  Step
+ * launches, single ones here, run one extra small kernel each (27 ny stores);
+ * long calls replay them from CUDA graphs.  A persistent launch is never used.  A driven grid cannot join a batch: lbm_batch_create and
  * lbm_batch_step return LBM_EINVAL.  Waits for the grid's stream; returns
  * LBM_EINVAL for a bad argument. */
 int lbm_set_drive(lbm_t h, int on, double amplitude, double period);
@@ -215,8 +215,8 @@ int lbm_set_drive(lbm_t h, int on, double amplitude, double period);
  * [ny][nx] array of c_e^2 > 0 (host if on_device == 0, else device; host
  * values are checked); the force at site x uses alpha(x) = 1/3 - c2(x) in
  * Eq. 5.  NULL returns to the grid's uniform c2.  The field costs one more
- * 4-byte read per site and step.  While a field is set the single-grid step
- * kernel uses at most 4 sites per lane, no bulk-copy pipeline and nearest
+ * 4-byte read per site and pass.  While a field is set single-step launches
+ * use at most 4 sites per lane, no bulk-copy pipeline and nearest
  * rounding (an FP32 grid configured for 4 sites per lane steps with 2 sites
  * per lane and one row of loads prefetched, its tile height raised to fill
  * one wave of resident warps where that helps).  The grid can join a batch,
@@ -276,9 +276,11 @@ int lbm_set_state(lbm_t h, const void *src_host, long long t);
  * (down to 2) when the grid has too few tiles to occupy them, more (up to
  * 32) when its tiles need between one and two waves; lbm_get_config reports
  * the configured 16.  In the default configuration, and after lbm_tune where
- * it measured faster, step calls on large grids (nx a multiple of 4 in FP32, of
- * 8 in 16-bit storage) take two or three steps per launch; bitwise the same.  A configuration or pipeline set by the caller steps once
- * per launch. */
+ * it measured faster, step calls take two or three steps per launch where that is
+ * estimated to be the faster, mostly on large grids; bitwise the same.  FP32 grids
+ * of any width from 4 and 16-bit grids of even widths from 8 can; with a c2 field
+ * widths that are multiples of 4 and of 8.  A configuration or pipeline set by the
+ * caller steps once per launch. */
 int lbm_set_config(lbm_t h, int vec, int rows, int warps);
 int lbm_get_config(lbm_t h, int *vec, int *rows, int *warps);
 
@@ -300,10 +302,10 @@ int lbm_get_pipeline(lbm_t h, int *stages, int *active);
  * fraction (as many random bits as dropped bits: 13 for FP16, 16 for BF16),
  * so each stored value is the FP32 result in expectation; the random bits are
  * a hash of (pair of sites, direction, step), so runs stay deterministic and
- * independent of the tile configuration and of batching.  Stochastic rounding
- * uses the register walks (vec 1, 2 or 4) and the shared-memory walk at vec 8
- * with 4 warps; it moves other vec-8 configurations to 4 and turns the
- * bulk-copy pipeline off.  FP32 storage
+ * independent of the tile configuration and of batching.  In single-step
+ * launches stochastic rounding uses the register walks (vec 1, 2 or 4) and the
+ * shared-memory walk at vec 8 with 4 warps; it moves other vec-8 configurations
+ * to 4 and turns the bulk-copy pipeline off.  FP32 storage
  * accepts only LBM_ROUND_NEAREST.  Because the dither differs from site to
  * site, it breaks symmetries a deterministic rounding keeps exactly: above c2
  * of about 1.16 (c_e > 1.08) a grid started uniform in y has transverse modes
@@ -347,8 +349,8 @@ int lbm_kernel_ms(lbm_t h, double *ms, long long *launches);
 
 /* Groups n >= 1 existing handles (any sizes, tau, c2, storage and rounding;
  * all on the same device) into a batch stepped by persistent cooperative
- * kernels over a tile work-list, with a grid-wide barrier between time steps
- * (one launch per kind group, see lbm_batch_get_groups).  Every grid reaches
+ * kernels over a tile work-list, with a grid-wide barrier between passes of one to
+ * three time steps (one launch per kind group, see lbm_batch_get_groups).  Every grid reaches
  * bitwise the state it reaches when stepped alone.  The batch refers to the
  * handles; they must outlive it and must not be stepped individually while
  * it is being stepped.  The batch's work runs on the stream grids[0] had
@@ -362,8 +364,9 @@ int lbm_batch_destroy(lbm_batch_t b);
 
 /* Advances grid g of the batch by min(n, limits[g]) steps (limits may be NULL:
  * n steps each), one persistent launch per kind group, replayed from a CUDA
- * graph (see lbm_batch_set_launch).  Asynchronous.  A barrier wait that exceeds its time limit makes the
- * kernel stop and the next synchronising batch call return LBM_ETIMEOUT.
+ * graph (see lbm_batch_set_launch).  Asynchronous.  A barrier wait that exceeds
+ * its time limit makes the kernel stop and the next synchronising batch call
+ * return LBM_ETIMEOUT.
  * If a grid's c2 field or rounding mode changed since the batch was built,
  * the work-list is rebuilt first (the call then waits for the stream).
  * LBM_EINVAL if a grid has gained a drive or the forward-difference gradient. */
@@ -380,10 +383,12 @@ int lbm_batch_sync(lbm_batch_t b);
  * and the error returned).  Until one of them is called, a lockstep batch
  * whose tiles at 16 rows would fill less than 3/4 of the resident warps
  * (16 per SM) takes shorter tiles, down to 2 rows, as many as those warps
- * hold, and kind groups whose walk takes two or three steps per pass over memory (FP32
- * grids with nx a multiple of 4, 16-bit grids under LBM_WALK16_AUTO with nx a
- * multiple of 8, unless their tiles are paired; slabs never) get the height
- * that balances their tiles over the resident warps.  The tuner times those too. */
+ * hold, and kind groups that take two or three steps per pass over memory get the
+ * height that balances their tiles over the resident warps.  The tuner times those
+ * too.  Such passes are for FP32 grids with nx a multiple of 4 (small batches whose
+ * strips of 120 columns are badly filled step singly) and 16-bit grids under
+ * LBM_WALK16_AUTO with nx a multiple of 8, unless their tiles are paired; never for
+ * slabs. */
 int lbm_batch_set_config(lbm_batch_t b, int rows, int blocks_per_sm);
 int lbm_batch_tune(lbm_batch_t b);
 /* Tile height of the first kind group as built (in the flow schedule, where grids have
@@ -435,7 +440,7 @@ int lbm_batch_get_walk16(lbm_batch_t b, int *walk);
 /* Schedule of lbm_batch_step:
  *   LBM_SCHEDULE_LOCKSTEP  the default: one persistent launch per kind group
  *                          runs every time step of all its grids, with a
- *                          grid-wide barrier between steps
+ *                          grid-wide barrier between passes
  *   LBM_SCHEDULE_FLOW      one launch over all grids with no barrier: each
  *                          grid advances on its own, a tile's step starting
  *                          as soon as the tiles it reads from have finished

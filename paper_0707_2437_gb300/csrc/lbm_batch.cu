@@ -1,14 +1,9 @@
 // Host side of the batched form (the kernels are in lbm_batch_kernels.cuh):
-// many uneven grids (any size, tau, c2 and storage) advanced by
-// one persistent cooperative kernel over a tile work-list, with a grid-wide
-// barrier between time steps, replayed from a CUDA graph.
-//
-// Work-list: every grid is cut into tiles of (32*vec columns) x (rows rows),
-// one warp per tile per step; within a step the resident warps take tiles in
-// list order from an atomic counter.  Within a time step tiles are independent (each reads its grid's
-// input buffer and writes the other one); between steps every block waits at
-// a barrier, because a tile's pull reaches two rows and one column into its
-// neighbours and its store overwrites what they read one step earlier.
+// many uneven grids (any size, tau, c2 and storage) advanced by persistent kernels over a
+// tile work-list, replayed from a CUDA graph: one cooperative launch per kind group with
+// a grid-wide barrier between passes (lockstep), or one launch with progress counters per
+// tile (flow).  This file plans: which kernel each group runs, whether its passes take
+// one, two or three steps, how tall its tiles are.
 //
 // Every barrier wait is bounded (wall-clock limit read from %globaltimer): a
 // block that gives up sets a status word and returns, all other blocks see the

@@ -1,15 +1,16 @@
 // Device side of the batched form: the grid descriptor and tile records,
-// the bounded grid barrier, the per-step tile counters and the persistent
-// batch kernels (the general k_batch and the specialised k_batch_one), plus
-// the table that picks a kernel for a set of grid kinds.  Included by
-// lbm_batch.cu only.
+// the bounded grid barrier, the tile counters, the persistent batch kernels (the
+// fused walk's k_batch_fused, single steps of one walk in k_batch_one and of any in
+// k_batch; their k_flow counterparts), and the tables that pick a kernel for a set of
+// grid kinds.  Included by lbm_batch.cu only.
 //
-// Work-list: every grid is cut into tiles of (32*vec columns) x (rows rows),
-// one warp per tile per step; within a step the resident warps take tiles in
-// list order from an atomic counter.  Within a time step tiles are independent (each reads its grid's
-// input buffer and writes the other one); between steps every block waits at
-// a barrier, because a tile's pull reaches two rows and one column into its
-// neighbours and its store overwrites what they read one step earlier.
+// Work-list: every grid is cut into tiles of a strip's columns and some rows, one warp
+// per tile and pass; a pass takes one step in the single-step kernels (strips of 32*vec
+// columns) and two or three on the fused walk (lbm_fused.cuh).  In lockstep the resident
+// warps take a pass's tiles in list order from an atomic counter.  Within a pass tiles are
+// independent (each reads its grid's input buffer and writes the other one); between
+// passes every block waits at a barrier, because a tile reaches two rows and columns a
+// step into its neighbours and its store overwrites what they read one pass earlier.
 //
 // Every barrier wait is bounded (wall-clock limit read from %globaltimer): a
 // block that gives up sets a status word and returns, all other blocks see the
@@ -726,14 +727,15 @@ __global__ void __launch_bounds__(32 * kBatchWarps, PD == 2 ? 3 : 4)
     }
 }
 
-// The same for grids on the fused walk: a pass takes several steps of every grid
-// that has them left, and the rest of a grid's steps at its end.  Bound as
+// The same for grids on the fused walk: a pass takes several steps of every grid that
+// has them left, and the rest of a grid's steps at its end.  Bound as
 // k_step_fused is, at its occupancy and two rows of copies in flight; a half or a
 // third as many barriers as single steps.  Measured, lockstep, 100 steps a call,
 // single steps before and passes now: nine 2048^2 grids FP32 93k -> 187k MLUPS, FP16
 // 170k -> 241k, BF16 with stochastic rounding 168k -> 216k, FP32 with a c2 field 85k
 // -> 168k; 512 uneven grids FP32 93k -> 178k, FP16 159k -> 229k, half and half 115k
-// -> 191k.  Flow schedule: nine 2048^2 FP32 92k -> 174k, FP16 168k -> 237k; 512 uneven,
+// -> 191k.  (The loop over tiles costs the 16-bit kernels registers: they spill 40
+// bytes with nearest rounding and 8 with stochastic, k_step_fused none.)  Flow schedule: nine 2048^2 FP32 92k -> 174k, FP16 168k -> 237k; 512 uneven,
 // half and half, 83k -> 145k.
 template <int S, int RND, int VA, int TS>
 __global__ void __launch_bounds__(32 * kBatchWarps, 2)

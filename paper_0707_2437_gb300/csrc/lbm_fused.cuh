@@ -7,8 +7,8 @@
 // density), T steps reach 2 T, which the halo lanes' columns cover (one lane a
 // side for T = 2, two for FP32's T = 3), so the strip needs no other halo work:
 // every shuffle stays inside the warp, and what the outer lanes compute from their
-// missing neighbours reaches no stored site.  Columns wrap lane by lane, so nx must
-// be a multiple of V.
+// missing neighbours reaches no stored site.  Columns wrap lane by lane where nx is a
+// multiple of V, and 4-byte word by word where it is not (RAG below).
 //
 // Down the rows the walk is a pipeline of T stages.  Each iteration takes a row of
 // stored values, copied ahead into shared memory (cp.async), and for each stage
@@ -120,8 +120,9 @@ constexpr int fused_most_rows(int storage, int steps) {
     return storage == ST_F32 && steps == 2 ? 64 : 512;
 }
 
-// The strips of nx columns (a multiple of fused_vec where tiles are packed).  Packing saves walks of mostly
-// idle lanes, which pays in the 16-bit kinds, bound by issue: FP16 4096^2 76.2 -> 71.8
+// The strips of nx columns (a multiple of fused_vec where tiles are packed).  Packing
+// saves walks of mostly idle lanes, which pays in the 16-bit kinds, bound by issue: FP16
+// 4096^2 76.2 -> 71.8
 // us a step, 8192^2 279 -> 272, 512 uneven FP16 grids in a batch 209k -> 229k MLUPS.
 // FP32 passes are bound by memory and gain nothing (2048^2 with three steps 26.3 /
 // 26.4 us; 512 uneven grids 178k / 174k), and as the lanes of a packed tile read and

@@ -86,9 +86,10 @@ struct FusedStrips {
     }
 };
 // Several steps per launch (lbm_step_fused.cu): the tiles of a grid's passes, and
-// one launch of 1 .. p.steps steps.  ok is false where the fused walk does not apply
-// (nx not a multiple of its 16-byte lanes) or single steps are the faster.  Uniform
-// alpha with either rounding, or a c2 field with nearest rounding.
+// one launch of 1 .. p.steps steps.  ok is false where the fused walk does not apply (odd
+// 16-bit widths; with a c2 field widths that are no multiple of its 16-byte lanes) or
+// single steps are estimated to be the faster.  Uniform alpha with either rounding, or a
+// c2 field with nearest rounding.
 struct FusedPlan {
     bool ok = false;
     int steps = 1;  // of a pass

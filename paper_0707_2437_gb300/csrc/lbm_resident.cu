@@ -11,8 +11,10 @@ namespace {
 struct Shape {
     int threads, rows;
 };
-// Block shapes: at most `threads` threads of `rows` rows each, none of which spills
-// registers; the order is that of the kernels (resident_of).
+// Block shapes: at most `threads` threads of `rows` rows each, as many rows as their
+// registers hold: no kernel spills but FP32 768 x 3 without and 384 x 10 with a field (4
+// and 20 bytes), FP16 384 x 10 with a field (16) and BF16 384 x 10 (4 to 44).  The order
+// is that of the kernels (resident_of).
 constexpr Shape kShapes[] = {{512, 1}, {512, 2}, {768, 2}, {768, 3}, {640, 4}, {512, 6}, {384, 10}};
 constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
 
